@@ -93,7 +93,8 @@ typedef struct {
  *                      signature compare); results are identical in both modes
  *   validate           1: check offsets and ids on the device before refining
  *   small_task_vertices vertices each warp of the small-vertex kernel takes per task
- *                      (tile size); 0 -> default 128, else 32..65536
+ *                      (tile size); 0 -> default 128, fewer for graphs too small
+ *                      to give every SM work with that; else 32..65536
  *   hub_chunk_edges    edges of one hub that one CTA dedups in shared memory before
  *                      merging into the hub's global set (tile size of the hub
  *                      path); 0 -> default 512, else 256, 512 or 1024

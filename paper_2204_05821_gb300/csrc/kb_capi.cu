@@ -136,7 +136,7 @@ struct Plan {
     int hub_chunk = kb::kDefaultHubChunk;
     int med_split = kb::kDefaultMedSplit;
     int small_max = kb::kSmallDegree;
-    int warp_verts = kb::kDefaultWarpVerts;
+    int warp_verts = 0;  // 0: by the graph's size (launch_small_round)
     int32_t size_class = 0;  // key of the tuning cache
     uint64_t cap = 0;
     bool reorder = false;  // locality order of the gather (RoundParams::perm)
@@ -421,7 +421,7 @@ void resolve_call_fields(Plan& P, const kb_options* opt, int rounds, bool multi,
     P.freeze = (rounds >= 0 || multi) && P.subject == KB_SUBJECT_PREVIOUS && opt->rekey_all == 0;
     P.dense0 = !multi;
     P.med_split = pick_field(opt->medium_split, T ? T->medium_split : 0, kb::kDefaultMedSplit);
-    P.warp_verts = pick_field(opt->small_task_vertices, T ? T->small_task_vertices : 0, kb::kDefaultWarpVerts);
+    P.warp_verts = pick_field(opt->small_task_vertices, T ? T->small_task_vertices : 0, 0);
     float lf = opt->load_factor > 0.f ? opt->load_factor : (T ? T->load_factor : 0.f);
     if (!(lf > 0.f)) lf = 0.5f;
     P.cap = table_capacity(P.n, lf);
@@ -809,7 +809,7 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
     if (dense) {
         kb::launch_dense_level0(R.p, key, R.dense_min, R.dense_pair, R.prefix, R.scan_tmp, out, s);
     } else {
-        kb::launch_small_round(R.p, true, false, s);
+        kb::launch_small_round(R.p, true, kb::SmallWindows::kConsecutive, s);
         kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, s);
     }
     // a starting level may mix edgeless vertices with others in one block:
@@ -837,15 +837,10 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
     if (hub && !p.frozen && R.set_bytes) KB_CUDA(ctx, cudaMemsetAsync(p.hub_sets, 0xff, R.set_bytes, s));
     if (T) T->end();
     if (T) T->begin(KB_KERNEL_SMALL);
-    if (R.sparse) {
-        // few vertices refine: long warp tasks, so that far fewer CTAs set up
-        // and flush a join map for a handful of vertices each
-        kb::RoundParams q = p;
-        q.warp_verts = 4096;
-        kb::launch_small_round(q, false, true, s);
-    } else {
-        kb::launch_small_round(p, false, R.compact, s);
-    }
+    kb::launch_small_round(p, false,
+                           R.sparse ? kb::SmallWindows::kSparse
+                                    : (R.compact ? kb::SmallWindows::kCompact : kb::SmallWindows::kConsecutive),
+                           s);
     if (T) T->end();
     if (med) {
         if (T) T->begin(KB_KERNEL_MEDIUM);
@@ -2447,13 +2442,22 @@ kb_status kb_autotune(kb_context* ctx, const kb_graph* g, const int64_t* voff, i
     const int32_t cls = size_class(m_proc, batch ? G : 1, batch);
 
     // every tuning field explicit, so no cached tuning is consulted while timing
+    // (the warp task size starts at 0, by the graph's size, so the cache is set
+    // aside meanwhile)
+    struct CacheAside {
+        kb_context* ctx;
+        std::map<int32_t, kb_tuning> kept;
+        explicit CacheAside(kb_context* c) : ctx(c) { kept.swap(ctx->tuned); }
+        ~CacheAside() { ctx->tuned.swap(kept); }
+    };
+    std::unique_ptr<CacheAside> aside(new CacheAside(ctx));
     kb_options base = *opt;
     base.early_stop = 0;
     base.validate = 0;
     kb_options dflt = base;
     dflt.load_factor = 0.5f;
     dflt.hub_threshold = kb::kDefaultHubThreshold;
-    dflt.small_task_vertices = kb::kDefaultWarpVerts;
+    dflt.small_task_vertices = 0;
     dflt.hub_chunk_edges = kb::kDefaultHubChunk;
     dflt.medium_split = kb::kDefaultMedSplit;
     dflt.small_max_degree = kb::kSmallDegree;
@@ -2530,7 +2534,9 @@ kb_status kb_autotune(kb_context* ctx, const kb_graph* g, const int64_t* voff, i
     T.ms = best;
     T.default_ms = default_ms;
     T.size_class = cls;
+    aside.reset();
     ctx->tuned[cls] = T;
+    if (T.small_task_vertices == 0) T.small_task_vertices = kb::kDefaultWarpVerts;  // the default, as a value
     if (out) *out = T;
     return KB_OK;
 }

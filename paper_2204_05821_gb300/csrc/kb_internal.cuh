@@ -102,7 +102,7 @@ struct RoundParams {
     uint32_t* moved;
     int32_t hub_threshold;
     int32_t small_max;    // largest degree of the small-vertex kernel (<= kSmallDegree, <= hub_threshold)
-    int32_t warp_verts;   // vertices per warp task of the small-vertex kernel
+    int32_t warp_verts;   // vertices per warp task of the small-vertex kernel; 0: by the graph's size
     int32_t hub_chunk;    // edges per hub-chunk CTA: 256, 512 or 1024
     int32_t med_split;    // medium vertices up to this degree take a warp, larger a CTA (1..kMaxMedSplit)
     int32_t hash_mode;
@@ -247,9 +247,10 @@ void launch_round_work(const RoundParams& p, cudaStream_t s);
 void launch_count_refining(const RoundParams& p, const uint32_t* frozen, Counters* ctr, cudaStream_t s);
 // Bit v set iff v has no edges in the processed CSR.
 void launch_edgeless_bits(int64_t n, const int64_t* row, uint32_t* bits, cudaStream_t s);
-// compact: windows are packed from the vertices that refine (worth it when
-// many are frozen), else from consecutive vertices.
-void launch_small_round(const RoundParams& p, bool level0, bool compact, cudaStream_t s);
+// Windows of consecutive vertices, or packed from the vertices that refine
+// (kCompact: worth it when many are frozen; kSparse: nearly all are).
+enum class SmallWindows { kConsecutive, kCompact, kSparse };
+void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s);
 void launch_medium_round(const RoundParams& p, cudaStream_t s);  // kb_medium.cu
 // Per-device kernel attributes (shared-memory carveouts); call once per device
 // before the first launch and outside any stream capture.

@@ -17,6 +17,8 @@
 //      vertices -- are skipped by steps 1-2 there and keep their minima.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kb_device.cuh"
 #include "kb_internal.cuh"
 
@@ -818,13 +820,13 @@ __global__ void edgeless_bits_kernel(int64_t n, const int64_t* row, uint32_t* bi
 constexpr int kClearTile = 65536;
 constexpr int kClearHubs = kClearTile / 64 + 1;
 
-__global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p) {
+__global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p, int64_t tile) {
     __shared__ int s_h0;
     __shared__ int64_t s_end[kClearHubs];
     __shared__ uint8_t s_ref[kClearHubs];
     const int64_t total = p.hub_set_off[p.n_hubs];
-    const int64_t t0 = (int64_t)blockIdx.x * kClearTile;
-    const int64_t t1 = min(total, t0 + kClearTile);
+    const int64_t t0 = (int64_t)blockIdx.x * tile;
+    const int64_t t1 = min(total, t0 + tile);
     if (threadIdx.x == 0) {
         int lo = 0, hi = p.n_hubs - 1;  // first hub whose set ends after t0
         while (lo < hi) {
@@ -1036,7 +1038,11 @@ void launch_clear_round(const RoundParams& p, cudaStream_t s) {
 
 void launch_clear_hub_sets(const RoundParams& p, int64_t total_slots, cudaStream_t s) {
     if (p.n_hubs <= 0 || total_slots <= 0) return;
-    clear_hub_sets_kernel<<<(unsigned)((total_slots + kClearTile - 1) / kClearTile), 256, 0, s>>>(p);
+    // short tiles while the sets are small, so that every SM stores (18 us for
+    // 3 x 10^5 slots in tiles of 65536, 5 us in tiles of 2048)
+    const int64_t per = total_slots / (152 * 8);
+    const int64_t tile = std::min<int64_t>(kClearTile, std::max<int64_t>(2048, (per + 1023) & ~(int64_t)1023));
+    clear_hub_sets_kernel<<<(unsigned)((total_slots + tile - 1) / tile), 256, 0, s>>>(p, tile);
 }
 
 void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,

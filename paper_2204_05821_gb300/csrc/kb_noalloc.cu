@@ -170,7 +170,7 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     if (host_cnts[1] > 0) return KB_ERR_INVALID_ARG;  // a degree outside [0, hub threshold]
     p.n_med = host_cnts[0];
 
-    kb::launch_small_round(p, false, false, s);
+    kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
     kb::launch_medium_round(p, s);
     kb::launch_renumber(p, reinterpret_cast<uint2*>(base + kOffPrefix), reinterpret_cast<uint32_t*>(base + kOffScan),
                         out, s);

@@ -26,6 +26,8 @@
 // aggregation leaves the result unchanged.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "kb_device.cuh"
 #include "kb_internal.cuh"
 
@@ -37,6 +39,7 @@ constexpr int kSmallThreads = 256;
 #define KB_SMALL_MIN_BLOCKS 6  // caps registers at 40: 48 warps per SM (a few bytes spill)
 #endif
 constexpr int kSmallWarps = kSmallThreads / 32;
+constexpr int64_t kResidentWarps = 152 * KB_SMALL_MIN_BLOCKS * kSmallWarps;  // warps the chip holds at once
 // Joins a CTA can aggregate (1 x its vertices at the default task size; a
 // join that finds no room goes to global memory at once).  The map is kept
 // small on purpose: shared memory comes out of the SM's L1, and the L1 also
@@ -413,9 +416,29 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
 
 }  // namespace
 
-void launch_small_round(const RoundParams& p, bool level0, bool compact, cudaStream_t s) {
+// Vertices per warp task when the caller gives none: the vertices spread over
+// two waves of resident warps, between lo and hi.  A warp walks its task window
+// after window, each a chain of dependent loads (offsets, neighbours, blocks,
+// table, representative), so a graph that fills only part of the chip with
+// tasks of 128 is bound by the length of that chain: one round of 10^4 vertices
+// and 5 x 10^4 edges took 104 us with tasks of 128 (10 CTAs) and 18 us with
+// tasks of 8.  From about 1.9 x 10^6 vertices on every task has 128.  One and
+// four waves measured the same, except one wave at 10^6 vertices (2374 -> 2522
+// us for a whole backward refinement: its second, nearly empty wave).
+static int64_t task_vertices(int64_t n, int64_t lo, int64_t hi) {
+    const int64_t per = (n + 2 * kResidentWarps - 1) / (2 * kResidentWarps);
+    return std::min(hi, std::max(lo, (per + 7) & ~(int64_t)7));
+}
+
+void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s) {
     if (p.n <= 0) return;
-    const int64_t wv = p.warp_verts > 0 ? p.warp_verts : kDefaultWarpVerts;
+    const bool compact = windows != SmallWindows::kConsecutive;
+    // consecutive windows hold about six vertices (32 edges), packed and
+    // level-0 windows up to 32
+    int64_t wv = p.warp_verts > 0 ? p.warp_verts : task_vertices(p.n, (level0 || compact) ? 32 : 8, kDefaultWarpVerts);
+    // few vertices refine: long warp tasks, so that far fewer CTAs set up and
+    // flush a join map for a handful of vertices each
+    if (windows == SmallWindows::kSparse) wv = task_vertices(p.n, kDefaultWarpVerts, 4096);
     const int64_t per_cta = wv * kSmallWarps;
     const int64_t blocks = (p.n + per_cta - 1) / per_cta;
     RoundParams q = p;
