@@ -162,7 +162,7 @@ struct Plan {
     size_t csr_bytes = 0;
     size_t o_emin = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
-           o_frozen = 0, o_fmin = 0, o_edgeless = 0, o_shared = 0, o_minof = 0, o_bm2 = 0, o_moved = 0, o_mark = 0,
+           o_frozen = 0, o_fmin = 0, o_edgeless = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0,
            o_dense = 0;
     size_t total = 0;
 };
@@ -249,6 +249,7 @@ void layout_round(Plan& P) {
     P.o_fmin = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_shared = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_minof = take(own_freeze ? sizeof(uint32_t) * (size_t)P.n : 0);
+    P.o_joined = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_bm2 = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_moved = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_mark = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
@@ -751,6 +752,8 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         R.bm[0] = p.bitmap;
         R.bm[1] = reinterpret_cast<uint32_t*>(ws + P.o_bm2);
         R.bm_cur = 0;
+        p.joined = reinterpret_cast<uint32_t*>(ws + P.o_joined);  // all clear between rounds
+        KB_CUDA(ctx, cudaMemsetAsync(p.joined, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
         if (R.ext_frozen) {
             // the caller's state, kept as it is
             R.frozen = R.ext_frozen;

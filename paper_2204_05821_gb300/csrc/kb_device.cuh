@@ -22,16 +22,37 @@ __device__ __forceinline__ void toggle_min(uint32_t* bitmap, uint32_t v) {
     atomicXor(&bitmap[v >> 5], 1u << (v & 31));
 }
 
-// Join slot `pos` (same epoch and tag as ours) with vertex v.
-__device__ __forceinline__ void join_slot(const RoundParams& p, uint64_t pos, uint32_t hi, uint32_t v) {
-    const uint64_t want = ((uint64_t)hi << 32) | v;
-    const uint64_t old = atomicMin(reinterpret_cast<unsigned long long*>(&p.table[pos]),
-                                   (unsigned long long)want);
-    const uint32_t prev_min = (uint32_t)old;
-    if (v < prev_min) {
+// A table entry's low word holds the smallest member of its block so far; the
+// bit above it is set while the block has only the vertex that inserted it.
+constexpr uint32_t kSingleBit = 0x80000000u;
+constexpr uint32_t kVertexMask = 0x7fffffffu;
+
+// Lower the smallest member of slot `pos` (same epoch and tag as ours) to v.
+// A block's minimum only decreases during a round, so an entry that another
+// vertex joined already and whose minimum is at or below v needs no atomic:
+// hot keys would otherwise take one serialised atomic per join.  The one join
+// that finds the entry single records its inserter in p.joined: the
+// renumbering turns that bit into the mark of the block's minimum, one atomic
+// per shared block (marks sent by every other member, through a cache per
+// CTA, were most of the renumbering: 450 -> 260 us in round 1 of the 2 x 10^8
+// edge graph, 283 -> 99 us with 10^8 edges and one label class).
+__device__ __forceinline__ void join_block(const RoundParams& p, uint64_t pos, uint32_t hi, uint32_t v) {
+    const uint32_t seen = (uint32_t)volatile_load(&p.table[pos]);
+    if (seen <= v) return;  // the single bit is above every vertex
+    const uint32_t want = min(v, seen & kVertexMask);
+    const uint32_t old = (uint32_t)atomicMin(reinterpret_cast<unsigned long long*>(&p.table[pos]),
+                                             (unsigned long long)(((uint64_t)hi << 32) | want));
+    const uint32_t prev_min = old & kVertexMask;
+    if ((old & kSingleBit) && p.joined) atomicOr(&p.joined[prev_min >> 5], 1u << (prev_min & 31));
+    if (want < prev_min) {
         toggle_min(p.bitmap, v);
         toggle_min(p.bitmap, prev_min);
     }
+}
+
+// Vertex v joins slot `pos`.
+__device__ __forceinline__ void join_slot(const RoundParams& p, uint64_t pos, uint32_t hi, uint32_t v) {
+    join_block(p, pos, hi, v);
     p.slot_of[v] = (int32_t)pos;
 }
 
@@ -61,22 +82,6 @@ __device__ __forceinline__ bool same_graph(const RoundParams& p, int64_t a, int6
     return !p.vgraph || p.vgraph[a] == p.vgraph[b];
 }
 
-// A vertex without edges in the processed direction has the key (own block,
-// empty set): it is grouped by its own block exactly, without hashing or a
-// signature compare.  emin[own] keeps the smallest such vertex of this round;
-// entries of earlier rounds carry a larger high word and lose every atomicMin.
-__device__ __forceinline__ void join_empty(const RoundParams& p, int32_t own, uint32_t v) {
-    const uint64_t want = ((uint64_t)p.ehigh << 32) | v;
-    const uint64_t old = atomicMin(reinterpret_cast<unsigned long long*>(&p.emin[own]), (unsigned long long)want);
-    if ((uint32_t)(old >> 32) != p.ehigh) {
-        toggle_min(p.bitmap, v);
-    } else if (v < (uint32_t)old) {
-        toggle_min(p.bitmap, v);
-        toggle_min(p.bitmap, (uint32_t)old);
-    }
-    p.slot_of[v] = (int32_t)(0x80000000u | (uint32_t)own);
-}
-
 // Probe the block table from *pos.  Returns 0 when v inserted a new key,
 // 1 with *rep set when a slot with our tag was found (a signature compare
 // decides), 2 when the probe limit was hit.
@@ -86,7 +91,7 @@ __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_i
     for (int it = 0; it < kProbeLimit; ++it) {
         uint64_t cur = volatile_load(&p.table[pos]);
         if ((uint32_t)(cur >> 56) != p.epoch) {
-            const uint64_t want = ((uint64_t)hi << 32) | v;
+            const uint64_t want = ((uint64_t)hi << 32) | kSingleBit | v;
             const uint64_t old = atomicCAS(reinterpret_cast<unsigned long long*>(&p.table[pos]),
                                            (unsigned long long)cur, (unsigned long long)want);
             if (old == cur) {
@@ -99,7 +104,7 @@ __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_i
             if ((uint32_t)(cur >> 56) != p.epoch) continue;
         }
         if ((uint32_t)(cur >> 32) == hi) {
-            *rep = (uint32_t)cur;
+            *rep = (uint32_t)cur & kVertexMask;
             *pos_io = pos;
             return 1;
         }

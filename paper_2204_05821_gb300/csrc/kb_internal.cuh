@@ -86,11 +86,15 @@ struct RoundParams {
     // the round kernels; frozen_min holds the minima of frozen blocks and
     // starts the round's bitmap of minima; a skipped vertex that is not a
     // minimum keeps its slot_of entry of the round that formed its block.  The
-    // renumbering sets bit b of shared for every block minimum b that another
-    // vertex points to.  All nullptr when every vertex is re-keyed.
+    // renumbering sets bit b of shared for the minimum b of every block of
+    // several vertices (blocks of edgeless vertices aside: those are frozen
+    // whatever their size), from joined: bit v for the vertex v that inserted
+    // the table entry of such a block, set by the round kernels and cleared by
+    // the renumbering.  All nullptr when every vertex is re-keyed.
     const uint32_t* frozen;
     const uint32_t* frozen_min;
     uint32_t* shared;
+    uint32_t* joined;
     // Clean blocks (with frozen blocks).  minof[v] is the smallest member of
     // v's block whenever v is not that member; the renumbering writes it for
     // every re-keyed vertex, and a frozen vertex keeps it.  moved (when set)
@@ -268,7 +272,7 @@ size_t scan_tmp_words(int64_t n_items);
 // are all in [0, kDenseLabels): the label partition straight from each
 // label's smallest vertex, without the block table.  launch_dense_labels
 // lowers lmin[label] (all ones for an unused label) to the label's smallest
-// vertex and sets ctr->dense_bad if some key lies outside the range (the
+// vertex (bit 31 set while it is the label's only one) and sets ctr->dense_bad if some key lies outside the range (the
 // caller then takes the general path).  launch_dense_level0 then writes what
 // the general level-0 pass writes: the minima bitmap and the shared-block
 // marks of p, the rank words, ctr->count, the level (out), minof and the

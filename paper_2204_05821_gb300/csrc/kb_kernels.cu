@@ -408,23 +408,17 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
     }
 }
 
-// Shared-block marks (RoundParams::shared) go through a small direct-mapped
-// cache of the minima this CTA marked already: a block with millions of
-// members (all edgeless vertices with one label) would otherwise send one
-// atomic per member to a single word.
-constexpr int kMarkCache = 1024;
-constexpr uint32_t kNoMark = 0xffffffffu;
+// The smallest member of v's block when v is not that member.
+__device__ __forceinline__ uint32_t block_min(const RoundParams& p, int64_t v) {
+    const uint32_t sl = (uint32_t)p.slot_of[v];
+    if (sl & 0x80000000u) return (uint32_t)p.emin[(sl & 0x7fffffffu) % (uint32_t)p.n];
+    return (uint32_t)p.table[(uint64_t)sl & p.mask] & kVertexMask;
+}
 
 __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const uint2* rank, int32_t* out) {
-    __shared__ uint32_t s_mark[kMarkCache];
-    if (p.shared) {
-        for (int i = threadIdx.x; i < kMarkCache; i += blockDim.x) s_mark[i] = kNoMark;
-        __syncthreads();
-    }
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < p.n; v += stride) {
         uint32_t mn = (uint32_t)v;
-        uint32_t mark = kNoMark;
         if (!vertex_active(p, v)) {
             if (!p.vmask) {  // a batched graph that stopped: its ids shift with the graphs before it
                 // (batched runs never use the locality order)
@@ -435,33 +429,13 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
             mn = p.kmin[p.keep_old[v]];  // incremental: the smallest kept member of its old block
             if ((int64_t)mn >= p.n) mn = (uint32_t)v;
         } else if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
-            const uint32_t sl = (uint32_t)p.slot_of[v];
-            if (sl & 0x80000000u)
-                mn = (uint32_t)p.emin[(sl & 0x7fffffffu) % (uint32_t)p.n];
-            else
-                mn = (uint32_t)(p.table[(uint64_t)sl & p.mask] & 0xffffffffu);
+            mn = block_min(p, v);
             if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
-            mark = mn;  // v is not the minimum: its block has another member
         }
         const uint2 rw = rank[mn >> 5];
         const int32_t b = (int32_t)(rw.x + __popc(rw.y & ((1u << (mn & 31)) - 1u)));
         out[v] = b;
         if (p.perm) p.gat[p.perm[v]] = (int32_t)mn;  // the block by its smallest member
-        if (p.shared) {
-            // one lane per distinct minimum in the warp, then the CTA's cache,
-            // then an L2 read: an atomic on a bit already set costs far more
-            // than the read (batched and incremental runs, which leave the
-            // loop early above, have no shared marks)
-            const unsigned grp = __match_any_sync(__activemask(), mark);
-            if (mark != kNoMark && (int)(threadIdx.x & 31) == __ffs(grp) - 1) {
-                const uint32_t c = (mark * 2654435761u) >> 22;
-                if (s_mark[c] != mark) {
-                    s_mark[c] = mark;
-                    const uint32_t bit = 1u << (mark & 31);
-                    if (!(__ldcg(p.shared + (mark >> 5)) & bit)) atomicOr(&p.shared[mark >> 5], bit);
-                }
-            }
-        }
     }
 }
 
@@ -490,21 +464,19 @@ __global__ void __launch_bounds__(256) stable_copy_kernel(const RoundParams p, i
 // vertices whose smallest block member changed: v itself or minof[v] at the
 // previous level, read before minof[v] is rewritten) leave as one word per
 // warp.  Frozen vertices keep minof, and their blocks keep their shared marks
-// (the freeze pass carries them over), so only re-keyed vertices mark.  moved
-// may be null (the starting level).
+// (the freeze pass carries them over); the mark of a re-keyed block comes from
+// the vertex that inserted its table entry (RoundParams::joined).  moved may be
+// null (the starting level).
 __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p, const uint2* rank, int32_t* out,
                                                              uint32_t* moved, int64_t stable_count) {
-    __shared__ uint32_t s_mark[kMarkCache];
     // a round that kept the block count is copied by stable_copy_kernel
     if (stable_count >= 0 && p.ctr->count == stable_count) return;
-    for (int i = threadIdx.x; i < kMarkCache; i += blockDim.x) s_mark[i] = kNoMark;
-    __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < p.n; base += stride) {
         const int64_t v = base + lane;
         bool mv = false;
-        uint32_t mark = kNoMark;
+        const uint32_t joined = p.joined[base >> 5];
         if (v < p.n && !vertex_active(p, v)) {
             // a batched graph that stopped: its ids shift with the graphs before it
             const int32_t g = p.vgraph[v];
@@ -513,21 +485,11 @@ __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p,
             const bool fz = vertex_frozen(p, v);
             uint32_t mn = (uint32_t)v;
             if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
-                if (fz) {
-                    mn = p.minof[v];  // a frozen block keeps its members and smallest member
-                } else {
-                    const uint32_t sl = (uint32_t)p.slot_of[v];
-                    if (sl & 0x80000000u)
-                        mn = (uint32_t)p.emin[(sl & 0x7fffffffu) % (uint32_t)p.n];
-                    else
-                        mn = (uint32_t)(p.table[(uint64_t)sl & p.mask] & 0xffffffffu);
-                    mark = mn;  // v is not the minimum: its block has another member
-                }
-                if ((int64_t)mn >= p.n) {  // only after a reported device error
-                    mn = (uint32_t)v;
-                    mark = kNoMark;
-                }
+                // a frozen block keeps its members and smallest member
+                mn = fz ? p.minof[v] : block_min(p, v);
+                if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
             }
+            if ((joined >> lane) & 1u) atomicOr(&p.shared[mn >> 5], 1u << (mn & 31));
             const uint2 rw = rank[mn >> 5];
             const int32_t b = (int32_t)(rw.x + __popc(rw.y & ((1u << (mn & 31)) - 1u)));
             out[v] = b;
@@ -546,17 +508,9 @@ __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p,
                 if (mn != (uint32_t)v) p.minof[v] = mn;
             }
         }
-        // one lane per distinct minimum in the warp, then the CTA's cache,
-        // then an L2 read: an atomic on a bit already set costs far more
-        // than the read
-        const unsigned grp = __match_any_sync(kFull, mark);
-        if (mark != kNoMark && lane == __ffs(grp) - 1) {
-            const uint32_t c = (mark * 2654435761u) >> 22;
-            if (s_mark[c] != mark) {
-                s_mark[c] = mark;
-                const uint32_t bit = 1u << (mark & 31);
-                if (!(__ldcg(p.shared + (mark >> 5)) & bit)) atomicOr(&p.shared[mark >> 5], bit);
-            }
+        if (joined) {  // read by every lane above
+            __syncwarp();
+            if (lane == 0) p.joined[base >> 5] = 0u;
         }
         if (moved) {
             const unsigned w = __ballot_sync(kFull, mv);
@@ -854,24 +808,39 @@ __global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p
 }
 
 // ----------------------------------------------------------------------------
-// Level 0 over small labels.  A shared minimum is read before the atomicMin
-// that would lower it: after a label's first members, a CTA's later (larger)
-// vertices leave its minimum alone.
+// Level 0 over small labels.  A label's entry is its smallest vertex so far,
+// with kSingleBit while it has only that one (all ones: none yet).  A shared
+// entry is read before the atomicMin that would lower it: after a label's first
+// members, a CTA's later (larger) vertices leave it alone.  Knowing here which
+// labels have several members saves the assignment its marks of shared blocks
+// (one atomic per label and CTA on the few words that hold the labels' smallest
+// vertices): 171 -> 13 us for it at 2.5 x 10^6 vertices, 569 -> 113 us at
+// 2 x 10^7 with the locality order (the minima pass itself 21 -> 31 us).
 // ----------------------------------------------------------------------------
 constexpr int kDenseThreads = 512;
+
+constexpr uint32_t kNoMember = 0xffffffffu;
+
+// Lower an entry to `member`: a vertex, with kSingleBit when it is the only one
+// its side has seen.
+__device__ __forceinline__ void see_member(uint32_t* entry, uint32_t member) {
+    const uint32_t old = atomicMin(entry, member);
+    if (old != kNoMember && ((member | old) & kSingleBit))  // several members together: the entry loses the bit
+        atomicMin(entry, min(member & kVertexMask, old & kVertexMask));
+}
 
 __device__ __forceinline__ void see_label(uint32_t* s_min, int64_t v, int32_t l, bool& bad) {
     if ((uint32_t)l >= (uint32_t)kDenseLabels) {
         bad = true;
         return;
     }
-    if ((uint32_t)v < s_min[l]) atomicMin(&s_min[l], (uint32_t)v);
+    if (s_min[l] > (uint32_t)v) see_member(&s_min[l], (uint32_t)v | kSingleBit);
 }
 
 __global__ void __launch_bounds__(kDenseThreads) dense_label_min_kernel(int64_t n, const int32_t* key, uint32_t* lmin,
                                                                          Counters* ctr) {
     __shared__ uint32_t s_min[kDenseLabels];
-    for (int i = threadIdx.x; i < kDenseLabels; i += blockDim.x) s_min[i] = 0xffffffffu;
+    for (int i = threadIdx.x; i < kDenseLabels; i += blockDim.x) s_min[i] = kNoMember;
     __syncthreads();
     bool bad = false;
     const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -893,38 +862,38 @@ __global__ void __launch_bounds__(kDenseThreads) dense_label_min_kernel(int64_t 
     if (bad) atomicOr(&ctr->dense_bad, 1);
     __syncthreads();
     for (int i = threadIdx.x; i < kDenseLabels; i += blockDim.x)
-        if (s_min[i] != 0xffffffffu) atomicMin(&lmin[i], s_min[i]);
+        if (s_min[i] != kNoMember && __ldcg(lmin + i) > (s_min[i] & kVertexMask)) see_member(&lmin[i], s_min[i]);
 }
 
-// Every used label's smallest vertex is a block minimum.
+// Every used label's smallest vertex is a block minimum, marked as shared when
+// the label has other members.
 __global__ void dense_mark_kernel(const RoundParams p, const uint32_t* lmin) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= kDenseLabels) return;
-    const uint32_t m = lmin[l];
-    if (m != 0xffffffffu) atomicOr(&p.bitmap[m >> 5], 1u << (m & 31));
+    const uint32_t e = lmin[l];
+    if (e == kNoMember) return;
+    const uint32_t m = e & kVertexMask;
+    atomicOr(&p.bitmap[m >> 5], 1u << (m & 31));
+    if (p.shared && !(e & kSingleBit)) atomicOr(&p.shared[m >> 5], 1u << (m & 31));
 }
 
 // (smallest vertex, canonical id) of every used label
 __global__ void dense_ids_kernel(const uint32_t* lmin, const uint2* rank, uint2* lpair) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= kDenseLabels) return;
-    const uint32_t m = lmin[l];
+    const uint32_t m = lmin[l] & kVertexMask;
     uint32_t id = 0u;
-    if (m != 0xffffffffu) {
+    if (lmin[l] != kNoMember) {
         const uint2 rw = rank[m >> 5];
         id = rw.x + __popc(rw.y & ((1u << (m & 31)) - 1u));
     }
     lpair[l] = make_uint2(m, id);
 }
 
-// The level, minof, the locality order's copy and the shared-block marks (a
-// block is shared when a vertex other than its smallest member has its label;
-// each CTA marks a label once).  The 64 KB label table stays in L1.
+// The level, minof and the locality order's copy.  The 64 KB label table stays
+// in L1.
 __global__ void __launch_bounds__(256) dense_assign_kernel(const RoundParams p, const int32_t* key,
                                                            const uint2* lpair, int32_t* out) {
-    __shared__ uint32_t s_marked[kDenseLabels / 32];
-    for (int i = threadIdx.x; i < kDenseLabels / 32; i += blockDim.x) s_marked[i] = 0u;
-    __syncthreads();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < p.n; v += stride) {
         const uint32_t l = (uint32_t)__ldcs(key + v);
@@ -936,12 +905,7 @@ __global__ void __launch_bounds__(256) dense_assign_kernel(const RoundParams p, 
         const uint32_t mn = e.x;
         out[v] = (int32_t)e.y;
         if (p.perm) p.gat[p.perm[v]] = (int32_t)mn;  // the block by its smallest member
-        if (mn != (uint32_t)v) {
-            if (p.minof) p.minof[v] = mn;
-            const uint32_t bit = 1u << (l & 31);
-            if (p.shared && !(s_marked[l >> 5] & bit) && !(atomicOr(&s_marked[l >> 5], bit) & bit))
-                atomicOr(&p.shared[mn >> 5], 1u << (mn & 31));
-        }
+        if (mn != (uint32_t)v && p.minof) p.minof[v] = mn;
     }
 }
 

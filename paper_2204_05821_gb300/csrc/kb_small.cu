@@ -84,10 +84,10 @@ __device__ __forceinline__ bool map_join(JoinMap& M, uint64_t key, uint32_t hi, 
     return false;
 }
 
-// Global atomicMin of a CTA's smallest joining vertex, with minimum toggles.
-// A block's minimum only decreases during a round, so a read that finds it at
-// or below v makes the atomic (and its toggles) a no-op, and it is skipped:
-// hot keys would otherwise take one serialised atomic per CTA.
+// A CTA's smallest joining vertex of one key, with minimum toggles.  Edgeless
+// blocks (vertices with the key (own block, empty set), grouped by the own
+// block exactly) keep their smallest vertex of this round in emin[own]; entries
+// of earlier rounds carry a larger high word and lose every atomicMin.
 __device__ __forceinline__ void flush_join(const RoundParams& p, uint64_t key, uint32_t hi, uint32_t v) {
     if (key & kEmptyKeyBit) {
         const int32_t own = (int32_t)(uint32_t)key;
@@ -102,14 +102,7 @@ __device__ __forceinline__ void flush_join(const RoundParams& p, uint64_t key, u
             toggle_min(p.bitmap, (uint32_t)old);
         }
     } else {
-        const uint64_t want = ((uint64_t)hi << 32) | v;
-        const uint64_t seen = volatile_load(&p.table[key]);
-        if ((uint32_t)(seen >> 32) == hi && (uint32_t)seen <= v) return;  // minima only decrease
-        const uint64_t old = atomicMin(reinterpret_cast<unsigned long long*>(&p.table[key]), (unsigned long long)want);
-        if (v < (uint32_t)old) {
-            toggle_min(p.bitmap, v);
-            toggle_min(p.bitmap, (uint32_t)old);
-        }
+        join_block(p, key, hi, v);
     }
 }
 
