@@ -162,7 +162,7 @@ struct Plan {
     size_t csr_bytes = 0;
     size_t o_emin = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
-           o_frozen = 0, o_fmin = 0, o_edgeless = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0,
+           o_frozen = 0, o_edgeless = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0,
            o_dense = 0;
     size_t total = 0;
 };
@@ -246,7 +246,6 @@ void layout_round(Plan& P) {
     P.o_ownkey = take(P.subject ? sizeof(int32_t) * (size_t)P.n : 0);
     const bool own_freeze = P.freeze && !P.ext_freeze;
     P.o_frozen = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
-    P.o_fmin = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_shared = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_minof = take(own_freeze ? sizeof(uint32_t) * (size_t)P.n : 0);
     P.o_joined = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
@@ -540,6 +539,8 @@ struct Prepared {
     // (dirty) blocks; RoundParams::minof
     uint32_t* bm[2] = {nullptr, nullptr};
     int bm_cur = 0;
+    bool bitmap_ready = false;  // the next round's bitmap holds the minima of its frozen blocks (next_minima)
+    bool counters_clear = false;  // the round need not clear the counters (no errors so far; see launch_renumber)
     uint32_t* moved = nullptr;
     uint32_t* mark = nullptr;
     uint32_t* dense_min = nullptr;  // launch_dense_labels / launch_dense_level0 (Plan::dense0)
@@ -766,14 +767,14 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
             // nothing frozen before the starting level; shared starts empty
             const size_t bw = sizeof(uint32_t) * (size_t)((n >> 5) + 1);
             R.frozen = reinterpret_cast<uint32_t*>(ws + P.o_frozen);
-            R.frozen_min = reinterpret_cast<uint32_t*>(ws + P.o_fmin);
             p.shared = reinterpret_cast<uint32_t*>(ws + P.o_shared);
             p.minof = reinterpret_cast<uint32_t*>(ws + P.o_minof);
             R.moved = reinterpret_cast<uint32_t*>(ws + P.o_moved);
             R.mark = reinterpret_cast<uint32_t*>(ws + P.o_mark);
             KB_CUDA(ctx, cudaMemsetAsync(R.frozen, 0, bw, s));
-            KB_CUDA(ctx, cudaMemsetAsync(R.frozen_min, 0, bw, s));
             KB_CUDA(ctx, cudaMemsetAsync(p.shared, 0, bw, s));
+            // the locality order's moved bits are set one by one
+            if (P.reorder) KB_CUDA(ctx, cudaMemsetAsync(R.moved, 0, bw, s));
         }
         KB_CUDA(ctx, cudaGetLastError());
     }
@@ -790,6 +791,11 @@ kb_status next_epoch(kb_context* ctx, Prepared& R, cudaStream_t s) {
     R.p.epoch = ++R.epoch;
     return KB_OK;
 }
+
+// Where the minima of the next round's frozen blocks go: straight into the
+// bitmap that round builds its minima in (the server, which can admit and move
+// graphs in between, keeps them apart).
+uint32_t* next_minima(const Prepared& R) { return R.ext_frozen ? R.frozen_min : R.bm[R.bm_cur ^ 1]; }
 
 // Starting level: canonical renumbering of `key` (labels or a given
 // partition; all-zero partition when key is NULL in a batched run).
@@ -813,13 +819,14 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
         kb::launch_dense_level0(R.p, key, R.dense_min, R.dense_pair, R.prefix, R.scan_tmp, out, s);
     } else {
         kb::launch_small_round(R.p, true, kb::SmallWindows::kConsecutive, s);
-        kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, s);
+        kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, nullptr, s);
     }
     // a starting level may mix edgeless vertices with others in one block:
     // only its singletons are frozen in the first round
     if (R.p.shared) {
-        kb::launch_freeze_clean(R.p.n, R.p.bitmap, R.p.shared, nullptr, out, nullptr, R.frozen, R.frozen_min,
+        kb::launch_freeze_clean(R.p.n, R.p.bitmap, R.p.shared, nullptr, out, nullptr, R.frozen, next_minima(R), nullptr,
                                 ctx->d_ctr, s);
+        R.bitmap_ready = !R.ext_frozen;
         kb::launch_count_refining(R.p, R.frozen, ctx->d_ctr, s);
     }
     KB_CUDA(ctx, cudaGetLastError());
@@ -835,9 +842,9 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
     const bool med = p.n_med && (!p.frozen || R.med_on);
     const bool hub = p.n_hubs && (!p.frozen || R.hub_on);
     if (T) T->begin(KB_KERNEL_OTHER);
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-    kb::launch_clear_round(p, s);
-    if (hub && !p.frozen && R.set_bytes) KB_CUDA(ctx, cudaMemsetAsync(p.hub_sets, 0xff, R.set_bytes, s));
+    if (!R.counters_clear) KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
+    if (!R.bitmap_ready) kb::launch_clear_round(p, s);
+    R.bitmap_ready = false;
     if (T) T->end();
     if (T) T->begin(KB_KERNEL_SMALL);
     kb::launch_small_round(p, false,
@@ -852,7 +859,7 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
     }
     if (hub) {
         if (T) T->begin(KB_KERNEL_HUB_CHUNK);
-        if (p.frozen) kb::launch_clear_hub_sets(p, (int64_t)(R.set_bytes / sizeof(uint64_t)), s);
+        kb::launch_clear_hubs(p, (int64_t)(R.set_bytes / sizeof(uint64_t)), s);
         kb::launch_hub_chunk(p, R.total_chunks, s);
         if (T) T->end();
         if (T) T->begin(KB_KERNEL_HUB_FINAL);
@@ -883,10 +890,10 @@ struct LevelRows {
     int32_t* row(int i) const { return levels ? levels + (size_t)i * (size_t)n : ping[i & 1]; }
 };
 
-// Queue the device-to-host copy of rows first..last (final on ctx->stream).
+// Queue the device-to-host copy of rows first..last, final on ctx->stream since
+// ctx->row_ev was recorded.
 kb_status emit_rows(kb_context* ctx, const LevelRows& rows, int first, int last) {
     if (!rows.host || rows.n == 0 || last < first) return KB_OK;
-    KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, ctx->stream));
     KB_CUDA(ctx, cudaStreamWaitEvent(ctx->copy_stream, ctx->row_ev, 0));
     KB_CUDA(ctx, cudaMemcpyAsync(rows.host + (size_t)first * (size_t)rows.n, rows.row(first),
                                  sizeof(int32_t) * (size_t)rows.n * (size_t)(last - first + 1), cudaMemcpyDeviceToHost,
@@ -968,9 +975,11 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     }
     if (counts) counts[i_start] = prev_count;
     if (last_count) *last_count = prev_count;
+    if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
     KB_TRY(emit_rows(ctx, rows, i_start, i_start));
 
     // ---- refinement rounds
+    R.counters_clear = !ctx->work && !R.P.subject;
     for (int i = i_start + 1; i <= k; ++i) {
         Timer T(ctx);
         KB_TRY(next_epoch(ctx, R, s));
@@ -992,17 +1001,17 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         T.begin(KB_KERNEL_RENUMBER);
         // under early stop a round that keeps the count is the last one
         const int64_t stable = (opt->early_stop || fixpoint) && !R.P.subject ? prev_count : -1;
-        kb::launch_renumber(p, R.prefix, R.scan_tmp, out, s, stable);
-        KB_TRY(emit_rows(ctx, rows, i, i));
+        kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, s, stable);
+        if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
         // the next round's frozen blocks: singletons; a block formed by this
         // round that holds an edgeless vertex holds only edgeless vertices with
         // one previous block; and clean blocks, none of whose members has an
         // edge to a vertex whose smallest block member this round changed
-        if (p.shared) {
-            KB_CUDA(ctx, cudaMemsetAsync(R.mark, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
+        if (p.shared && i < k) {
             kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, s, stable);
-            kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen, R.frozen_min,
-                                    ctx->d_ctr, s, nullptr, nullptr, stable);
+            kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen, next_minima(R),
+                                    p.perm ? R.moved : nullptr, ctx->d_ctr, s, nullptr, nullptr, stable);
+            R.bitmap_ready = true;
             kb::launch_count_refining(p, R.frozen, ctx->d_ctr, s);
         }
         T.end();
@@ -1031,15 +1040,21 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
             // stratified levels only split blocks, so an unchanged count means an
             // unchanged partition; generic CSE levels were compared entry by entry
             if (stopped_stable) *stopped_stable = true;
-            if (!fixpoint && i < k) {
-                kb::launch_copy_rows(rows.levels, n, i, i + 1, k, s);
-                KB_TRY(emit_rows(ctx, rows, i + 1, k));
+            // with frozen blocks the renumbering left this row to be copied too
+            const int src = p.minof ? i - 1 : i;
+            if (!fixpoint) {
+                kb::launch_copy_rows(rows.levels, n, src, src + 1, k, s);
+                if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
+                KB_TRY(emit_rows(ctx, rows, i, k));
+            } else if (p.minof) {
+                KB_CUDA(ctx, cudaMemcpyAsync(out, p.prev, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
             }
             if (counts)
                 for (int j = i + 1; j <= k; ++j) counts[j] = c;
             KB_CUDA(ctx, cudaGetLastError());
             break;
         }
+        KB_TRY(emit_rows(ctx, rows, i, i));
         prev_count = c;
     }
     KB_CUDA(ctx, cudaStreamSynchronize(s));
@@ -1181,7 +1196,7 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_TRY(launch_round_body(ctx, R, s, &T));
         kb::launch_keep_bits(n, wmask, keep, kmin, p.bitmap, s);
         T.begin(KB_KERNEL_RENUMBER);
-        kb::launch_renumber(p, R.prefix, R.scan_tmp, row(i), s);
+        kb::launch_renumber(p, R.prefix, R.scan_tmp, row(i), nullptr, s);
         T.end();
         kb::launch_moved(n, wmask, keep, row(i), ranges, moved, s);
         kb::launch_count_bits(moved, nw, &ctx->d_ctr->moved, s);
@@ -1409,7 +1424,7 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
     int32_t* sticky = reinterpret_cast<int32_t*>(b + o_sticky);
     uint32_t* bases = reinterpret_cast<uint32_t*>(b + o_bases);
     uint32_t* bm_a = p.bitmap;
-    uint32_t* bm_b = reinterpret_cast<uint32_t*>(b + o_bm2);
+    uint32_t* bm_b = R.bm[1] ? R.bm[1] : reinterpret_cast<uint32_t*>(b + o_bm2);
     std::vector<uint8_t> act_h((size_t)G), early_h((size_t)G, (uint8_t)(opt->early_stop ? 1 : 0));
     for (int64_t j = 0; j < G; ++j) act_h[(size_t)j] = k_h[j] > 0 ? 1 : 0;
     KB_CUDA(ctx, cudaMemcpyAsync(voff, voff_h, sizeof(int64_t) * (size_t)(G + 1), cudaMemcpyHostToDevice, s));
@@ -1432,6 +1447,7 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
 
     // rounds 1..kmax, captured once
     p.gactive = gact;
+    R.counters_clear = true;
     if (kmax > 0) {
         if (!ctx->cap_stream) KB_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
         cudaStream_t cs = ctx->cap_stream;
@@ -1459,15 +1475,12 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
             st = launch_round_body(ctx, R, cs, nullptr);
             if (st != KB_OK) break;
             kb::launch_carry_minima(p, cs);
-            kb::launch_renumber(p, R.prefix, R.scan_tmp, out, cs);
-            if (p.shared) {
-                if (cudaMemsetAsync(R.mark, 0, sizeof(uint32_t) * (size_t)nw, cs) != cudaSuccess) {
-                    st = fail(ctx, KB_ERR_CUDA, "memset failed");
-                    break;
-                }
+            kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, cs);
+            if (p.shared && i < kmax) {
                 kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, cs);
-                kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen, R.frozen_min,
-                                        ctx->d_ctr, cs);
+                kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen,
+                                        (i & 1) ? bm_a : bm_b, nullptr, ctx->d_ctr, cs);
+                R.bitmap_ready = true;
             }
             kb::launch_graph_stop(p, i, kd, early, gact, glast, sticky, cs);
         }
@@ -2026,17 +2039,16 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         p.moved = sv->history ? sv->R.moved : nullptr;
         SV_TRY(sv, launch_round_body(ctx, sv->R, s, nullptr));
         kb::launch_carry_minima(p, s);
-        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, out, s);
+        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, out, p.moved ? sv->R.mark : nullptr, s);
         kb::launch_emit(sv->n_used, sv->vgraph, out, p.gbase_cur, sv->slot_levels, sv->slot_row, sv->slot_n, sv->voff, s);
         if (p.shared) {
             const uint32_t* mark = nullptr;
             if (p.moved) {
-                SV_CUDA(sv, cudaMemsetAsync(sv->R.mark, 0, sizeof(uint32_t) * (size_t)((sv->n_used >> 5) + 1), s));
                 kb::launch_dirty_blocks(p, sv->R.edgeless, sv->R.moved, out, kb::kMaxHubThreshold, sv->R.mark, s);
                 mark = sv->R.mark;
             }
             kb::launch_freeze_clean(sv->n_used, p.bitmap, p.shared, sv->R.edgeless, out, mark, sv->R.frozen,
-                                    sv->R.frozen_min, ctx->d_ctr, s, sv->vgraph, sv->gmode);
+                                    sv->R.frozen_min, nullptr, ctx->d_ctr, s, sv->vgraph, sv->gmode);
         }
         sv->history = true;
         SV_CUDA(sv, cudaGetLastError());

@@ -214,8 +214,8 @@ __device__ __forceinline__ uint32_t table_hi(uint64_t h, uint32_t epoch) {
 // Signature rounds (kb_kernels.cu).  The round's bitmap of block minima starts
 // as p.frozen_min (or empty).
 void launch_clear_round(const RoundParams& p, cudaStream_t s);
-// Empty the hub sets of the hubs that refine this round.
-void launch_clear_hub_sets(const RoundParams& p, int64_t total_slots, cudaStream_t s);
+// Empty the sets of the hubs that refine this round; clear the hubs' sums.
+void launch_clear_hubs(const RoundParams& p, int64_t total_slots, cudaStream_t s);
 // Clean blocks (RoundParams::minof).  After the renumbering of level i
 // (`level`, whose minima are in p.bitmap, moved vertices in `moved`): mark =
 // blocks of level i holding a vertex with an edge to a moved vertex (bit =
@@ -234,12 +234,12 @@ void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const u
 // in a level-i block without a mark bit (mark != null, unless more than an
 // eighth of the vertices moved).  frozen_min receives the minima of frozen
 // blocks; shared keeps exactly their marks; ctr->frozen counts the frozen
-// vertices.
+// vertices.  moved_clear (or nullptr): a bitmap to clear.
 // Serving (vgraph, gmode given): the vertices of graphs that computed their
 // level 0 in this step are not frozen by the edgeless rule.
 void launch_freeze_clean(int64_t n, const uint32_t* bitmap, uint32_t* shared, const uint32_t* edgeless,
                          const int32_t* level, const uint32_t* mark, uint32_t* frozen, uint32_t* frozen_min,
-                         Counters* ctr, cudaStream_t s, const int32_t* vgraph = nullptr,
+                         uint32_t* moved_clear, Counters* ctr, cudaStream_t s, const int32_t* vgraph = nullptr,
                          const uint8_t* gmode = nullptr, int64_t stable_count = -1);
 // Clear bits a..b-1 of a bitmap.
 void launch_clear_bits(uint32_t* words, int64_t a, int64_t b, cudaStream_t s);
@@ -263,10 +263,13 @@ void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s
 void launch_hub_final(const RoundParams& p, cudaStream_t s);
 // Canonical renumbering: prefix of block minima, then ids.
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
-// stable_count >= 0 (frozen-block rounds under early stop): a round whose
-// count equals it copies the previous level (it is the last round).
-void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, cudaStream_t s,
-                     int64_t stable_count = -1);
+// The frozen, med_on, hub_on and moved counters restart at 0; with frozen
+// blocks moved vertices are counted, and mark (or nullptr) is cleared.
+// stable_count >= 0 (frozen-block rounds under early stop): in a round whose
+// count equals it (the last round) the ids are those of the previous level, and
+// out is left for the caller to copy.
+void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
+                     cudaStream_t s, int64_t stable_count = -1);
 size_t scan_tmp_words(int64_t n_items);
 // Level 0 of one graph whose keys (vertex labels, or a starting partition)
 // are all in [0, kDenseLabels): the label partition straight from each
@@ -365,7 +368,7 @@ void launch_count_bits(const uint32_t* words, int64_t nw, int64_t* out, cudaStre
 void launch_set_bits(int64_t n, int64_t count, const int32_t* ids, uint32_t* bits, Counters* ctr, cudaStream_t s);
 void launch_classify(int64_t n, const int64_t* row, int32_t lo, int32_t hi, int32_t* out, int64_t* n_out,
                      cudaStream_t s);
-// Copy row src of the level store to the rows [first, last] of levels.
+// Copy row src of the level store to the rows [first, last] of levels (src not among them).
 void launch_copy_rows(int32_t* levels, int64_t n, int src, int first, int last, cudaStream_t s);
 
 // ---- serving arena (kb_serve.cu)

@@ -362,27 +362,26 @@ __global__ void __launch_bounds__(kScanThreads) popc_reduce_kernel(const uint32_
     if (threadIdx.x == 0) block_sums[blockIdx.x] = s;
 }
 
-__global__ void __launch_bounds__(kScanThreads) scan_block_sums_kernel(uint32_t* block_sums, int64_t nb,
-                                                                      Counters* ctr) {
-    __shared__ uint32_t tmp[32];
-    uint32_t carry = 0;
-    for (int64_t base = 0; base < nb; base += kScanThreads) {
-        const int64_t i = base + threadIdx.x;
-        const uint32_t x = i < nb ? block_sums[i] : 0u;
-        uint32_t total;
-        const uint32_t ex = block_exscan_u32(x, tmp, &total);
-        if (i < nb) block_sums[i] = carry + ex;
-        carry += total;
-    }
-    if (threadIdx.x == 0) ctr->count = (int64_t)carry;
-}
-
-// prefix[w] = set bits before word w; with rank given instead, rank[w] =
-// (prefix[w], bitmap[w]), so a rank lookup is one 8-byte load.
+// Rank of every set bit: prefix[w] = set bits before word w, or with rank
+// given instead, rank[w] = (prefix[w], bitmap[w]), so a rank lookup is one
+// 8-byte load.  Every block finds the set bits before its tile by itself: from
+// the tiles' sums (popc_reduce_kernel), or with block_sums null from the words
+// of the tiles before it.  The last block writes the total (and, for several
+// graphs, rank[nw]) and clears the counters that the passes after the
+// renumbering add to.
 __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t* bitmap, int64_t nw,
                                                                 const uint32_t* block_sums, uint32_t* prefix,
-                                                                uint2* rank) {
+                                                                uint2* rank, bool rank_total, Counters* ctr) {
     __shared__ uint32_t tmp[32];
+    __shared__ uint32_t s_before;
+    uint32_t before = 0;
+    if (block_sums) {
+        for (int64_t i = threadIdx.x; i < blockIdx.x; i += kScanThreads) before += block_sums[i];
+    } else {
+        for (int64_t i = threadIdx.x; i < (int64_t)blockIdx.x * kScanTile; i += kScanThreads) before += __popc(bitmap[i]);
+    }
+    before = block_sum_u32(before, tmp);
+    if (threadIdx.x == 0) s_before = before;
     const int64_t base = (int64_t)blockIdx.x * kScanTile + (int64_t)threadIdx.x * kScanItems;
     uint32_t w[kScanItems], c[kScanItems];
     uint32_t s = 0;
@@ -394,7 +393,17 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
         s += c[u];
     }
     uint32_t total;
-    uint32_t ex = block_exscan_u32(s, tmp, &total) + block_sums[blockIdx.x];
+    uint32_t ex = block_exscan_u32(s, tmp, &total);  // its barriers publish s_before
+    ex += s_before;
+    if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
+        const uint32_t all = s_before + total;
+        ctr->count = (int64_t)all;
+        ctr->frozen = 0;
+        ctr->med_on = 0;
+        ctr->hub_on = 0;
+        ctr->moved = 0;
+        if (rank_total) rank[nw] = make_uint2(all, 0u);
+    }
 #pragma unroll
     for (int u = 0; u < kScanItems; ++u) {
         const int64_t i = base + u;
@@ -406,6 +415,20 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
         }
         ex += c[u];
     }
+}
+
+// Up to this many tiles one launch does the scan, each block counting the words
+// before its tile: the last of 8 reads 28,672 words (7 per thread and tile
+// before it), less than the 3 us that the launch of a reduction costs.
+constexpr int64_t kScanDirect = 8;
+
+void rank_scan(const uint32_t* bitmap, int64_t nw, uint32_t* scan_tmp, uint32_t* prefix, uint2* rank, bool rank_total,
+               Counters* ctr, cudaStream_t s) {
+    const int64_t nb = (nw + kScanTile - 1) / kScanTile;
+    const bool direct = nb <= kScanDirect;
+    if (!direct) popc_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(bitmap, nw, scan_tmp);
+    popc_scan_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(bitmap, nw, direct ? nullptr : scan_tmp, prefix, rank,
+                                                           rank_total, ctr);
 }
 
 // The smallest member of v's block when v is not that member.
@@ -439,25 +462,6 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
     }
 }
 
-// The round kept the block count: blocks only split, so it kept every block
-// and its ids are the previous level's.  Under early stop it is the last
-// round, and nothing else of it is needed.  (Apart from assign_frozen_kernel,
-// whose registers bound its occupancy.)
-__global__ void __launch_bounds__(256) stable_copy_kernel(const RoundParams p, int32_t* out, int64_t stable_count) {
-    if (p.ctr->count != stable_count) return;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    int64_t done = 0;
-    if (((reinterpret_cast<uintptr_t>(p.prev) | reinterpret_cast<uintptr_t>(out)) & 15) == 0) {
-        const int64_t n4 = p.n >> 2;  // 16-byte copies while both rows allow them
-        const int4* src = reinterpret_cast<const int4*>(p.prev);
-        int4* dst = reinterpret_cast<int4*>(out);
-        for (int64_t i = t; i < n4; i += stride) dst[i] = __ldcs(src + i);
-        done = n4 << 2;
-    }
-    for (int64_t v = done + t; v < p.n; v += stride) out[v] = p.prev[v];
-}
-
 // Canonical ids of a stratified round with frozen blocks (RoundParams::minof;
 // one graph, or several at once): assign_kernel's work with every lane of a warp on one
 // bitmap word (a warp-uniform loop), so that the moved vertices (re-keyed
@@ -466,12 +470,18 @@ __global__ void __launch_bounds__(256) stable_copy_kernel(const RoundParams p, i
 // warp.  Frozen vertices keep minof, and their blocks keep their shared marks
 // (the freeze pass carries them over); the mark of a re-keyed block comes from
 // the vertex that inserted its table entry (RoundParams::joined).  moved may be
-// null (the starting level).
+// null (the starting level); mark, when given, is cleared for the dirty pass.
 __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p, const uint2* rank, int32_t* out,
-                                                             uint32_t* moved, int64_t stable_count) {
-    // a round that kept the block count is copied by stable_copy_kernel
+                                                             uint32_t* moved, uint32_t* mark,
+                                                             int64_t stable_count) {
+    // a round that kept the block count kept every block (blocks only split):
+    // under early stop it is the last one, and the caller copies the level
     if (stable_count >= 0 && p.ctr->count == stable_count) return;
+    __shared__ uint32_t s_moved;
+    if (threadIdx.x == 0) s_moved = 0u;
+    __syncthreads();
     const int lane = threadIdx.x & 31;
+    uint32_t n_moved = 0;
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < p.n; base += stride) {
         const int64_t v = base + lane;
@@ -512,6 +522,7 @@ __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p,
             __syncwarp();
             if (lane == 0) p.joined[base >> 5] = 0u;
         }
+        if (mark && lane == 0) mark[base >> 5] = 0u;
         if (moved) {
             const unsigned w = __ballot_sync(kFull, mv);
             if (p.perm) {
@@ -519,8 +530,14 @@ __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p,
             } else if (lane == 0) {
                 moved[base >> 5] = w;
             }
+            n_moved += __popc(w);
         }
     }
+    if (!moved) return;  // uniform over the grid
+    if (lane == 0 && n_moved) atomicAdd(&s_moved, n_moved);
+    __syncthreads();
+    if (threadIdx.x == 0 && s_moved)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctr->moved), (unsigned long long)s_moved);
 }
 
 // Vertices of bitmap word w that are neither alone in their block nor
@@ -534,8 +551,9 @@ __device__ __forceinline__ uint32_t candidate_word(const uint32_t* bitmap, const
     return c;
 }
 
-// A warp takes 32 consecutive bitmap words (1024 vertices) and deals their
-// candidate vertices (candidate_word) to its lanes, 32 at a time: *v receives
+// A warp takes up to 32 consecutive bitmap words (1024 vertices; fewer while
+// the graph is too small to fill the chip with that) and deals their candidate
+// vertices (candidate_word) to its lanes, 32 at a time: *v receives
 // the vertex of rank r among them, or -1.  excl / c are this lane's word's
 // exclusive candidate prefix and candidate bits.
 __device__ __forceinline__ int64_t dealt_vertex(int64_t w0, uint32_t excl, uint32_t c, int r, int total) {
@@ -564,14 +582,16 @@ __device__ __forceinline__ bool few_moved(const RoundParams& p) { return p.ctr->
 
 __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, const uint32_t* edgeless,
                                                             const uint32_t* moved, const int32_t* level,
-                                                            int32_t max_scan, uint32_t* mark, int64_t stable_count) {
+                                                            int32_t max_scan, uint32_t* mark, int per_warp,
+                                                            int64_t stable_count) {
     if (!few_moved(p)) return;
     if (stable_count >= 0 && p.ctr->count == stable_count) return;  // the last round: nothing follows
     const int lane = threadIdx.x & 31;
     const int64_t nw = (p.n >> 5) + 1;
-    const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+    const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per_warp;
     if (w0 >= nw) return;  // uniform over the warp
-    const uint32_t c = w0 + lane < nw ? candidate_word(p.bitmap, p.shared, edgeless, w0 + lane, p.n) : 0u;
+    const uint32_t c =
+        lane < per_warp && w0 + lane < nw ? candidate_word(p.bitmap, p.shared, edgeless, w0 + lane, p.n) : 0u;
     uint32_t incl = __popc(c);
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -608,23 +628,29 @@ __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, 
 // and no more than an eighth of the vertices moved).  frozen_min holds the
 // minima of frozen blocks, and the shared marks of exactly those minima are
 // kept for the next round (their blocks keep their members; the others are
-// marked afresh).  A warp takes 32 bitmap words and deals the candidates
+// marked afresh).  A warp takes up to 32 bitmap words and deals the candidates
 // whose block it must look up to its lanes, as dirty_blocks_kernel does.
+// moved_clear, when given, is a bitmap that starts the next round empty.
 __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint32_t* bitmap, uint32_t* shared,
                                                             const uint32_t* edgeless, const int32_t* level,
                                                             const uint32_t* mark, uint32_t* frozen,
-                                                            uint32_t* frozen_min, Counters* ctr, const int32_t* vgraph,
+                                                            uint32_t* frozen_min, uint32_t* moved_clear, int per_warp,
+                                                            Counters* ctr, const int32_t* vgraph,
                                                             const uint8_t* gmode, int64_t stable_count) {
     __shared__ uint32_t s_clean[8][32];
+    __shared__ uint32_t s_frozen;
+    if (stable_count >= 0 && ctr->count == stable_count) return;  // the last round: nothing follows
+    if (threadIdx.x == 0) s_frozen = 0u;
+    __syncthreads();
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (n >> 5) + 1;
-    const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * 32;
-    if (w0 >= nw) return;  // uniform over the warp
-    if (stable_count >= 0 && ctr->count == stable_count) return;  // the last round: nothing follows
+    // a warp past the end keeps to the barriers with no words of its own
+    const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + warp) * per_warp;
     if (mark && ctr->moved * 8 > n) mark = nullptr;  // the dirty pass scanned nothing
     const int64_t w = w0 + lane;
+    const bool own = lane < per_warp && w < nw;
     uint32_t b = 0, sh = 0, e = 0, c = 0;
-    if (w < nw) {
+    if (own) {
         b = bitmap[w];
         sh = shared[w];
         e = edgeless ? edgeless[w] : 0u;
@@ -663,7 +689,7 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint
         if (!((mark[l >> 5] >> (l & 31)) & 1u)) atomicOr(&s_clean[warp][(v >> 5) - w0], 1u << (v & 31));
     }
     __syncwarp();
-    if (w < nw) {
+    if (own) {
         // no bit past the last vertex survives (rank scans count whole words)
         const uint32_t valid = w * 32 + 32 <= n ? 0xffffffffu : (n > w * 32 ? (1u << (uint32_t)(n - w * 32)) - 1u : 0u);
         const uint32_t single = b & ~sh & valid;
@@ -673,7 +699,12 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint
         frozen[w] = fz;
         frozen_min[w] = fm;
         shared[w] = sh & fm;
+        if (moved_clear) moved_clear[w] = 0u;
+        if (fz) atomicAdd(&s_frozen, (uint32_t)__popc(fz));
     }
+    __syncthreads();
+    if (threadIdx.x == 0 && s_frozen)
+        atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->frozen), (unsigned long long)s_frozen);
 }
 
 // The vertices a round re-keys (those not in frozen; all when frozen is null)
@@ -958,10 +989,6 @@ __global__ void vertex_graph_kernel(const int64_t* voff, int32_t G, int64_t n, i
     for (int64_t v = voff[g] + threadIdx.x; v < voff[g + 1]; v += blockDim.x) vgraph[v] = g;
 }
 
-__global__ void write_total_kernel(uint2* rank, int64_t nw, const Counters* ctr) {
-    rank[nw] = make_uint2((uint32_t)ctr->count, 0u);
-}
-
 __global__ void fill_i32_kernel(int32_t* out, int64_t n, int32_t value) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) out[i] = value;
@@ -994,14 +1021,17 @@ void launch_clear_round(const RoundParams& p, cudaStream_t s) {
         cudaMemcpyAsync(p.bitmap, p.frozen_min, bytes, cudaMemcpyDeviceToDevice, s);
     else
         cudaMemsetAsync(p.bitmap, 0, bytes, s);
-    if (p.n_hubs > 0) {
-        cudaMemsetAsync(p.hub_acc, 0, sizeof(uint64_t) * (size_t)p.n_hubs, s);
-        cudaMemsetAsync(p.hub_cnt, 0, sizeof(uint32_t) * (size_t)p.n_hubs, s);
-    }
 }
 
-void launch_clear_hub_sets(const RoundParams& p, int64_t total_slots, cudaStream_t s) {
-    if (p.n_hubs <= 0 || total_slots <= 0) return;
+void launch_clear_hubs(const RoundParams& p, int64_t total_slots, cudaStream_t s) {
+    if (p.n_hubs <= 0) return;
+    cudaMemsetAsync(p.hub_acc, 0, sizeof(uint64_t) * (size_t)p.n_hubs, s);
+    cudaMemsetAsync(p.hub_cnt, 0, sizeof(uint32_t) * (size_t)p.n_hubs, s);
+    if (total_slots <= 0) return;
+    if (!p.frozen) {
+        cudaMemsetAsync(p.hub_sets, 0xff, sizeof(uint64_t) * (size_t)total_slots, s);
+        return;
+    }
     // short tiles while the sets are small, so that every SM stores (18 us for
     // 3 x 10^5 slots in tiles of 65536, 5 us in tiles of 2048)
     const int64_t per = total_slots / (152 * 8);
@@ -1009,24 +1039,34 @@ void launch_clear_hub_sets(const RoundParams& p, int64_t total_slots, cudaStream
     clear_hub_sets_kernel<<<(unsigned)((total_slots + tile - 1) / tile), 256, 0, s>>>(p, tile);
 }
 
+// Bitmap words per warp of the dirty and freeze passes: 32, fewer while that
+// leaves SMs idle (a lane walks up to as many candidates as its warp has words:
+// 17 and 11 us for 3 x 10^5 vertices on the 37 CTAs that 32 words give).
+static int words_per_warp(int64_t nw) {
+    return (int)std::min<int64_t>(32, std::max<int64_t>(1, nw / (152 * 32)));
+}
+
 void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,
                          int32_t max_scan, uint32_t* mark, cudaStream_t s, int64_t stable_count) {
     if (p.n <= 0) return;
-    const int64_t warps = ((p.n >> 5) + 1 + 31) / 32;  // 32 bitmap words each
-    dirty_blocks_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(p, edgeless, moved, level, max_scan, mark,
+    const int64_t nw = (p.n >> 5) + 1;
+    const int per = words_per_warp(nw);
+    const int64_t warps = (nw + per - 1) / per;
+    dirty_blocks_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(p, edgeless, moved, level, max_scan, mark, per,
                                                                      stable_count);
 }
 
 void launch_freeze_clean(int64_t n, const uint32_t* bitmap, uint32_t* shared, const uint32_t* edgeless,
                          const int32_t* level, const uint32_t* mark, uint32_t* frozen, uint32_t* frozen_min,
-                         Counters* ctr, cudaStream_t s, const int32_t* vgraph, const uint8_t* gmode,
-                         int64_t stable_count) {
+                         uint32_t* moved_clear, Counters* ctr, cudaStream_t s, const int32_t* vgraph,
+                         const uint8_t* gmode, int64_t stable_count) {
     if (n <= 0) return;
-    const int64_t warps = ((n >> 5) + 1 + 31) / 32;  // 32 bitmap words each
-    freeze_clean_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(n, bitmap, shared, edgeless, level, mark, frozen,
-                                                                     frozen_min, ctr, vgraph, gmode, stable_count);
     const int64_t nw = (n >> 5) + 1;
-    count_bits_kernel<<<grid_for(nw, 256) < 1216 ? grid_for(nw, 256) : 1216, 256, 0, s>>>(frozen, nw, &ctr->frozen);
+    const int per = words_per_warp(nw);
+    const int64_t warps = (nw + per - 1) / per;
+    freeze_clean_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(n, bitmap, shared, edgeless, level, mark, frozen,
+                                                                     frozen_min, moved_clear, per, ctr, vgraph, gmode,
+                                                                     stable_count);
 }
 
 void launch_round_work(const RoundParams& p, cudaStream_t s) {
@@ -1075,37 +1115,19 @@ size_t scan_tmp_words(int64_t n_items) { return (size_t)((n_items + kScanTile - 
 
 void launch_bitmap_rank(const uint32_t* bitmap, int64_t nw, uint32_t* scan_tmp, uint32_t* prefix, Counters* ctr,
                         cudaStream_t s) {
-    const int64_t nb = (nw + kScanTile - 1) / kScanTile;
-    popc_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(bitmap, nw, scan_tmp);
-    scan_block_sums_kernel<<<1, kScanThreads, 0, s>>>(scan_tmp, nb, ctr);
-    popc_scan_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(bitmap, nw, scan_tmp, prefix, nullptr);
+    rank_scan(bitmap, nw, scan_tmp, prefix, nullptr, false, ctr, s);
 }
 
-void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, cudaStream_t s,
-                     int64_t stable_count) {
+void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
+                     cudaStream_t s, int64_t stable_count) {
     const int64_t nw = (p.n >> 5) + 1;
-    const int64_t nb = (nw + kScanTile - 1) / kScanTile;
-    popc_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(p.bitmap, nw, scan_tmp);
-    scan_block_sums_kernel<<<1, kScanThreads, 0, s>>>(scan_tmp, nb, p.ctr);
-    popc_scan_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(p.bitmap, nw, scan_tmp, nullptr, rank);
-    if (batched(p)) {
-        // rank[nw] (one past the last word) is not written by the scan: the
-        // total sits in the counters, and graph_base_kernel reads it there
-        // for a graph that starts at n.
-        write_total_kernel<<<1, 1, 0, s>>>(rank, nw, p.ctr);
-        graph_base_kernel<<<(p.n_graphs + 1 + 255) / 256, 256, 0, s>>>(p, rank);
-    }
-    if (p.minof) {
-        if (p.moved && p.perm) cudaMemsetAsync(p.moved, 0, sizeof(uint32_t) * (size_t)nw, s);
-        if (p.n > 0 && stable_count >= 0)
-            stable_copy_kernel<<<grid_for(p.n, 256) < 1216 ? grid_for(p.n, 256) : 1216, 256, 0, s>>>(p, out,
-                                                                                                 stable_count);
-        if (p.n > 0) assign_frozen_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out, p.moved, stable_count);
-        if (p.moved) count_bits_kernel<<<grid_for(nw, 256) < 1216 ? grid_for(nw, 256) : 1216, 256, 0, s>>>(
-            p.moved, nw, &p.ctr->moved);
-        return;
-    }
-    if (p.n > 0) assign_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out);
+    rank_scan(p.bitmap, nw, scan_tmp, nullptr, rank, batched(p), p.ctr, s);
+    if (batched(p)) graph_base_kernel<<<(p.n_graphs + 1 + 255) / 256, 256, 0, s>>>(p, rank);
+    if (p.n <= 0) return;
+    if (p.minof)
+        assign_frozen_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out, p.moved, mark, stable_count);
+    else
+        assign_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out);
 }
 
 void launch_dense_labels(int64_t n, const int32_t* key, uint32_t* lmin, Counters* ctr, cudaStream_t s) {
@@ -1119,11 +1141,8 @@ void launch_dense_level0(const RoundParams& p, const int32_t* key, const uint32_
                          uint32_t* scan_tmp, int32_t* out, cudaStream_t s) {
     if (p.n <= 0) return;
     const int64_t nw = (p.n >> 5) + 1;
-    const int64_t nb = (nw + kScanTile - 1) / kScanTile;
     dense_mark_kernel<<<(kDenseLabels + 255) / 256, 256, 0, s>>>(p, lmin);
-    popc_reduce_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(p.bitmap, nw, scan_tmp);
-    scan_block_sums_kernel<<<1, kScanThreads, 0, s>>>(scan_tmp, nb, p.ctr);
-    popc_scan_kernel<<<(unsigned)nb, kScanThreads, 0, s>>>(p.bitmap, nw, scan_tmp, nullptr, rank);
+    rank_scan(p.bitmap, nw, scan_tmp, nullptr, rank, false, p.ctr, s);
     dense_ids_kernel<<<(kDenseLabels + 255) / 256, 256, 0, s>>>(lmin, rank, lpair);
     dense_assign_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, key, lpair, out);
 }

@@ -173,7 +173,7 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
     kb::launch_medium_round(p, s);
     kb::launch_renumber(p, reinterpret_cast<uint2*>(base + kOffPrefix), reinterpret_cast<uint32_t*>(base + kOffScan),
-                        out, s);
+                        out, nullptr, s);
     NA_CUDA(cudaGetLastError());
     NA_CUDA(cudaMemcpyAsync(&host_ctr, ctr, sizeof(host_ctr), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));

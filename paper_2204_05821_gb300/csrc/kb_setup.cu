@@ -281,6 +281,16 @@ __global__ void __launch_bounds__(kT) scan_down_kernel(const int64_t* in, int64_
     }
 }
 
+// rows consecutive rows of n entries, each a copy of src, which is read once
+template <typename T>
+__global__ void __launch_bounds__(256) copy_rows_kernel(const T* src, int64_t n, int rows, T* dst) {
+    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) {
+        const T x = __ldcs(src + i);
+        for (int r = 0; r < rows; ++r) dst[(int64_t)r * n + i] = x;
+    }
+}
+
 __global__ void write_total_kernel(const int64_t* sums, int64_t nb, int64_t* out, int64_t n) { out[n] = sums[nb]; }
 
 }  // namespace
@@ -354,10 +364,14 @@ void launch_classify(int64_t n, const int64_t* row, int32_t lo, int32_t hi, int3
 }
 
 void launch_copy_rows(int32_t* levels, int64_t n, int src, int first, int last, cudaStream_t s) {
-    for (int r = first; r <= last; ++r)
-        if (r != src)
-            cudaMemcpyAsync(levels + (size_t)r * (size_t)n, levels + (size_t)src * (size_t)n,
-                            sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s);
+    if (n <= 0 || last < first) return;
+    int32_t* from = levels + (size_t)src * (size_t)n;
+    int32_t* to = levels + (size_t)first * (size_t)n;
+    if (((reinterpret_cast<uintptr_t>(levels) | (uintptr_t)(4 * n)) & 15) == 0)  // every row starts on 16 bytes
+        copy_rows_kernel<<<grid_for(n / 4, 256), 256, 0, s>>>(reinterpret_cast<const int4*>(from), n / 4, last - first + 1,
+                                                              reinterpret_cast<int4*>(to));
+    else
+        copy_rows_kernel<<<grid_for(n, 256), 256, 0, s>>>(from, n, last - first + 1, to);
 }
 
 }  // namespace kb
