@@ -31,12 +31,10 @@ struct kb_context {
     // small persistent device state
     kb::Counters* d_ctr = nullptr;
     kb::Counters* h_ctr = nullptr;  // pinned
-    int32_t* d_hub_n = nullptr;
-    int32_t* h_hub_n = nullptr;  // pinned
-    int64_t* d_med_n = nullptr;
-    int64_t* h_med_n = nullptr;  // pinned
-    void* hub_tmp = nullptr;     // unordered hub list during planning
-    size_t hub_tmp_bytes = 0;
+    uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
+    char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
+    void* class_tmp = nullptr;    // degree-class bitmaps, tile counts and hub list during planning
+    size_t class_tmp_bytes = 0;
     void* plan_tmp = nullptr;    // in-degree scratch used by kb_workspace_size
     size_t plan_tmp_bytes = 0;
     // host-buffer refinement staging (library-owned)
@@ -107,6 +105,9 @@ kb_status fail(kb_context* ctx, kb_status st, const char* fmt, ...) {
         if (s_ != KB_OK) return s_;        \
     } while (0)
 
+// Hubs whose list comes back in the same copy as the counts of the plan.
+constexpr int64_t kEagerHubs = 4096;
+
 size_t align_up(size_t x) { return (x + 255) & ~(size_t)255; }
 
 uint64_t next_pow2(uint64_t x) {
@@ -153,18 +154,19 @@ struct Plan {
     // hubs (host copies, ascending vertex id)
     std::vector<int32_t> hub_v;
     std::vector<int64_t> chunk_off, set_off;
-    std::vector<int32_t> chunk_hub;
     // their sizes (the lists themselves are dropped once on the device)
     size_t n_hubs = 0;
     int64_t n_chunks = 0, set_slots = 0;
+    int64_t n_med = 0;  // medium vertices
     // layout
     size_t o_rowp = 0, o_colp = 0, o_labp = 0, o_cursor = 0, o_inpref = 0, o_i64tmp = 0;
     size_t csr_bytes = 0;
     size_t o_emin = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
-           o_frozen = 0, o_edgeless = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0,
-           o_dense = 0;
+           o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0;
     size_t total = 0;
+    // bytes of one degree-class bitmap; three follow one another: edgeless, medium, hub
+    size_t class_bytes() const { return align_up(sizeof(uint32_t) * (size_t)((n >> 5) + 1)); }
 };
 
 bool needs_in_csr(int dir) { return dir == KB_DIR_IN || dir == KB_DIR_BOTH; }
@@ -181,7 +183,6 @@ struct kb_prepared {
     Plan P;             // graph_ext layout; host hub lists dropped after upload
     char* csr = nullptr;   // processed CSR (IN / BOTH)
     char* gbuf = nullptr;  // per-graph part
-    int64_t n_med = 0;
     float build_ms = 0.f;
     ~kb_prepared() {
         if (!csr && !gbuf) return;
@@ -218,7 +219,7 @@ void layout_round(Plan& P) {
     auto takeg = [&](size_t bytes) { size_t o = goff; goff += align_up(bytes); return o; };
     const int64_t nw = (P.n >> 5) + 1;
     const size_t H = P.n_hubs;
-    P.o_med = takeg(sizeof(int32_t) * (size_t)(std::min<int64_t>(P.n, P.m_proc / 2 + 1) + 1));
+    P.o_med = takeg(sizeof(int32_t) * (size_t)P.n_med);
     P.o_hubv = takeg(sizeof(int32_t) * H);
     P.o_chunk = takeg(sizeof(int64_t) * (H + 1));
     P.o_setoff = takeg(sizeof(int64_t) * (H + 1));
@@ -229,7 +230,7 @@ void layout_round(Plan& P) {
     // CSR is reordered in place
     P.o_colr = takeg(P.reorder && !needs_in_csr(P.dir) ? sizeof(int32_t) * (size_t)P.m_proc : 0);
     P.o_hist = takeg(P.reorder ? sizeof(unsigned long long) * 512 : 0);
-    P.o_edgeless = takeg((P.freeze || P.graph_ext) ? sizeof(uint32_t) * (size_t)nw : 0);
+    P.o_classes = takeg((P.freeze || P.graph_ext) ? 3 * P.class_bytes() : 0);
     P.graph_bytes = P.graph_ext ? goff : 0;
     size_t off = P.graph_ext ? 0 : goff;
     auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
@@ -252,7 +253,6 @@ void layout_round(Plan& P) {
     P.o_bm2 = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_moved = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_mark = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
-    P.o_dense = take(P.dense0 ? (sizeof(uint32_t) + sizeof(uint2)) * (size_t)kb::kDenseLabels : 0);
     P.total = off;
 }
 
@@ -332,51 +332,66 @@ kb_status build_processed_csr(kb_context* ctx, const kb_graph* g, Plan& P, char*
     return KB_OK;
 }
 
-// Discover hubs of the processed CSR and fill the host side of the plan.
-kb_status plan_hubs(kb_context* ctx, Plan& P, const int64_t* row_p) {
+// Where launch_classes put its results (ctx->class_tmp), for a plan's n.
+struct ClassScratch {
+    size_t bits = 0, counts = 0, hub_v = 0, hub_deg = 0, total = 0;
+    int64_t hub_cap = 0;
+    explicit ClassScratch(const Plan& P) {
+        counts = 3 * P.class_bytes();
+        hub_v = counts + align_up(2 * sizeof(uint32_t) * kb::class_tiles(P.n));
+        hub_cap = std::min<int64_t>(P.n, P.m_proc / (P.thr + 1) + 1);
+        hub_deg = hub_v + align_up(sizeof(int32_t) * (size_t)hub_cap);
+        total = hub_deg + align_up(sizeof(int64_t) * (size_t)hub_cap);
+    }
+};
+
+// Degree classes of the processed CSR and the host side of the plan: hubs,
+// their chunks and sets, the number of medium vertices.  One round trip, which
+// also brings back ctx->h_ctr (errors of the validation, the level-0 key
+// check).
+kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::CheckRows check) {
+    cudaStream_t s = ctx->stream;
     P.hub_v.clear();
     P.chunk_off.assign(1, 0);
     P.set_off.assign(1, 0);
-    P.chunk_hub.clear();
     P.n_hubs = 0;
-    P.n_chunks = P.set_slots = 0;
-    if (P.n == 0 || P.m_proc == 0) return KB_OK;
-    const int64_t hmax = std::min<int64_t>(P.n, P.m_proc / (P.thr + 1) + 1);
-    const size_t deg_off = align_up(sizeof(int32_t) * (size_t)hmax);
-    KB_TRY(ensure_buffer(ctx, &ctx->hub_tmp, &ctx->hub_tmp_bytes, deg_off + sizeof(int64_t) * (size_t)hmax));
-    int32_t* d_v = reinterpret_cast<int32_t*>(ctx->hub_tmp);
-    int64_t* d_deg = reinterpret_cast<int64_t*>(reinterpret_cast<char*>(ctx->hub_tmp) + deg_off);
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_hub_n, 0, sizeof(int32_t), ctx->stream));
-    kb::launch_find_hubs(P.n, row_p, P.thr, d_v, d_deg, ctx->d_hub_n, ctx->stream);
+    P.n_chunks = P.set_slots = P.n_med = 0;
+    if (P.n == 0) return read_counters(ctx);
+    const ClassScratch C(P);
+    KB_TRY(ensure_buffer(ctx, &ctx->class_tmp, &ctx->class_tmp_bytes, C.total));
+    char* b = reinterpret_cast<char*>(ctx->class_tmp);
+    uint32_t* counts = reinterpret_cast<uint32_t*>(b + C.counts);
+    auto bits = [&](int i) { return reinterpret_cast<uint32_t*>(b + (size_t)i * P.class_bytes()); };
+    kb::launch_classes(P.n, P.m_proc, row_p, P.small_max, P.thr, bits(0), bits(1), bits(2), counts, check, ctx->d_ctr, s);
+    kb::launch_class_list(P.n, row_p, bits(2), counts, 1, C.hub_cap, reinterpret_cast<int32_t*>(b + C.hub_v),
+                          reinterpret_cast<int64_t*>(b + C.hub_deg), s);
     KB_CUDA(ctx, cudaGetLastError());
-    KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_hub_n, ctx->d_hub_n, sizeof(int32_t), cudaMemcpyDeviceToHost, ctx->stream));
-    KB_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
-    const int32_t H = *ctx->h_hub_n;
+    const int64_t eager = std::min(C.hub_cap, kEagerHubs);
+    char* h_deg = ctx->h_hubs + sizeof(int32_t) * kEagerHubs;
+    KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_hubs, b + C.hub_v, sizeof(int32_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
+    KB_CUDA(ctx, cudaMemcpyAsync(h_deg, b + C.hub_deg, sizeof(int64_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
+    KB_TRY(read_counters(ctx));
+    KB_TRY(device_error(ctx));
+    const int64_t H = ctx->h_ctr->n_hubs;
+    P.n_med = ctx->h_ctr->n_med;
+    if (H > C.hub_cap || P.n_med > P.n) return fail(ctx, KB_ERR_DEVICE_CHECK, "degree class larger than the graph allows");
     if (H <= 0) return KB_OK;
-    if (H > hmax) return fail(ctx, KB_ERR_DEVICE_CHECK, "hub count exceeds bound");
-    std::vector<int32_t> hv((size_t)H);
-    std::vector<int64_t> hd((size_t)H);
-    KB_CUDA(ctx, cudaMemcpy(hv.data(), d_v, sizeof(int32_t) * (size_t)H, cudaMemcpyDeviceToHost));
-    KB_CUDA(ctx, cudaMemcpy(hd.data(), d_deg, sizeof(int64_t) * (size_t)H, cudaMemcpyDeviceToHost));
-    std::vector<int32_t> order((size_t)H);
-    for (int32_t i = 0; i < H; ++i) order[(size_t)i] = i;
-    std::sort(order.begin(), order.end(), [&](int32_t a, int32_t b) { return hv[(size_t)a] < hv[(size_t)b]; });
     P.hub_v.resize((size_t)H);
     std::vector<int64_t> deg((size_t)H);
-    for (int32_t i = 0; i < H; ++i) {
-        P.hub_v[(size_t)i] = hv[(size_t)order[(size_t)i]];
-        deg[(size_t)i] = hd[(size_t)order[(size_t)i]];
+    if (H <= eager) {
+        std::memcpy(P.hub_v.data(), ctx->h_hubs, sizeof(int32_t) * (size_t)H);
+        std::memcpy(deg.data(), h_deg, sizeof(int64_t) * (size_t)H);
+    } else {
+        KB_CUDA(ctx, cudaMemcpyAsync(P.hub_v.data(), b + C.hub_v, sizeof(int32_t) * (size_t)H, cudaMemcpyDeviceToHost, s));
+        KB_CUDA(ctx, cudaMemcpyAsync(deg.data(), b + C.hub_deg, sizeof(int64_t) * (size_t)H, cudaMemcpyDeviceToHost, s));
+        KB_CUDA(ctx, cudaStreamSynchronize(s));
     }
     P.chunk_off.resize((size_t)H + 1);
     P.set_off.resize((size_t)H + 1);
-    for (int32_t i = 0; i < H; ++i) {
-        const int64_t d = deg[(size_t)i];
-        P.chunk_off[(size_t)i + 1] = P.chunk_off[(size_t)i] + (d + P.hub_chunk - 1) / P.hub_chunk;
-        P.set_off[(size_t)i + 1] = P.set_off[(size_t)i] + kb::hub_set_capacity(d);
+    for (size_t i = 0; i < (size_t)H; ++i) {
+        P.chunk_off[i + 1] = P.chunk_off[i] + (deg[i] + P.hub_chunk - 1) / P.hub_chunk;
+        P.set_off[i + 1] = P.set_off[i] + kb::hub_set_capacity(deg[i]);
     }
-    P.chunk_hub.resize((size_t)P.chunk_off[(size_t)H]);
-    for (int32_t i = 0; i < H; ++i)
-        for (int64_t c = P.chunk_off[(size_t)i]; c < P.chunk_off[(size_t)i + 1]; ++c) P.chunk_hub[(size_t)c] = i;
     P.n_hubs = (size_t)H;
     P.n_chunks = P.chunk_off[(size_t)H];
     P.set_slots = P.set_off[(size_t)H];
@@ -464,7 +479,7 @@ kb_status make_plan(kb_context* ctx, const kb_graph* g, const kb_options* opt, P
         KB_TRY(build_processed_csr(ctx, g, P, csr_base));
         row_p = reinterpret_cast<const int64_t*>(csr_base + P.o_rowp);
     }
-    KB_TRY(plan_hubs(ctx, P, row_p));
+    KB_TRY(plan_classes(ctx, P, row_p, opt->validate && !for_query ? kb::CheckRows::kAll : kb::CheckRows::kNone));
     layout_round(P);
     return KB_OK;
 }
@@ -543,8 +558,10 @@ struct Prepared {
     bool counters_clear = false;  // the round need not clear the counters (no errors so far; see launch_renumber)
     uint32_t* moved = nullptr;
     uint32_t* mark = nullptr;
-    uint32_t* dense_min = nullptr;  // launch_dense_labels / launch_dense_level0 (Plan::dense0)
-    uint2* dense_pair = nullptr;
+    const int32_t* key_checked = nullptr;  // level-0 keys whose label minima are in ctx->d_dense,
+    bool key_dense = false;                //   and whether they are all small (launch_dense_labels)
+    const uint32_t* medium_bits = nullptr;  // degree classes (Plan::class_bytes); nullptr: an empty class
+    const uint32_t* hub_bits = nullptr;
     bool compact = false;  // small-kernel windows skip frozen vertices (many frozen)
     bool sparse = false;   // fewer than 1/64 of the vertices refine: long warp tasks
     // A caller-held block table (ext_cap slots) and empty-signature minima
@@ -571,9 +588,8 @@ struct Prepared {
 // Bind the per-graph part of a plan into p: the processed CSR (csr: IN /
 // BOTH), the hub lists, the locality order and the medium list (gws: graph
 // part base).  build: also fill them (hub lists uploaded, chunk extents, the
-// locality order, using `count_tmp` (n words) as scratch, the medium list
-// and, with `edgeless`, the edgeless bits); else they hold a prepared graph's
-// contents.  Synchronises when building.
+// locality order, using `count_tmp` (n words) as scratch, the medium list and
+// the degree-class bitmaps); else they hold a prepared graph's contents.
 kb_status bind_graph_part(kb_context* ctx, const kb_graph* g, const Plan& P, char* csr, char* gws, bool build,
                           uint32_t* count_tmp, kb::RoundParams& p, cudaStream_t s) {
     const int64_t n = g->n;
@@ -594,14 +610,15 @@ kb_status bind_graph_part(kb_context* ctx, const kb_graph* g, const Plan& P, cha
     p.chunk_hub = reinterpret_cast<const int32_t*>(gws + P.o_chunkhub);
     p.chunk_ext = reinterpret_cast<const uint64_t*>(gws + P.o_chunkext);
     if (build && H) {
-        KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_hubv, P.hub_v.data(), sizeof(int32_t) * H, cudaMemcpyHostToDevice, s));
-        KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_chunk, P.chunk_off.data(), sizeof(int64_t) * (H + 1),
-                                     cudaMemcpyHostToDevice, s));
-        KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_setoff, P.set_off.data(), sizeof(int64_t) * (H + 1),
-                                     cudaMemcpyHostToDevice, s));
-        KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_chunkhub, P.chunk_hub.data(), sizeof(int32_t) * P.chunk_hub.size(),
-                                     cudaMemcpyHostToDevice, s));
-        kb::launch_chunk_ext((int64_t)P.chunk_hub.size(), p.chunk_hub, p.hub_v, p.hub_chunk_off, p.row, P.hub_chunk,
+        // the three lists lie one after another: one copy
+        std::vector<char> up(P.o_setoff + sizeof(int64_t) * (H + 1) - P.o_hubv);
+        std::memcpy(up.data(), P.hub_v.data(), sizeof(int32_t) * H);
+        std::memcpy(up.data() + (P.o_chunk - P.o_hubv), P.chunk_off.data(), sizeof(int64_t) * (H + 1));
+        std::memcpy(up.data() + (P.o_setoff - P.o_hubv), P.set_off.data(), sizeof(int64_t) * (H + 1));
+        // pageable memory: staged before the call returns
+        KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_hubv, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+        kb::launch_chunk_ext(P.n_chunks, (int32_t)H, p.hub_v, p.hub_chunk_off, p.row, P.hub_chunk,
+                             reinterpret_cast<int32_t*>(gws + P.o_chunkhub),
                              reinterpret_cast<uint64_t*>(gws + P.o_chunkext), s);
         KB_CUDA(ctx, cudaGetLastError());
     }
@@ -620,29 +637,49 @@ kb_status bind_graph_part(kb_context* ctx, const kb_graph* g, const Plan& P, cha
         p.perm = perm;
     }
     p.med_v = reinterpret_cast<int32_t*>(gws + P.o_med);
+    p.n_med = P.n_med;
     if (build) {
-        p.n_med = 0;
-        if (g->m > 0) {
-            KB_CUDA(ctx, cudaMemsetAsync(ctx->d_med_n, 0, sizeof(int64_t), s));
-            kb::launch_classify(n, p.row, p.small_max, P.thr, const_cast<int32_t*>(p.med_v), ctx->d_med_n, s);
-            KB_CUDA(ctx, cudaGetLastError());
-            KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_med_n, ctx->d_med_n, sizeof(int64_t), cudaMemcpyDeviceToHost, s));
-            KB_CUDA(ctx, cudaStreamSynchronize(s));
-            p.n_med = *ctx->h_med_n;
-        }
+        // the plan's scratch still holds the classes (plan_classes)
+        const ClassScratch C(P);
+        const char* b = reinterpret_cast<const char*>(ctx->class_tmp);
+        kb::launch_class_list(n, p.row, reinterpret_cast<const uint32_t*>(b + P.class_bytes()),
+                              reinterpret_cast<const uint32_t*>(b + C.counts), 0, P.n_med, const_cast<int32_t*>(p.med_v),
+                              nullptr, s);
         if (P.freeze || P.graph_ext)  // laid out only then
-            kb::launch_edgeless_bits(n, p.row, reinterpret_cast<uint32_t*>(gws + P.o_edgeless), s);
+            KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_classes, b, 3 * P.class_bytes(), cudaMemcpyDeviceToDevice, s));
         KB_CUDA(ctx, cudaGetLastError());
     }
+    return KB_OK;
+}
+
+// Queue the validation of the caller's CSR.  Its verdict comes back with the
+// degree classes (plan_classes), which only read the offsets of an out-edge CSR;
+// before in-edges are counted it has to be known.
+kb_status check_input(kb_context* ctx, const kb_graph* g, const kb_options* opt) {
+    if (!opt->validate) return KB_OK;
+    const bool in = needs_in_csr(opt->direction);
+    kb::launch_validate(g->n, g->m, in ? g->row_offsets : nullptr, g->col_indices, ctx->d_ctr, ctx->stream);
+    KB_CUDA(ctx, cudaGetLastError());
+    if (!in) return KB_OK;
+    KB_TRY(read_counters(ctx));
+    return device_error(ctx);
+}
+
+// Queue the small-label minima of a level 0 (launch_dense_labels).
+kb_status check_small_labels(kb_context* ctx, int64_t n, const int32_t* key) {
+    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_dense, 0xff, sizeof(uint32_t) * kb::kDenseLabels, ctx->stream));
+    kb::launch_dense_labels(n, key, ctx->d_dense, ctx->d_ctr, ctx->stream);
+    KB_CUDA(ctx, cudaGetLastError());
     return KB_OK;
 }
 
 // Validate, plan, acquire the workspace, bind the round parameters, list the
 // medium vertices and reset the per-call state (block table, empty-signature
 // minima).  With a prepared graph (pg) only the per-call part is planned and
-// reset.  Synchronises.
+// reset.  key0: level 0's keys, or nullptr; without pg they are checked for the
+// small-label path in the plan's round trip.  Synchronises.
 kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Prepared& R, int rounds,
-                  bool multi = false, const kb_prepared* pg = nullptr) {
+                  bool multi = false, const kb_prepared* pg = nullptr, const int32_t* key0 = nullptr) {
     cudaStream_t s = ctx->stream;
     const int64_t n = g->n;
     KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
@@ -665,13 +702,11 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         csr = pg->csr;
         gws = pg->gbuf;
         KB_TRY(bind_graph_part(ctx, g, P, csr, gws, false, nullptr, p, s));
-        p.n_med = pg->n_med;
     } else {
-        if (opt->validate) {
-            kb::launch_validate(n, g->m, g->row_offsets, g->col_indices, ctx->d_ctr, s);
-            KB_CUDA(ctx, cudaGetLastError());
-            KB_TRY(read_counters(ctx));
-            KB_TRY(device_error(ctx));
+        KB_TRY(check_input(ctx, g, opt));
+        if (key0) {
+            R.key_checked = key0;
+            KB_TRY(check_small_labels(ctx, n, key0));
         }
         // The processed CSR sits at the head of the workspace, so its size is known
         // before the hub layout.
@@ -710,6 +745,7 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         csr = base;
         gws = ws;
         p.small_max = P.small_max;
+        R.key_dense = R.key_checked && ctx->h_ctr->dense_bad == 0;
         // the slot array serves as the count buffer of the locality order:
         // every round rewrites it
         KB_TRY(bind_graph_part(ctx, g, P, csr, gws, true, reinterpret_cast<uint32_t*>(ws + P.o_slot), p, s));
@@ -738,10 +774,6 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     if (P.reorder) p.gat = reinterpret_cast<int32_t*>(ws + P.o_gat);
     R.prefix = reinterpret_cast<uint2*>(ws + P.o_prefix);
     R.scan_tmp = reinterpret_cast<uint32_t*>(ws + P.o_scan);
-    if (P.dense0) {
-        R.dense_min = reinterpret_cast<uint32_t*>(ws + P.o_dense);
-        R.dense_pair = reinterpret_cast<uint2*>(ws + P.o_dense + align_up(sizeof(uint32_t) * kb::kDenseLabels));
-    }
     R.total_chunks = P.n_chunks;
     R.set_bytes = sizeof(uint64_t) * (size_t)P.set_slots;
     if (!R.ext_table) {
@@ -749,7 +781,9 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         R.epoch = 0;
     }
     if (P.freeze) {
-        R.edgeless = reinterpret_cast<uint32_t*>(gws + P.o_edgeless);
+        R.edgeless = reinterpret_cast<uint32_t*>(gws + P.o_classes);
+        R.medium_bits = P.n_med ? reinterpret_cast<uint32_t*>(gws + P.o_classes + P.class_bytes()) : nullptr;
+        R.hub_bits = P.n_hubs ? reinterpret_cast<uint32_t*>(gws + P.o_classes + 2 * P.class_bytes()) : nullptr;
         R.bm[0] = p.bitmap;
         R.bm[1] = reinterpret_cast<uint32_t*>(ws + P.o_bm2);
         R.bm_cur = 0;
@@ -797,9 +831,29 @@ kb_status next_epoch(kb_context* ctx, Prepared& R, cudaStream_t s) {
 // graphs in between, keeps them apart).
 uint32_t* next_minima(const Prepared& R) { return R.ext_frozen ? R.frozen_min : R.bm[R.bm_cur ^ 1]; }
 
+// The freeze pass after a signature round of one graph or a batch.
+kb::FreezePass freeze_pass(kb_context* ctx, const Prepared& R, const int32_t* level) {
+    kb::FreezePass f;
+    f.n = R.p.n;
+    f.bitmap = R.p.bitmap;
+    f.shared = R.p.shared;
+    f.edgeless = R.edgeless;
+    f.level = level;
+    f.mark = R.mark;
+    f.frozen = R.frozen;
+    f.frozen_min = next_minima(R);
+    f.moved_clear = R.p.perm ? R.moved : nullptr;
+    f.medium = R.medium_bits;
+    f.hub = R.hub_bits;
+    f.ctr = ctx->d_ctr;
+    return f;
+}
+
 // Starting level: canonical renumbering of `key` (labels or a given
 // partition; all-zero partition when key is NULL in a batched run).
-kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_t* out, cudaStream_t s) {
+// dense_path: set when the small-label path was taken.
+kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_t* out, cudaStream_t s,
+                        bool* dense_path = nullptr) {
     KB_TRY(next_epoch(ctx, R, s));
     KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
     KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
@@ -807,27 +861,36 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
     R.p.frozen = nullptr;
     R.p.frozen_min = nullptr;
     // small non-negative keys (one graph): each label's smallest vertex
-    // directly; the check for the range costs one host round trip
+    // directly; the check for the range costs one host round trip, unless it
+    // came with the plan's
     bool dense = false;
-    if (key && R.dense_min && !kb::batched(R.p) && R.p.n > 0) {
-        KB_CUDA(ctx, cudaMemsetAsync(R.dense_min, 0xff, sizeof(uint32_t) * kb::kDenseLabels, s));
-        kb::launch_dense_labels(R.p.n, key, R.dense_min, ctx->d_ctr, s);
-        KB_TRY(read_counters(ctx));
-        dense = ctx->h_ctr->dense_bad == 0;
+    if (key && R.P.dense0 && R.p.n > 0) {
+        if (key == R.key_checked) {
+            dense = R.key_dense;
+            R.key_checked = nullptr;
+        } else {
+            KB_TRY(check_small_labels(ctx, R.p.n, key));
+            KB_TRY(read_counters(ctx));
+            dense = ctx->h_ctr->dense_bad == 0;
+        }
     }
+    if (dense_path) *dense_path = dense;
     if (dense) {
-        kb::launch_dense_level0(R.p, key, R.dense_min, R.dense_pair, R.prefix, R.scan_tmp, out, s);
+        kb::launch_dense_level0(R.p, key, ctx->d_dense, reinterpret_cast<uint2*>(ctx->d_dense + kb::kDenseLabels),
+                                R.prefix, R.scan_tmp, out, s);
     } else {
         kb::launch_small_round(R.p, true, kb::SmallWindows::kConsecutive, s);
-        kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, nullptr, s);
+        kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, nullptr, false, s);
     }
     // a starting level may mix edgeless vertices with others in one block:
     // only its singletons are frozen in the first round
     if (R.p.shared) {
-        kb::launch_freeze_clean(R.p.n, R.p.bitmap, R.p.shared, nullptr, out, nullptr, R.frozen, next_minima(R), nullptr,
-                                ctx->d_ctr, s);
+        kb::FreezePass f = freeze_pass(ctx, R, out);
+        f.edgeless = nullptr;
+        f.mark = nullptr;
+        f.moved_clear = nullptr;
+        kb::launch_freeze_clean(f, s);
         R.bitmap_ready = !R.ext_frozen;
-        kb::launch_count_refining(R.p, R.frozen, ctx->d_ctr, s);
     }
     KB_CUDA(ctx, cudaGetLastError());
     return KB_OK;
@@ -931,7 +994,8 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     ctx->round_keyed.clear();
     RowCopyGuard copies{rows.host ? ctx->copy_stream : nullptr};
     Prepared R;
-    KB_TRY(prepare(ctx, g, opt, R, k - i_start, false, pg));
+    const int32_t* init_key = start ? start : (opt->use_vertex_labels ? g->vertex_labels : nullptr);
+    KB_TRY(prepare(ctx, g, opt, R, k - i_start, false, pg, opt->subject == KB_SUBJECT_LABEL ? nullptr : init_key));
     kb::RoundParams& p = R.p;
 
     // ---- the subject part of every key (generic CSE rounds)
@@ -952,18 +1016,27 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
 
     // ---- the starting level
     int32_t* row0 = rows.row(i_start);
-    const int32_t* init_key = start ? start : (opt->use_vertex_labels ? g->vertex_labels : nullptr);
     int64_t prev_count = 1;
+    bool count_known = true;  // the starting level's block count is on the host
     if (init_key) {
-        KB_TRY(launch_level0(ctx, R, init_key, row0, s));
-        KB_TRY(read_counters(ctx));
-        KB_TRY(device_error(ctx));
-        prev_count = ctx->h_ctr->count;
-        R.compact = R.P.freeze && ctx->h_ctr->frozen * 4 > n;
-        R.sparse = R.P.freeze && (n - ctx->h_ctr->frozen) * 64 < n;
-        R.med_on = ctx->h_ctr->med_on > 0;
-        R.hub_on = ctx->h_ctr->hub_on > 0;
+        bool dense = false;
+        KB_TRY(launch_level0(ctx, R, init_key, row0, s, &dense));
+        // At most kDenseLabels blocks after the small-label path: how many are
+        // frozen decides nothing about the first round, and the count comes
+        // back with that round's.
+        count_known = !(dense && R.P.freeze && !ctx->work && k > i_start);
+        if (count_known) {
+            KB_TRY(read_counters(ctx));
+            KB_TRY(device_error(ctx));
+            prev_count = ctx->h_ctr->count;
+            R.compact = R.P.freeze && ctx->h_ctr->frozen * 4 > n;
+            R.sparse = R.P.freeze && (n - ctx->h_ctr->frozen) * 64 < n;
+            R.med_on = ctx->h_ctr->med_on > 0;
+            R.hub_on = ctx->h_ctr->hub_on > 0;
+        }
     } else {
+        // the count's low byte, for the rounds that compare with the previous one
+        KB_CUDA(ctx, cudaMemsetAsync(&ctx->d_ctr->count, 1, 1, s));
         kb::launch_fill_i32(row0, n, 0, s);
         if (p.perm) kb::launch_fill_i32(p.gat, n, 0, s);
         if (p.minof) {
@@ -979,7 +1052,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     KB_TRY(emit_rows(ctx, rows, i_start, i_start));
 
     // ---- refinement rounds
-    R.counters_clear = !ctx->work && !R.P.subject;
+    R.counters_clear = !R.P.subject;
     for (int i = i_start + 1; i <= k; ++i) {
         Timer T(ctx);
         KB_TRY(next_epoch(ctx, R, s));
@@ -997,22 +1070,25 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         }
         int32_t* out = rows.row(i);
         KB_TRY(launch_round_body(ctx, R, s, &T));
-        if (ctx->work) kb::launch_round_work(p, s);
+        if (ctx->work) {
+            KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr->keyed_v, 0, 6 * sizeof(int64_t), s));
+            kb::launch_round_work(p, s);
+        }
         T.begin(KB_KERNEL_RENUMBER);
         // under early stop a round that keeps the count is the last one
-        const int64_t stable = (opt->early_stop || fixpoint) && !R.P.subject ? prev_count : -1;
-        kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, s, stable);
+        const bool stop_stable = (opt->early_stop || fixpoint) && p.minof;
+        kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, stop_stable, s);
         if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
         // the next round's frozen blocks: singletons; a block formed by this
         // round that holds an edgeless vertex holds only edgeless vertices with
         // one previous block; and clean blocks, none of whose members has an
         // edge to a vertex whose smallest block member this round changed
         if (p.shared && i < k) {
-            kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, s, stable);
-            kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen, next_minima(R),
-                                    p.perm ? R.moved : nullptr, ctx->d_ctr, s, nullptr, nullptr, stable);
+            kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, stop_stable, s);
+            kb::FreezePass f = freeze_pass(ctx, R, out);
+            f.stop_stable = stop_stable;
+            kb::launch_freeze_clean(f, s);
             R.bitmap_ready = true;
-            kb::launch_count_refining(p, R.frozen, ctx->d_ctr, s);
         }
         T.end();
         // CSE levels need not refine each other: compare whole levels
@@ -1032,6 +1108,11 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         ctx->round_ms.push_back(T.collect());
         KB_TRY(device_error(ctx));
         const int64_t c = ctx->h_ctr->count;
+        if (!count_known) {
+            prev_count = ctx->h_ctr->prev_count;
+            if (counts) counts[i_start] = prev_count;
+            count_known = true;
+        }
         if (counts) counts[i] = c;
         if (last_count) *last_count = c;
         if (levels_computed) *levels_computed = i;
@@ -1133,7 +1214,8 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
 
     Prepared R;
     // no locality order: the dirty pass reads neighbour ids, not ranks
-    KB_TRY(prepare(ctx, g, opt, R, -1));
+    const int32_t* init_key = opt->use_vertex_labels ? g->vertex_labels : nullptr;
+    KB_TRY(prepare(ctx, g, opt, R, -1, false, nullptr, init_key));
     kb::RoundParams& p = R.p;
     uint32_t* changed_bits = reinterpret_cast<uint32_t*>(b);
     uint32_t* dirty = reinterpret_cast<uint32_t*>(b + szb);
@@ -1157,7 +1239,6 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         return fail(ctx, KB_ERR_INVALID_ARG, "old levels or changed vertices hold ids outside [0, n)");
 
     // level 0 from scratch; its moved vertices start the dirty set
-    const int32_t* init_key = opt->use_vertex_labels ? g->vertex_labels : nullptr;
     if (init_key) {
         KB_TRY(launch_level0(ctx, R, init_key, level0, s));
         KB_TRY(read_counters(ctx));
@@ -1196,7 +1277,7 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_TRY(launch_round_body(ctx, R, s, &T));
         kb::launch_keep_bits(n, wmask, keep, kmin, p.bitmap, s);
         T.begin(KB_KERNEL_RENUMBER);
-        kb::launch_renumber(p, R.prefix, R.scan_tmp, row(i), nullptr, s);
+        kb::launch_renumber(p, R.prefix, R.scan_tmp, row(i), nullptr, false, s);
         T.end();
         kb::launch_moved(n, wmask, keep, row(i), ranges, moved, s);
         kb::launch_count_bits(moved, nw, &ctx->d_ctr->moved, s);
@@ -1475,11 +1556,12 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
             st = launch_round_body(ctx, R, cs, nullptr);
             if (st != KB_OK) break;
             kb::launch_carry_minima(p, cs);
-            kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, cs);
+            kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, false, cs);
             if (p.shared && i < kmax) {
-                kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, cs);
-                kb::launch_freeze_clean(n, p.bitmap, p.shared, R.edgeless, out, R.mark, R.frozen,
-                                        (i & 1) ? bm_a : bm_b, nullptr, ctx->d_ctr, cs);
+                kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, false, cs);
+                kb::FreezePass f = freeze_pass(ctx, R, out);
+                f.frozen_min = (i & 1) ? bm_a : bm_b;
+                kb::launch_freeze_clean(f, cs);
                 R.bitmap_ready = true;
             }
             kb::launch_graph_stop(p, i, kd, early, gact, glast, sticky, cs);
@@ -2039,16 +2121,16 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         p.moved = sv->history ? sv->R.moved : nullptr;
         SV_TRY(sv, launch_round_body(ctx, sv->R, s, nullptr));
         kb::launch_carry_minima(p, s);
-        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, out, p.moved ? sv->R.mark : nullptr, s);
+        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, out, p.moved ? sv->R.mark : nullptr, false, s);
         kb::launch_emit(sv->n_used, sv->vgraph, out, p.gbase_cur, sv->slot_levels, sv->slot_row, sv->slot_n, sv->voff, s);
         if (p.shared) {
-            const uint32_t* mark = nullptr;
-            if (p.moved) {
-                kb::launch_dirty_blocks(p, sv->R.edgeless, sv->R.moved, out, kb::kMaxHubThreshold, sv->R.mark, s);
-                mark = sv->R.mark;
-            }
-            kb::launch_freeze_clean(sv->n_used, p.bitmap, p.shared, sv->R.edgeless, out, mark, sv->R.frozen,
-                                    sv->R.frozen_min, nullptr, ctx->d_ctr, s, sv->vgraph, sv->gmode);
+            if (p.moved)
+                kb::launch_dirty_blocks(p, sv->R.edgeless, sv->R.moved, out, kb::kMaxHubThreshold, sv->R.mark, false, s);
+            kb::FreezePass f = freeze_pass(ctx, sv->R, out);
+            f.mark = p.moved ? sv->R.mark : nullptr;
+            f.vgraph = sv->vgraph;
+            f.gmode = sv->gmode;
+            kb::launch_freeze_clean(f, s);
         }
         sv->history = true;
         SV_CUDA(sv, cudaGetLastError());
@@ -2145,11 +2227,9 @@ kb_status kb_create(kb_context** out, int device, void* stream) {
     ctx->device = device;
     ctx->stream = reinterpret_cast<cudaStream_t>(stream);
     if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&ctx->d_ctr, sizeof(Counters)) != cudaSuccess ||
-        cudaMalloc(&ctx->d_hub_n, sizeof(int32_t)) != cudaSuccess ||
-        cudaMalloc(&ctx->d_med_n, sizeof(int64_t)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_med_n, sizeof(int64_t)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_ctr, sizeof(Counters)) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_hub_n, sizeof(int32_t)) != cudaSuccess) {
+        cudaMalloc(&ctx->d_dense, (sizeof(uint32_t) + sizeof(uint2)) * kb::kDenseLabels) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_hubs, (sizeof(int32_t) + sizeof(int64_t)) * kEagerHubs) != cudaSuccess ||
+        cudaMallocHost(&ctx->h_ctr, sizeof(Counters)) != cudaSuccess) {
         cudaGetLastError();
         kb_destroy(ctx);
         return KB_ERR_CUDA;
@@ -2166,13 +2246,11 @@ kb_status kb_destroy(kb_context* ctx) {
     cudaSetDevice(ctx->device);
     if (ctx->stream) cudaStreamSynchronize(ctx->stream); else cudaDeviceSynchronize();
     cudaFree(ctx->d_ctr);
-    cudaFree(ctx->d_hub_n);
-    cudaFree(ctx->d_med_n);
-    cudaFreeHost(ctx->h_med_n);
+    cudaFree(ctx->d_dense);
+    cudaFreeHost(ctx->h_hubs);
     cudaFreeHost(ctx->h_ctr);
-    cudaFreeHost(ctx->h_hub_n);
     cudaFree(ctx->own_ws);
-    cudaFree(ctx->hub_tmp);
+    cudaFree(ctx->class_tmp);
     cudaFree(ctx->plan_tmp);
     cudaFree(ctx->stage);
     cudaFree(ctx->batch_ws);
@@ -2203,6 +2281,7 @@ kb_status kb_workspace_size(kb_context* ctx, const kb_graph* g, const kb_options
     }
     Plan P;
     char* unused = nullptr;
+    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), ctx->stream));
     KB_TRY(make_plan(ctx, g, opt, P, &unused, true, k));
     *bytes = P.total;
     return KB_OK;
@@ -2243,12 +2322,7 @@ kb_status kb_graph_prepare(kb_context* ctx, const kb_graph* g, const kb_options*
     pg->edge_labels = opt->use_edge_labels ? 1 : 0;
     const int64_t n = g->n;
     KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-    if (opt->validate && n > 0) {
-        kb::launch_validate(n, g->m, g->row_offsets, g->col_indices, ctx->d_ctr, s);
-        KB_CUDA(ctx, cudaGetLastError());
-        KB_TRY(read_counters(ctx));
-        KB_TRY(device_error(ctx));
-    }
+    if (n > 0) KB_TRY(check_input(ctx, g, opt));
     Plan& P = pg->P;
     P.graph_ext = true;
     Plan probe;
@@ -2282,13 +2356,11 @@ kb_status kb_graph_prepare(kb_context* ctx, const kb_graph* g, const kb_options*
         cudaFree(count_tmp);
         KB_TRY(st);
         if (e != cudaSuccess) return fail(ctx, KB_ERR_CUDA, "prepare: %s", cudaGetErrorString(e));
-        pg->n_med = p.n_med;
     }
     // the hub lists are on the device now
     std::vector<int32_t>().swap(P.hub_v);
     std::vector<int64_t>().swap(P.chunk_off);
     std::vector<int64_t>().swap(P.set_off);
-    std::vector<int32_t>().swap(P.chunk_hub);
     pg->build_ms = std::chrono::duration<float, std::milli>(std::chrono::steady_clock::now() - t0).count();
     *out = pg.release();
     return KB_OK;
@@ -2305,7 +2377,7 @@ kb_status kb_prepared_get_info(const kb_prepared* pg, kb_prepared_info* info) {
     info->device_bytes = (pg->csr ? pg->P.csr_bytes : 0) + pg->P.graph_bytes;
     info->n_hubs = (int64_t)pg->P.n_hubs;
     info->n_hub_chunks = pg->P.n_chunks;
-    info->n_medium = pg->n_med;
+    info->n_medium = pg->P.n_med;
     info->reorder = pg->P.reorder ? 1 : 0;
     info->hub_threshold = pg->P.thr;
     info->small_max_degree = pg->P.small_max;

@@ -40,14 +40,17 @@ struct Counters {
     int32_t diff;   // set when two compared levels differ (launch_levels_differ)
     int64_t count;  // blocks at the level just assigned
     int64_t frozen; // vertices frozen for the next round (launch_freeze_clean)
-    int64_t med_on; // medium vertices that refine next round (launch_count_refining)
-    int64_t hub_on; // hubs that refine next round (launch_count_refining)
+    int64_t med_on; // medium vertices that refine next round (launch_freeze_clean)
+    int64_t hub_on; // hubs that refine next round (launch_freeze_clean)
     int64_t moved;  // re-keyed vertices whose smallest block member changed (renumbering)
     // vertices re-keyed this round and their edges in the processed
     // direction, per kernel family: small, medium, hub
     int64_t keyed_v[3];
     int64_t keyed_e[3];
     int32_t dense_bad;  // a level-0 key outside [0, kDenseLabels) (launch_dense_labels)
+    int64_t prev_count; // blocks at the level before
+    int64_t n_med;      // medium vertices and hubs of the graph (launch_classes)
+    int64_t n_hubs;
 };
 
 // Everything one refinement round reads and writes.
@@ -222,35 +225,42 @@ void launch_clear_hubs(const RoundParams& p, int64_t total_slots, cudaStream_t s
 // level-i id; a vertex above max_scan edges counts as such).  Only vertices
 // that are neither alone in their block (bitmap & ~shared) nor edgeless are
 // scanned, and nothing when more than an eighth of the vertices moved.
-// stable_count >= 0: the pass does nothing when this round's count equals it
-// (a stable round under early stop is the last one).
+// stop_stable: the pass does nothing after a round that kept the block count (a
+// stable round under early stop is the last one).
 void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,
-                         int32_t max_scan, uint32_t* mark, cudaStream_t s, int64_t stable_count = -1);
-// After the renumbering (single-graph stratified rounds): the frozen blocks
-// of the next round.  A vertex is frozen when it is alone in its block (a
-// minimum in bitmap that no other vertex marked in shared), edgeless
-// (edgeless != null: from the first signature round on, a block holding an
-// edgeless vertex holds only edgeless vertices with one previous block), or
-// in a level-i block without a mark bit (mark != null, unless more than an
-// eighth of the vertices moved).  frozen_min receives the minima of frozen
-// blocks; shared keeps exactly their marks; ctr->frozen counts the frozen
-// vertices.  moved_clear (or nullptr): a bitmap to clear.
-// Serving (vgraph, gmode given): the vertices of graphs that computed their
-// level 0 in this step are not frozen by the edgeless rule.
-void launch_freeze_clean(int64_t n, const uint32_t* bitmap, uint32_t* shared, const uint32_t* edgeless,
-                         const int32_t* level, const uint32_t* mark, uint32_t* frozen, uint32_t* frozen_min,
-                         uint32_t* moved_clear, Counters* ctr, cudaStream_t s, const int32_t* vgraph = nullptr,
-                         const uint8_t* gmode = nullptr, int64_t stable_count = -1);
+                         int32_t max_scan, uint32_t* mark, bool stop_stable, cudaStream_t s);
+// After the renumbering (stratified rounds): the frozen blocks of the next
+// round.  A vertex is frozen when it is alone in its block (a minimum in bitmap
+// without a mark in shared), edgeless (edgeless != null: from the first
+// signature round on, a block holding an edgeless vertex holds only edgeless
+// vertices with one previous block), or in a level-i block without a mark bit
+// (mark != null, unless more than an eighth of the vertices moved).
+struct FreezePass {
+    int64_t n = 0;
+    const uint32_t* bitmap = nullptr;    // block minima of the level
+    uint32_t* shared = nullptr;          // in: minima of blocks of several vertices; out: exactly the frozen ones
+    const uint32_t* edgeless = nullptr;
+    const int32_t* level = nullptr;
+    const uint32_t* mark = nullptr;
+    uint32_t* frozen = nullptr;          // out: frozen vertices, counted in ctr->frozen
+    uint32_t* frozen_min = nullptr;      // out: the minima of frozen blocks
+    uint32_t* moved_clear = nullptr;     // a bitmap to clear, or nullptr
+    const uint32_t* medium = nullptr;    // degree classes: those not frozen are counted in ctr->med_on and hub_on
+    const uint32_t* hub = nullptr;       //   (nullptr: an empty class)
+    Counters* ctr = nullptr;
+    // serving: the vertices of graphs that computed their level 0 in this step
+    // (gmode) are not frozen by the edgeless rule
+    const int32_t* vgraph = nullptr;
+    const uint8_t* gmode = nullptr;
+    bool stop_stable = false;            // a round that kept the count is the last one: nothing to do after it
+    int per_warp = 32;                   // bitmap words per warp (set by the launcher)
+};
+void launch_freeze_clean(const FreezePass& f, cudaStream_t s);
 // Clear bits a..b-1 of a bitmap.
 void launch_clear_bits(uint32_t* words, int64_t a, int64_t b, cudaStream_t s);
 // The vertices this round re-keys (not in p.frozen) and their edges, per
 // kernel family, into ctr->keyed_v / keyed_e (work accounting only).
 void launch_round_work(const RoundParams& p, cudaStream_t s);
-// After launch_freeze_clean: the medium vertices and hubs that are not frozen, into
-// ctr->med_on and ctr->hub_on (their kernels are skipped when none refine).
-void launch_count_refining(const RoundParams& p, const uint32_t* frozen, Counters* ctr, cudaStream_t s);
-// Bit v set iff v has no edges in the processed CSR.
-void launch_edgeless_bits(int64_t n, const int64_t* row, uint32_t* bits, cudaStream_t s);
 // Windows of consecutive vertices, or packed from the vertices that refine
 // (kCompact: worth it when many are frozen; kSparse: nearly all are).
 enum class SmallWindows { kConsecutive, kCompact, kSparse };
@@ -265,11 +275,11 @@ void launch_hub_final(const RoundParams& p, cudaStream_t s);
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
 // The frozen, med_on, hub_on and moved counters restart at 0; with frozen
 // blocks moved vertices are counted, and mark (or nullptr) is cleared.
-// stable_count >= 0 (frozen-block rounds under early stop): in a round whose
-// count equals it (the last round) the ids are those of the previous level, and
-// out is left for the caller to copy.
+// stop_stable (frozen-block rounds under early stop): in a round that kept the
+// block count (the last round) the ids are those of the previous level, and out
+// is left for the caller to copy.
 void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
-                     cudaStream_t s, int64_t stable_count = -1);
+                     bool stop_stable, cudaStream_t s);
 size_t scan_tmp_words(int64_t n_items);
 // Level 0 of one graph whose keys (vertex labels, or a starting partition)
 // are all in [0, kDenseLabels): the label partition straight from each
@@ -297,6 +307,7 @@ void launch_localize(int32_t* row, int64_t n, const int32_t* vgraph, const uint3
 void launch_vertex_graph(const int64_t* voff, int32_t G, int64_t n, int32_t* vgraph, cudaStream_t s);
 
 // Setup (kb_setup.cu)
+// Neighbour ids in [0, n); with row also offsets monotone from 0 to m.
 void launch_validate(int64_t n, int64_t m, const int64_t* row, const int32_t* col, Counters* ctr,
                      cudaStream_t s);
 // in-degree histogram: deg[w] += 1 per edge (deg must be zeroed)
@@ -309,14 +320,23 @@ size_t scan_i64_tmp(int64_t n);
 void launch_build_csr(int64_t n, int64_t m, const int64_t* row, const int32_t* col, const int32_t* lab,
                       const int64_t* in_prefix, int include_out, int64_t* row_p, int32_t* col_p,
                       int32_t* lab_p, int64_t* cursor, cudaStream_t s);
-// Compact the vertices with more than thr edges (unordered) into out_v with
-// their degrees in out_deg; count in *n_out.
-void launch_find_hubs(int64_t n, const int64_t* row, int32_t thr, int32_t* out_v, int64_t* out_deg,
-                      int32_t* n_out, cudaStream_t s);
-// Append the vertices with lo < degree <= hi to out (order within a warp
-// preserved); count in *n_out.
-void launch_chunk_ext(int64_t chunks, const int32_t* chunk_hub, const int32_t* hub_v, const int64_t* chunk_off,
-                      const int64_t* row, int32_t chunk, uint64_t* out, cudaStream_t s);
+// Degree classes of the processed CSR: bitmaps of (n >> 5) + 1 words of the
+// vertices without edges, with lo < degree <= hi (medium) and above (hubs),
+// their numbers in ctr->n_med and n_hubs, and both per tile in tile_counts (two
+// words per tile, class_tiles(n) tiles).  check: report offsets out of order
+// (kOrder), or also not from 0 to m (kAll), in ctr->err.
+enum class CheckRows { kNone, kOrder, kAll };
+size_t class_tiles(int64_t n);
+void launch_classes(int64_t n, int64_t m, const int64_t* row, int32_t lo, int32_t hi, uint32_t* edgeless,
+                    uint32_t* medium, uint32_t* hub, uint32_t* tile_counts, CheckRows check, Counters* ctr,
+                    cudaStream_t s);
+// The vertices of a class (which: 0 medium, 1 hub), ascending, at most cap of
+// them, with their degrees unless deg is nullptr.
+void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, const uint32_t* tile_counts, int which,
+                       int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s);
+// Hub and packed extent of every hub chunk (RoundParams::chunk_hub, chunk_ext).
+void launch_chunk_ext(int64_t chunks, int32_t n_hubs, const int32_t* hub_v, const int64_t* chunk_off,
+                      const int64_t* row, int32_t chunk, int32_t* chunk_hub, uint64_t* out, cudaStream_t s);
 void launch_locality_order(int64_t n, int64_t m, const int32_t* col, uint32_t* cnt, unsigned long long* hist,
                            int32_t* perm, cudaStream_t s);
 void launch_remap_cols(int64_t m, const int32_t* col, const int32_t* perm, int32_t* out, cudaStream_t s);
@@ -366,8 +386,6 @@ void launch_touched_size(int64_t n, int64_t count, const int32_t* ids, const int
 // *out += set bits of words[0..nw) (kb_kernels.cu)
 void launch_count_bits(const uint32_t* words, int64_t nw, int64_t* out, cudaStream_t s);
 void launch_set_bits(int64_t n, int64_t count, const int32_t* ids, uint32_t* bits, Counters* ctr, cudaStream_t s);
-void launch_classify(int64_t n, const int64_t* row, int32_t lo, int32_t hi, int32_t* out, int64_t* n_out,
-                     cudaStream_t s);
 // Copy row src of the level store to the rows [first, last] of levels (src not among them).
 void launch_copy_rows(int32_t* levels, int64_t n, int src, int first, int last, cudaStream_t s);
 

@@ -397,6 +397,7 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
     ex += s_before;
     if (blockIdx.x == gridDim.x - 1 && threadIdx.x == 0) {
         const uint32_t all = s_before + total;
+        ctr->prev_count = ctr->count;
         ctr->count = (int64_t)all;
         ctr->frozen = 0;
         ctr->med_on = 0;
@@ -472,11 +473,10 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
 // the vertex that inserted its table entry (RoundParams::joined).  moved may be
 // null (the starting level); mark, when given, is cleared for the dirty pass.
 __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p, const uint2* rank, int32_t* out,
-                                                             uint32_t* moved, uint32_t* mark,
-                                                             int64_t stable_count) {
+                                                             uint32_t* moved, uint32_t* mark, bool stop_stable) {
     // a round that kept the block count kept every block (blocks only split):
     // under early stop it is the last one, and the caller copies the level
-    if (stable_count >= 0 && p.ctr->count == stable_count) return;
+    if (stop_stable && p.ctr->count == p.ctr->prev_count) return;
     __shared__ uint32_t s_moved;
     if (threadIdx.x == 0) s_moved = 0u;
     __syncthreads();
@@ -583,9 +583,9 @@ __device__ __forceinline__ bool few_moved(const RoundParams& p) { return p.ctr->
 __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, const uint32_t* edgeless,
                                                             const uint32_t* moved, const int32_t* level,
                                                             int32_t max_scan, uint32_t* mark, int per_warp,
-                                                            int64_t stable_count) {
+                                                            bool stop_stable) {
     if (!few_moved(p)) return;
-    if (stable_count >= 0 && p.ctr->count == stable_count) return;  // the last round: nothing follows
+    if (stop_stable && p.ctr->count == p.ctr->prev_count) return;  // the last round: nothing follows
     const int lane = threadIdx.x & 31;
     const int64_t nw = (p.n >> 5) + 1;
     const int64_t w0 = ((int64_t)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * per_warp;
@@ -622,26 +622,24 @@ __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, 
     }
 }
 
-// The frozen blocks of the next round: a vertex is frozen when it is alone in
-// its block (a minimum that no other vertex marked shared), edgeless
-// (edgeless != null), or in a level-i block without a mark bit (mark != null
-// and no more than an eighth of the vertices moved).  frozen_min holds the
+// The frozen blocks of the next round (see FreezePass).  frozen_min holds the
 // minima of frozen blocks, and the shared marks of exactly those minima are
 // kept for the next round (their blocks keep their members; the others are
 // marked afresh).  A warp takes up to 32 bitmap words and deals the candidates
 // whose block it must look up to its lanes, as dirty_blocks_kernel does.
-// moved_clear, when given, is a bitmap that starts the next round empty.
-__global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint32_t* bitmap, uint32_t* shared,
-                                                            const uint32_t* edgeless, const int32_t* level,
-                                                            const uint32_t* mark, uint32_t* frozen,
-                                                            uint32_t* frozen_min, uint32_t* moved_clear, int per_warp,
-                                                            Counters* ctr, const int32_t* vgraph,
-                                                            const uint8_t* gmode, int64_t stable_count) {
+__global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
     __shared__ uint32_t s_clean[8][32];
-    __shared__ uint32_t s_frozen;
-    if (stable_count >= 0 && ctr->count == stable_count) return;  // the last round: nothing follows
-    if (threadIdx.x == 0) s_frozen = 0u;
+    __shared__ uint32_t s_on[3];  // frozen vertices, refining medium vertices and hubs of this CTA
+    Counters* ctr = f.ctr;
+    if (f.stop_stable && ctr->count == ctr->prev_count) return;  // the last round: nothing follows
+    if (threadIdx.x < 3) s_on[threadIdx.x] = 0u;
     __syncthreads();
+    const int64_t n = f.n;
+    const int per_warp = f.per_warp;
+    const uint32_t* bitmap = f.bitmap;
+    uint32_t* shared = f.shared;
+    const uint32_t* edgeless = f.edgeless;
+    const uint32_t* mark = f.mark;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t nw = (n >> 5) + 1;
     // a warp past the end keeps to the barriers with no words of its own
@@ -656,13 +654,13 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint
         e = edgeless ? edgeless[w] : 0u;
         c = mark ? candidate_word(bitmap, shared, edgeless, w, n) : 0u;
     }
-    if (gmode && edgeless) {
+    if (f.gmode && edgeless) {
         // serving: a graph that computed its level 0 in this step has not had
         // its edgeless blocks formed by a round yet
         for (int j = 0; j < 32; ++j) {
             const uint32_t ej = __shfl_sync(kFull, e, j);
             const int64_t vj = (w0 + j) * 32 + lane;
-            const bool lvl0 = vj < n && ((ej >> lane) & 1u) && gmode[vgraph[vj]] == 1;
+            const bool lvl0 = vj < n && ((ej >> lane) & 1u) && f.gmode[f.vgraph[vj]] == 1;
             const uint32_t drop = __ballot_sync(kFull, lvl0);
             if (lane == j) {
                 e &= ~drop;
@@ -685,7 +683,7 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint
     for (int t = 0; t < total; t += 32) {
         const int64_t v = dealt_vertex(w0, excl, c, t + lane, total);
         if (v < 0) continue;
-        const uint32_t l = (uint32_t)level[v];
+        const uint32_t l = (uint32_t)f.level[v];
         if (!((mark[l >> 5] >> (l & 31)) & 1u)) atomicOr(&s_clean[warp][(v >> 5) - w0], 1u << (v & 31));
     }
     __syncwarp();
@@ -696,15 +694,21 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(int64_t n, const uint
         const uint32_t cl = s_clean[warp][lane];
         const uint32_t fz = single | (e & valid) | cl;
         const uint32_t fm = single | (b & (e | cl) & valid);
-        frozen[w] = fz;
-        frozen_min[w] = fm;
+        f.frozen[w] = fz;
+        f.frozen_min[w] = fm;
         shared[w] = sh & fm;
-        if (moved_clear) moved_clear[w] = 0u;
-        if (fz) atomicAdd(&s_frozen, (uint32_t)__popc(fz));
+        if (f.moved_clear) f.moved_clear[w] = 0u;
+        if (fz) atomicAdd(&s_on[0], (uint32_t)__popc(fz));
+        const uint32_t md = f.medium ? f.medium[w] & ~fz : 0u;
+        const uint32_t hb = f.hub ? f.hub[w] & ~fz : 0u;
+        if (md) atomicAdd(&s_on[1], (uint32_t)__popc(md));
+        if (hb) atomicAdd(&s_on[2], (uint32_t)__popc(hb));
     }
     __syncthreads();
-    if (threadIdx.x == 0 && s_frozen)
-        atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->frozen), (unsigned long long)s_frozen);
+    if (threadIdx.x < 3 && s_on[threadIdx.x]) {
+        int64_t* dst = threadIdx.x == 0 ? &ctr->frozen : (threadIdx.x == 1 ? &ctr->med_on : &ctr->hub_on);
+        atomicAdd(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)s_on[threadIdx.x]);
+    }
 }
 
 // The vertices a round re-keys (those not in frozen; all when frozen is null)
@@ -763,36 +767,6 @@ __global__ void __launch_bounds__(256) count_bits_kernel(const uint32_t* words, 
         unsigned long long t = 0;
         for (int w = 0; w < 8; ++w) t += s_sum[w];
         if (t) atomicAdd(reinterpret_cast<unsigned long long*>(out), t);
-    }
-}
-
-__global__ void count_refining_kernel(const int32_t* med_v, int64_t n_med, const int32_t* hub_v, int64_t n_hubs,
-                                      const uint32_t* frozen, Counters* ctr) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long cm = 0, ch = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_med + n_hubs; i += stride) {
-        const int32_t v = i < n_med ? med_v[i] : hub_v[i - n_med];
-        const bool on = !((frozen[v >> 5] >> (v & 31)) & 1u);
-        if (i < n_med) cm += on; else ch += on;
-    }
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-        cm += __shfl_xor_sync(kFull, cm, o);
-        ch += __shfl_xor_sync(kFull, ch, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (cm) atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->med_on), cm);
-        if (ch) atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->hub_on), ch);
-    }
-}
-
-__global__ void edgeless_bits_kernel(int64_t n, const int64_t* row, uint32_t* bits) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < n; base += stride) {
-        const int64_t v = base + threadIdx.x;  // blockDim is a multiple of 32: a warp covers one word
-        const bool e = v < n && row[v + 1] == row[v];
-        const unsigned w = __ballot_sync(kFull, e);
-        if ((threadIdx.x & 31) == 0 && (v >> 5) <= (n >> 5)) bits[v >> 5] = w;
     }
 }
 
@@ -1047,26 +1021,22 @@ static int words_per_warp(int64_t nw) {
 }
 
 void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,
-                         int32_t max_scan, uint32_t* mark, cudaStream_t s, int64_t stable_count) {
+                         int32_t max_scan, uint32_t* mark, bool stop_stable, cudaStream_t s) {
     if (p.n <= 0) return;
     const int64_t nw = (p.n >> 5) + 1;
     const int per = words_per_warp(nw);
     const int64_t warps = (nw + per - 1) / per;
     dirty_blocks_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(p, edgeless, moved, level, max_scan, mark, per,
-                                                                     stable_count);
+                                                                     stop_stable);
 }
 
-void launch_freeze_clean(int64_t n, const uint32_t* bitmap, uint32_t* shared, const uint32_t* edgeless,
-                         const int32_t* level, const uint32_t* mark, uint32_t* frozen, uint32_t* frozen_min,
-                         uint32_t* moved_clear, Counters* ctr, cudaStream_t s, const int32_t* vgraph,
-                         const uint8_t* gmode, int64_t stable_count) {
-    if (n <= 0) return;
-    const int64_t nw = (n >> 5) + 1;
-    const int per = words_per_warp(nw);
-    const int64_t warps = (nw + per - 1) / per;
-    freeze_clean_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(n, bitmap, shared, edgeless, level, mark, frozen,
-                                                                     frozen_min, moved_clear, per, ctr, vgraph, gmode,
-                                                                     stable_count);
+void launch_freeze_clean(const FreezePass& f, cudaStream_t s) {
+    if (f.n <= 0) return;
+    const int64_t nw = (f.n >> 5) + 1;
+    FreezePass g = f;
+    g.per_warp = words_per_warp(nw);
+    const int64_t warps = (nw + g.per_warp - 1) / g.per_warp;
+    freeze_clean_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(g);
 }
 
 void launch_round_work(const RoundParams& p, cudaStream_t s) {
@@ -1084,16 +1054,6 @@ void launch_clear_bits(uint32_t* words, int64_t a, int64_t b, cudaStream_t s) {
     if (b <= a) return;
     const int64_t w0 = a >> 5, w1 = (b - 1) >> 5;
     clear_bits_kernel<<<grid_for(w1 - w0 + 1, 256), 256, 0, s>>>(words, a, b);
-}
-
-void launch_count_refining(const RoundParams& p, const uint32_t* frozen, Counters* ctr, cudaStream_t s) {
-    const int64_t items = p.n_med + p.n_hubs;
-    if (items > 0)
-        count_refining_kernel<<<grid_for(items, 256), 256, 0, s>>>(p.med_v, p.n_med, p.hub_v, p.n_hubs, frozen, ctr);
-}
-
-void launch_edgeless_bits(int64_t n, const int64_t* row, uint32_t* bits, cudaStream_t s) {
-    if (n > 0) edgeless_bits_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, row, bits);
 }
 
 void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s) {
@@ -1119,13 +1079,13 @@ void launch_bitmap_rank(const uint32_t* bitmap, int64_t nw, uint32_t* scan_tmp, 
 }
 
 void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
-                     cudaStream_t s, int64_t stable_count) {
+                     bool stop_stable, cudaStream_t s) {
     const int64_t nw = (p.n >> 5) + 1;
     rank_scan(p.bitmap, nw, scan_tmp, nullptr, rank, batched(p), p.ctr, s);
     if (batched(p)) graph_base_kernel<<<(p.n_graphs + 1 + 255) / 256, 256, 0, s>>>(p, rank);
     if (p.n <= 0) return;
     if (p.minof)
-        assign_frozen_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out, p.moved, mark, stable_count);
+        assign_frozen_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out, p.moved, mark, stop_stable);
     else
         assign_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out);
 }

@@ -1,6 +1,6 @@
 // kb_refine_round_noalloc: one refinement round that allocates no device
 // memory.  Its scratch (block table, slot per vertex, empty-signature minima,
-// bitmap of block minima and its prefix, medium-vertex list, counters) lives
+// bitmap of block minima and its prefix, degree classes, counters) lives
 // in one file-scope device array of fixed size, shared by every call on a
 // device and kept until the process exits.
 #include <cuda_runtime.h>
@@ -19,13 +19,15 @@ constexpr size_t kAlign = 256;
 constexpr size_t up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 constexpr int64_t kWords = (kMaxVertices >> 5) + 1;
 // layout of the scratch array
-constexpr size_t kOffCtr = 0;                                        // kb::Counters
-constexpr size_t kOffCounts = kOffCtr + up(sizeof(kb::Counters));    // int64 medium count, int64 oversize count
-constexpr size_t kOffTable = kOffCounts + up(2 * sizeof(int64_t));
+constexpr size_t kOffCtr = 0;  // kb::Counters, tile counts and minima bitmap: one memset clears all three
+constexpr size_t kTiles = (size_t)((kMaxVertices + 131071) / 131072);
+constexpr size_t kOffTiles = kOffCtr + up(sizeof(kb::Counters));
+constexpr size_t kOffBitmap = kOffTiles + up(2 * sizeof(uint32_t) * kTiles);
+constexpr size_t kOffClasses = kOffBitmap + up(sizeof(uint32_t) * kWords);  // edgeless, medium, hub bits
+constexpr size_t kOffTable = kOffClasses + 3 * up(sizeof(uint32_t) * kWords);
 constexpr size_t kOffSlot = kOffTable + up(sizeof(uint64_t) * kTableCap);
 constexpr size_t kOffEmin = kOffSlot + up(sizeof(int32_t) * kMaxVertices);
-constexpr size_t kOffBitmap = kOffEmin + up(sizeof(uint64_t) * kMaxVertices);
-constexpr size_t kOffPrefix = kOffBitmap + up(sizeof(uint32_t) * kWords);
+constexpr size_t kOffPrefix = kOffEmin + up(sizeof(uint64_t) * kMaxVertices);
 constexpr size_t kOffScan = kOffPrefix + up(sizeof(uint2) * (kWords + 1));  // rank words
 constexpr size_t kScanWords = (size_t)((kWords + 4095) / 4096) + 1;
 constexpr size_t kOffMed = kOffScan + up(sizeof(uint32_t) * kScanWords);
@@ -57,26 +59,16 @@ kb_status scratch_address(int device, unsigned char** out) {
     return KB_OK;
 }
 
-// Level i-1 must hold ids in [0, n): they index the empty-signature minima.
-__global__ void check_prev_kernel(int64_t n, const int32_t* prev, kb::Counters* ctr) {
+// Level i-1 must hold ids in [0, n) (they index the empty-signature minima);
+// with col given, the neighbour ids too.
+__global__ void check_ids_kernel(int64_t n, int64_t m, const int32_t* prev, const int32_t* col, kb::Counters* ctr) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
+    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     bool bad = false;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-        if (prev[v] < 0 || (int64_t)prev[v] >= n) bad = true;
+    for (int64_t v = t; v < n; v += stride) bad |= prev[v] < 0 || (int64_t)prev[v] >= n;
+    if (col)
+        for (int64_t e = t; e < m; e += stride) bad |= col[e] < 0 || (int64_t)col[e] >= n;
     if (bad) atomicOr(&ctr->err, kb::kErrInvalid);
-}
-
-// Vertices this entry point cannot take: a degree above the hub threshold (no
-// hub path here) or a negative one (offsets not monotone, when validation is
-// off).  Counted into *bad.
-__global__ void check_degree_kernel(int64_t n, const int64_t* row, int32_t thr, unsigned long long* bad) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long c = 0;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const int64_t d = row[v + 1] - row[v];
-        if (d < 0 || d > thr) ++c;
-    }
-    if (c) atomicAdd(bad, c);
 }
 
 uint64_t next_pow2(uint64_t x) {
@@ -123,7 +115,6 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     const int32_t thr = opt->hub_threshold > 0 ? opt->hub_threshold : kb::kDefaultHubThreshold;
     const uint64_t cap = std::max<uint64_t>(1024, next_pow2((uint64_t)(2 * n)));
     kb::Counters* ctr = reinterpret_cast<kb::Counters*>(base + kOffCtr);
-    int64_t* cnts = reinterpret_cast<int64_t*>(base + kOffCounts);
 
     kb::RoundParams p{};
     p.n = n;
@@ -149,31 +140,30 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     p.n_hubs = 0;
 
     // The array keeps the previous call's contents: reset what must start clean.
-    NA_CUDA(cudaMemsetAsync(ctr, 0, sizeof(kb::Counters), s));
-    NA_CUDA(cudaMemsetAsync(cnts, 0, 2 * sizeof(int64_t), s));
+    NA_CUDA(cudaMemsetAsync(base, 0, kOffBitmap + sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
     NA_CUDA(cudaMemsetAsync(p.table, 0, sizeof(uint64_t) * cap, s));
     NA_CUDA(cudaMemsetAsync(p.emin, 0xff, sizeof(uint64_t) * (size_t)n, s));
-    NA_CUDA(cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
-    if (opt->validate) kb::launch_validate(n, g->m, g->row_offsets, g->col_indices, ctr, s);
-    const unsigned grid = (unsigned)std::min<int64_t>((n + 255) / 256, 1024);
-    check_prev_kernel<<<grid, 256, 0, s>>>(n, prev, ctr);
-    check_degree_kernel<<<grid, 256, 0, s>>>(n, p.row, thr, reinterpret_cast<unsigned long long*>(&cnts[1]));
-    if (g->m > 0)
-        kb::launch_classify(n, p.row, p.small_max, thr, reinterpret_cast<int32_t*>(base + kOffMed), &cnts[0], s);
+    const unsigned grid = (unsigned)std::min<int64_t>((std::max(n, g->m) + 255) / 256, 152 * 8);
+    check_ids_kernel<<<grid, 256, 0, s>>>(n, g->m, prev, opt->validate ? g->col_indices : nullptr, ctr);
+    // the degree classes: no vertex may lie above the hub threshold (no hub path
+    // here) or have a negative degree
+    auto bits = [&](int i) { return reinterpret_cast<uint32_t*>(base + kOffClasses + (size_t)i * up(sizeof(uint32_t) * kWords)); };
+    uint32_t* tiles = reinterpret_cast<uint32_t*>(base + kOffTiles);
+    kb::launch_classes(n, g->m, p.row, p.small_max, thr, bits(0), bits(1), bits(2), tiles,
+                       opt->validate ? kb::CheckRows::kAll : kb::CheckRows::kOrder, ctr, s);
+    kb::launch_class_list(n, p.row, bits(1), tiles, 0, kMaxVertices, reinterpret_cast<int32_t*>(base + kOffMed), nullptr, s);
     NA_CUDA(cudaGetLastError());
-    int64_t host_cnts[2] = {0, 0};
     kb::Counters host_ctr{};
-    NA_CUDA(cudaMemcpyAsync(host_cnts, cnts, sizeof(host_cnts), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaMemcpyAsync(&host_ctr, ctr, sizeof(host_ctr), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     if (host_ctr.err & kb::kErrInvalid) return KB_ERR_INVALID_ARG;
-    if (host_cnts[1] > 0) return KB_ERR_INVALID_ARG;  // a degree outside [0, hub threshold]
-    p.n_med = host_cnts[0];
+    if (host_ctr.n_hubs > 0) return KB_ERR_INVALID_ARG;  // a degree above the hub threshold
+    p.n_med = host_ctr.n_med;
 
     kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
     kb::launch_medium_round(p, s);
     kb::launch_renumber(p, reinterpret_cast<uint2*>(base + kOffPrefix), reinterpret_cast<uint32_t*>(base + kOffScan),
-                        out, nullptr, s);
+                        out, nullptr, false, s);
     NA_CUDA(cudaGetLastError());
     NA_CUDA(cudaMemcpyAsync(&host_ctr, ctr, sizeof(host_ctr), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
