@@ -102,8 +102,8 @@ typedef struct {
  *                      hub_threshold) with at most this many edges take a warp each,
  *                      larger ones a CTA each; 0 -> default 256, else 1..256
  *   small_max_degree   vertices with at most this many edges take the small-vertex
- *                      (warp-per-task) kernel; 0 -> default 32, else 1..32 (and at
- *                      most hub_threshold)
+ *                      kernels (a lane each up to 8 edges, eight lanes each above);
+ *                      0 -> default 32, else 1..32 (and at most hub_threshold)
  *                      The five tuning fields above, load_factor and hub_threshold,
  *                      when 0, take the values kb_autotune cached for the call's size
  *                      class, else the defaults.  None of them changes any result.
@@ -364,7 +364,7 @@ kb_status kb_refine_host(kb_context* ctx, const kb_graph* g, const kb_options* o
  *   kernel_ms[j] / kernel_launches[j] for j < KB_KERNEL_COUNT: summed device time
  *   and launches of each kernel family inside the rounds. */
 enum {
-    KB_KERNEL_SMALL = 0,       /* warp kernel: vertices with <= 32 edges (signature, dedup, hash, insert) */
+    KB_KERNEL_SMALL = 0,       /* vertices with <= 32 edges (signature, dedup, hash, insert) */
     KB_KERNEL_MEDIUM = 1,      /* tile kernel: vertices with 33..hub_threshold edges */
     KB_KERNEL_HUB_CHUNK = 2,   /* hub pairs: chunk dedup + global set insert */
     KB_KERNEL_HUB_FINAL = 3,   /* hub hash + block-table insert */

@@ -44,6 +44,15 @@ struct kb_context {
     // count of the batched call being planned
     std::map<int32_t, kb_tuning> tuned;
     int64_t plan_graphs = 1;
+    // block table and empty-signature minima, kept between calls (grow-only)
+    // unless the caller gives the workspace: entries of earlier rounds lose by
+    // their epoch or round word, so a call clears neither
+    void* tab = nullptr;
+    size_t tab_bytes = 0;
+    uint32_t tab_epoch = 0;
+    void* emin = nullptr;
+    size_t emin_bytes = 0;
+    uint32_t emin_round = 0;
     // batched refinement
     void* batch_ws = nullptr;
     size_t batch_ws_bytes = 0;
@@ -136,7 +145,7 @@ struct Plan {
     int thr = kb::kDefaultHubThreshold;
     int hub_chunk = kb::kDefaultHubChunk;
     int med_split = kb::kDefaultMedSplit;
-    int small_max = kb::kSmallDegree;
+    int small_max = kb::kMidDegree;  // small_max_degree: small and mid vertices
     int warp_verts = 0;  // 0: by the graph's size (launch_small_round)
     int32_t size_class = 0;  // key of the tuning cache
     uint64_t cap = 0;
@@ -157,16 +166,17 @@ struct Plan {
     // their sizes (the lists themselves are dropped once on the device)
     size_t n_hubs = 0;
     int64_t n_chunks = 0, set_slots = 0;
-    int64_t n_med = 0;  // medium vertices
+    int64_t n_mid = 0, n_med = 0;  // mid and medium vertices
     // layout
     size_t o_rowp = 0, o_colp = 0, o_labp = 0, o_cursor = 0, o_inpref = 0, o_i64tmp = 0;
     size_t csr_bytes = 0;
-    size_t o_emin = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
+    size_t o_emin = 0, o_mid = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
            o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0;
     size_t total = 0;
-    // bytes of one degree-class bitmap; three follow one another: edgeless, medium, hub
+    // bytes of one degree-class bitmap; four follow one another (kb::DegreeClass)
     size_t class_bytes() const { return align_up(sizeof(uint32_t) * (size_t)((n >> 5) + 1)); }
+    static constexpr int kClassBitmaps = 1 + kb::kClassLists;
 };
 
 bool needs_in_csr(int dir) { return dir == KB_DIR_IN || dir == KB_DIR_BOTH; }
@@ -219,6 +229,7 @@ void layout_round(Plan& P) {
     auto takeg = [&](size_t bytes) { size_t o = goff; goff += align_up(bytes); return o; };
     const int64_t nw = (P.n >> 5) + 1;
     const size_t H = P.n_hubs;
+    P.o_mid = takeg(sizeof(int32_t) * (size_t)P.n_mid);
     P.o_med = takeg(sizeof(int32_t) * (size_t)P.n_med);
     P.o_hubv = takeg(sizeof(int32_t) * H);
     P.o_chunk = takeg(sizeof(int64_t) * (H + 1));
@@ -230,7 +241,7 @@ void layout_round(Plan& P) {
     // CSR is reordered in place
     P.o_colr = takeg(P.reorder && !needs_in_csr(P.dir) ? sizeof(int32_t) * (size_t)P.m_proc : 0);
     P.o_hist = takeg(P.reorder ? sizeof(unsigned long long) * 512 : 0);
-    P.o_classes = takeg((P.freeze || P.graph_ext) ? 3 * P.class_bytes() : 0);
+    P.o_classes = takeg((P.freeze || P.graph_ext) ? Plan::kClassBitmaps * P.class_bytes() : 0);
     P.graph_bytes = P.graph_ext ? goff : 0;
     size_t off = P.graph_ext ? 0 : goff;
     auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
@@ -280,8 +291,8 @@ kb_status check_graph(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         return fail(ctx, KB_ERR_INVALID_ARG, "hub_chunk_edges must be 0, 256, 512 or 1024");
     if (opt->medium_split < 0 || opt->medium_split > kb::kMaxMedSplit)
         return fail(ctx, KB_ERR_INVALID_ARG, "medium_split must be in [0, %d]", kb::kMaxMedSplit);
-    if (opt->small_max_degree < 0 || opt->small_max_degree > kb::kSmallDegree)
-        return fail(ctx, KB_ERR_INVALID_ARG, "small_max_degree must be in [0, %d]", kb::kSmallDegree);
+    if (opt->small_max_degree < 0 || opt->small_max_degree > kb::kMidDegree)
+        return fail(ctx, KB_ERR_INVALID_ARG, "small_max_degree must be in [0, %d]", kb::kMidDegree);
     if (opt->direction == KB_DIR_BOTH && g->m > (int64_t)1 << 62)
         return fail(ctx, KB_ERR_INVALID_ARG, "too many edges");
     return KB_OK;
@@ -337,8 +348,8 @@ struct ClassScratch {
     size_t bits = 0, counts = 0, hub_v = 0, hub_deg = 0, total = 0;
     int64_t hub_cap = 0;
     explicit ClassScratch(const Plan& P) {
-        counts = 3 * P.class_bytes();
-        hub_v = counts + align_up(2 * sizeof(uint32_t) * kb::class_tiles(P.n));
+        counts = Plan::kClassBitmaps * P.class_bytes();
+        hub_v = counts + align_up(kb::kClassLists * sizeof(uint32_t) * kb::class_tiles(P.n));
         hub_cap = std::min<int64_t>(P.n, P.m_proc / (P.thr + 1) + 1);
         hub_deg = hub_v + align_up(sizeof(int32_t) * (size_t)hub_cap);
         total = hub_deg + align_up(sizeof(int64_t) * (size_t)hub_cap);
@@ -355,15 +366,17 @@ kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::Check
     P.chunk_off.assign(1, 0);
     P.set_off.assign(1, 0);
     P.n_hubs = 0;
-    P.n_chunks = P.set_slots = P.n_med = 0;
+    P.n_chunks = P.set_slots = P.n_mid = P.n_med = 0;
     if (P.n == 0) return read_counters(ctx);
     const ClassScratch C(P);
     KB_TRY(ensure_buffer(ctx, &ctx->class_tmp, &ctx->class_tmp_bytes, C.total));
     char* b = reinterpret_cast<char*>(ctx->class_tmp);
     uint32_t* counts = reinterpret_cast<uint32_t*>(b + C.counts);
-    auto bits = [&](int i) { return reinterpret_cast<uint32_t*>(b + (size_t)i * P.class_bytes()); };
-    kb::launch_classes(P.n, P.m_proc, row_p, P.small_max, P.thr, bits(0), bits(1), bits(2), counts, check, ctx->d_ctr, s);
-    kb::launch_class_list(P.n, row_p, bits(2), counts, 1, C.hub_cap, reinterpret_cast<int32_t*>(b + C.hub_v),
+    uint32_t* bits = reinterpret_cast<uint32_t*>(b);
+    const int64_t pitch = (int64_t)(P.class_bytes() / sizeof(uint32_t));
+    const kb::ClassBounds bounds{std::min(P.small_max, kb::kSmallDegree), P.small_max, P.thr};
+    kb::launch_classes(P.n, P.m_proc, row_p, bounds, bits, pitch, counts, check, ctx->d_ctr, s);
+    kb::launch_class_list(P.n, row_p, bits, pitch, counts, kb::kHub, C.hub_cap, reinterpret_cast<int32_t*>(b + C.hub_v),
                           reinterpret_cast<int64_t*>(b + C.hub_deg), s);
     KB_CUDA(ctx, cudaGetLastError());
     const int64_t eager = std::min(C.hub_cap, kEagerHubs);
@@ -372,9 +385,10 @@ kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::Check
     KB_CUDA(ctx, cudaMemcpyAsync(h_deg, b + C.hub_deg, sizeof(int64_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
     KB_TRY(read_counters(ctx));
     KB_TRY(device_error(ctx));
-    const int64_t H = ctx->h_ctr->n_hubs;
-    P.n_med = ctx->h_ctr->n_med;
-    if (H > C.hub_cap || P.n_med > P.n) return fail(ctx, KB_ERR_DEVICE_CHECK, "degree class larger than the graph allows");
+    P.n_mid = ctx->h_ctr->n_class[0];
+    P.n_med = ctx->h_ctr->n_class[1];
+    const int64_t H = ctx->h_ctr->n_class[2];
+    if (H > C.hub_cap || P.n_mid + P.n_med > P.n) return fail(ctx, KB_ERR_DEVICE_CHECK, "degree class larger than the graph allows");
     if (H <= 0) return KB_OK;
     P.hub_v.resize((size_t)H);
     std::vector<int64_t> deg((size_t)H);
@@ -462,7 +476,7 @@ kb_status make_plan(kb_context* ctx, const kb_graph* g, const kb_options* opt, P
     const kb_tuning* T = tuned_for(ctx, P.size_class);
     P.thr = pick_field(opt->hub_threshold, T ? T->hub_threshold : 0, kb::kDefaultHubThreshold);
     P.hub_chunk = pick_field(opt->hub_chunk_edges, T ? T->hub_chunk_edges : 0, kb::kDefaultHubChunk);
-    P.small_max = std::min(pick_field(opt->small_max_degree, T ? T->small_max_degree : 0, kb::kSmallDegree), P.thr);
+    P.small_max = std::min(pick_field(opt->small_max_degree, T ? T->small_max_degree : 0, kb::kMidDegree), P.thr);
     resolve_call_fields(P, opt, rounds, multi, T);
     layout_csr(P);
     const int64_t* row_p = g->row_offsets;
@@ -543,7 +557,10 @@ struct Prepared {
     uint32_t* scan_tmp = nullptr;
     int64_t total_chunks = 0;
     size_t set_bytes = 0;
-    uint32_t epoch = 0;
+    uint32_t epoch_own = 0, round_own = 0;
+    uint32_t* epoch = nullptr;  // last table epoch used, and rounds since the minima were cleared: the two
+    uint32_t* round = nullptr;  //   above, or the context's with its table
+    size_t table_bytes = 0, emin_bytes = 0;
     // frozen blocks for the next round and their minima, edgeless vertices
     // (Plan::freeze; RoundParams::frozen)
     uint32_t* frozen = nullptr;
@@ -560,8 +577,7 @@ struct Prepared {
     uint32_t* mark = nullptr;
     const int32_t* key_checked = nullptr;  // level-0 keys whose label minima are in ctx->d_dense,
     bool key_dense = false;                //   and whether they are all small (launch_dense_labels)
-    const uint32_t* medium_bits = nullptr;  // degree classes (Plan::class_bytes); nullptr: an empty class
-    const uint32_t* hub_bits = nullptr;
+    const uint32_t* class_bits[3] = {};  // mid, medium and hub vertices; nullptr: an empty class
     bool compact = false;  // small-kernel windows skip frozen vertices (many frozen)
     bool sparse = false;   // fewer than 1/64 of the vertices refine: long warp tasks
     // A caller-held block table (ext_cap slots) and empty-signature minima
@@ -581,8 +597,7 @@ struct Prepared {
     uint32_t* ext_minof = nullptr;
     uint32_t* ext_moved = nullptr;
     uint32_t* ext_mark = nullptr;
-    bool med_on = true;    // some medium vertex refines this round
-    bool hub_on = true;    // some hub refines this round
+    bool class_on[3] = {true, true, true};  // some mid vertex, medium vertex, hub refines this round
 };
 
 // Bind the per-graph part of a plan into p: the processed CSR (csr: IN /
@@ -636,19 +651,69 @@ kb_status bind_graph_part(kb_context* ctx, const kb_graph* g, const Plan& P, cha
         p.col = colr;
         p.perm = perm;
     }
+    p.mid_v = reinterpret_cast<int32_t*>(gws + P.o_mid);
+    p.n_mid = P.n_mid;
     p.med_v = reinterpret_cast<int32_t*>(gws + P.o_med);
     p.n_med = P.n_med;
     if (build) {
         // the plan's scratch still holds the classes (plan_classes)
         const ClassScratch C(P);
         const char* b = reinterpret_cast<const char*>(ctx->class_tmp);
-        kb::launch_class_list(n, p.row, reinterpret_cast<const uint32_t*>(b + P.class_bytes()),
-                              reinterpret_cast<const uint32_t*>(b + C.counts), 0, P.n_med, const_cast<int32_t*>(p.med_v),
-                              nullptr, s);
+        const uint32_t* bits = reinterpret_cast<const uint32_t*>(b);
+        const uint32_t* counts = reinterpret_cast<const uint32_t*>(b + C.counts);
+        const int64_t pitch = (int64_t)(P.class_bytes() / sizeof(uint32_t));
+        kb::launch_class_list(n, p.row, bits, pitch, counts, kb::kMid, P.n_mid, const_cast<int32_t*>(p.mid_v), nullptr, s);
+        kb::launch_class_list(n, p.row, bits, pitch, counts, kb::kMedium, P.n_med, const_cast<int32_t*>(p.med_v), nullptr,
+                              s);
         if (P.freeze || P.graph_ext)  // laid out only then
-            KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_classes, b, 3 * P.class_bytes(), cudaMemcpyDeviceToDevice, s));
+            KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_classes, b, Plan::kClassBitmaps * P.class_bytes(),
+                                         cudaMemcpyDeviceToDevice, s));
         KB_CUDA(ctx, cudaGetLastError());
     }
+    return KB_OK;
+}
+
+// Bind the block table and the empty-signature minima: the caller's (the
+// server's arena), the context's, or with a caller-owned workspace a part of it.
+kb_status bind_table(kb_context* ctx, const Plan& P, Prepared& R, cudaStream_t s) {
+    kb::RoundParams& p = R.p;
+    R.epoch = &R.epoch_own;
+    R.round = &R.round_own;
+    const size_t table_need = sizeof(uint64_t) * (size_t)P.cap, emin_need = sizeof(uint64_t) * (size_t)P.n;
+    if (R.ext_table) {
+        p.table = R.ext_table;
+        p.mask = R.ext_cap - 1;
+        p.emin = R.ext_emin;
+        R.table_bytes = sizeof(uint64_t) * (size_t)R.ext_cap;
+        return KB_OK;
+    }
+    p.mask = P.cap - 1;
+    if (ctx->user_ws) {
+        p.table = reinterpret_cast<uint64_t*>(R.ws + P.o_table);
+        p.emin = reinterpret_cast<uint64_t*>(R.ws + P.o_emin);
+        R.table_bytes = table_need;
+        R.emin_bytes = emin_need;
+        R.epoch_own = R.round_own = 0;
+        KB_CUDA(ctx, cudaMemsetAsync(p.table, 0, table_need, s));
+        KB_CUDA(ctx, cudaMemsetAsync(p.emin, 0xff, emin_need, s));
+        return KB_OK;
+    }
+    if (ctx->tab_bytes < table_need) {
+        KB_TRY(ensure_buffer(ctx, &ctx->tab, &ctx->tab_bytes, table_need));
+        KB_CUDA(ctx, cudaMemsetAsync(ctx->tab, 0, ctx->tab_bytes, s));
+        ctx->tab_epoch = 0;
+    }
+    if (ctx->emin_bytes < emin_need) {
+        KB_TRY(ensure_buffer(ctx, &ctx->emin, &ctx->emin_bytes, emin_need));
+        KB_CUDA(ctx, cudaMemsetAsync(ctx->emin, 0xff, ctx->emin_bytes, s));
+        ctx->emin_round = 0;
+    }
+    p.table = reinterpret_cast<uint64_t*>(ctx->tab);
+    p.emin = reinterpret_cast<uint64_t*>(ctx->emin);
+    R.table_bytes = ctx->tab_bytes;
+    R.emin_bytes = ctx->emin_bytes;
+    R.epoch = &ctx->tab_epoch;
+    R.round = &ctx->emin_round;
     return KB_OK;
 }
 
@@ -693,12 +758,11 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     p.ctr = ctx->d_ctr;
     if (pg) {
         P = pg->P;
-        P.ext_table = R.ext_table != nullptr;
+        P.ext_table = R.ext_table || !ctx->user_ws;
         P.ext_freeze = R.ext_frozen != nullptr;
         resolve_call_fields(P, opt, rounds, multi, tuned_for(ctx, P.size_class));
         layout_round(P);
         KB_TRY(acquire_workspace(ctx, P.total, &ws));
-        p.small_max = P.small_max;
         csr = pg->csr;
         gws = pg->gbuf;
         KB_TRY(bind_graph_part(ctx, g, P, csr, gws, false, nullptr, p, s));
@@ -728,7 +792,7 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
                 base = reinterpret_cast<char*>(ctx->plan_tmp);
             }
         }
-        P.ext_table = R.ext_table != nullptr;
+        P.ext_table = R.ext_table || !ctx->user_ws;
         P.ext_freeze = R.ext_frozen != nullptr;
         KB_TRY(make_plan(ctx, g, opt, P, &base, false, rounds, multi));
         if (ctx->user_ws) {
@@ -744,7 +808,6 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         }
         csr = base;
         gws = ws;
-        p.small_max = P.small_max;
         R.key_dense = R.key_checked && ctx->h_ctr->dense_bad == 0;
         // the slot array serves as the count buffer of the locality order:
         // every round rewrites it
@@ -752,20 +815,14 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     }
     R.ws = ws;
     p.hub_threshold = P.thr;
-    p.small_max = P.small_max;
+    p.small_max = std::min(P.small_max, kb::kSmallDegree);
+    p.mid_max = P.small_max;
     p.warp_verts = P.warp_verts;
     p.hub_chunk = P.hub_chunk;
     p.med_split = P.med_split;
     p.hash_mode = opt->hash_mode;
-    p.table = R.ext_table ? R.ext_table : reinterpret_cast<uint64_t*>(ws + P.o_table);
-    p.mask = (R.ext_table ? R.ext_cap : P.cap) - 1;
     p.slot_of = reinterpret_cast<int32_t*>(ws + P.o_slot);
-    if (R.ext_table) {
-        p.emin = R.ext_emin;  // entries of earlier rounds carry a larger round word and lose
-    } else {
-        p.emin = reinterpret_cast<uint64_t*>(ws + P.o_emin);
-        KB_CUDA(ctx, cudaMemsetAsync(p.emin, 0xff, sizeof(uint64_t) * (size_t)n, s));
-    }
+    KB_TRY(bind_table(ctx, P, R, s));
     p.bitmap = reinterpret_cast<uint32_t*>(ws + P.o_bitmap);
     p.ctr = ctx->d_ctr;
     p.hub_sets = reinterpret_cast<uint64_t*>(ws + P.o_sets);
@@ -776,14 +833,12 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     R.scan_tmp = reinterpret_cast<uint32_t*>(ws + P.o_scan);
     R.total_chunks = P.n_chunks;
     R.set_bytes = sizeof(uint64_t) * (size_t)P.set_slots;
-    if (!R.ext_table) {
-        KB_CUDA(ctx, cudaMemsetAsync(p.table, 0, sizeof(uint64_t) * (size_t)P.cap, s));
-        R.epoch = 0;
-    }
     if (P.freeze) {
         R.edgeless = reinterpret_cast<uint32_t*>(gws + P.o_classes);
-        R.medium_bits = P.n_med ? reinterpret_cast<uint32_t*>(gws + P.o_classes + P.class_bytes()) : nullptr;
-        R.hub_bits = P.n_hubs ? reinterpret_cast<uint32_t*>(gws + P.o_classes + 2 * P.class_bytes()) : nullptr;
+        const int64_t members[3] = {P.n_mid, P.n_med, (int64_t)P.n_hubs};
+        for (int c = 0; c < 3; ++c)
+            R.class_bits[c] = members[c] ? reinterpret_cast<uint32_t*>(gws + P.o_classes + (size_t)(c + 1) * P.class_bytes())
+                                         : nullptr;
         R.bm[0] = p.bitmap;
         R.bm[1] = reinterpret_cast<uint32_t*>(ws + P.o_bm2);
         R.bm_cur = 0;
@@ -818,11 +873,22 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
 // Advance the table epoch (entries of other epochs read as empty); the table
 // is cleared once every 255 rounds.
 kb_status next_epoch(kb_context* ctx, Prepared& R, cudaStream_t s) {
-    if (R.epoch == 255) {
-        KB_CUDA(ctx, cudaMemsetAsync(R.p.table, 0, sizeof(uint64_t) * (size_t)(R.p.mask + 1), s));
-        R.epoch = 0;
+    if (*R.epoch == 255) {
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.table, 0, R.table_bytes, s));
+        *R.epoch = 0;
     }
-    R.p.epoch = ++R.epoch;
+    R.p.epoch = ++*R.epoch;
+    return KB_OK;
+}
+
+// The round word of the next round's empty-signature minima: smaller than any
+// before.
+kb_status next_empty_round(kb_context* ctx, Prepared& R, cudaStream_t s) {
+    if (*R.round >= 0xfffffff0u) {
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.emin, 0xff, R.emin_bytes, s));
+        *R.round = 0;
+    }
+    R.p.ehigh = 0xffffffffu - ++*R.round;
     return KB_OK;
 }
 
@@ -843,8 +909,7 @@ kb::FreezePass freeze_pass(kb_context* ctx, const Prepared& R, const int32_t* le
     f.frozen = R.frozen;
     f.frozen_min = next_minima(R);
     f.moved_clear = R.p.perm ? R.moved : nullptr;
-    f.medium = R.medium_bits;
-    f.hub = R.hub_bits;
+    for (int c = 0; c < 3; ++c) f.classes[c] = R.class_bits[c];
     f.ctr = ctx->d_ctr;
     return f;
 }
@@ -899,11 +964,12 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
 // One refinement round up to (not including) the renumbering.
 kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer* T) {
     kb::RoundParams& p = R.p;
-    // with frozen blocks, the medium and hub kernels run only while some of
-    // their vertices refine (after the first rounds, hubs are mostly alone in
-    // their blocks)
-    const bool med = p.n_med && (!p.frozen || R.med_on);
-    const bool hub = p.n_hubs && (!p.frozen || R.hub_on);
+    // with frozen blocks, the mid, medium and hub kernels run only while some
+    // of their vertices refine (after the first rounds, hubs are mostly alone
+    // in their blocks)
+    const bool mid = p.n_mid && (!p.frozen || R.class_on[0]);
+    const bool med = p.n_med && (!p.frozen || R.class_on[1]);
+    const bool hub = p.n_hubs && (!p.frozen || R.class_on[2]);
     if (T) T->begin(KB_KERNEL_OTHER);
     if (!R.counters_clear) KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
     if (!R.bitmap_ready) kb::launch_clear_round(p, s);
@@ -914,6 +980,7 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
                            R.sparse ? kb::SmallWindows::kSparse
                                     : (R.compact ? kb::SmallWindows::kCompact : kb::SmallWindows::kConsecutive),
                            s);
+    if (mid) kb::launch_mid_round(p, s);
     if (T) T->end();
     if (med) {
         if (T) T->begin(KB_KERNEL_MEDIUM);
@@ -1031,8 +1098,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
             prev_count = ctx->h_ctr->count;
             R.compact = R.P.freeze && ctx->h_ctr->frozen * 4 > n;
             R.sparse = R.P.freeze && (n - ctx->h_ctr->frozen) * 64 < n;
-            R.med_on = ctx->h_ctr->med_on > 0;
-            R.hub_on = ctx->h_ctr->hub_on > 0;
+            for (int c = 0; c < 3; ++c) R.class_on[c] = ctx->h_ctr->class_on[c] > 0;
         }
     } else {
         // the count's low byte, for the rounds that compare with the previous one
@@ -1056,7 +1122,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     for (int i = i_start + 1; i <= k; ++i) {
         Timer T(ctx);
         KB_TRY(next_epoch(ctx, R, s));
-        p.ehigh = 0xffffffffu - (uint32_t)(i - i_start);
+        KB_TRY(next_empty_round(ctx, R, s));
         p.prev = rows.row(i - 1);
         p.own_key = R.P.subject ? reinterpret_cast<const int32_t*>(R.ws + R.P.o_ownkey) : nullptr;
         p.frozen = R.frozen;
@@ -1103,8 +1169,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         // compacted small-kernel windows pay once a quarter of the vertices are frozen
         R.compact = R.P.freeze && ctx->h_ctr->frozen * 4 > n;
         R.sparse = R.P.freeze && (n - ctx->h_ctr->frozen) * 64 < n;
-        R.med_on = ctx->h_ctr->med_on > 0;
-        R.hub_on = ctx->h_ctr->hub_on > 0;
+        for (int c = 0; c < 3; ++c) R.class_on[c] = ctx->h_ctr->class_on[c] > 0;
         ctx->round_ms.push_back(T.collect());
         KB_TRY(device_error(ctx));
         const int64_t c = ctx->h_ctr->count;
@@ -1269,7 +1334,7 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_CUDA(ctx, cudaMemcpyAsync(keep, row(i), sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
         kb::launch_keep_min(n, wmask, keep, kmin, s);
         KB_TRY(next_epoch(ctx, R, s));
-        p.ehigh = 0xffffffffu - (uint32_t)i;
+        KB_TRY(next_empty_round(ctx, R, s));
         p.prev = row(i - 1);
         p.vmask = wmask;
         p.keep_old = keep;
@@ -1536,8 +1601,8 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
         kb_status st = KB_OK;
         for (int i = 1; i <= kmax && st == KB_OK; ++i) {
             st = next_epoch(ctx, R, cs);
+            if (st == KB_OK) st = next_empty_round(ctx, R, cs);
             if (st != KB_OK) break;
-            p.ehigh = 0xffffffffu - (uint32_t)i;
             p.prev = levels + (size_t)(i - 1) * (size_t)n;
             p.bitmap = (i & 1) ? bm_b : bm_a;
             p.bitmap_prev = (i & 1) ? bm_a : bm_b;
@@ -1683,7 +1748,6 @@ struct kb_server {
     uint64_t* table = nullptr;
     uint64_t table_cap = 0;
     uint64_t* emin = nullptr;
-    uint64_t round_counter = 0;  // rounds run; decreasing round words of the minima
     // Frozen-block state of the arena, sized for a full arena and kept across
     // re-plans: frozen vertices, minima of frozen blocks, shared marks,
     // smallest members, moved vertices, dirty blocks, and the two bitmaps of
@@ -2049,6 +2113,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
             o.hash_mode = sv->cfg.hash_mode;
             sv->R.ext_table = sv->table;
             sv->R.ext_cap = sv->table_cap;
+            sv->R.emin_bytes = sizeof(uint64_t) * (size_t)sv->cfg.max_vertices;
             sv->R.ext_emin = sv->emin;
             sv->R.ext_frozen = sv->frz[0];
             sv->R.ext_frozen_min = sv->frz[1];
@@ -2101,7 +2166,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         SV_CUDA(sv, cudaMemcpyAsync(sv->slot_n, sn.data(), sizeof(int64_t) * (size_t)G, cudaMemcpyHostToDevice, s));
         // one round for everything in flight
         SV_TRY(sv, next_epoch(ctx, sv->R, s));
-        p.ehigh = 0xffffffffu - (uint32_t)(++sv->round_counter);
+        SV_TRY(sv, next_empty_round(ctx, sv->R, s));
         p.vgraph = sv->vgraph;
         p.voff = sv->voff;
         p.n_graphs = G;
@@ -2253,6 +2318,8 @@ kb_status kb_destroy(kb_context* ctx) {
     cudaFree(ctx->class_tmp);
     cudaFree(ctx->plan_tmp);
     cudaFree(ctx->stage);
+    cudaFree(ctx->tab);
+    cudaFree(ctx->emin);
     cudaFree(ctx->batch_ws);
     cudaFree(ctx->tune_buf);
     cudaFree(ctx->fix_buf);
@@ -2349,7 +2416,6 @@ kb_status kb_graph_prepare(kb_context* ctx, const kb_graph* g, const kb_options*
         if (P.reorder) KB_TRY(alloc(&count_tmp, sizeof(uint32_t) * (size_t)n));
         kb::RoundParams p{};
         p.n = n;
-        p.small_max = P.small_max;
         const kb_status st = bind_graph_part(ctx, g, P, pg->csr, pg->gbuf, true,
                                              reinterpret_cast<uint32_t*>(count_tmp), p, s);
         const cudaError_t e = cudaStreamSynchronize(s);
@@ -2547,7 +2613,7 @@ kb_status kb_autotune(kb_context* ctx, const kb_graph* g, const int64_t* voff, i
     dflt.small_task_vertices = 0;
     dflt.hub_chunk_edges = kb::kDefaultHubChunk;
     dflt.medium_split = kb::kDefaultMedSplit;
-    dflt.small_max_degree = kb::kSmallDegree;
+    dflt.small_max_degree = kb::kMidDegree;
     kb_options start = dflt;
     if (base.load_factor > 0.f) start.load_factor = base.load_factor;
     if (base.hub_threshold) start.hub_threshold = base.hub_threshold;

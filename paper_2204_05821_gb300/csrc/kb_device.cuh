@@ -86,7 +86,7 @@ __device__ __forceinline__ bool same_graph(const RoundParams& p, int64_t a, int6
 // 1 with *rep set when a slot with our tag was found (a signature compare
 // decides), 2 when the probe limit was hit.
 __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_io, uint32_t hi, uint32_t v,
-                                           uint32_t* rep, bool toggle = true) {
+                                           uint32_t* rep) {
     uint64_t pos = *pos_io;
     for (int it = 0; it < kProbeLimit; ++it) {
         uint64_t cur = volatile_load(&p.table[pos]);
@@ -96,7 +96,7 @@ __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_i
                                            (unsigned long long)cur, (unsigned long long)want);
             if (old == cur) {
                 p.slot_of[v] = (int32_t)pos;
-                if (toggle) toggle_min(p.bitmap, v);
+                toggle_min(p.bitmap, v);
                 *pos_io = pos;
                 return 0;
             }
@@ -112,6 +112,4 @@ __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_i
     }
     return 2;
 }
-
-
 }  // namespace kb

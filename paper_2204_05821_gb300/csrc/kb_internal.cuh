@@ -27,7 +27,8 @@ constexpr int kMaxMedSplit = 256;
 constexpr int kDefaultMedSplit = kMaxMedSplit;
 constexpr int kHubFinalThreads = 256;
 constexpr int kProbeLimit = 1 << 22;  // bound on block-table probes per vertex
-constexpr int kSmallDegree = 32;      // vertices with at most this many edges take the warp kernel
+constexpr int kSmallDegree = 8;       // vertices with at most this many edges take a lane each (kb_small.cu),
+constexpr int kMidDegree = 32;        // with at most this many eight lanes each (kb_medium.cu)
 constexpr int kDefaultWarpVerts = 128;
 
 constexpr uint64_t kEmptyPair = ~0ull;  // block field 0x7fffffff never occurs (n <= 2^31-2)
@@ -40,8 +41,7 @@ struct Counters {
     int32_t diff;   // set when two compared levels differ (launch_levels_differ)
     int64_t count;  // blocks at the level just assigned
     int64_t frozen; // vertices frozen for the next round (launch_freeze_clean)
-    int64_t med_on; // medium vertices that refine next round (launch_freeze_clean)
-    int64_t hub_on; // hubs that refine next round (launch_freeze_clean)
+    int64_t class_on[3]; // mid and medium vertices and hubs that refine next round (launch_freeze_clean)
     int64_t moved;  // re-keyed vertices whose smallest block member changed (renumbering)
     // vertices re-keyed this round and their edges in the processed
     // direction, per kernel family: small, medium, hub
@@ -49,8 +49,7 @@ struct Counters {
     int64_t keyed_e[3];
     int32_t dense_bad;  // a level-0 key outside [0, kDenseLabels) (launch_dense_labels)
     int64_t prev_count; // blocks at the level before
-    int64_t n_med;      // medium vertices and hubs of the graph (launch_classes)
-    int64_t n_hubs;
+    int64_t n_class[3]; // mid and medium vertices and hubs of the graph (launch_classes)
 };
 
 // Everything one refinement round reads and writes.
@@ -108,13 +107,14 @@ struct RoundParams {
     uint32_t* minof;
     uint32_t* moved;
     int32_t hub_threshold;
-    int32_t small_max;    // largest degree of the small-vertex kernel (<= kSmallDegree, <= hub_threshold)
+    int32_t small_max;    // largest degree of the small-vertex kernel (<= kSmallDegree, <= mid_max)
+    int32_t mid_max;      // largest degree of the mid kernel (<= kMidDegree, <= hub_threshold)
     int32_t warp_verts;   // vertices per warp task of the small-vertex kernel; 0: by the graph's size
     int32_t hub_chunk;    // edges per hub-chunk CTA: 256, 512 or 1024
     int32_t med_split;    // medium vertices up to this degree take a warp, larger a CTA (1..kMaxMedSplit)
     int32_t hash_mode;
     uint32_t epoch;       // 1..255, tags this round's table entries
-    uint64_t* table;      // [mask+1] block table
+    uint64_t* table;      // [mask+1] block table: [epoch 8 | tag 24 | single bit, smallest member 32]
     uint64_t mask;
     int32_t* slot_of;     // [n] table slot of every vertex; 0x80000000|own for an empty signature
     uint64_t* emin;       // [n] smallest vertex with an empty signature per own block:
@@ -122,7 +122,10 @@ struct RoundParams {
     uint32_t ehigh;
     uint32_t* bitmap;     // [n/32+1] bit v set iff v is the smallest member of its block
     Counters* ctr;
-    // medium vertices (small_max < degree <= hub_threshold), processed by the tile kernel
+    // mid (small_max < degree <= mid_max) and medium vertices (up to
+    // hub_threshold), ascending
+    const int32_t* mid_v;
+    int64_t n_mid;
     const int32_t* med_v;
     int64_t n_med;
     // hubs (vertices with more than hub_threshold edges)
@@ -245,8 +248,8 @@ struct FreezePass {
     uint32_t* frozen = nullptr;          // out: frozen vertices, counted in ctr->frozen
     uint32_t* frozen_min = nullptr;      // out: the minima of frozen blocks
     uint32_t* moved_clear = nullptr;     // a bitmap to clear, or nullptr
-    const uint32_t* medium = nullptr;    // degree classes: those not frozen are counted in ctr->med_on and hub_on
-    const uint32_t* hub = nullptr;       //   (nullptr: an empty class)
+    const uint32_t* classes[3] = {};     // mid, medium, hub: those not frozen are counted in ctr->class_on
+                                         // (nullptr: an empty class)
     Counters* ctr = nullptr;
     // serving: the vertices of graphs that computed their level 0 in this step
     // (gmode) are not frozen by the edgeless rule
@@ -265,7 +268,8 @@ void launch_round_work(const RoundParams& p, cudaStream_t s);
 // (kCompact: worth it when many are frozen; kSparse: nearly all are).
 enum class SmallWindows { kConsecutive, kCompact, kSparse };
 void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s);
-void launch_medium_round(const RoundParams& p, cudaStream_t s);  // kb_medium.cu
+void launch_mid_round(const RoundParams& p, cudaStream_t s);     // kb_medium.cu: after the small vertices,
+void launch_medium_round(const RoundParams& p, cudaStream_t s);  //   after the mid ones
 // Per-device kernel attributes (shared-memory carveouts); call once per device
 // before the first launch and outside any stream capture.
 void set_medium_kernel_attributes();
@@ -273,7 +277,7 @@ void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s
 void launch_hub_final(const RoundParams& p, cudaStream_t s);
 // Canonical renumbering: prefix of block minima, then ids.
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
-// The frozen, med_on, hub_on and moved counters restart at 0; with frozen
+// The frozen, class_on and moved counters restart at 0; with frozen
 // blocks moved vertices are counted, and mark (or nullptr) is cleared.
 // stop_stable (frozen-block rounds under early stop): in a round that kept the
 // block count (the last round) the ids are those of the previous level, and out
@@ -320,20 +324,26 @@ size_t scan_i64_tmp(int64_t n);
 void launch_build_csr(int64_t n, int64_t m, const int64_t* row, const int32_t* col, const int32_t* lab,
                       const int64_t* in_prefix, int include_out, int64_t* row_p, int32_t* col_p,
                       int32_t* lab_p, int64_t* cursor, cudaStream_t s);
-// Degree classes of the processed CSR: bitmaps of (n >> 5) + 1 words of the
-// vertices without edges, with lo < degree <= hi (medium) and above (hubs),
-// their numbers in ctr->n_med and n_hubs, and both per tile in tile_counts (two
+// Degree classes of the processed CSR: vertices without edges, mid, medium and
+// hub vertices, a bitmap of (n >> 5) + 1 words each, pitch words apart.  The last
+// three are counted in ctr->n_class and per tile in tile_counts (kClassLists
 // words per tile, class_tiles(n) tiles).  check: report offsets out of order
 // (kOrder), or also not from 0 to m (kAll), in ctr->err.
+enum DegreeClass { kEdgeless, kMid, kMedium, kHub };
+constexpr int kClassLists = 3;  // classes that are also listed
+struct ClassBounds {
+    int32_t small;   // largest degree of the small-vertex kernel
+    int32_t mid;     // of the mid class
+    int32_t medium;  // of the medium class
+};
 enum class CheckRows { kNone, kOrder, kAll };
 size_t class_tiles(int64_t n);
-void launch_classes(int64_t n, int64_t m, const int64_t* row, int32_t lo, int32_t hi, uint32_t* edgeless,
-                    uint32_t* medium, uint32_t* hub, uint32_t* tile_counts, CheckRows check, Counters* ctr,
-                    cudaStream_t s);
-// The vertices of a class (which: 0 medium, 1 hub), ascending, at most cap of
-// them, with their degrees unless deg is nullptr.
-void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, const uint32_t* tile_counts, int which,
-                       int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s);
+void launch_classes(int64_t n, int64_t m, const int64_t* row, const ClassBounds& bounds, uint32_t* bits, int64_t pitch,
+                    uint32_t* tile_counts, CheckRows check, Counters* ctr, cudaStream_t s);
+// The vertices of a class, ascending, at most cap of them, with their degrees
+// unless deg is nullptr.
+void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
+                       DegreeClass c, int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s);
 // Hub and packed extent of every hub chunk (RoundParams::chunk_hub, chunk_ext).
 void launch_chunk_ext(int64_t chunks, int32_t n_hubs, const int32_t* hub_v, const int64_t* chunk_off,
                       const int64_t* row, int32_t chunk, int32_t* chunk_hub, uint64_t* out, cudaStream_t s);

@@ -400,8 +400,7 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
         ctr->prev_count = ctr->count;
         ctr->count = (int64_t)all;
         ctr->frozen = 0;
-        ctr->med_on = 0;
-        ctr->hub_on = 0;
+        for (int k = 0; k < 3; ++k) ctr->class_on[k] = 0;
         ctr->moved = 0;
         if (rank_total) rank[nw] = make_uint2(all, 0u);
     }
@@ -629,10 +628,10 @@ __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, 
 // whose block it must look up to its lanes, as dirty_blocks_kernel does.
 __global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
     __shared__ uint32_t s_clean[8][32];
-    __shared__ uint32_t s_on[3];  // frozen vertices, refining medium vertices and hubs of this CTA
+    __shared__ uint32_t s_on[4];  // frozen vertices, refining mid and medium vertices and hubs of this CTA
     Counters* ctr = f.ctr;
     if (f.stop_stable && ctr->count == ctr->prev_count) return;  // the last round: nothing follows
-    if (threadIdx.x < 3) s_on[threadIdx.x] = 0u;
+    if (threadIdx.x < 4) s_on[threadIdx.x] = 0u;
     __syncthreads();
     const int64_t n = f.n;
     const int per_warp = f.per_warp;
@@ -699,14 +698,15 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
         shared[w] = sh & fm;
         if (f.moved_clear) f.moved_clear[w] = 0u;
         if (fz) atomicAdd(&s_on[0], (uint32_t)__popc(fz));
-        const uint32_t md = f.medium ? f.medium[w] & ~fz : 0u;
-        const uint32_t hb = f.hub ? f.hub[w] & ~fz : 0u;
-        if (md) atomicAdd(&s_on[1], (uint32_t)__popc(md));
-        if (hb) atomicAdd(&s_on[2], (uint32_t)__popc(hb));
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            const uint32_t on = f.classes[k] ? f.classes[k][w] & ~fz : 0u;
+            if (on) atomicAdd(&s_on[1 + k], (uint32_t)__popc(on));
+        }
     }
     __syncthreads();
-    if (threadIdx.x < 3 && s_on[threadIdx.x]) {
-        int64_t* dst = threadIdx.x == 0 ? &ctr->frozen : (threadIdx.x == 1 ? &ctr->med_on : &ctr->hub_on);
+    if (threadIdx.x < 4 && s_on[threadIdx.x]) {
+        int64_t* dst = threadIdx.x == 0 ? &ctr->frozen : &ctr->class_on[threadIdx.x - 1];
         atomicAdd(reinterpret_cast<unsigned long long*>(dst), (unsigned long long)s_on[threadIdx.x]);
     }
 }
@@ -1042,7 +1042,7 @@ void launch_freeze_clean(const FreezePass& f, cudaStream_t s) {
 void launch_round_work(const RoundParams& p, cudaStream_t s) {
     if (p.n <= 0) return;
     const int g = grid_for(p.n, 256) < 1216 ? grid_for(p.n, 256) : 1216;
-    round_work_kernel<<<g, 256, 0, s>>>(p.n, p.row, p.frozen, p.small_max, p.hub_threshold, p.ctr);
+    round_work_kernel<<<g, 256, 0, s>>>(p.n, p.row, p.frozen, p.mid_max, p.hub_threshold, p.ctr);
 }
 
 void launch_count_bits(const uint32_t* words, int64_t nw, int64_t* out, cudaStream_t s) {

@@ -39,6 +39,160 @@ static_assert(kMaxHubThreshold <= 1024, "the second class holds degrees up to 10
 // enters the hash sum, so each new pair costs one mix.
 __device__ __forceinline__ uint32_t med_slot(uint64_t pm, uint32_t cmask) { return (uint32_t)(pm >> 24) & cmask; }
 
+// The same for the mid vertices (at most kMidDegree edges): eight lanes each,
+// four edges per lane, so a warp has four vertices and all their edges' loads in
+// flight at once.  A warp per vertex spends most of its instructions on empty
+// lanes at these degrees, a lane per vertex needs room for all its pairs.
+constexpr int kGroup = 8;
+constexpr int kMidWarps = 8;
+constexpr int kMidCap = 2 * kMidDegree;
+
+__global__ void __launch_bounds__(kMidWarps * 32) mid_round_kernel(const RoundParams p, int32_t per_task) {
+    constexpr int U = kMidDegree / kGroup;
+    constexpr uint32_t cmask = kMidCap - 1;
+    __shared__ uint64_t s_set[kMidWarps * 4][kMidCap];
+    __shared__ uint32_t s_mark[kMidWarps * 4][kMidCap / 32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int g = lane / kGroup, gl = lane % kGroup;
+    uint64_t* set = s_set[warp * 4 + g];
+    uint32_t* mark = s_mark[warp * 4 + g];
+    const int64_t t0 = ((int64_t)blockIdx.x * kMidWarps + warp) * per_task;
+    if (t0 >= p.n_mid) return;  // uniform over the warp
+    const int nt = (int)min((int64_t)per_task, p.n_mid - t0);
+
+    // the task's vertices, row offsets and own blocks, loaded at once
+    int32_t tv = 0, town = 0, td = 0;
+    int64_t trs = 0;
+    bool take = false;
+    if (lane < nt) {
+        tv = p.mid_v[t0 + lane];
+        take = vertex_refines(p, tv);
+        if (take) {
+            trs = p.row[tv];
+            td = (int32_t)(p.row[(int64_t)tv + 1] - trs);
+            town = own_of(p, tv);
+        }
+    }
+    unsigned todo = __ballot_sync(kFull, take);
+
+    while (todo) {
+        // the next four vertices, one per group
+        unsigned mine = todo;
+        for (int i = 0; i < g; ++i) mine &= mine - 1;
+        for (int i = 0; i < 4; ++i) todo &= todo - 1;
+        bool pending = mine != 0u;
+        const int j = pending ? __ffs(mine) - 1 : 0;
+        const int32_t v = __shfl_sync(kFull, tv, j);
+        const int32_t own = __shfl_sync(kFull, town, j);
+        const int64_t rs = __shfl_sync(kFull, trs, j);
+        int d = __shfl_sync(kFull, td, j);
+        if (!pending) d = 0;
+        int32_t w[U], l[U], b[U];
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const int e = u * kGroup + gl;
+            w[u] = l[u] = 0;
+            if (e < d) {
+                w[u] = __ldcs(p.col + rs + e);
+                if (p.lab) l[u] = __ldcs(p.lab + rs + e);
+            }
+        }
+#pragma unroll
+        for (int i = 0; i < kMidCap / kGroup; ++i) set[i * kGroup + gl] = kEmptyPair;
+#pragma unroll
+        for (int u = 0; u < U; ++u)
+            if (u * kGroup + gl < d) b[u] = gather_block(p, w[u]);
+        __syncwarp();
+        uint64_t acc = 0;
+        uint32_t cnt = 0;
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (u * kGroup + gl >= d) continue;
+            const uint64_t pr = pack_pair(l[u], (uint32_t)w[u], b[u]);
+            const uint64_t pm = pair_mix(pr);
+            uint32_t slot = med_slot(pm, cmask);
+            while (true) {
+                const unsigned long long old = atomicCAS(reinterpret_cast<unsigned long long*>(set + slot),
+                                                         (unsigned long long)kEmptyPair, (unsigned long long)pr);
+                if (old == (unsigned long long)kEmptyPair) {
+                    acc += pm;
+                    ++cnt;
+                    break;
+                }
+                if (old == (unsigned long long)pr) break;
+                slot = (slot + 1) & cmask;
+            }
+        }
+#pragma unroll
+        for (int o = kGroup / 2; o > 0; o >>= 1) {
+            acc += __shfl_xor_sync(kFull, (unsigned long long)acc, o);
+            cnt += __shfl_xor_sync(kFull, cnt, o);
+        }
+        __syncwarp();
+
+        // find or insert, with the full signature compare on every tag match
+        const uint64_t h = vertex_hash(own, cnt, acc, p.hash_mode);
+        uint64_t pos = h & p.mask;
+        const uint32_t hi = table_hi(h, p.epoch);
+        const unsigned gmask = ((1u << kGroup) - 1u) << (g * kGroup);
+        while (__any_sync(kFull, pending)) {
+            int r = 0;
+            uint32_t rep = 0;
+            if (pending && gl == 0) {
+                r = probe_table(p, &pos, hi, (uint32_t)v, &rep);
+                if (r == 2) set_error(p.ctr, kErrTableFull);
+            }
+            if (gl < kMidCap / 32) mark[gl] = 0u;
+            r = __shfl_sync(kFull, r, lane - gl);
+            rep = __shfl_sync(kFull, rep, lane - gl);
+            pos = __shfl_sync(kFull, (unsigned long long)pos, lane - gl);
+            if (r != 1) pending = false;  // inserted, or the probe limit
+            bool ok = pending && same_graph(p, rep, v) && own_of(p, rep) == own;
+            int64_t rb = 0, rend = 0;
+            if (ok) {
+                rb = p.row[rep];
+                rend = p.row[(int64_t)rep + 1];
+            }
+            uint32_t nf = 0;
+            for (; __any_sync(kFull, rb < rend); rb += kMidDegree) {
+                bool found = true;
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int64_t e = rb + u * kGroup + gl;
+                    if (e >= rend) continue;
+                    const int32_t ww = __ldg(p.col + e);
+                    const int32_t ll = p.lab ? __ldg(p.lab + e) : 0;
+                    const uint64_t pr = pack_pair(ll, (uint32_t)ww, gather_block(p, ww));
+                    uint32_t slot = med_slot(pair_mix(pr), cmask);
+                    uint64_t cur;
+                    while ((cur = set[slot]) != pr && cur != kEmptyPair) slot = (slot + 1) & cmask;
+                    if (cur == pr) {
+                        const uint32_t bit = 1u << (slot & 31);
+                        if (!(atomicOr(&mark[slot >> 5], bit) & bit)) ++nf;
+                    } else {
+                        found = false;
+                    }
+                }
+                if (__ballot_sync(kFull, !found) & gmask) {
+                    ok = false;
+                    rend = rb;
+                }
+            }
+#pragma unroll
+            for (int o = kGroup / 2; o > 0; o >>= 1) nf += __shfl_xor_sync(kFull, nf, o);
+            if (pending) {
+                if (ok && nf == cnt) {
+                    if (gl == 0) join_slot(p, pos, hi, (uint32_t)v);
+                    pending = false;
+                } else {
+                    pos = (pos + 1) & p.mask;
+                }
+            }
+            __syncwarp();
+        }
+    }
+}
+
 template <int kCap, int kWarps>
 __global__ void __launch_bounds__(kWarps * 32) medium_round_kernel(const RoundParams p, int32_t dlo, int32_t dhi, int32_t per_task) {
     __shared__ uint64_t s_set[kWarps][kCap];
@@ -422,21 +576,29 @@ static int32_t task_entries(int64_t n_med, int64_t tasks) {
     return (int32_t)std::min<int64_t>(kMedTask, (n_med + tasks - 1) / tasks);
 }
 
+void launch_mid_round(const RoundParams& p, cudaStream_t s) {
+    if (p.n_mid <= 0) return;
+    const int32_t per = task_entries(p.n_mid, 152 * 6 * kMidWarps * 2);
+    const int64_t ctas = (p.n_mid + (int64_t)per * kMidWarps - 1) / ((int64_t)per * kMidWarps);
+    mid_round_kernel<<<(unsigned)ctas, kMidWarps * 32, 0, s>>>(p, per);
+}
+
 void launch_medium_round(const RoundParams& p, cudaStream_t s) {
     if (p.n_med <= 0) return;
     const int32_t thr = std::min(p.hub_threshold, (int32_t)kMaxHubThreshold);
     const int32_t split = std::min(std::max(p.med_split, 1), (int32_t)kMedSplit);
-    if (p.small_max < split) {
+    const int32_t lo = p.mid_max;
+    if (lo < std::min(thr, split)) {
         constexpr int kW = 4;
         const int32_t per = task_entries(p.n_med, 152 * 13 * kW);
         const int64_t ctas = (p.n_med + (int64_t)per * kW - 1) / ((int64_t)per * kW);
         medium_round_kernel<2 * kMedSplit, kW>
-            <<<(unsigned)ctas, kW * 32, 0, s>>>(p, p.small_max, std::min(thr, split), per);
+            <<<(unsigned)ctas, kW * 32, 0, s>>>(p, lo, std::min(thr, split), per);
     }
     if (thr > split) {
         const int32_t per = task_entries(p.n_med, 152 * 7 * 2);
         medium_cta_kernel<2 * kMaxHubThreshold, kMedCtaThreads>
-            <<<(unsigned)((p.n_med + per - 1) / per), kMedCtaThreads, 0, s>>>(p, std::max(p.small_max, split), thr, per);
+            <<<(unsigned)((p.n_med + per - 1) / per), kMedCtaThreads, 0, s>>>(p, std::max(lo, split), thr, per);
     }
 }
 

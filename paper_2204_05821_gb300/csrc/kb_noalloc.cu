@@ -22,9 +22,9 @@ constexpr int64_t kWords = (kMaxVertices >> 5) + 1;
 constexpr size_t kOffCtr = 0;  // kb::Counters, tile counts and minima bitmap: one memset clears all three
 constexpr size_t kTiles = (size_t)((kMaxVertices + 131071) / 131072);
 constexpr size_t kOffTiles = kOffCtr + up(sizeof(kb::Counters));
-constexpr size_t kOffBitmap = kOffTiles + up(2 * sizeof(uint32_t) * kTiles);
-constexpr size_t kOffClasses = kOffBitmap + up(sizeof(uint32_t) * kWords);  // edgeless, medium, hub bits
-constexpr size_t kOffTable = kOffClasses + 3 * up(sizeof(uint32_t) * kWords);
+constexpr size_t kOffBitmap = kOffTiles + up(kb::kClassLists * sizeof(uint32_t) * kTiles);
+constexpr size_t kOffClasses = kOffBitmap + up(sizeof(uint32_t) * kWords);  // kb::DegreeClass
+constexpr size_t kOffTable = kOffClasses + (1 + kb::kClassLists) * up(sizeof(uint32_t) * kWords);
 constexpr size_t kOffSlot = kOffTable + up(sizeof(uint64_t) * kTableCap);
 constexpr size_t kOffEmin = kOffSlot + up(sizeof(int32_t) * kMaxVertices);
 constexpr size_t kOffPrefix = kOffEmin + up(sizeof(uint64_t) * kMaxVertices);
@@ -98,7 +98,7 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     if (opt->small_task_vertices != 0 && (opt->small_task_vertices < 32 || opt->small_task_vertices > 65536))
         return KB_ERR_INVALID_ARG;
     if (opt->medium_split < 0 || opt->medium_split > kb::kMaxMedSplit) return KB_ERR_INVALID_ARG;
-    if (opt->small_max_degree < 0 || opt->small_max_degree > kb::kSmallDegree) return KB_ERR_INVALID_ARG;
+    if (opt->small_max_degree < 0 || opt->small_max_degree > kb::kMidDegree) return KB_ERR_INVALID_ARG;
     if (g->n == 0) {
         *count = 0;
         return KB_OK;
@@ -123,7 +123,8 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     p.lab = opt->use_edge_labels ? g->edge_labels : nullptr;
     p.prev = prev;
     p.hub_threshold = thr;
-    p.small_max = std::min(opt->small_max_degree > 0 ? opt->small_max_degree : kb::kSmallDegree, thr);
+    p.mid_max = std::min(opt->small_max_degree > 0 ? opt->small_max_degree : kb::kMidDegree, thr);
+    p.small_max = std::min(p.mid_max, kb::kSmallDegree);
     p.warp_verts = opt->small_task_vertices;
     p.hub_chunk = kb::kDefaultHubChunk;  // no hubs here
     p.med_split = opt->medium_split > 0 ? opt->medium_split : kb::kDefaultMedSplit;
@@ -136,7 +137,6 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     p.ehigh = 0xfffffffeu;  // emin is reset to all ones below, so this round's entries win
     p.bitmap = reinterpret_cast<uint32_t*>(base + kOffBitmap);
     p.ctr = ctr;
-    p.med_v = reinterpret_cast<const int32_t*>(base + kOffMed);
     p.n_hubs = 0;
 
     // The array keeps the previous call's contents: reset what must start clean.
@@ -147,20 +147,29 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     check_ids_kernel<<<grid, 256, 0, s>>>(n, g->m, prev, opt->validate ? g->col_indices : nullptr, ctr);
     // the degree classes: no vertex may lie above the hub threshold (no hub path
     // here) or have a negative degree
-    auto bits = [&](int i) { return reinterpret_cast<uint32_t*>(base + kOffClasses + (size_t)i * up(sizeof(uint32_t) * kWords)); };
+    uint32_t* bits = reinterpret_cast<uint32_t*>(base + kOffClasses);
+    const int64_t pitch = (int64_t)(up(sizeof(uint32_t) * kWords) / sizeof(uint32_t));
     uint32_t* tiles = reinterpret_cast<uint32_t*>(base + kOffTiles);
-    kb::launch_classes(n, g->m, p.row, p.small_max, thr, bits(0), bits(1), bits(2), tiles,
+    const kb::ClassBounds bounds{p.small_max, p.mid_max, thr};
+    kb::launch_classes(n, g->m, p.row, bounds, bits, pitch, tiles,
                        opt->validate ? kb::CheckRows::kAll : kb::CheckRows::kOrder, ctr, s);
-    kb::launch_class_list(n, p.row, bits(1), tiles, 0, kMaxVertices, reinterpret_cast<int32_t*>(base + kOffMed), nullptr, s);
     NA_CUDA(cudaGetLastError());
     kb::Counters host_ctr{};
     NA_CUDA(cudaMemcpyAsync(&host_ctr, ctr, sizeof(host_ctr), cudaMemcpyDeviceToHost, s));
     NA_CUDA(cudaStreamSynchronize(s));
     if (host_ctr.err & kb::kErrInvalid) return KB_ERR_INVALID_ARG;
-    if (host_ctr.n_hubs > 0) return KB_ERR_INVALID_ARG;  // a degree above the hub threshold
-    p.n_med = host_ctr.n_med;
+    if (host_ctr.n_class[2] > 0) return KB_ERR_INVALID_ARG;  // a degree above the hub threshold
+    // the two lists share the array: together they hold at most n vertices
+    p.n_mid = host_ctr.n_class[0];
+    p.n_med = host_ctr.n_class[1];
+    int32_t* lists = reinterpret_cast<int32_t*>(base + kOffMed);
+    p.mid_v = lists;
+    p.med_v = lists + p.n_mid;
+    kb::launch_class_list(n, p.row, bits, pitch, tiles, kb::kMid, p.n_mid, lists, nullptr, s);
+    kb::launch_class_list(n, p.row, bits, pitch, tiles, kb::kMedium, p.n_med, lists + p.n_mid, nullptr, s);
 
     kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
+    kb::launch_mid_round(p, s);
     kb::launch_medium_round(p, s);
     kb::launch_renumber(p, reinterpret_cast<uint2*>(base + kOffPrefix), reinterpret_cast<uint32_t*>(base + kOffScan),
                         out, nullptr, false, s);

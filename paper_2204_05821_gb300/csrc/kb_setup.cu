@@ -288,50 +288,53 @@ __global__ void remap_cols_kernel(int64_t m, const int32_t* col, const int32_t* 
 }
 
 // ---- degree classes
-// One pass over the row offsets: bit v of edgeless / medium / hub says which
-// class v's degree falls in (no bit: 1 .. lo edges), counted per tile of
-// kListTile vertices and in ctr.  A CTA
-// counts its classes before it touches global memory (an atomic per warp on one
-// counter was 130 us of the pass over 10^7 vertices).
+// One pass over the row offsets: a bitmap per class (DegreeClass) says which one
+// a vertex's degree falls in (no bit: 1 .. bounds.small edges), counted per tile
+// of kListTile vertices and in ctr.  A CTA counts its classes before it touches
+// global memory (an atomic per warp on one counter was 130 us of the pass over
+// 10^7 vertices).
 constexpr int kListTile = 131072;  // vertices whose words one CTA of the list kernel turns into ids
 constexpr int kClassPer = 4096;    // vertices per CTA of the class kernel, at most; a divisor of kListTile
 
-__global__ void __launch_bounds__(256) classes_kernel(int64_t n, int64_t m, const int64_t* row, int32_t lo, int32_t hi,
-                                                      uint32_t* edgeless, uint32_t* medium, uint32_t* hub,
-                                                      uint32_t* tile_counts, int per, CheckRows check, Counters* ctr) {
-    __shared__ uint32_t s_n[2];
-    if (threadIdx.x < 2) s_n[threadIdx.x] = 0u;
+__global__ void __launch_bounds__(256) classes_kernel(int64_t n, int64_t m, const int64_t* row, ClassBounds bounds,
+                                                      uint32_t* bits, int64_t pitch, uint32_t* tile_counts, int per,
+                                                      CheckRows check, Counters* ctr) {
+    __shared__ uint32_t s_n[kClassLists];
+    if (threadIdx.x < kClassLists) s_n[threadIdx.x] = 0u;
     __syncthreads();
     const int lane = threadIdx.x & 31;
     const int64_t v0 = (int64_t)blockIdx.x * per;
     const int64_t nw = (n >> 5) + 1;
     bool bad = check == CheckRows::kAll && blockIdx.x == 0 && threadIdx.x == 0 && (row[0] != 0 || row[n] != m);
-    uint32_t nm = 0, nh = 0;
+    uint32_t c[kClassLists] = {0, 0, 0};
 #pragma unroll 4
     for (int i = 0; i < per / 256; ++i) {
         const int64_t v = v0 + i * 256 + threadIdx.x;
-        const int64_t d = v < n ? row[v + 1] - row[v] : lo;
+        const int64_t d = v < n ? row[v + 1] - row[v] : 1;
         bad |= d < 0;
-        const unsigned be = __ballot_sync(kFull, v < n && d == 0);
-        const unsigned bm = __ballot_sync(kFull, v < n && d > lo && d <= hi);
-        const unsigned bh = __ballot_sync(kFull, v < n && d > hi);
+        const bool mid = v < n && d > bounds.small && d <= bounds.mid, hub = v < n && d > bounds.medium;
+        unsigned w[1 + kClassLists];
+        w[kEdgeless] = __ballot_sync(kFull, d == 0);
+        w[kMid] = __ballot_sync(kFull, mid);
+        w[kMedium] = __ballot_sync(kFull, v < n && d > bounds.small && !mid && !hub);
+        w[kHub] = __ballot_sync(kFull, hub);
         if (lane == 0 && (v >> 5) < nw) {
-            edgeless[v >> 5] = be;
-            medium[v >> 5] = bm;
-            hub[v >> 5] = bh;
+#pragma unroll
+            for (int k = 0; k <= kClassLists; ++k) bits[k * pitch + (v >> 5)] = w[k];
         }
-        nm += __popc(bm);
-        nh += __popc(bh);
+#pragma unroll
+        for (int k = 0; k < kClassLists; ++k) c[k] += __popc(w[k + 1]);
     }
     if (lane == 0) {
-        if (nm) atomicAdd(&s_n[0], nm);
-        if (nh) atomicAdd(&s_n[1], nh);
+#pragma unroll
+        for (int k = 0; k < kClassLists; ++k)
+            if (c[k]) atomicAdd(&s_n[k], c[k]);
     }
     if (check != CheckRows::kNone && bad) atomicOr(&ctr->err, kErrInvalid);
     __syncthreads();
-    if (threadIdx.x < 2 && s_n[threadIdx.x]) {
-        atomicAdd(&tile_counts[2 * (v0 / kListTile) + threadIdx.x], s_n[threadIdx.x]);
-        atomicAdd(reinterpret_cast<unsigned long long*>(threadIdx.x ? &ctr->n_hubs : &ctr->n_med),
+    if (threadIdx.x < kClassLists && s_n[threadIdx.x]) {
+        atomicAdd(&tile_counts[kClassLists * (v0 / kListTile) + threadIdx.x], s_n[threadIdx.x]);
+        atomicAdd(reinterpret_cast<unsigned long long*>(&ctr->n_class[threadIdx.x]),
                   (unsigned long long)s_n[threadIdx.x]);
     }
 }
@@ -369,16 +372,15 @@ __device__ __forceinline__ int64_t block_exscan_i64(int64_t x, int64_t* tmp, int
 
 // The set bits of a class bitmap as ascending vertex ids (with their degrees
 // when deg is given): a CTA takes the words of one tile and finds its place from
-// the counts of the tiles before it (which: 0 medium, 1 hub).  Nothing is
-// written at or past cap.
+// the counts of the tiles before it.  Nothing is written at or past cap.
 static_assert(kListTile == kT * 4 * 32, "four words per thread");
 __global__ void __launch_bounds__(kT) class_list_kernel(int64_t n, const int64_t* row, const uint32_t* bits,
-                                                        const uint32_t* tile_counts, int which, int64_t cap,
-                                                        int32_t* out, int64_t* deg) {
+                                                        const uint32_t* tile_counts, int64_t cap, int32_t* out,
+                                                        int64_t* deg) {
     __shared__ int64_t tmp[32];
-    if (tile_counts[2 * (int64_t)blockIdx.x + which] == 0) return;  // uniform over the CTA
+    if (tile_counts[kClassLists * (int64_t)blockIdx.x] == 0) return;  // uniform over the CTA
     int64_t before = 0, base;
-    for (int64_t t = threadIdx.x; t < blockIdx.x; t += kT) before += tile_counts[2 * t + which];
+    for (int64_t t = threadIdx.x; t < blockIdx.x; t += kT) before += tile_counts[kClassLists * t];
     block_exscan_i64(before, tmp, &base);
     const int64_t nw = (n >> 5) + 1;
     const int64_t w0 = (int64_t)blockIdx.x * (kListTile / 32) + (int64_t)threadIdx.x * 4;
@@ -501,22 +503,22 @@ void launch_chunk_ext(int64_t chunks, int32_t n_hubs, const int32_t* hub_v, cons
 
 size_t class_tiles(int64_t n) { return (size_t)((n + kListTile - 1) / kListTile); }
 
-void launch_classes(int64_t n, int64_t m, const int64_t* row, int32_t lo, int32_t hi, uint32_t* edgeless,
-                    uint32_t* medium, uint32_t* hub, uint32_t* tile_counts, CheckRows check, Counters* ctr,
-                    cudaStream_t s) {
+void launch_classes(int64_t n, int64_t m, const int64_t* row, const ClassBounds& bounds, uint32_t* bits, int64_t pitch,
+                    uint32_t* tile_counts, CheckRows check, Counters* ctr, cudaStream_t s) {
     if (n <= 0) return;
-    cudaMemsetAsync(tile_counts, 0, 2 * sizeof(uint32_t) * class_tiles(n), s);
-    int per = 256;  // short CTAs on small graphs (11 us for 10^5 vertices in CTAs of 4096, 3 us in CTAs of 256)
+    cudaMemsetAsync(tile_counts, 0, kClassLists * sizeof(uint32_t) * class_tiles(n), s);
+    int per = 256;  // short CTAs on small graphs (11 us for 10^5 vertices in CTAs of 4096, 4 us in CTAs of 256)
     while (per < kClassPer && n > (int64_t)per * 152 * 8) per *= 2;
     // (n >> 5) + 1 words: the last one may lie past the last vertex
-    classes_kernel<<<(unsigned)((n + per) / per), 256, 0, s>>>(n, m, row, lo, hi, edgeless, medium, hub, tile_counts, per,
-                                                               check, ctr);
+    classes_kernel<<<(unsigned)((n + per) / per), 256, 0, s>>>(n, m, row, bounds, bits, pitch, tile_counts, per, check,
+                                                               ctr);
 }
 
-void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, const uint32_t* tile_counts, int which,
-                       int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s) {
+void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
+                       DegreeClass c, int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s) {
     if (n <= 0 || cap <= 0) return;
-    class_list_kernel<<<(unsigned)class_tiles(n), kT, 0, s>>>(n, row, bits, tile_counts, which, cap, out, deg);
+    class_list_kernel<<<(unsigned)class_tiles(n), kT, 0, s>>>(n, row, bits + c * pitch, tile_counts + c - 1, cap, out,
+                                                              deg);
 }
 
 void launch_locality_order(int64_t n, int64_t m, const int32_t* col, uint32_t* cnt, unsigned long long* hist,

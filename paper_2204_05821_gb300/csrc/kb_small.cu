@@ -1,19 +1,25 @@
-// Warp kernel for the vertices with at most 32 edges in the processed
+// Kernel for the vertices with at most kSmallDegree edges in the processed
 // direction (the large majority of vertices in power-law graphs), and for
 // level 0 (no edges; the key is the vertex label or a starting partition).
 //
-// One warp packs consecutive small vertices into its 32 lanes, one edge per
-// lane, so loads of neighbour ids and labels stay coalesced.  Everything after
-// the loads stays in registers:
-//   * duplicate pairs of a vertex (set semantics, Def. "signature") are found
-//     with two __match_any_sync calls, on the pair and on the owning vertex;
-//   * per-vertex counts and pair-mix sums come from one warp scan;
-//   * the full signature compare against a table representative (which is
-//     itself a small vertex: larger ones enter the table after this kernel)
-//     runs on every lane at once: each lane re-derives its representative's
-//     pairs and looks each up among its own vertex's pairs, which the warp
-//     parks in a 256-byte shared buffer; equality needs every pair of each
-//     side found on the other.
+// One lane per vertex: it loads four neighbours, labels and blocks at a time,
+// keeps its distinct pairs (set semantics, Def. "signature") in a column of
+// shared memory, sums their mixes, probes the table and, on a tag match, derives
+// the representative's pairs and looks each up among its own (the full
+// signature compare).  Representatives are small vertices too: larger ones enter
+// the table after this kernel.  Neighbouring lanes read neighbouring edges, so
+// the lines that one lane's load brings serve the others from L1.
+//
+// What bounds it: random 4-8 byte accesses (blocks, table, representatives) and
+// the instructions around them.  One edge per lane, with vertices packed into
+// windows of 32 edges by warp scans and matches, issued 730 warp instructions
+// per window of about six vertices and filled 55-61% of the issue slots; a lane
+// per vertex needs about a fifth of them and has four loads in flight per lane.
+// Round 1: 2871 -> 895 us with 10^8 power-law edges (and 207 us more in the mid
+// kernel, which takes 9 to 32 edges), 2733 -> 1385 us with 2 x 10^8 (+ 415 us),
+// 1795 -> 733 us on a batch of 5.5 x 10^7 Erdos-Renyi edges (+ 160 us).  Vertices
+// of up to 16 edges in this kernel lose (7311 against 6938 us for a whole call
+// when this was tried): their pairs take the L1 that the random loads need.
 //
 // Hot keys.  In power-law graphs millions of vertices share a key (all
 // edgeless vertices with the same label, all vertices with one edge to the
@@ -36,24 +42,18 @@ namespace {
 
 constexpr int kSmallThreads = 256;
 #ifndef KB_SMALL_MIN_BLOCKS
-#define KB_SMALL_MIN_BLOCKS 6  // caps registers at 40: 48 warps per SM (a few bytes spill)
+#define KB_SMALL_MIN_BLOCKS 5  // 48 registers, nothing spills; 6 CTAs per SM spill and cost a tenth of a whole call
 #endif
 constexpr int kSmallWarps = kSmallThreads / 32;
 constexpr int64_t kResidentWarps = 152 * KB_SMALL_MIN_BLOCKS * kSmallWarps;  // warps the chip holds at once
 // Joins a CTA can aggregate (1 x its vertices at the default task size; a
-// join that finds no room goes to global memory at once).  The map is kept
-// small on purpose: shared memory comes out of the SM's L1, and the L1 also
-// tracks the kernel's many outstanding random loads.
-#ifndef KB_MAP_CAP
-#define KB_MAP_CAP 1024
-#endif
-constexpr int kMapCap = KB_MAP_CAP;
+// join that finds no room goes to global memory at once).  Shared memory comes
+// out of the SM's L1, which the many outstanding random loads need, so no more;
+// 512 and 256 entries lose 2% and 7% of a whole call to hot keys.
+constexpr int kMapBits = 10;
+constexpr int kMapCap = 1 << kMapBits;
 constexpr uint64_t kMapEmpty = ~0ull;
 constexpr uint64_t kEmptyKeyBit = 1ull << 63;  // map key of an empty-signature join: bit 63 | own
-
-__device__ __forceinline__ uint64_t shfl64(uint64_t x, int src) {
-    return __shfl_sync(kFull, (unsigned long long)x, src);
-}
 
 struct JoinMap {
     uint64_t key[kMapCap];
@@ -64,7 +64,7 @@ struct JoinMap {
 // Record that v joins `key`; false when the map has no room (the caller then
 // joins globally right away).
 __device__ __forceinline__ bool map_join(JoinMap& M, uint64_t key, uint32_t hi, uint32_t v) {
-    uint32_t slot = (uint32_t)(mix64(key) >> 32) & (kMapCap - 1);
+    uint32_t slot = ((uint32_t)key * 2654435761u ^ (uint32_t)(key >> 63)) >> (32 - kMapBits);
     for (int t = 0; t < 32; ++t) {
         uint64_t cur = M.key[slot];
         if (cur == kMapEmpty) {
@@ -108,11 +108,12 @@ __device__ __forceinline__ void flush_join(const RoundParams& p, uint64_t key, u
 
 template <bool kLevel0, bool kCompact>
 __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_round_kernel(const RoundParams p) {
-    __shared__ uint64_t s_pairs[kSmallThreads];
+    __shared__ uint64_t s_pairs[kLevel0 ? 1 : kSmallDegree][kSmallThreads];
     __shared__ JoinMap M;
     __shared__ unsigned long long s_l0[kLevel0 ? 256 : 1];
+    __shared__ uint16_t s_off[kSmallWarps][kCompact ? 32 : 1];
     const int lane = threadIdx.x & 31;
-    uint64_t* wpairs = s_pairs + (threadIdx.x & ~31);
+    uint64_t* pairs = &s_pairs[0][threadIdx.x];  // this lane's distinct pairs, kSmallThreads apart
     for (int i = threadIdx.x; i < kMapCap; i += kSmallThreads) {
         M.key[i] = kMapEmpty;
         M.vmin[i] = 0xffffffffu;
@@ -129,20 +130,17 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
     // ones, or (kCompact, when many vertices are frozen) the next ones that
     // refine this round among the next kLook, so that frozen and inactive
     // vertices take no lane.  The next window is picked, and its row offsets
-    // and own blocks loaded, while the current one works (its start is known
-    // once the current one is packed).
+    // and own blocks loaded, before the current one works.
     constexpr int kLook = kCompact ? 128 : 32;
-    const int span = (int)(ve - vb);  // task vertices (at most 65536)
-    // next window: this lane's vertex as an offset from vb (-1: none), and
-    // packed: vertices picked (bits 0..5), more than 32 candidates in the span
-    // (bit 6), offset of the first vertex after the span (bits 7..)
-    int pf_off = -1;
-    int pf_win = 0;
+    const int span = (int)max(ve - vb, (int64_t)0);  // task vertices (at most 65536)
+    int pf_off = -1;  // next window: this lane's vertex as an offset from vb (-1: none)
+    int pf_next = 0;  // and where the window after it starts
     int64_t pf_a = 0;
     int32_t pf_d = 0, pf_own = 0;
     auto pick = [&](int c) {
         if (!kCompact) {  // the next 32 vertices
             pf_off = c + lane < span ? c + lane : -1;
+            pf_next = c + 32;
         } else {  // the next 32 that refine, among the next kLook
             unsigned bk[kLook / 32];
 #pragma unroll
@@ -150,16 +148,20 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
                 const int u = c + 32 * k + lane;
                 bk[k] = __ballot_sync(kFull, u < span && vertex_active(p, vb + u) && !vertex_frozen(p, vb + u));
             }
-            int rem = lane, total = 0;
-            pf_off = -1;
+            // every candidate hands its offset to the lane of its rank
+            uint16_t* offs = s_off[threadIdx.x >> 5];
+            int total = 0;
 #pragma unroll
             for (int k = 0; k < kLook / 32; ++k) {
-                const int ck = __popc(bk[k]);
-                if (pf_off < 0 && rem < ck) pf_off = c + 32 * k + __fns(bk[k], 0, rem + 1);
-                if (pf_off < 0) rem -= ck;
-                total += ck;
+                const int r = total + __popc(bk[k] & ((1u << lane) - 1u));
+                if (((bk[k] >> lane) & 1u) && r < 32) offs[r] = (uint16_t)(c + 32 * k + lane);
+                total += __popc(bk[k]);
             }
-            pf_win = min(total, 32) | (total > 32 ? 64 : 0) | (min(span, c + kLook) << 7);
+            __syncwarp();
+            const int o = offs[lane], last = offs[31];
+            __syncwarp();
+            pf_off = lane < total ? o : -1;
+            pf_next = total > 32 ? last + 1 : c + kLook;
         }
         if (pf_off >= 0) {
             const int64_t pv = vb + pf_off;
@@ -173,111 +175,59 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
     pick(0);
     for (int wc = 0; wc < span;) {
         const int64_t v0 = vb + wc;  // first vertex of a window of consecutive vertices (not kCompact)
-        const int nvw = kCompact ? pf_win & 63 : min(span - wc, 32);
-        const int64_t v = kCompact ? vb + pf_off : v0 + lane;  // meaningful for lanes < nvw
-        if (kCompact && nvw == 0) {  // nothing to key in this span
-            wc = pf_win >> 7;
-            if (wc < span) pick(wc);
-            continue;
-        }
-        const bool more = (pf_win & 64) != 0;
-        const int span_end = pf_win >> 7;
-        int cd = 0;
-        bool small = false;
-        int64_t a = 0;
-        int32_t own = 0;
+        const int64_t v = vb + pf_off;  // meaningful when this lane has a vertex
+        const int64_t a = pf_a;
+        int d = pf_d;
+        int32_t own = pf_own;
         bool l0 = kLevel0;
-        const int64_t cur_a = pf_a;
-        const int32_t cur_d = pf_d, cur_own = pf_own;
-        if (lane < nvw && (kCompact || (vertex_active(p, v) && !vertex_frozen(p, v)))) {
-            if (!kLevel0 && vertex_level0(p, v)) {
-                l0 = true;
-                own = p.vlab ? p.vlab[v] : 0;
-                small = true;
-            } else if (kLevel0) {
-                own = cur_own;
-                small = true;
-            } else {
-                own = cur_own;
-                a = cur_a;
-                small = cur_d <= p.small_max;
-                cd = small ? cur_d : 0;
-            }
+        bool pending = pf_off >= 0 && (kCompact || (vertex_active(p, v) && !vertex_frozen(p, v)));
+        if (!kLevel0 && pending && vertex_level0(p, v)) {
+            l0 = true;
+            own = p.vlab ? p.vlab[v] : 0;
         }
-        // pack whole vertices while their edges fit in 32 lanes
-        int incl = cd;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-            const int y = __shfl_up_sync(kFull, incl, o);
-            if (lane >= o) incl += y;
-        }
-        const unsigned fit = __ballot_sync(kFull, lane < nvw && incl <= 32);
-        const int nfit = __popc(fit);  // incl is non-decreasing, so the fitting lanes are 0..nfit-1
-        const int E = __shfl_sync(kFull, incl, nfit - 1);
-        const int start = incl - cd;
-        // the next window starts at the first vertex that did not fit, else
-        // after the last one picked, else after the span
-        if (!kCompact) {
-            wc += nfit;
-        } else {
-            const int o_nf = __shfl_sync(kFull, pf_off, nfit < 32 ? nfit : 31);
-            const int o_last = __shfl_sync(kFull, pf_off, 31);
-            wc = nfit < nvw ? o_nf : (more ? o_last + 1 : span_end);
-        }
+        if (kLevel0 || l0) d = 0;
+        pending = pending && d <= p.small_max;
+        wc = pf_next;
         if (wc < span) pick(wc);
 
-        uint64_t pr = 0;
-        int j = 0;
-        uint64_t c = 0;
-        uint32_t cu = 0;
-        if (!kLevel0) {
-            const bool owns = lane < nfit && cd > 0;
-            const unsigned heads = __reduce_or_sync(kFull, owns ? (1u << start) : 0u);
-            const unsigned has_e = __ballot_sync(kFull, owns);
-            if (lane < E) {
-                const unsigned upto = lane == 31 ? kFull : ((2u << lane) - 1u);
-                j = (int)__fns(has_e, 0, __popc(heads & upto));
-            }
-            const int64_t aj = __shfl_sync(kFull, (long long)a, j);
-            const int sj = __shfl_sync(kFull, start, j);
-            if (lane < E) {
-                const int64_t e = aj + (lane - sj);
-                const int32_t w = __ldcs(p.col + e);
-                const int32_t l = p.lab ? __ldcs(p.lab + e) : 0;
-                pr = pack_pair(l, (uint32_t)w, gather_block(p, w));
-                const unsigned act = E == 32 ? kFull : ((1u << E) - 1u);
-                const unsigned m = __match_any_sync(act, (unsigned long long)pr) & __match_any_sync(act, (unsigned)j);
-                if (__ffs(m) - 1 == lane) {
-                    c = pair_mix(pr);
-                    cu = 1;
-                }
-            }
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const uint64_t c2 = shfl64(c, lane >= o ? lane - o : lane);
-                const uint32_t u2 = __shfl_sync(kFull, cu, lane >= o ? lane - o : lane);
-                if (lane >= o) {
-                    c += c2;
-                    cu += u2;
-                }
-            }
-        }
-        const int src_end = max(start + cd - 1, 0), src_pre = max(start - 1, 0);
-        const uint64_t c_end = shfl64(c, src_end), c_pre = shfl64(c, src_pre);
-        const uint32_t u_end = __shfl_sync(kFull, cu, src_end), u_pre = __shfl_sync(kFull, cu, src_pre);
+        // this lane's distinct pairs and the sum of their mixes, four edges at a time
+        int cnt = 0;
         uint64_t acc = 0;
-        uint32_t cnt = 0;
-        if (cd > 0) {
-            acc = c_end - (start > 0 ? c_pre : 0ull);
-            cnt = u_end - (start > 0 ? u_pre : 0u);
+        if (!kLevel0) {
+            const int de = pending ? d : 0;
+            for (int k = 0; __any_sync(kFull, k < de); k += 4) {
+                int32_t w[4], l[4], b[4];
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    w[u] = l[u] = 0;
+                    if (k + u < de) {
+                        w[u] = __ldg(p.col + a + k + u);
+                        if (p.lab) l[u] = __ldg(p.lab + a + k + u);
+                    }
+                }
+#pragma unroll
+                for (int u = 0; u < 4; ++u)
+                    if (k + u < de) b[u] = gather_block(p, w[u]);
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    if (k + u >= de) break;
+                    const uint64_t x = pack_pair(l[u], (uint32_t)w[u], b[u]);
+                    bool seen = false;
+                    for (int t = 0; t < cnt; ++t) seen |= pairs[t * kSmallThreads] == x;
+                    if (!seen) {
+                        pairs[cnt * kSmallThreads] = x;
+                        acc += pair_mix(x);
+                        ++cnt;
+                    }
+                }
+            }
         }
 
-        bool pending = lane < nfit && small;
         bool inserted = false;
         uint64_t pos = 0;
-        uint32_t hi = 0, rep = 0;
+        uint32_t hi = 0;
         if (pending) {
-            if (!l0 && cd == 0) {
+            if (!l0 && d == 0) {
                 // (own block, empty set): grouped by the own block exactly
                 const uint64_t key = kEmptyKeyBit | (uint32_t)own;
                 if (!map_join(M, key, 0u, (uint32_t)v)) flush_join(p, key, 0u, (uint32_t)v);
@@ -285,16 +235,11 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
                 pending = false;
             } else {
                 // at level 0 of a multi-graph run the key is (graph, label)
-                const uint32_t c2 = (l0 && batched(p)) ? (uint32_t)p.vgraph[v] : cnt;
+                const uint32_t c2 = (l0 && batched(p)) ? (uint32_t)p.vgraph[v] : (uint32_t)cnt;
                 const uint64_t h = vertex_hash(own, c2, acc, p.hash_mode);
                 pos = h & p.mask;
                 hi = table_hi(h, p.epoch);
             }
-        }
-        if (!kLevel0) {
-            __syncwarp();
-            wpairs[lane] = pr;  // lanes >= E hold unused values
-            __syncwarp();
         }
         // Level 0 of one graph: the key is the label alone, so a slot that a
         // lane of this CTA found (or claimed) for a label serves later lanes
@@ -314,57 +259,61 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
                 }
             }
         }
-        const unsigned vmask = cd >= 32 ? kFull : ((1u << cd) - 1u);
-        while (__any_sync(kFull, pending)) {
+        for (int probes = 0; __any_sync(kFull, pending); ++probes) {
             if (!pending) continue;
-            const int r = probe_table(p, &pos, hi, (uint32_t)v, &rep, false);
-            if (r == 0) {
-                inserted = true;
-                pending = false;
-                continue;
-            }
-            if (r == 2) {
+            if (probes > kProbeLimit) {
                 set_error(p.ctr, kErrTableFull);
                 pending = false;
                 continue;
             }
-            // full signature compare with the representative, on this lane;
-            // its key and its row offsets are loaded together
-            const int32_t* keys = (l0 && !kLevel0) ? p.vlab : ((!kLevel0 && p.own_key) ? p.own_key : p.prev);
-            const int32_t rkey = keys ? __ldg(keys + rep) : 0;
-            int64_t rb = 0, re = 0;
-            if (!l0) {
-                rb = p.row[rep];
-                re = p.row[(int64_t)rep + 1];
+            const uint64_t cur = volatile_load(&p.table[pos]);
+            if ((uint32_t)(cur >> 56) != p.epoch) {
+                const unsigned long long want = ((uint64_t)hi << 32) | kSingleBit | (uint32_t)v;
+                if (atomicCAS(reinterpret_cast<unsigned long long*>(&p.table[pos]), (unsigned long long)cur, want) != cur)
+                    continue;  // taken
+                p.slot_of[v] = (int32_t)pos;
+                inserted = true;
+                pending = false;
+                continue;
             }
-            bool eq = same_graph(p, rep, v) && rkey == own;
-            if (!l0 && eq) {
-                unsigned vfound = 0;
-                for (int64_t e0 = rb; e0 < re && eq; e0 += 4) {
-                    uint64_t x[4];
+            bool eq = false;
+            if ((uint32_t)(cur >> 32) == hi) {
+                // full signature compare with the representative: its key and its
+                // row offsets are loaded together
+                const uint32_t rep = (uint32_t)cur & kVertexMask;
+                const int32_t* keys = (l0 && !kLevel0) ? p.vlab : ((!kLevel0 && p.own_key) ? p.own_key : p.prev);
+                const int32_t rkey = keys ? __ldg(keys + rep) : 0;
+                int64_t rb = 0, re = 0;
+                if (!l0) {
+                    rb = p.row[rep];
+                    re = p.row[(int64_t)rep + 1];
+                }
+                eq = same_graph(p, rep, v) && rkey == own;
+                if (!l0 && eq) {
+                    unsigned found = 0;
+                    for (int64_t e0 = rb; e0 < re && eq; e0 += 4) {
+                        uint64_t x[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        x[u] = 0;
-                        if (e0 + u < re) {
-                            const int32_t w = __ldg(p.col + e0 + u);
-                            const int32_t l = p.lab ? __ldg(p.lab + e0 + u) : 0;
-                            x[u] = pack_pair(l, (uint32_t)w, gather_block(p, w));
-                        }
-                    }
-#pragma unroll
-                    for (int u = 0; u < 4; ++u) {
-                        if (e0 + u >= re) break;
-                        bool found = false;
-                        for (int t = 0; t < cd; ++t) {
-                            if (wpairs[start + t] == x[u]) {
-                                vfound |= 1u << t;
-                                found = true;
+                        for (int u = 0; u < 4; ++u) {
+                            x[u] = 0;
+                            if (e0 + u < re) {
+                                const int32_t w = __ldg(p.col + e0 + u);
+                                const int32_t l = p.lab ? __ldg(p.lab + e0 + u) : 0;
+                                x[u] = pack_pair(l, (uint32_t)w, gather_block(p, w));
                             }
                         }
-                        if (!found) eq = false;
+#pragma unroll
+                        for (int u = 0; u < 4; ++u) {
+                            if (e0 + u >= re) break;
+                            unsigned hit = 0;
+                            for (int t = 0; t < cnt; ++t)
+                                if (pairs[t * kSmallThreads] == x[u]) hit = 1u << t;
+                            if (!hit) eq = false;
+                            found |= hit;
+                        }
                     }
+                    if (found != (1u << cnt) - 1u) eq = false;
                 }
-                if (vfound != vmask) eq = false;
             }
             if (eq) {
                 if (!map_join(M, pos, hi, (uint32_t)v)) flush_join(p, pos, hi, (uint32_t)v);
@@ -382,12 +331,10 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
         if (!kCompact) {
             const uint32_t sh = (uint32_t)(v0 & 31);
             const int64_t w0 = v0 >> 5;
-            const bool in0 = (v >> 5) == w0;
-            const unsigned m0 = __ballot_sync(kFull, inserted && in0);
-            const unsigned m1 = __ballot_sync(kFull, inserted && !in0);
-            if (lane == 0) {
-                if (m0) atomicXor(&p.bitmap[w0], m0 << sh);
-                if (m1) atomicXor(&p.bitmap[w0 + 1], m1 >> (32 - sh));
+            const unsigned m = __ballot_sync(kFull, inserted);
+            if (lane == 0 && m) {
+                atomicXor(&p.bitmap[w0], m << sh);
+                if (sh && (m >> (32 - sh))) atomicXor(&p.bitmap[w0 + 1], m >> (32 - sh));
             }
         } else {
             unsigned todo = __ballot_sync(kFull, inserted);
@@ -413,11 +360,9 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
 // two waves of resident warps, between lo and hi.  A warp walks its task window
 // after window, each a chain of dependent loads (offsets, neighbours, blocks,
 // table, representative), so a graph that fills only part of the chip with
-// tasks of 128 is bound by the length of that chain: one round of 10^4 vertices
-// and 5 x 10^4 edges took 104 us with tasks of 128 (10 CTAs) and 18 us with
-// tasks of 8.  From about 1.9 x 10^6 vertices on every task has 128.  One and
-// four waves measured the same, except one wave at 10^6 vertices (2374 -> 2522
-// us for a whole backward refinement: its second, nearly empty wave).
+// tasks of 128 is bound by the length of that chain (104 against 18 us for a
+// round of 10^4 vertices when windows held six of them).  From about 1.6 x 10^6
+// vertices on every task has 128.
 static int64_t task_vertices(int64_t n, int64_t lo, int64_t hi) {
     const int64_t per = (n + 2 * kResidentWarps - 1) / (2 * kResidentWarps);
     return std::min(hi, std::max(lo, (per + 7) & ~(int64_t)7));
@@ -426,9 +371,7 @@ static int64_t task_vertices(int64_t n, int64_t lo, int64_t hi) {
 void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s) {
     if (p.n <= 0) return;
     const bool compact = windows != SmallWindows::kConsecutive;
-    // consecutive windows hold about six vertices (32 edges), packed and
-    // level-0 windows up to 32
-    int64_t wv = p.warp_verts > 0 ? p.warp_verts : task_vertices(p.n, (level0 || compact) ? 32 : 8, kDefaultWarpVerts);
+    int64_t wv = p.warp_verts > 0 ? p.warp_verts : task_vertices(p.n, 32, kDefaultWarpVerts);
     // few vertices refine: long warp tasks, so that far fewer CTAs set up and
     // flush a join map for a handful of vertices each
     if (windows == SmallWindows::kSparse) wv = task_vertices(p.n, kDefaultWarpVerts, 4096);
