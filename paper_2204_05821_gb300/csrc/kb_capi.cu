@@ -1418,10 +1418,9 @@ kb_status summary_impl(kb_context* ctx, const kb_graph* g, int direction, int us
     const int64_t m = g->m;
     const uint64_t cap = std::max<uint64_t>(1024, next_pow2((uint64_t)(m + m / 4 + 64)));
     const int64_t nw = (m >> 5) + 1;
-    const size_t sz_table = 16 * (size_t)cap, sz_first = 8 * (size_t)cap, sz_bitmap = 4 * (size_t)nw,
+    const size_t sz_table = 16 * (size_t)cap, sz_bitmap = 4 * (size_t)nw,
                  sz_prefix = 4 * (size_t)(nw + 1), sz_scan = 4 * kb::scan_tmp_words(nw);
-    const size_t total = align_up(sz_table) + align_up(sz_first) + align_up(sz_bitmap) + align_up(sz_prefix) +
-                         align_up(sz_scan);
+    const size_t total = align_up(sz_table) + align_up(sz_bitmap) + align_up(sz_prefix) + align_up(sz_scan);
     KB_TRY(ensure_buffer(ctx, &ctx->sum_buf, &ctx->sum_buf_bytes, total));
     char* base = reinterpret_cast<char*>(ctx->sum_buf);
     kb::SummaryParams q{};
@@ -1436,8 +1435,6 @@ kb_status summary_impl(kb_context* ctx, const kb_graph* g, int direction, int us
     size_t off = 0;
     q.table = reinterpret_cast<unsigned long long*>(base + off);
     off += align_up(sz_table);
-    q.first = reinterpret_cast<unsigned long long*>(base + off);
-    off += align_up(sz_first);
     q.bitmap = reinterpret_cast<uint32_t*>(base + off);
     off += align_up(sz_bitmap);
     uint32_t* prefix = reinterpret_cast<uint32_t*>(base + off);
@@ -1449,14 +1446,10 @@ kb_status summary_impl(kb_context* ctx, const kb_graph* g, int direction, int us
     auto run = [&]() -> kb_status {
         KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
         KB_CUDA(ctx, cudaMemsetAsync(q.table, 0, sz_table, s));
-        KB_CUDA(ctx, cudaMemsetAsync(q.first, 0xff, sz_first, s));
         KB_CUDA(ctx, cudaMemsetAsync(q.bitmap, 0, sz_bitmap, s));
         kb::launch_validate(g->n, m, g->row_offsets, g->col_indices, ctx->d_ctr, s);
-        KB_CUDA(ctx, cudaGetLastError());
-        KB_TRY(read_counters(ctx));
-        KB_TRY(device_error(ctx));
+        // (the insert does nothing when that found something)
         kb::launch_summary_insert(q, s);
-        kb::launch_summary_mark(q, s);
         kb::launch_bitmap_rank(q.bitmap, nw, scan_tmp, prefix, ctx->d_ctr, s);
         KB_CUDA(ctx, cudaGetLastError());
         KB_TRY(read_counters(ctx));

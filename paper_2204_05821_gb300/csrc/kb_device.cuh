@@ -112,4 +112,65 @@ __device__ __forceinline__ int probe_table(const RoundParams& p, uint64_t* pos_i
     }
     return 2;
 }
+// ---- tiles of consecutive edges
+// Source vertex of edge e, the largest v with row[v] <= e, by a whole warp: each
+// step reads 32 offsets at once and keeps one of 33 parts (a search by halves is
+// 20 dependent loads, 12 us, that a tile's CTA has to wait for).
+__device__ __forceinline__ int64_t edge_source(const int64_t* row, int64_t n, int64_t e) {
+    const int lane = threadIdx.x & 31;
+    int64_t lo = 0, hi = n;  // row[lo] <= e < row[hi]
+    while (hi - lo > 1) {
+        const int64_t at = lo + (lane + 1) * (hi - lo) / 33;
+        const int c = __popc(__ballot_sync(kFull, row[at] <= e));  // ascending over the lanes
+        const int64_t below = __shfl_sync(kFull, (long long)at, max(c - 1, 0));
+        const int64_t above = __shfl_sync(kFull, (long long)at, min(c, 31));
+        if (c > 0) lo = below;
+        if (c < 32) hi = above;
+    }
+    return lo;
+}
+
+// Sources of the edges [e0, e1) of a tile of kThreads x kPer edges, for a whole
+// CTA of kThreads: s_src[i] = source of edge e0 + i.  Two warps search for the
+// first and last edge's source, every vertex between them that has edges marks
+// its first one, and a running maximum fills the rest (a search per edge reads
+// a dozen offsets each).  Begins and ends with a barrier.
+template <int kThreads, int kPer>
+__device__ __forceinline__ void tile_sources(int64_t n, const int64_t* row, int64_t e0, int64_t e1, int32_t* s_src) {
+    __shared__ int64_t s_v[2];
+    __shared__ int32_t s_warp[kThreads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    __syncthreads();
+    if (warp < 2) {
+        const int64_t v = edge_source(row, n, warp ? e1 - 1 : e0);
+        if (lane == 0) s_v[warp] = v;
+    }
+    for (int i = tid; i < kThreads * kPer; i += kThreads) s_src[i] = -1;
+    __syncthreads();
+    for (int64_t v = s_v[0] + tid; v <= s_v[1]; v += kThreads) {
+        const int64_t a = row[v], b = row[v + 1];
+        if (b > a && b > e0 && a < e1) s_src[max(a, e0) - e0] = (int32_t)v;
+    }
+    __syncthreads();
+    int32_t run[kPer], mx = -1;
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) {
+        mx = max(mx, s_src[tid * kPer + u]);
+        run[u] = mx;
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int32_t y = __shfl_up_sync(kFull, mx, o);
+        if (lane >= o) mx = max(mx, y);
+    }
+    if (lane == 31) s_warp[warp] = mx;
+    int32_t before = __shfl_up_sync(kFull, mx, 1);
+    if (lane == 0) before = -1;
+    __syncthreads();
+    for (int i = 0; i < warp; ++i) before = max(before, s_warp[i]);
+#pragma unroll
+    for (int u = 0; u < kPer; ++u) s_src[tid * kPer + u] = max(run[u], before);
+    __syncthreads();
+}
+
 }  // namespace kb

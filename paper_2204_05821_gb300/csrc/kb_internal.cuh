@@ -363,14 +363,12 @@ struct SummaryParams {
     int32_t dir;                // 0: x = source, y = target; 1: reversed
     const int32_t* lsrc;        // [n] block of x
     const int32_t* ldst;        // [n] block of y
-    unsigned long long* table;  // [2 * cap] 16-byte slots; both words zero = empty
-    unsigned long long* first;  // [cap] smallest edge index of the slot's triple
+    unsigned long long* table;  // [2 * cap] 16-byte slots (summary_insert_kernel); both words zero = empty
     uint64_t mask;              // cap - 1
     uint32_t* bitmap;           // [m/32+1] edges that are first occurrences
     Counters* ctr;
 };
 void launch_summary_insert(const SummaryParams& q, cudaStream_t s);
-void launch_summary_mark(const SummaryParams& q, cudaStream_t s);
 void launch_summary_emit(const SummaryParams& q, const uint32_t* prefix, int32_t* out_src, int32_t* out_label,
                          int32_t* out_dst, cudaStream_t s);
 // fill out[i] = i (kb_kernels.cu)

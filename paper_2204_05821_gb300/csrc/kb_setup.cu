@@ -4,12 +4,11 @@
 // hub discovery, an int64 prefix scan and level-row copies.
 #include <cuda_runtime.h>
 
+#include "kb_device.cuh"
 #include "kb_internal.cuh"
 
 namespace kb {
 namespace {
-
-constexpr uint32_t kFull = 0xffffffffu;
 
 int grid_for(int64_t n, int threads) {
     int64_t b = (n + threads - 1) / threads;
@@ -84,16 +83,6 @@ __global__ void __launch_bounds__(kCsrThreads) in_degree_kernel(int64_t m, const
     }
 }
 
-// Source vertex of edge e: the largest v with row[v] <= e.
-__device__ __forceinline__ int64_t edge_source(const int64_t* row, int64_t n, int64_t e) {
-    int64_t lo = 0, hi = n;  // row[lo] <= e < row[hi]
-    while (hi - lo > 1) {
-        const int64_t mid = (lo + hi) >> 1;
-        if (row[mid] <= e) lo = mid; else hi = mid;
-    }
-    return lo;
-}
-
 __global__ void rows_kernel(int64_t n, const int64_t* row, const int64_t* in_prefix, int include_out,
                             int64_t* row_p, int64_t* cursor) {
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
@@ -105,18 +94,14 @@ __global__ void rows_kernel(int64_t n, const int64_t* row, const int64_t* in_pre
 }
 
 // Writes every edge at its target's cursor (and, for both directions, at its
-// place among the source's out-edges, e + in_prefix[source]).  The tile's
-// sources come from the offsets between its first and its last edge's: every
-// vertex with edges marks its first one, a running maximum does the rest.
+// place among the source's out-edges, e + in_prefix[source]).
 __global__ void __launch_bounds__(kCsrThreads) place_edges_kernel(int64_t n, int64_t m, const int64_t* row,
                                                                   const int32_t* col, const int32_t* lab,
                                                                   int include_out, const int64_t* in_prefix,
                                                                   int32_t* col_p, int32_t* lab_p, int64_t* cursor) {
     __shared__ uint2 tab[kCsrSlots];  // (target, edges), then the target's first position in the tile
     __shared__ int32_t s_src[kCsrTile];
-    __shared__ int64_t s_v[2];
-    __shared__ int32_t s_warp[kCsrThreads / 32];
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tid = threadIdx.x;
     const int64_t e0 = (int64_t)blockIdx.x * kCsrTile;
     const int64_t e1 = min(m, e0 + kCsrTile);
     uint32_t w[kCsrPer];
@@ -127,9 +112,7 @@ __global__ void __launch_bounds__(kCsrThreads) place_edges_kernel(int64_t n, int
         w[u] = e < e1 ? (uint32_t)__ldcs(col + e) : kNoTarget;
         l[u] = lab && e < e1 ? __ldcs(lab + e) : 0;
     }
-    if (tid < 2) s_v[tid] = edge_source(row, n, tid ? e1 - 1 : e0);
     clear_tile(tab);
-    for (int i = tid; i < kCsrTile; i += kCsrThreads) s_src[i] = -1;
     __syncthreads();
     uint32_t at[kCsrPer];  // slot << 16 | edges of the tile with this target before this one
 #pragma unroll
@@ -139,10 +122,6 @@ __global__ void __launch_bounds__(kCsrThreads) place_edges_kernel(int64_t n, int
         const int slot = tile_slot(tab, w[u]);
         at[u] = ((uint32_t)slot << 16) | atomicAdd(&tab[slot].y, 1u);
     }
-    for (int64_t v = s_v[0] + tid; v <= s_v[1]; v += kCsrThreads) {
-        const int64_t a = row[v], b = row[v + 1];
-        if (b > a && b > e0 && a < e1) s_src[max(a, e0) - e0] = (int32_t)v;
-    }
     __syncthreads();
     for (int i = tid; i < kCsrSlots; i += kCsrThreads) {
         const uint2 t = tab[i];
@@ -151,26 +130,7 @@ __global__ void __launch_bounds__(kCsrThreads) place_edges_kernel(int64_t n, int
             atomicAdd(reinterpret_cast<unsigned long long*>(&cursor[t.x]), (unsigned long long)t.y);
         tab[i] = make_uint2((uint32_t)first, (uint32_t)(first >> 32));
     }
-    // running maximum over the tile, kCsrPer consecutive entries per thread
-    int32_t run[kCsrPer], mx = -1;
-#pragma unroll
-    for (int u = 0; u < kCsrPer; ++u) {
-        mx = max(mx, s_src[tid * kCsrPer + u]);
-        run[u] = mx;
-    }
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-        const int32_t y = __shfl_up_sync(kFull, mx, o);
-        if (lane >= o) mx = max(mx, y);
-    }
-    if (lane == 31) s_warp[warp] = mx;
-    int32_t before = __shfl_up_sync(kFull, mx, 1);
-    if (lane == 0) before = -1;
-    __syncthreads();
-    for (int i = 0; i < warp; ++i) before = max(before, s_warp[i]);
-#pragma unroll
-    for (int u = 0; u < kCsrPer; ++u) s_src[tid * kCsrPer + u] = max(run[u], before);
-    __syncthreads();
+    tile_sources<kCsrThreads, kCsrPer>(n, row, e0, e1, s_src);
 #pragma unroll
     for (int u = 0; u < kCsrPer; ++u) {
         if (w[u] == kNoTarget) continue;
