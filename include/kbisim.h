@@ -405,8 +405,8 @@ kb_status kb_get_round_work(const kb_context* ctx, int64_t* vertices, int64_t* e
  *   counts                 HOST int64[G*(k_max+1)]; counts[j*(k_max+1)+i]
  *   levels_computed        HOST int32[G] or NULL
  * Rounds run for all active graphs at once: one signature launch per round over
- * the union, the whole k_max-round loop captured once in a CUDA graph and
- * replayed, and a device-side per-graph stop flag (no host sync per round). */
+ * the union, a per-graph stop test on the device, and a host that queues each
+ * round before it looks at the one before, until no graph refines. */
 kb_status kb_refine_batch(kb_context* ctx, const kb_graph* union_graph,
                           const int64_t* graph_vertex_offsets, int64_t G,
                           const int32_t* k_per_graph, const kb_options* opt, int32_t* levels,

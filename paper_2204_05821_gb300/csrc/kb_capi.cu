@@ -30,7 +30,8 @@ struct kb_context {
     size_t own_ws_bytes = 0;
     // small persistent device state
     kb::Counters* d_ctr = nullptr;
-    kb::Counters* h_ctr = nullptr;  // pinned
+    kb::Counters* h_ctr = nullptr;  // pinned: the last counters read, and a slot per round in flight (queue_counters)
+    cudaEvent_t slot_ev[4] = {};
     uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
     char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
     void* class_tmp = nullptr;    // degree-class bitmaps, tile counts and hub list during planning
@@ -68,7 +69,6 @@ struct kb_context {
     void* upd_buf = nullptr;
     size_t upd_buf_bytes = 0;
     unsigned long long* d_work = nullptr;  // |W| of the current round
-    cudaStream_t cap_stream = nullptr;  // non-default stream used only to capture CUDA graphs
     cudaStream_t copy_stream = nullptr;  // level rows back to the host (kb_refine_host)
     cudaEvent_t row_ev = nullptr;
     // timing: CUDA events per kernel family; with work, also the vertices and
@@ -172,7 +172,7 @@ struct Plan {
     size_t csr_bytes = 0;
     size_t o_emin = 0, o_mid = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
-           o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_bm2 = 0, o_moved = 0, o_mark = 0;
+           o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_moved = 0, o_mark = 0;
     size_t total = 0;
     // bytes of one degree-class bitmap; four follow one another (kb::DegreeClass)
     size_t class_bytes() const { return align_up(sizeof(uint32_t) * (size_t)((n >> 5) + 1)); }
@@ -261,7 +261,6 @@ void layout_round(Plan& P) {
     P.o_shared = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_minof = take(own_freeze ? sizeof(uint32_t) * (size_t)P.n : 0);
     P.o_joined = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
-    P.o_bm2 = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_moved = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_mark = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.total = off;
@@ -315,6 +314,24 @@ kb_status ensure_buffer(kb_context* ctx, void** buf, size_t* have, size_t need) 
 kb_status read_counters(kb_context* ctx) {
     KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(Counters), cudaMemcpyDeviceToHost, ctx->stream));
     KB_CUDA(ctx, cudaStreamSynchronize(ctx->stream));
+    return KB_OK;
+}
+
+// The counters as they are after what is queued now (`round`), and waiting for
+// them (into ctx->h_ctr) while later rounds are queued already.
+constexpr int kCounterSlots = 4;
+
+kb_status queue_counters(kb_context* ctx, int round) {
+    const int slot = round % kCounterSlots;
+    KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_ctr + 1 + slot, ctx->d_ctr, sizeof(Counters), cudaMemcpyDeviceToHost, ctx->stream));
+    KB_CUDA(ctx, cudaEventRecord(ctx->slot_ev[slot], ctx->stream));
+    return KB_OK;
+}
+
+kb_status wait_counters(kb_context* ctx, int round) {
+    const int slot = round % kCounterSlots;
+    KB_CUDA(ctx, cudaEventSynchronize(ctx->slot_ev[slot]));
+    *ctx->h_ctr = ctx->h_ctr[1 + slot];
     return KB_OK;
 }
 
@@ -444,10 +461,10 @@ int32_t pick_field(int32_t given, int32_t cached, int32_t dflt) { return given ?
 // blocks, table size, medium split and warp task size.
 void resolve_call_fields(Plan& P, const kb_options* opt, int rounds, bool multi, const kb_tuning* T) {
     P.subject = opt->subject;
-    // stratified rounds of one graph or (multi) of batched and served graphs;
-    // incremental refinement plans without, and generic CSE keys need not
-    // hold the own previous block
-    P.freeze = (rounds >= 0 || multi) && P.subject == KB_SUBJECT_PREVIOUS && opt->rekey_all == 0;
+    // stratified rounds of one graph, and always of batched and served graphs
+    // (multi); incremental refinement plans without, and generic CSE keys need
+    // not hold the own previous block
+    P.freeze = multi || (rounds >= 0 && P.subject == KB_SUBJECT_PREVIOUS && opt->rekey_all == 0);
     P.dense0 = !multi;
     P.med_split = pick_field(opt->medium_split, T ? T->medium_split : 0, kb::kDefaultMedSplit);
     P.warp_verts = pick_field(opt->small_task_vertices, T ? T->small_task_vertices : 0, 0);
@@ -555,6 +572,7 @@ struct Prepared {
     kb::RoundParams p{};
     uint2* prefix = nullptr;  // rank words of the renumbering (launch_renumber)
     uint32_t* scan_tmp = nullptr;
+    uint8_t* gactive = nullptr;  // several graphs: those that refine
     int64_t total_chunks = 0;
     size_t set_bytes = 0;
     uint32_t epoch_own = 0, round_own = 0;
@@ -566,12 +584,9 @@ struct Prepared {
     uint32_t* frozen = nullptr;
     uint32_t* frozen_min = nullptr;
     uint32_t* edgeless = nullptr;
-    // clean blocks (frozen blocks on): the two bitmaps of block minima used in
-    // turn (this level's and the previous level's), moved vertices and marked
-    // (dirty) blocks; RoundParams::minof
-    uint32_t* bm[2] = {nullptr, nullptr};
-    int bm_cur = 0;
-    bool bitmap_ready = false;  // the next round's bitmap holds the minima of its frozen blocks (next_minima)
+    // clean blocks (frozen blocks on): moved vertices and marked (dirty)
+    // blocks; RoundParams::minof
+    bool bitmap_ready = false;  // the round's bitmap holds the minima of its frozen blocks already
     bool counters_clear = false;  // the round need not clear the counters (no errors so far; see launch_renumber)
     uint32_t* moved = nullptr;
     uint32_t* mark = nullptr;
@@ -839,9 +854,6 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
         for (int c = 0; c < 3; ++c)
             R.class_bits[c] = members[c] ? reinterpret_cast<uint32_t*>(gws + P.o_classes + (size_t)(c + 1) * P.class_bytes())
                                          : nullptr;
-        R.bm[0] = p.bitmap;
-        R.bm[1] = reinterpret_cast<uint32_t*>(ws + P.o_bm2);
-        R.bm_cur = 0;
         p.joined = reinterpret_cast<uint32_t*>(ws + P.o_joined);  // all clear between rounds
         KB_CUDA(ctx, cudaMemsetAsync(p.joined, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
         if (R.ext_frozen) {
@@ -892,22 +904,21 @@ kb_status next_empty_round(kb_context* ctx, Prepared& R, cudaStream_t s) {
     return KB_OK;
 }
 
-// Where the minima of the next round's frozen blocks go: straight into the
-// bitmap that round builds its minima in (the server, which can admit and move
-// graphs in between, keeps them apart).
-uint32_t* next_minima(const Prepared& R) { return R.ext_frozen ? R.frozen_min : R.bm[R.bm_cur ^ 1]; }
-
 // The freeze pass after a signature round of one graph or a batch.
-kb::FreezePass freeze_pass(kb_context* ctx, const Prepared& R, const int32_t* level) {
+kb::FreezePass freeze_pass(kb_context* ctx, const Prepared& R) {
     kb::FreezePass f;
     f.n = R.p.n;
     f.bitmap = R.p.bitmap;
     f.shared = R.p.shared;
     f.edgeless = R.edgeless;
-    f.level = level;
+    f.names = R.p.minof;
     f.mark = R.mark;
     f.frozen = R.frozen;
-    f.frozen_min = next_minima(R);
+    // straight into the bitmap, which the next round builds on (the server, which
+    // can admit and move graphs in between, keeps the minima apart)
+    f.frozen_min = R.ext_frozen ? R.frozen_min : R.p.bitmap;
+    f.vgraph = R.p.lgraph;
+    f.gactive = R.gactive;
     f.moved_clear = R.p.perm ? R.moved : nullptr;
     for (int c = 0; c < 3; ++c) f.classes[c] = R.class_bits[c];
     f.ctr = ctx->d_ctr;
@@ -950,7 +961,7 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
     // a starting level may mix edgeless vertices with others in one block:
     // only its singletons are frozen in the first round
     if (R.p.shared) {
-        kb::FreezePass f = freeze_pass(ctx, R, out);
+        kb::FreezePass f = freeze_pass(ctx, R);
         f.edgeless = nullptr;
         f.mark = nullptr;
         f.moved_clear = nullptr;
@@ -1128,10 +1139,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         p.frozen = R.frozen;
         p.frozen_min = R.frozen_min;
         if (p.minof) {
-            // the minima of level i-1 stay readable while level i's are built
-            p.bitmap_prev = R.bm[R.bm_cur];
-            R.bm_cur ^= 1;
-            p.bitmap = R.bm[R.bm_cur];
+            p.prev = reinterpret_cast<const int32_t*>(p.minof);  // blocks by name
             p.moved = R.moved;
         }
         int32_t* out = rows.row(i);
@@ -1150,8 +1158,8 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         // one previous block; and clean blocks, none of whose members has an
         // edge to a vertex whose smallest block member this round changed
         if (p.shared && i < k) {
-            kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, stop_stable, s);
-            kb::FreezePass f = freeze_pass(ctx, R, out);
+            kb::launch_dirty_blocks(p, R.edgeless, R.moved, kb::kMaxHubThreshold, R.mark, nullptr, stop_stable, s);
+            kb::FreezePass f = freeze_pass(ctx, R);
             f.stop_stable = stop_stable;
             kb::launch_freeze_clean(f, s);
             R.bitmap_ready = true;
@@ -1193,7 +1201,8 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
                 if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
                 KB_TRY(emit_rows(ctx, rows, i, k));
             } else if (p.minof) {
-                KB_CUDA(ctx, cudaMemcpyAsync(out, p.prev, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
+                KB_CUDA(ctx, cudaMemcpyAsync(out, rows.row(i - 1), sizeof(int32_t) * (size_t)n,
+                                             cudaMemcpyDeviceToDevice, s));
             }
             if (counts)
                 for (int j = i + 1; j <= k; ++j) counts[j] = c;
@@ -1501,11 +1510,12 @@ kb_status fixpoint_impl(kb_context* ctx, const kb_graph* g, const kb_options* op
 }
 
 // Batched refinement of G graphs held as one disjoint union (see
-// kb_refine_batch in kbisim.h).  Block ids are union-global while the rounds
-// run: the own previous block is part of every key, so vertices of different
-// graphs never share a block, and level 0 hashes the graph id into the key.
-// Rounds 1..k_max are captured once into a CUDA graph; per-graph stopping is
-// decided on the device, so the loop needs no host synchronisation.
+// kb_refine_batch in kbisim.h).  Blocks go by their smallest member while the
+// rounds run: the own previous block is part of every key, so vertices of
+// different graphs never share a block, and level 0 hashes the graph id into the
+// key.  Stopping is decided per graph on the device, which freezes all blocks of
+// a stopped graph.  The host queues every round before it looks at the one
+// before, and stops once no graph refines.
 kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, int64_t G, const int32_t* k_h,
                      const kb_options* opt, int32_t* levels, int64_t* counts, int32_t* lc_out) {
     if (!g || !opt) return fail(ctx, KB_ERR_INVALID_ARG, "graph and options must not be NULL");
@@ -1540,133 +1550,99 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
     kb::RoundParams& p = R.p;
 
     // batch scratch
-    const int64_t nw = (n >> 5) + 1;
     size_t off = 0;
     auto take = [&](size_t b) { size_t o = off; off += align_up(b); return o; };
     const size_t o_vgraph = take(sizeof(int32_t) * (size_t)n);
     const size_t o_voff = take(sizeof(int64_t) * (size_t)(G + 1));
     const size_t o_k = take(sizeof(int32_t) * (size_t)G);
     const size_t o_act = take((size_t)G);
-    const size_t o_early = take((size_t)G);
     const size_t o_last = take(sizeof(int32_t) * (size_t)G);
-    const size_t o_sticky = take(sizeof(int32_t));
+    const size_t up_bytes = off - o_voff;  // voff .. glast come from the host in one copy
     const size_t o_bases = take(sizeof(uint32_t) * (size_t)(G + 1) * (size_t)(kmax + 1));
-    const size_t o_bm2 = take(sizeof(uint32_t) * (size_t)nw);
     KB_TRY(ensure_buffer(ctx, &ctx->batch_ws, &ctx->batch_ws_bytes, off));
     char* b = reinterpret_cast<char*>(ctx->batch_ws);
     int32_t* vgraph = reinterpret_cast<int32_t*>(b + o_vgraph);
     int64_t* voff = reinterpret_cast<int64_t*>(b + o_voff);
     int32_t* kd = reinterpret_cast<int32_t*>(b + o_k);
     uint8_t* gact = reinterpret_cast<uint8_t*>(b + o_act);
-    uint8_t* early = reinterpret_cast<uint8_t*>(b + o_early);
     int32_t* glast = reinterpret_cast<int32_t*>(b + o_last);
-    int32_t* sticky = reinterpret_cast<int32_t*>(b + o_sticky);
     uint32_t* bases = reinterpret_cast<uint32_t*>(b + o_bases);
-    uint32_t* bm_a = p.bitmap;
-    uint32_t* bm_b = R.bm[1] ? R.bm[1] : reinterpret_cast<uint32_t*>(b + o_bm2);
-    std::vector<uint8_t> act_h((size_t)G), early_h((size_t)G, (uint8_t)(opt->early_stop ? 1 : 0));
-    for (int64_t j = 0; j < G; ++j) act_h[(size_t)j] = k_h[j] > 0 ? 1 : 0;
-    KB_CUDA(ctx, cudaMemcpyAsync(voff, voff_h, sizeof(int64_t) * (size_t)(G + 1), cudaMemcpyHostToDevice, s));
-    KB_CUDA(ctx, cudaMemcpyAsync(kd, k_h, sizeof(int32_t) * (size_t)G, cudaMemcpyHostToDevice, s));
-    KB_CUDA(ctx, cudaMemcpyAsync(gact, act_h.data(), (size_t)G, cudaMemcpyHostToDevice, s));
-    KB_CUDA(ctx, cudaMemcpyAsync(early, early_h.data(), (size_t)G, cudaMemcpyHostToDevice, s));
-    KB_CUDA(ctx, cudaMemsetAsync(glast, 0, sizeof(int32_t) * (size_t)G, s));
-    KB_CUDA(ctx, cudaMemsetAsync(sticky, 0, sizeof(int32_t), s));
+    std::vector<char> up(up_bytes, 0);
+    std::memcpy(up.data(), voff_h, sizeof(int64_t) * (size_t)(G + 1));
+    std::memcpy(up.data() + (o_k - o_voff), k_h, sizeof(int32_t) * (size_t)G);
+    for (int64_t j = 0; j < G; ++j) up[o_act - o_voff + (size_t)j] = k_h[j] > 0 ? 1 : 0;
+    KB_CUDA(ctx, cudaMemcpyAsync(voff, up.data(), up_bytes, cudaMemcpyHostToDevice, s));  // staged before it returns
     kb::launch_vertex_graph(voff, (int32_t)G, n, vgraph, s);
-    p.vgraph = vgraph;
     p.voff = voff;
     p.n_graphs = (int32_t)G;
+    p.lgraph = vgraph;
+    R.gactive = gact;
 
     // level 0 for every graph: key (graph, label) or (graph) without labels
-    p.gactive = nullptr;
+    p.vgraph = vgraph;
     p.gbase_cur = bases;
     KB_TRY(launch_level0(ctx, R, opt->use_vertex_labels ? g->vertex_labels : nullptr, levels, s));
+
+    // rounds 1..kmax
+    p.vgraph = nullptr;  // block names tell the graphs apart
+    R.counters_clear = true;
+    cudaEvent_t e0 = ctx->ev[20], e1 = ctx->ev[21];
+    KB_CUDA(ctx, cudaEventRecord(e0, s));
+    int last = 0;  // last round queued
+    for (int i = 1; i <= kmax; ++i) {
+        KB_TRY(next_epoch(ctx, R, s));
+        KB_TRY(next_empty_round(ctx, R, s));
+        p.prev = reinterpret_cast<const int32_t*>(p.minof);
+        p.gbase_prev = bases + (size_t)(i - 1) * (size_t)(G + 1);
+        p.gbase_cur = bases + (size_t)i * (size_t)(G + 1);
+        // frozen blocks as in a single-graph call (blocks never span graphs); the
+        // mid, medium and hub kernels always launch (nothing is known of the
+        // round before yet)
+        p.frozen = R.frozen;
+        p.frozen_min = R.frozen_min;
+        p.moved = R.moved;
+        // from round 2 on, windows packed from the vertices that refine
+        // (frozen blocks and stopped graphs take no lane)
+        R.compact = i >= 2;
+        KB_TRY(launch_round_body(ctx, R, s, nullptr));
+        kb::GraphStop stop;
+        stop.active = gact;
+        stop.round = i;
+        stop.k = kd;
+        stop.early = opt->early_stop != 0;
+        stop.last = glast;
+        kb::launch_renumber(p, R.prefix, R.scan_tmp, levels + (size_t)i * (size_t)n, R.mark, false, s, stop);
+        if (i < kmax) {
+            kb::launch_dirty_blocks(p, R.edgeless, R.moved, kb::kMaxHubThreshold, R.mark, gact, false, s);
+            kb::launch_freeze_clean(freeze_pass(ctx, R), s);
+            R.bitmap_ready = true;
+        }
+        KB_CUDA(ctx, cudaGetLastError());
+        KB_TRY(queue_counters(ctx, i));
+        last = i;
+        if (i >= 2) {
+            KB_TRY(wait_counters(ctx, i - 1));
+            if (ctx->h_ctr->graphs_on == 0) break;  // this round repeated the last levels
+        }
+    }
+    KB_CUDA(ctx, cudaEventRecord(e1, s));
+    // the remaining rows repeat the last one
+    kb::launch_copy_rows(levels, n, last, last + 1, kmax, s);
+
+    // results: per-graph counts, last refined level
+    std::vector<uint32_t> bases_h((size_t)(G + 1) * (size_t)(last + 1));
+    KB_CUDA(ctx, cudaMemcpyAsync(bases_h.data(), bases, sizeof(uint32_t) * bases_h.size(), cudaMemcpyDeviceToHost, s));
+    if (lc_out) KB_CUDA(ctx, cudaMemcpyAsync(lc_out, glast, sizeof(int32_t) * (size_t)G, cudaMemcpyDeviceToHost, s));
     KB_TRY(read_counters(ctx));
     KB_TRY(device_error(ctx));
-
-    // rounds 1..kmax, captured once
-    p.gactive = gact;
-    R.counters_clear = true;
     if (kmax > 0) {
-        if (!ctx->cap_stream) KB_CUDA(ctx, cudaStreamCreateWithFlags(&ctx->cap_stream, cudaStreamNonBlocking));
-        cudaStream_t cs = ctx->cap_stream;
-        KB_CUDA(ctx, cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal));
-        kb_status st = KB_OK;
-        for (int i = 1; i <= kmax && st == KB_OK; ++i) {
-            st = next_epoch(ctx, R, cs);
-            if (st == KB_OK) st = next_empty_round(ctx, R, cs);
-            if (st != KB_OK) break;
-            p.prev = levels + (size_t)(i - 1) * (size_t)n;
-            p.bitmap = (i & 1) ? bm_b : bm_a;
-            p.bitmap_prev = (i & 1) ? bm_a : bm_b;
-            p.gbase_prev = bases + (size_t)(i - 1) * (size_t)(G + 1);
-            p.gbase_cur = bases + (size_t)i * (size_t)(G + 1);
-            // frozen blocks as in a single-graph call (blocks never span
-            // graphs); the medium and hub kernels always launch (no host
-            // reads inside the captured rounds)
-            p.frozen = R.frozen;
-            p.frozen_min = R.frozen_min;
-            p.moved = R.moved;
-            // from round 2 on, windows packed from the vertices that refine
-            // (frozen blocks and stopped graphs take no lane)
-            R.compact = i >= 2;
-            int32_t* out = levels + (size_t)i * (size_t)n;
-            st = launch_round_body(ctx, R, cs, nullptr);
-            if (st != KB_OK) break;
-            kb::launch_carry_minima(p, cs);
-            kb::launch_renumber(p, R.prefix, R.scan_tmp, out, R.mark, false, cs);
-            if (p.shared && i < kmax) {
-                kb::launch_dirty_blocks(p, R.edgeless, R.moved, out, kb::kMaxHubThreshold, R.mark, false, cs);
-                kb::FreezePass f = freeze_pass(ctx, R, out);
-                f.frozen_min = (i & 1) ? bm_a : bm_b;
-                kb::launch_freeze_clean(f, cs);
-                R.bitmap_ready = true;
-            }
-            kb::launch_graph_stop(p, i, kd, early, gact, glast, sticky, cs);
-        }
-        cudaGraph_t graph = nullptr;
-        const cudaError_t ce = cudaStreamEndCapture(cs, &graph);
-        if (st != KB_OK) {
-            if (graph) cudaGraphDestroy(graph);
-            return st;
-        }
-        if (ce != cudaSuccess) return fail(ctx, KB_ERR_CUDA, "graph capture failed: %s", cudaGetErrorString(ce));
-        cudaGraphExec_t exec = nullptr;
-        const cudaError_t ie = cudaGraphInstantiate(&exec, graph, 0);
-        cudaGraphDestroy(graph);
-        if (ie != cudaSuccess) return fail(ctx, KB_ERR_CUDA, "graph instantiation failed: %s", cudaGetErrorString(ie));
-        cudaEvent_t e0 = ctx->ev[20], e1 = ctx->ev[21];
-        cudaEventRecord(e0, s);
-        const cudaError_t le = cudaGraphLaunch(exec, s);
-        cudaEventRecord(e1, s);
-        if (le != cudaSuccess) {
-            cudaGraphExecDestroy(exec);
-            return fail(ctx, KB_ERR_CUDA, "graph launch failed: %s", cudaGetErrorString(le));
-        }
-        const cudaError_t se = cudaStreamSynchronize(s);
-        cudaGraphExecDestroy(exec);
-        if (se != cudaSuccess) return fail(ctx, KB_ERR_CUDA, "batched rounds failed: %s", cudaGetErrorString(se));
         float ms = 0.f;
         cudaEventElapsedTime(&ms, e0, e1);
         ctx->round_ms.push_back(ms);
     }
-    p.bitmap = bm_a;
-
-    // results: graph-local ids, per-graph counts, last refined level
-    std::vector<uint32_t> bases_h((size_t)(G + 1) * (size_t)(kmax + 1));
-    int32_t sticky_h = 0;
-    KB_CUDA(ctx, cudaMemcpyAsync(bases_h.data(), bases, sizeof(uint32_t) * bases_h.size(), cudaMemcpyDeviceToHost, s));
-    KB_CUDA(ctx, cudaMemcpyAsync(&sticky_h, sticky, sizeof(int32_t), cudaMemcpyDeviceToHost, s));
-    if (lc_out) KB_CUDA(ctx, cudaMemcpyAsync(lc_out, glast, sizeof(int32_t) * (size_t)G, cudaMemcpyDeviceToHost, s));
-    for (int i = 0; i <= kmax; ++i)
-        kb::launch_localize(levels + (size_t)i * (size_t)n, n, vgraph, bases + (size_t)i * (size_t)(G + 1), s);
-    KB_CUDA(ctx, cudaGetLastError());
-    KB_CUDA(ctx, cudaStreamSynchronize(s));
-    if (sticky_h & kb::kErrTableFull) return fail(ctx, KB_ERR_TABLE_FULL, "block table probe limit reached");
-    if (sticky_h) return fail(ctx, KB_ERR_DEVICE_CHECK, "device consistency check failed (%d)", sticky_h);
     for (int64_t j = 0; j < G; ++j)
         for (int i = 0; i <= kmax; ++i) {
-            const uint32_t* bi = bases_h.data() + (size_t)i * (size_t)(G + 1);
+            const uint32_t* bi = bases_h.data() + (size_t)std::min(i, last) * (size_t)(G + 1);
             counts[j * (kmax + 1) + i] = (int64_t)(bi[j + 1] - bi[j]);
         }
     return KB_OK;
@@ -1684,7 +1660,7 @@ struct Arena {
     int32_t* col = nullptr;   // [Mcap]
     int32_t* lab = nullptr;   // [Mcap]
     int32_t* vlab = nullptr;  // [Ncap]
-    int32_t* B[2] = {nullptr, nullptr};  // [Ncap] current / next level, union-global ids
+    uint32_t* name = nullptr;  // [Ncap] smallest member of every vertex's block (RoundParams::minof)
 };
 
 struct ServeRequest {
@@ -1728,7 +1704,6 @@ struct kb_server {
     std::mutex mu;  // guards queue, requests, stats (submit vs step)
     Arena arena[2];
     int cur = 0;  // active arena buffer
-    int bsel = 0;  // which B buffer of the arena holds the current level
     int64_t n_used = 0, m_used = 0;
     std::vector<Slot> slots;
     std::deque<int64_t> waiting;
@@ -1742,29 +1717,25 @@ struct kb_server {
     uint64_t table_cap = 0;
     uint64_t* emin = nullptr;
     // Frozen-block state of the arena, sized for a full arena and kept across
-    // re-plans: frozen vertices, minima of frozen blocks, shared marks,
-    // smallest members, moved vertices, dirty blocks, and the two bitmaps of
-    // block minima used in turn.
+    // re-plans: frozen vertices, minima of frozen blocks, shared marks, moved
+    // vertices, dirty blocks (and Arena::name).
     uint32_t* frz[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};
-    uint32_t* minof = nullptr;
-    uint32_t* bitmap1 = nullptr;
     int64_t planned_n = 0;        // arena vertices at the last re-plan
     bool vertices_moved = false;  // a compaction since the last re-plan
-    // The last step's minima and smallest members are valid for this step's
-    // moved vertices (false after a compaction, which moves vertices and
-    // clears the frozen blocks)
+    // Block names are those of the last step, against which this step's moved
+    // vertices are told (false after a compaction, which renames blocks and
+    // clears the frozen ones)
     bool history = false;
     // per-slot device arrays (capacity max_requests + dead slots: sized by max_slots)
     int32_t max_slots = 0;
     int32_t* vgraph = nullptr;
     int64_t* voff = nullptr;
-    uint8_t* gactive = nullptr;
-    uint8_t* gmode = nullptr;
-    uint32_t* bases[2] = {nullptr, nullptr};
-    uint32_t* bitmap2 = nullptr;
-    int32_t** slot_levels = nullptr;
-    int32_t* slot_row = nullptr;
-    int64_t* slot_n = nullptr;
+    uint32_t* bases = nullptr;
+    // what the host says about every slot at a step, in one copy: where its level
+    // goes, its count before, then a byte each for active, level 0 and the stop
+    // mode (kb::GraphStop)
+    char* slot_up = nullptr;
+    std::vector<char> slot_up_h;
     std::vector<uint32_t> gbase_host;
     // staging for admission (raw graph, processed CSR for IN / BOTH)
     void* stage = nullptr;
@@ -1773,8 +1744,6 @@ struct kb_server {
     Prepared R;
     bool dirty = true;
 
-    int bmsel = 0;
-    uint32_t* bm_ws = nullptr;
     // stats
     double t_first = -1;
     int64_t submitted = 0, completed = 0, failed = 0, steps = 0, compactions = 0;
@@ -1916,20 +1885,18 @@ kb_status compact(kb_server* sv) {
         a.scol = S.col;
         a.slab = S.lab;
         a.svlab = S.vlab;
-        a.sB = S.B[sv->bsel];
+        a.sname = S.name;
         a.drow = D.row;
         a.dcol = D.col;
         a.dlab = D.lab;
         a.dvlab = D.vlab;
-        a.dB = D.B[0];
+        a.dname = D.name;
         a.n = o.n;
         a.m = o.m;
         a.src_vbase = o.vbase;
         a.src_ebase = o.ebase;
         a.dst_vbase = nv;
         a.dst_ebase = ne;
-        a.b_sub = sv->gbase_host.size() > j ? sv->gbase_host[j] : 0u;
-        a.b_add = (uint32_t)nv;
         kb::launch_place(a, s);
         Slot ns = o;
         ns.vbase = nv;
@@ -1944,8 +1911,6 @@ kb_status compact(kb_server* sv) {
     sv->n_used = nv;
     sv->m_used = ne;
     sv->cur = 1 - sv->cur;
-    sv->bsel = 0;
-    sv->gbase_host.clear();
     sv->dirty = true;
     sv->vertices_moved = true;
     ++sv->compactions;
@@ -2113,7 +2078,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
             sv->R.ext_shared = sv->frz[2];
             sv->R.ext_moved = sv->frz[3];
             sv->R.ext_mark = sv->frz[4];
-            sv->R.ext_minof = sv->minof;
+            sv->R.ext_minof = A.name;
             const size_t bw = sizeof(uint32_t) * (size_t)((sv->n_used >> 5) + 1);
             if (sv->vertices_moved) {
                 // compacted: vertex ids moved, nothing carries over
@@ -2128,7 +2093,6 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
                 for (int f = 0; f < 3; ++f) kb::launch_clear_bits(sv->frz[f], sv->planned_n, word_end, s);
             }
             SV_TRY(sv, prepare(ctx, &view, &o, sv->R, -1, true));
-            sv->bm_ws = sv->bitmap1;
             sv->planned_n = sv->n_used;
             std::vector<int64_t> voff((size_t)G + 1);
             for (int j = 0; j < G; ++j) voff[(size_t)j] = sv->slots[(size_t)j].vbase;
@@ -2137,59 +2101,56 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
             kb::launch_vertex_graph(sv->voff, G, sv->n_used, sv->vgraph, s);
             sv->dirty = false;
         }
-        // per-slot flags for this step
-        std::vector<uint8_t> act((size_t)G), mode((size_t)G);
-        std::vector<int32_t*> lev((size_t)G, nullptr);
-        std::vector<int32_t> row((size_t)G, -1);
-        std::vector<int64_t> sn((size_t)G, 0);
+        // per-slot words for this step
+        const size_t o_cnt = sizeof(int32_t*) * (size_t)G, o_act = o_cnt + sizeof(int64_t) * (size_t)G,
+                     o_mode = o_act + (size_t)G, o_stop = o_mode + (size_t)G;
+        std::vector<char>& up = sv->slot_up_h;
+        up.assign(o_stop + (size_t)G, 0);
+        int32_t** lev = reinterpret_cast<int32_t**>(up.data());
+        int64_t* before = reinterpret_cast<int64_t*>(up.data() + o_cnt);
         for (int j = 0; j < G; ++j) {
             const Slot& sl = sv->slots[(size_t)j];
-            sn[(size_t)j] = sl.n;
             if (sl.ticket < 0) continue;
             ServeRequest& r = sv->reqs[sl.ticket];
-            act[(size_t)j] = 1;
-            mode[(size_t)j] = r.round == 0 ? 1 : 0;
-            lev[(size_t)j] = r.d_levels;
-            row[(size_t)j] = r.round;
+            lev[j] = r.d_levels + (size_t)r.round * (size_t)r.n;
+            before[j] = r.round > 0 ? r.counts[(size_t)r.round - 1] : 0;
+            up[o_act + (size_t)j] = 1;
+            up[o_mode + (size_t)j] = r.round == 0 ? 1 : 0;
+            up[o_stop + (size_t)j] = r.round >= r.k ? 1 : (r.round > 0 && r.opt.early_stop ? 2 : 0);
         }
-        SV_CUDA(sv, cudaMemcpyAsync(sv->gactive, act.data(), (size_t)G, cudaMemcpyHostToDevice, s));
-        SV_CUDA(sv, cudaMemcpyAsync(sv->gmode, mode.data(), (size_t)G, cudaMemcpyHostToDevice, s));
-        SV_CUDA(sv, cudaMemcpyAsync(sv->slot_levels, lev.data(), sizeof(int32_t*) * (size_t)G, cudaMemcpyHostToDevice, s));
-        SV_CUDA(sv, cudaMemcpyAsync(sv->slot_row, row.data(), sizeof(int32_t) * (size_t)G, cudaMemcpyHostToDevice, s));
-        SV_CUDA(sv, cudaMemcpyAsync(sv->slot_n, sn.data(), sizeof(int64_t) * (size_t)G, cudaMemcpyHostToDevice, s));
+        SV_CUDA(sv, cudaMemcpyAsync(sv->slot_up, up.data(), up.size(), cudaMemcpyHostToDevice, s));
+        uint8_t* gactive = reinterpret_cast<uint8_t*>(sv->slot_up + o_act);
+        const uint8_t* gmode = reinterpret_cast<const uint8_t*>(sv->slot_up + o_mode);
         // one round for everything in flight
         SV_TRY(sv, next_epoch(ctx, sv->R, s));
         SV_TRY(sv, next_empty_round(ctx, sv->R, s));
         p.vgraph = sv->vgraph;
+        p.lgraph = sv->vgraph;
         p.voff = sv->voff;
         p.n_graphs = G;
-        p.gactive = sv->gactive;
-        p.gmode = sv->gmode;
+        p.gmode = gmode;
+        p.gout = reinterpret_cast<int32_t* const*>(sv->slot_up);
         p.vlab = A.vlab;
-        p.prev = A.B[sv->bsel];
-        // block-minima bitmaps alternate between the prepared one and the server's own
-        p.bitmap = sv->bmsel ? sv->bitmap2 : sv->bm_ws;
-        p.bitmap_prev = sv->bmsel ? sv->bm_ws : sv->bitmap2;
-        p.gbase_prev = sv->bases[1 - (sv->steps & 1)];
-        p.gbase_cur = sv->bases[sv->steps & 1];
-        int32_t* out = A.B[1 - sv->bsel];
+        p.prev = reinterpret_cast<const int32_t*>(A.name);
+        p.gbase_cur = sv->bases;
+        sv->R.gactive = gactive;
         // frozen blocks, as in a single-graph call (blocks never span graphs)
         p.frozen = sv->R.frozen;
         p.frozen_min = sv->R.frozen_min;
         p.moved = sv->history ? sv->R.moved : nullptr;
+        sv->R.compact = sv->history;  // retired graphs' vertices are frozen
         SV_TRY(sv, launch_round_body(ctx, sv->R, s, nullptr));
-        kb::launch_carry_minima(p, s);
-        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, out, p.moved ? sv->R.mark : nullptr, false, s);
-        kb::launch_emit(sv->n_used, sv->vgraph, out, p.gbase_cur, sv->slot_levels, sv->slot_row, sv->slot_n, sv->voff, s);
-        if (p.shared) {
-            if (p.moved)
-                kb::launch_dirty_blocks(p, sv->R.edgeless, sv->R.moved, out, kb::kMaxHubThreshold, sv->R.mark, false, s);
-            kb::FreezePass f = freeze_pass(ctx, sv->R, out);
-            f.mark = p.moved ? sv->R.mark : nullptr;
-            f.vgraph = sv->vgraph;
-            f.gmode = sv->gmode;
-            kb::launch_freeze_clean(f, s);
-        }
+        kb::GraphStop stop;
+        stop.active = gactive;
+        stop.mode = reinterpret_cast<const uint8_t*>(sv->slot_up + o_stop);
+        stop.prev_count = reinterpret_cast<const int64_t*>(sv->slot_up + o_cnt);
+        kb::launch_renumber(p, sv->R.prefix, sv->R.scan_tmp, nullptr, p.moved ? sv->R.mark : nullptr, false, s, stop);
+        if (p.moved)
+            kb::launch_dirty_blocks(p, sv->R.edgeless, sv->R.moved, kb::kMaxHubThreshold, sv->R.mark, gactive, false, s);
+        kb::FreezePass f = freeze_pass(ctx, sv->R);
+        f.mark = p.moved ? sv->R.mark : nullptr;
+        f.gmode = gmode;
+        kb::launch_freeze_clean(f, s);
         sv->history = true;
         SV_CUDA(sv, cudaGetLastError());
         sv->gbase_host.assign((size_t)G + 1, 0);
@@ -2200,8 +2161,6 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         if (ctx->h_ctr->err) {
             SV_TRY(sv, device_error(ctx));
         }
-        sv->bsel = 1 - sv->bsel;
-        sv->bmsel = 1 - sv->bmsel;
         // bookkeeping and retirement (one synchronisation for all copies)
         std::vector<std::pair<ServeRequest*, int>> finished;
         for (int j = 0; j < G; ++j) {
@@ -2287,12 +2246,13 @@ kb_status kb_create(kb_context** out, int device, void* stream) {
     if (cudaSetDevice(device) != cudaSuccess || cudaMalloc(&ctx->d_ctr, sizeof(Counters)) != cudaSuccess ||
         cudaMalloc(&ctx->d_dense, (sizeof(uint32_t) + sizeof(uint2)) * kb::kDenseLabels) != cudaSuccess ||
         cudaMallocHost(&ctx->h_hubs, (sizeof(int32_t) + sizeof(int64_t)) * kEagerHubs) != cudaSuccess ||
-        cudaMallocHost(&ctx->h_ctr, sizeof(Counters)) != cudaSuccess) {
+        cudaMallocHost(&ctx->h_ctr, sizeof(Counters) * (1 + kCounterSlots)) != cudaSuccess) {
         cudaGetLastError();
         kb_destroy(ctx);
         return KB_ERR_CUDA;
     }
     for (auto& e : ctx->ev) cudaEventCreate(&e);
+    for (auto& e : ctx->slot_ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     kb::set_medium_kernel_attributes();
     cudaGetLastError();
     *out = ctx;
@@ -2319,11 +2279,12 @@ kb_status kb_destroy(kb_context* ctx) {
     cudaFree(ctx->sum_buf);
     cudaFree(ctx->upd_buf);
     cudaFree(ctx->d_work);
-    if (ctx->cap_stream) cudaStreamDestroy(ctx->cap_stream);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->row_ev) cudaEventDestroy(ctx->row_ev);
 
     for (auto& e : ctx->ev)
+        if (e) cudaEventDestroy(e);
+    for (auto& e : ctx->slot_ev)
         if (e) cudaEventDestroy(e);
     delete ctx;
     return KB_OK;
@@ -2734,19 +2695,12 @@ kb_status kb_server_create(kb_server** out, int device, void* stream, const kb_s
         alloc((void**)&A.col, sizeof(int32_t) * (size_t)M);
         alloc((void**)&A.lab, sizeof(int32_t) * (size_t)M);
         alloc((void**)&A.vlab, sizeof(int32_t) * (size_t)N);
-        alloc((void**)&A.B[0], sizeof(int32_t) * (size_t)N);
-        alloc((void**)&A.B[1], sizeof(int32_t) * (size_t)N);
+        alloc((void**)&A.name, sizeof(uint32_t) * (size_t)N);
     }
     alloc((void**)&sv->vgraph, sizeof(int32_t) * (size_t)N);
     alloc((void**)&sv->voff, sizeof(int64_t) * (size_t)(S + 1));
-    alloc((void**)&sv->gactive, (size_t)S);
-    alloc((void**)&sv->gmode, (size_t)S);
-    alloc((void**)&sv->bases[0], sizeof(uint32_t) * (size_t)(S + 1));
-    alloc((void**)&sv->bases[1], sizeof(uint32_t) * (size_t)(S + 1));
-    alloc((void**)&sv->bitmap2, sizeof(uint32_t) * (size_t)((N >> 5) + 1));
-    alloc((void**)&sv->slot_levels, sizeof(int32_t*) * (size_t)S);
-    alloc((void**)&sv->slot_row, sizeof(int32_t) * (size_t)S);
-    alloc((void**)&sv->slot_n, sizeof(int64_t) * (size_t)S);
+    alloc((void**)&sv->bases, sizeof(uint32_t) * (size_t)(S + 1));
+    alloc((void**)&sv->slot_up, (sizeof(int32_t*) + sizeof(int64_t) + 3) * (size_t)S);
     // the arena's block table and empty-signature minima, sized for a full arena
     const float lf = cfg->load_factor > 0.f ? cfg->load_factor : 0.5f;
     sv->table_cap = table_capacity(N, lf);
@@ -2754,16 +2708,13 @@ kb_status kb_server_create(kb_server** out, int device, void* stream, const kb_s
     alloc((void**)&sv->emin, sizeof(uint64_t) * (size_t)N);
     const size_t bwN = sizeof(uint32_t) * (size_t)((N >> 5) + 1);
     for (int f = 0; f < 5; ++f) alloc((void**)&sv->frz[f], bwN);
-    alloc((void**)&sv->minof, sizeof(uint32_t) * (size_t)N);
-    alloc((void**)&sv->bitmap1, bwN);
     if (ok) {
         ok = cudaMemset(sv->arena[0].row, 0, sizeof(int64_t)) == cudaSuccess &&
              cudaMemset(sv->arena[1].row, 0, sizeof(int64_t)) == cudaSuccess &&
-             cudaMemset(sv->bitmap2, 0, sizeof(uint32_t) * (size_t)((N >> 5) + 1)) == cudaSuccess &&
              cudaMemset(sv->table, 0, sizeof(uint64_t) * (size_t)sv->table_cap) == cudaSuccess &&
              cudaMemset(sv->emin, 0xff, sizeof(uint64_t) * (size_t)N) == cudaSuccess &&
              cudaMemset(sv->frz[0], 0, bwN) == cudaSuccess && cudaMemset(sv->frz[1], 0, bwN) == cudaSuccess &&
-             cudaMemset(sv->frz[2], 0, bwN) == cudaSuccess && cudaMemset(sv->bitmap1, 0, bwN) == cudaSuccess;
+             cudaMemset(sv->frz[2], 0, bwN) == cudaSuccess;
     }
     if (!ok) {
         kb_server_destroy(sv);
@@ -2786,27 +2737,18 @@ kb_status kb_server_destroy(kb_server* sv) {
     cudaFree(sv->table);
     cudaFree(sv->emin);
     for (int f = 0; f < 5; ++f) cudaFree(sv->frz[f]);
-    cudaFree(sv->minof);
-    cudaFree(sv->bitmap1);
     for (int a = 0; a < 2; ++a) {
         Arena& A = sv->arena[a];
         cudaFree(A.row);
         cudaFree(A.col);
         cudaFree(A.lab);
         cudaFree(A.vlab);
-        cudaFree(A.B[0]);
-        cudaFree(A.B[1]);
+        cudaFree(A.name);
     }
     cudaFree(sv->vgraph);
     cudaFree(sv->voff);
-    cudaFree(sv->gactive);
-    cudaFree(sv->gmode);
-    cudaFree(sv->bases[0]);
-    cudaFree(sv->bases[1]);
-    cudaFree(sv->bitmap2);
-    cudaFree(sv->slot_levels);
-    cudaFree(sv->slot_row);
-    cudaFree(sv->slot_n);
+    cudaFree(sv->bases);
+    cudaFree(sv->slot_up);
     cudaFree(sv->stage);
     kb_destroy(sv->ctx);
     delete sv;

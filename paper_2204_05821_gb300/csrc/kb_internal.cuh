@@ -43,6 +43,7 @@ struct Counters {
     int64_t frozen; // vertices frozen for the next round (launch_freeze_clean)
     int64_t class_on[3]; // mid and medium vertices and hubs that refine next round (launch_freeze_clean)
     int64_t moved;  // re-keyed vertices whose smallest block member changed (renumbering)
+    int64_t graphs_on;  // graphs of a batch that refine next round (launch_graph_bases)
     // vertices re-keyed this round and their edges in the processed
     // direction, per kernel family: small, medium, hub
     int64_t keyed_v[3];
@@ -98,12 +99,12 @@ struct RoundParams {
     uint32_t* shared;
     uint32_t* joined;
     // Clean blocks (with frozen blocks).  minof[v] is the smallest member of
-    // v's block whenever v is not that member; the renumbering writes it for
-    // every re-keyed vertex, and a frozen vertex keeps it.  moved (when set)
-    // receives bit v for every re-keyed vertex whose smallest block member
-    // changed this round (read against bitmap_prev, the previous level's block
-    // minima, and minof), counted in ctr->moved; under the locality order the
-    // bit goes to v's position, which is what the neighbour ids hold.
+    // v's block at the level last assigned: the name its block goes by in the
+    // next round's keys (prev and gather), unique over all graphs of a run.  The
+    // renumbering writes it for re-keyed vertices whose block's smallest member
+    // changed; a frozen vertex keeps it.  moved (when set) receives bit v for
+    // every such vertex, counted in ctr->moved; under the locality order the bit
+    // goes to v's position, which is what the neighbour ids hold.
     uint32_t* minof;
     uint32_t* moved;
     int32_t hub_threshold;
@@ -138,19 +139,25 @@ struct RoundParams {
     uint64_t* hub_sets;
     uint64_t* hub_acc;  // [n_hubs] sum of pair mixes over unique pairs
     uint32_t* hub_cnt;  // [n_hubs] unique pairs
-    // several graphs at once (batched refinement, serving); all null for one graph
-    const int32_t* vgraph;     // [n] graph of every vertex
-    const uint8_t* gactive;    // [G] the graph refines this round (else it keeps its partition)
-    const int64_t* voff;       // [G+1] first vertex of every graph
+    // several graphs at once (batched refinement, serving); all null or 0 for one graph
     int32_t n_graphs;
+    const int64_t* voff;       // [G+1] first vertex of every graph
+    // vgraph: graph of every vertex, while keys need it: at a batch's level 0 and
+    // in serving, where graphs may compute their level 0 among others' rounds.
+    // (The names of blocks are unique over all graphs, so signature keys of
+    // different graphs differ by themselves.)
+    const int32_t* vgraph;
     const uint8_t* gmode;      // [G] 1: the graph computes its level 0 this round (serving), or nullptr
     const int32_t* vlab;       // [n] vertex labels read by graphs in level-0 mode, or nullptr (all 0)
-    const uint32_t* bitmap_prev;  // block minima of the previous level (batched: kept by inactive graphs)
+    // Where the levels go: ids local to the graph (lgraph: graph of every vertex),
+    // into one row, or (gout) to every graph's own row, nullptr for none.
+    const int32_t* lgraph;
+    int32_t* const* gout;
     const uint32_t* gbase_prev;   // [G+1] rank of every graph's first vertex at the previous level
     uint32_t* gbase_cur;          // [G+1] the same at this level (written by the renumbering)
 };
 
-__host__ __device__ __forceinline__ bool batched(const RoundParams& p) { return p.vgraph != nullptr; }
+__host__ __device__ __forceinline__ bool batched(const RoundParams& p) { return p.n_graphs > 0; }
 
 // The subject part of vertex v's key in a signature round.
 __host__ __device__ __forceinline__ int32_t own_of(const RoundParams& p, int64_t v) {
@@ -222,16 +229,18 @@ __device__ __forceinline__ uint32_t table_hi(uint64_t h, uint32_t epoch) {
 void launch_clear_round(const RoundParams& p, cudaStream_t s);
 // Empty the sets of the hubs that refine this round; clear the hubs' sums.
 void launch_clear_hubs(const RoundParams& p, int64_t total_slots, cudaStream_t s);
-// Clean blocks (RoundParams::minof).  After the renumbering of level i
-// (`level`, whose minima are in p.bitmap, moved vertices in `moved`): mark =
+// Clean blocks (RoundParams::minof).  After the renumbering of level i (minima
+// in p.bitmap, names in p.minof, moved vertices in `moved`): mark =
 // blocks of level i holding a vertex with an edge to a moved vertex (bit =
-// level-i id; a vertex above max_scan edges counts as such).  Only vertices
+// the block's name; a vertex above max_scan edges counts as such).  Only vertices
 // that are neither alone in their block (bitmap & ~shared) nor edgeless are
 // scanned, and nothing when more than an eighth of the vertices moved.
-// stop_stable: the pass does nothing after a round that kept the block count (a
+// gactive (or nullptr): graphs that stopped are not scanned.  stop_stable: the
+// pass does nothing after a round that kept the block count (a
 // stable round under early stop is the last one).
-void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,
-                         int32_t max_scan, uint32_t* mark, bool stop_stable, cudaStream_t s);
+void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved,
+                         int32_t max_scan, uint32_t* mark, const uint8_t* gactive, bool stop_stable,
+                         cudaStream_t s);
 // After the renumbering (stratified rounds): the frozen blocks of the next
 // round.  A vertex is frozen when it is alone in its block (a minimum in bitmap
 // without a mark in shared), edgeless (edgeless != null: from the first
@@ -243,7 +252,7 @@ struct FreezePass {
     const uint32_t* bitmap = nullptr;    // block minima of the level
     uint32_t* shared = nullptr;          // in: minima of blocks of several vertices; out: exactly the frozen ones
     const uint32_t* edgeless = nullptr;
-    const int32_t* level = nullptr;
+    const uint32_t* names = nullptr;     // RoundParams::minof
     const uint32_t* mark = nullptr;
     uint32_t* frozen = nullptr;          // out: frozen vertices, counted in ctr->frozen
     uint32_t* frozen_min = nullptr;      // out: the minima of frozen blocks
@@ -251,9 +260,11 @@ struct FreezePass {
     const uint32_t* classes[3] = {};     // mid, medium, hub: those not frozen are counted in ctr->class_on
                                          // (nullptr: an empty class)
     Counters* ctr = nullptr;
-    // serving: the vertices of graphs that computed their level 0 in this step
-    // (gmode) are not frozen by the edgeless rule
+    // several graphs: all vertices of a graph that stopped (not in gactive) are
+    // frozen, those of a graph that computed its level 0 in this step (gmode) are
+    // not by the edgeless rule
     const int32_t* vgraph = nullptr;
+    const uint8_t* gactive = nullptr;
     const uint8_t* gmode = nullptr;
     bool stop_stable = false;            // a round that kept the count is the last one: nothing to do after it
     int per_warp = 32;                   // bitmap words per warp (set by the launcher)
@@ -275,6 +286,20 @@ void launch_medium_round(const RoundParams& p, cudaStream_t s);  //   after the 
 void set_medium_kernel_attributes();
 void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s);
 void launch_hub_final(const RoundParams& p, cudaStream_t s);
+// Several graphs, after the rank scan: gbase_cur, and the stop test of every
+// graph still in `active` (cleared when it stops; ctr->graphs_on counts the
+// others).  `round`: the level just computed.
+struct GraphStop {
+    uint8_t* active = nullptr;        // [G]; nullptr: no test
+    int round = 0;
+    // a batch: stop at the graph's own k, or (early) at an unchanged count
+    const int32_t* k = nullptr;       // [G]
+    bool early = false;
+    int32_t* last = nullptr;          // [G] receives the round
+    // serving: mode 1 stops after this round, 2 when the count is prev_count's
+    const uint8_t* mode = nullptr;    // [G]
+    const int64_t* prev_count = nullptr;
+};
 // Canonical renumbering: prefix of block minima, then ids.
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
 // The frozen, class_on and moved counters restart at 0; with frozen
@@ -283,7 +308,7 @@ void launch_hub_final(const RoundParams& p, cudaStream_t s);
 // block count (the last round) the ids are those of the previous level, and out
 // is left for the caller to copy.
 void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
-                     bool stop_stable, cudaStream_t s);
+                     bool stop_stable, cudaStream_t s, const GraphStop& stop = GraphStop());
 size_t scan_tmp_words(int64_t n_items);
 // Level 0 of one graph whose keys (vertex labels, or a starting partition)
 // are all in [0, kDenseLabels): the label partition straight from each
@@ -299,14 +324,6 @@ void launch_dense_labels(int64_t n, const int32_t* key, uint32_t* lmin, Counters
 void launch_dense_level0(const RoundParams& p, const int32_t* key, const uint32_t* lmin, uint2* lpair, uint2* rank,
                          uint32_t* scan_tmp, int32_t* out, cudaStream_t s);
 void launch_fill_i32(int32_t* out, int64_t n, int32_t value, cudaStream_t s);
-// Batched runs: inactive graphs keep the block minima of the previous level.
-void launch_carry_minima(const RoundParams& p, cudaStream_t s);
-// Batched runs: per-graph stop test after round `round` (count unchanged with
-// early stop, or the graph's own k reached) -> gactive cleared, glast set.
-void launch_graph_stop(const RoundParams& p, int round, const int32_t* k_per_graph, const uint8_t* early,
-                       uint8_t* gactive, int32_t* glast, int32_t* sticky_err, cudaStream_t s);
-// Batched runs: row -= gbase[graph of v] (union-global ids to graph-local ids).
-void launch_localize(int32_t* row, int64_t n, const int32_t* vgraph, const uint32_t* gbase, cudaStream_t s);
 // vgraph[v] = graph owning v
 void launch_vertex_graph(const int64_t* voff, int32_t G, int64_t n, int32_t* vgraph, cudaStream_t s);
 
@@ -401,27 +418,20 @@ void launch_copy_rows(int32_t* levels, int64_t n, int src, int first, int last, 
 // Copy vertices [src_vbase, src_vbase+n] and edges [src_ebase, src_ebase+m)
 // of a CSR into an arena at dst_vbase / dst_ebase, rebasing row offsets and
 // neighbour ids (the in-edge bit of a neighbour id is kept).  Labels may be
-// null (written as 0).  When sB and dB are given, block ids move too, as
-// sB - b_sub + b_add.
+// null (written as 0).  When given, block names (RoundParams::minof) move too.
 struct PlaceArgs {
     const int64_t* srow;
     const int32_t* scol;
     const int32_t* slab;
     const int32_t* svlab;
-    const int32_t* sB;
+    const uint32_t* sname;
     int64_t* drow;
     int32_t* dcol;
     int32_t* dlab;
     int32_t* dvlab;
-    int32_t* dB;
+    uint32_t* dname;
     int64_t n, m;
     int64_t src_vbase, dst_vbase, src_ebase, dst_ebase;
-    uint32_t b_sub, b_add;
 };
 void launch_place(const PlaceArgs& a, cudaStream_t s);
-// For every arena vertex whose graph g has slot_row[g] >= 0:
-// slot_levels[g][slot_row[g] * slot_n[g] + (v - voff[g])] = B[v] - gbase[g].
-void launch_emit(int64_t n, const int32_t* vgraph, const int32_t* B, const uint32_t* gbase, int32_t* const* slot_levels,
-                 const int32_t* slot_row, const int64_t* slot_n, const int64_t* voff, cudaStream_t s);
-
 }  // namespace kb

@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kHubThreads) hub_chunk_kernel(const RoundParam
     const uint64_t ext = p.chunk_ext[c];
     const int64_t e0 = (int64_t)(ext >> 16);
     const int E = (int)(ext & 0xffffu);
-    if ((batched(p) || p.vmask || p.frozen) && !vertex_refines(p, p.hub_v[h])) return;  // uniform over the CTA
+    if ((p.gmode || p.vmask || p.frozen) && !vertex_refines(p, p.hub_v[h])) return;  // uniform over the CTA
     if (tid == 0) {
         s_nuniq = 0;
         s_nnew = 0;
@@ -402,6 +402,7 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
         ctr->frozen = 0;
         for (int k = 0; k < 3; ++k) ctr->class_on[k] = 0;
         ctr->moved = 0;
+        ctr->graphs_on = 0;
         if (rank_total) rank[nw] = make_uint2(all, 0u);
     }
 #pragma unroll
@@ -443,12 +444,6 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < p.n; v += stride) {
         uint32_t mn = (uint32_t)v;
         if (!vertex_active(p, v)) {
-            if (!p.vmask) {  // a batched graph that stopped: its ids shift with the graphs before it
-                // (batched runs never use the locality order)
-                const int32_t g = p.vgraph[v];
-                out[v] = (int32_t)((uint32_t)p.prev[v] - p.gbase_prev[g] + p.gbase_cur[g]);
-                continue;
-            }
             mn = p.kmin[p.keep_old[v]];  // incremental: the smallest kept member of its old block
             if ((int64_t)mn >= p.n) mn = (uint32_t)v;
         } else if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
@@ -463,14 +458,13 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
 }
 
 // Canonical ids of a stratified round with frozen blocks (RoundParams::minof;
-// one graph, or several at once): assign_kernel's work with every lane of a warp on one
-// bitmap word (a warp-uniform loop), so that the moved vertices (re-keyed
-// vertices whose smallest block member changed: v itself or minof[v] at the
-// previous level, read before minof[v] is rewritten) leave as one word per
-// warp.  Frozen vertices keep minof, and their blocks keep their shared marks
-// (the freeze pass carries them over); the mark of a re-keyed block comes from
-// the vertex that inserted its table entry (RoundParams::joined).  moved may be
-// null (the starting level); mark, when given, is cleared for the dirty pass.
+// one graph, or several at once): assign_kernel's work with every lane of a warp
+// on one bitmap word (a warp-uniform loop), so that the moved vertices (re-keyed
+// vertices whose smallest block member changed) leave as one word per warp.
+// Frozen vertices keep minof, and their blocks keep their shared marks (the
+// freeze pass carries them over); the mark of a re-keyed block comes from the
+// vertex that inserted its table entry (RoundParams::joined).  moved may be null
+// (the starting level); mark, when given, is cleared for the dirty pass.
 __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p, const uint2* rank, int32_t* out,
                                                              uint32_t* moved, uint32_t* mark, bool stop_stable) {
     // a round that kept the block count kept every block (blocks only split):
@@ -486,35 +480,37 @@ __global__ void __launch_bounds__(256) assign_frozen_kernel(const RoundParams p,
         const int64_t v = base + lane;
         bool mv = false;
         const uint32_t joined = p.joined[base >> 5];
-        if (v < p.n && !vertex_active(p, v)) {
-            // a batched graph that stopped: its ids shift with the graphs before it
-            const int32_t g = p.vgraph[v];
-            out[v] = (int32_t)((uint32_t)p.prev[v] - p.gbase_prev[g] + p.gbase_cur[g]);
-        } else if (v < p.n) {
+        if (v < p.n) {
             const bool fz = vertex_frozen(p, v);
+            // a frozen block keeps its members and smallest member; a graph that
+            // computed its level 0 here has no previous level
+            const bool history = fz || (moved && !vertex_level0(p, v));
+            const uint32_t before = history ? p.minof[v] : 0u;
             uint32_t mn = (uint32_t)v;
-            if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
-                // a frozen block keeps its members and smallest member
-                mn = fz ? p.minof[v] : block_min(p, v);
-                if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
-            }
+            if (fz)
+                mn = before;
+            else if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u))
+                mn = block_min(p, v);
+            if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
             if ((joined >> lane) & 1u) atomicOr(&p.shared[mn >> 5], 1u << (mn & 31));
             const uint2 rw = rank[mn >> 5];
-            const int32_t b = (int32_t)(rw.x + __popc(rw.y & ((1u << (mn & 31)) - 1u)));
-            out[v] = b;
-            if (!fz) {
-                // a graph that computed its level 0 here has no previous level
-                bool new_min = true;
-                if (moved && !vertex_level0(p, v)) {
-                    const uint32_t pm = ((p.bitmap_prev[v >> 5] >> (v & 31)) & 1u) ? (uint32_t)v : p.minof[v];
-                    mv = pm != mn;
-                    new_min = mv;
-                }
-                // the locality order's copy of the level names every block by
-                // its smallest member, which only moved vertices change (a
-                // frozen block keeps its members and its smallest member)
-                if (p.perm && new_min) p.gat[p.perm[v]] = (int32_t)mn;
-                if (mn != (uint32_t)v) p.minof[v] = mn;
+            uint32_t b = rw.x + __popc(rw.y & ((1u << (mn & 31)) - 1u));
+            if (!p.lgraph) {
+                out[v] = (int32_t)b;
+            } else {
+                const int32_t g = p.lgraph[v];
+                b -= p.gbase_cur[g];
+                if (!p.gout)
+                    out[v] = (int32_t)b;
+                else if (p.gout[g])
+                    p.gout[g][v - p.voff[g]] = (int32_t)b;
+            }
+            // the locality order's copy of the level names every block by its
+            // smallest member too
+            if (!history || before != mn) {
+                mv = history;
+                if (p.perm) p.gat[p.perm[v]] = (int32_t)mn;
+                p.minof[v] = mn;
             }
         }
         if (joined) {  // read by every lane above
@@ -573,16 +569,16 @@ __device__ __forceinline__ int64_t dealt_vertex(int64_t w0, uint32_t excl, uint3
 // level-(i-1) block B, and v has its label-l edges into B only outside C, in
 // another part C'.  So B split, and C or C' lacks B's smallest member: the
 // members of that part changed smallest member, and u or v has an edge to
-// one of them.  Mark (bit = level-i id) the blocks that hold such a member; a
+// one of them.  Mark (by the block's name) the blocks that hold such a member; a
 // vertex with more than max_scan edges marks its block unread.  When more
 // than an eighth of the vertices moved, nothing is scanned: the freeze pass
 // then takes every block as marked.
 __device__ __forceinline__ bool few_moved(const RoundParams& p) { return p.ctr->moved * 8 <= p.n; }
 
 __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, const uint32_t* edgeless,
-                                                            const uint32_t* moved, const int32_t* level,
+                                                            const uint32_t* moved,
                                                             int32_t max_scan, uint32_t* mark, int per_warp,
-                                                            bool stop_stable) {
+                                                            const uint8_t* gactive, bool stop_stable) {
     if (!few_moved(p)) return;
     if (stop_stable && p.ctr->count == p.ctr->prev_count) return;  // the last round: nothing follows
     const int lane = threadIdx.x & 31;
@@ -601,7 +597,7 @@ __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, 
     const uint32_t excl = incl - __popc(c);
     for (int t = 0; t < total; t += 32) {
         const int64_t v = dealt_vertex(w0, excl, c, t + lane, total);
-        if (v < 0 || !vertex_active(p, v)) continue;
+        if (v < 0 || (gactive && !gactive[p.lgraph[v]])) continue;
         const int64_t a = p.row[v], e_end = p.row[v + 1];
         // a graph that computed its level 0 here has no history: all dirty
         bool dirty = e_end - a > max_scan || vertex_level0(p, v);
@@ -614,7 +610,7 @@ __global__ void __launch_bounds__(256) dirty_blocks_kernel(const RoundParams p, 
                 if (w[u] >= 0 && ((moved[w[u] >> 5] >> (w[u] & 31)) & 1u)) dirty = true;
         }
         if (dirty) {
-            const uint32_t b = (uint32_t)level[v];
+            const uint32_t b = p.minof[v];
             const uint32_t mb = 1u << (b & 31);
             if (!(__ldcg(mark + (b >> 5)) & mb)) atomicOr(&mark[b >> 5], mb);
         }
@@ -653,6 +649,20 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
         e = edgeless ? edgeless[w] : 0u;
         c = mark ? candidate_word(bitmap, shared, edgeless, w, n) : 0u;
     }
+    uint32_t off = 0;  // vertices of graphs that stopped
+    if (f.gactive && own) {
+        const int64_t first = w * 32, last = min(n, first + 32) - 1;
+        if (first <= last) {
+            const int32_t g0 = f.vgraph[first], g1 = f.vgraph[last];
+            if (g0 == g1) {
+                off = f.gactive[g0] ? 0u : 0xffffffffu;
+            } else {
+                for (int64_t v = first; v <= last; ++v)
+                    if (!f.gactive[f.vgraph[v]]) off |= 1u << (v - first);
+            }
+        }
+        c &= ~off;
+    }
     if (f.gmode && edgeless) {
         // serving: a graph that computed its level 0 in this step has not had
         // its edgeless blocks formed by a round yet
@@ -682,7 +692,7 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
     for (int t = 0; t < total; t += 32) {
         const int64_t v = dealt_vertex(w0, excl, c, t + lane, total);
         if (v < 0) continue;
-        const uint32_t l = (uint32_t)f.level[v];
+        const uint32_t l = (uint32_t)f.names[v];
         if (!((mark[l >> 5] >> (l & 31)) & 1u)) atomicOr(&s_clean[warp][(v >> 5) - w0], 1u << (v & 31));
     }
     __syncwarp();
@@ -691,8 +701,9 @@ __global__ void __launch_bounds__(256) freeze_clean_kernel(const FreezePass f) {
         const uint32_t valid = w * 32 + 32 <= n ? 0xffffffffu : (n > w * 32 ? (1u << (uint32_t)(n - w * 32)) - 1u : 0u);
         const uint32_t single = b & ~sh & valid;
         const uint32_t cl = s_clean[warp][lane];
-        const uint32_t fz = single | (e & valid) | cl;
-        const uint32_t fm = single | (b & (e | cl) & valid);
+        const uint32_t keep = (e | cl | off) & valid;
+        const uint32_t fz = single | keep;
+        const uint32_t fm = single | (b & keep);
         f.frozen[w] = fz;
         f.frozen_min[w] = fm;
         shared[w] = sh & fm;
@@ -910,57 +921,46 @@ __global__ void __launch_bounds__(256) dense_assign_kernel(const RoundParams p, 
         const uint32_t mn = e.x;
         out[v] = (int32_t)e.y;
         if (p.perm) p.gat[p.perm[v]] = (int32_t)mn;  // the block by its smallest member
-        if (mn != (uint32_t)v && p.minof) p.minof[v] = mn;
+        if (p.minof) p.minof[v] = mn;
     }
 }
 
-// rank of every graph's first vertex (the first vertex of a graph is always
-// the smallest member of its block)
-__global__ void graph_base_kernel(const RoundParams p, const uint2* rank) {
+// Rank of every graph's first vertex (the first vertex of a graph is always the
+// smallest member of its block), and the graphs' stop test (GraphStop).
+__device__ __forceinline__ uint32_t rank_at(const RoundParams& p, const uint2* rank, int64_t x) {
+    if (x >= p.n) return rank[(p.n >> 5) + 1].x;
+    const uint2 rw = rank[x >> 5];
+    return rw.x + __popc(rw.y & ((1u << (x & 31)) - 1u));
+}
+
+__global__ void graph_base_kernel(const RoundParams p, const uint2* rank, const GraphStop st) {
     const int g = blockIdx.x * blockDim.x + threadIdx.x;
     if (g > p.n_graphs) return;
-    const int64_t x = p.voff[g];
-    uint32_t r;
-    if (x >= p.n) {
-        r = rank[(p.n >> 5) + 1].x;
+    const uint32_t base = rank_at(p, rank, p.voff[g]);
+    p.gbase_cur[g] = base;
+    if (!st.active || g == p.n_graphs || !st.active[g]) return;
+    const uint32_t count = rank_at(p, rank, p.voff[g + 1]) - base;
+    bool stop;
+    if (st.k) {
+        st.last[g] = st.round;
+        stop = st.round >= st.k[g] || (st.early && count == p.gbase_prev[g + 1] - p.gbase_prev[g]);
     } else {
-        const uint2 rw = rank[x >> 5];
-        r = rw.x + __popc(rw.y & ((1u << (x & 31)) - 1u));
+        stop = st.mode[g] == 1 || (st.mode[g] == 2 && (int64_t)count == st.prev_count[g]);
     }
-    p.gbase_cur[g] = r;
+    if (stop)
+        st.active[g] = 0;
+    else
+        atomicAdd(reinterpret_cast<unsigned long long*>(&p.ctr->graphs_on), 1ull);
 }
 
-__global__ void carry_minima_kernel(const RoundParams p) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < p.n; base += stride) {
-        const int64_t v = base + threadIdx.x;  // blockDim is a multiple of 32: a warp covers one bitmap word
-        const bool keep = v < p.n && !vertex_active(p, v) && ((p.bitmap_prev[v >> 5] >> (v & 31)) & 1u);
-        const unsigned b = __ballot_sync(kFull, keep);
-        if ((threadIdx.x & 31) == 0 && b) atomicOr(&p.bitmap[v >> 5], b);
-    }
-}
-
-__global__ void graph_stop_kernel(const RoundParams p, int round, const int32_t* k_per_graph, const uint8_t* early,
-                                  uint8_t* gactive, int32_t* glast, int32_t* sticky_err) {
-    const int g = blockIdx.x * blockDim.x + threadIdx.x;
-    if (g == 0 && p.ctr->err) atomicOr(sticky_err, p.ctr->err);
-    if (g >= p.n_graphs || !gactive[g]) return;
-    const uint32_t cur = p.gbase_cur[g + 1] - p.gbase_cur[g];
-    const uint32_t prv = p.gbase_prev[g + 1] - p.gbase_prev[g];
-    glast[g] = round;
-    if ((early[g] && cur == prv) || round >= k_per_graph[g]) gactive[g] = 0;
-}
-
-__global__ void localize_kernel(int32_t* row, int64_t n, const int32_t* vgraph, const uint32_t* gbase) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride)
-        row[v] = (int32_t)((uint32_t)row[v] - gbase[vgraph[v]]);
-}
-
-__global__ void vertex_graph_kernel(const int64_t* voff, int32_t G, int64_t n, int32_t* vgraph) {
-    const int g = blockIdx.x;
-    if (g >= G) return;
-    for (int64_t v = voff[g] + threadIdx.x; v < voff[g + 1]; v += blockDim.x) vgraph[v] = g;
+// vgraph[v] = graph owning v, in tiles (a CTA per graph leaves most of the chip
+// idle: 282 us for 16 graphs of 5 x 10^6 vertices together).
+constexpr int kGraphPer = 8;
+__global__ void __launch_bounds__(256) vertex_graph_kernel(const int64_t* voff, int64_t G, int64_t n, int32_t* vgraph) {
+    __shared__ int32_t s_g[256 * kGraphPer];
+    const int64_t v0 = (int64_t)blockIdx.x * 256 * kGraphPer;
+    tile_sources<256, kGraphPer>(G, voff, v0, min(n, v0 + 256 * kGraphPer), s_g);
+    for (int i = threadIdx.x; i < 256 * kGraphPer && v0 + i < n; i += 256) vgraph[v0 + i] = s_g[i];
 }
 
 __global__ void fill_i32_kernel(int32_t* out, int64_t n, int32_t value) {
@@ -1020,14 +1020,15 @@ static int words_per_warp(int64_t nw) {
     return (int)std::min<int64_t>(32, std::max<int64_t>(1, nw / (152 * 32)));
 }
 
-void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved, const int32_t* level,
-                         int32_t max_scan, uint32_t* mark, bool stop_stable, cudaStream_t s) {
+void launch_dirty_blocks(const RoundParams& p, const uint32_t* edgeless, const uint32_t* moved,
+                         int32_t max_scan, uint32_t* mark, const uint8_t* gactive, bool stop_stable,
+                         cudaStream_t s) {
     if (p.n <= 0) return;
     const int64_t nw = (p.n >> 5) + 1;
     const int per = words_per_warp(nw);
     const int64_t warps = (nw + per - 1) / per;
-    dirty_blocks_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(p, edgeless, moved, level, max_scan, mark, per,
-                                                                     stop_stable);
+    dirty_blocks_kernel<<<(unsigned)((warps + 7) / 8), 256, 0, s>>>(p, edgeless, moved, max_scan, mark, per,
+                                                                     gactive, stop_stable);
 }
 
 void launch_freeze_clean(const FreezePass& f, cudaStream_t s) {
@@ -1079,10 +1080,10 @@ void launch_bitmap_rank(const uint32_t* bitmap, int64_t nw, uint32_t* scan_tmp, 
 }
 
 void launch_renumber(const RoundParams& p, uint2* rank, uint32_t* scan_tmp, int32_t* out, uint32_t* mark,
-                     bool stop_stable, cudaStream_t s) {
+                     bool stop_stable, cudaStream_t s, const GraphStop& stop) {
     const int64_t nw = (p.n >> 5) + 1;
     rank_scan(p.bitmap, nw, scan_tmp, nullptr, rank, batched(p), p.ctr, s);
-    if (batched(p)) graph_base_kernel<<<(p.n_graphs + 1 + 255) / 256, 256, 0, s>>>(p, rank);
+    if (batched(p)) graph_base_kernel<<<(p.n_graphs + 1 + 255) / 256, 256, 0, s>>>(p, rank, stop);
     if (p.n <= 0) return;
     if (p.minof)
         assign_frozen_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, rank, out, p.moved, mark, stop_stable);
@@ -1107,26 +1108,10 @@ void launch_dense_level0(const RoundParams& p, const int32_t* key, const uint32_
     dense_assign_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p, key, lpair, out);
 }
 
-void launch_carry_minima(const RoundParams& p, cudaStream_t s) {
-    if (p.n <= 0) return;
-    carry_minima_kernel<<<grid_for(p.n, 256), 256, 0, s>>>(p);
-}
-
-void launch_graph_stop(const RoundParams& p, int round, const int32_t* k_per_graph, const uint8_t* early,
-                       uint8_t* gactive, int32_t* glast, int32_t* sticky_err, cudaStream_t s) {
-    if (p.n_graphs <= 0) return;
-    graph_stop_kernel<<<(p.n_graphs + 255) / 256, 256, 0, s>>>(p, round, k_per_graph, early, gactive, glast,
-                                                                sticky_err);
-}
-
-void launch_localize(int32_t* row, int64_t n, const int32_t* vgraph, const uint32_t* gbase, cudaStream_t s) {
-    if (n <= 0) return;
-    localize_kernel<<<grid_for(n, 256), 256, 0, s>>>(row, n, vgraph, gbase);
-}
-
 void launch_vertex_graph(const int64_t* voff, int32_t G, int64_t n, int32_t* vgraph, cudaStream_t s) {
-    if (G <= 0) return;
-    vertex_graph_kernel<<<(unsigned)G, 256, 0, s>>>(voff, G, n, vgraph);
+    if (G <= 0 || n <= 0) return;
+    const int64_t tile = 256 * kGraphPer;
+    vertex_graph_kernel<<<(unsigned)((n + tile - 1) / tile), 256, 0, s>>>(voff, G, n, vgraph);
 }
 
 void launch_iota_i32(int32_t* out, int64_t n, cudaStream_t s) {

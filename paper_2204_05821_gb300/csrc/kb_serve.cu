@@ -1,6 +1,5 @@
 // Device helpers of the serving arena: placing a request's CSR (and moving
-// it during compaction) with vertex and edge ids rebased, and writing every
-// running request's new level, in its own graph-local ids, to its level store.
+// it during compaction) with vertex and edge ids rebased.
 #include <cuda_runtime.h>
 
 #include "kb_internal.cuh"
@@ -21,7 +20,7 @@ __global__ void place_vertices_kernel(const PlaceArgs a) {
         a.drow[a.dst_vbase + i] = a.srow[a.src_vbase + i] - a.src_ebase + a.dst_ebase;
         if (i == a.n) continue;
         a.dvlab[a.dst_vbase + i] = a.svlab ? a.svlab[a.src_vbase + i] : 0;
-        if (a.sB && a.dB) a.dB[a.dst_vbase + i] = (int32_t)((uint32_t)a.sB[a.src_vbase + i] - a.b_sub + a.b_add);
+        if (a.sname) a.dname[a.dst_vbase + i] = a.sname[a.src_vbase + i] - (uint32_t)a.src_vbase + (uint32_t)a.dst_vbase;
     }
 }
 
@@ -35,30 +34,11 @@ __global__ void place_edges_kernel(const PlaceArgs a) {
     }
 }
 
-__global__ void emit_kernel(int64_t n, const int32_t* vgraph, const int32_t* B, const uint32_t* gbase,
-                            int32_t* const* slot_levels, const int32_t* slot_row, const int64_t* slot_n,
-                            const int64_t* voff) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n; v += stride) {
-        const int32_t g = vgraph[v];
-        const int32_t r = slot_row[g];
-        if (r < 0) continue;
-        const int64_t local = v - voff[g];
-        slot_levels[g][(int64_t)r * slot_n[g] + local] = (int32_t)((uint32_t)B[v] - gbase[g]);
-    }
-}
-
 }  // namespace
 
 void launch_place(const PlaceArgs& a, cudaStream_t s) {
     place_vertices_kernel<<<grid_for(a.n + 1, 256), 256, 0, s>>>(a);
     if (a.m > 0) place_edges_kernel<<<grid_for(a.m, 256), 256, 0, s>>>(a);
-}
-
-void launch_emit(int64_t n, const int32_t* vgraph, const int32_t* B, const uint32_t* gbase, int32_t* const* slot_levels,
-                 const int32_t* slot_row, const int64_t* slot_n, const int64_t* voff, cudaStream_t s) {
-    if (n <= 0) return;
-    emit_kernel<<<grid_for(n, 256), 256, 0, s>>>(n, vgraph, B, gbase, slot_levels, slot_row, slot_n, voff);
 }
 
 }  // namespace kb

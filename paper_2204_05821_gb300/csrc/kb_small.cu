@@ -235,7 +235,7 @@ __global__ void __launch_bounds__(kSmallThreads, KB_SMALL_MIN_BLOCKS) small_roun
                 pending = false;
             } else {
                 // at level 0 of a multi-graph run the key is (graph, label)
-                const uint32_t c2 = (l0 && batched(p)) ? (uint32_t)p.vgraph[v] : (uint32_t)cnt;
+                const uint32_t c2 = (l0 && p.vgraph) ? (uint32_t)p.vgraph[v] : (uint32_t)cnt;
                 const uint64_t h = vertex_hash(own, c2, acc, p.hash_mode);
                 pos = h & p.mask;
                 hi = table_hi(h, p.epoch);
