@@ -153,6 +153,7 @@ struct Plan {
     int subject = 0;       // kb_options::subject (generic CSE rounds when > 0)
     bool freeze = false;   // frozen blocks skip the rounds (RoundParams::frozen)
     bool dense0 = false;   // one graph: level 0 may take the small-label path (launch_dense_level0)
+    bool sketch = false;     // hub sketches ahead of the exact sets (launch_hub_sketch)
     bool ext_table = false;  // block table and empty-signature minima live outside the workspace
     bool ext_freeze = false;  // frozen-block state lives outside the workspace
     // the per-graph part (processed CSR, degree classes, hub plan, locality
@@ -171,7 +172,7 @@ struct Plan {
     size_t o_rowp = 0, o_colp = 0, o_labp = 0, o_cursor = 0, o_inpref = 0, o_i64tmp = 0;
     size_t csr_bytes = 0;
     size_t o_emin = 0, o_mid = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
-           o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0,
+           o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0, o_exact = 0, o_exactlist = 0, o_twin = 0,
            o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_moved = 0, o_mark = 0;
     size_t total = 0;
     // bytes of one degree-class bitmap; four follow one another (kb::DegreeClass)
@@ -254,6 +255,10 @@ void layout_round(Plan& P) {
     P.o_acc = take(sizeof(uint64_t) * H);
     P.o_cnt = take(sizeof(uint32_t) * H);
     P.o_sets = take(sizeof(uint64_t) * (size_t)P.set_slots);
+    P.sketch = P.n_chunks >= kb::kSketchMinChunks && P.thr >= kb::kSketchMinThreshold;
+    P.o_exact = take(P.sketch ? sizeof(uint32_t) * H : 0);
+    P.o_exactlist = take(P.sketch ? sizeof(int32_t) * (size_t)P.n_chunks : 0);
+    P.o_twin = take(P.sketch ? sizeof(uint32_t) * (size_t)next_pow2(2 * H) : 0);
     P.o_gat = take(P.reorder ? sizeof(int32_t) * (size_t)P.n : 0);
     P.o_ownkey = take(P.subject ? sizeof(int32_t) * (size_t)P.n : 0);
     const bool own_freeze = P.freeze && !P.ext_freeze;
@@ -843,6 +848,12 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     p.hub_sets = reinterpret_cast<uint64_t*>(ws + P.o_sets);
     p.hub_acc = reinterpret_cast<uint64_t*>(ws + P.o_acc);
     p.hub_cnt = reinterpret_cast<uint32_t*>(ws + P.o_cnt);
+    if (P.sketch) {
+        p.hub_exact = reinterpret_cast<uint32_t*>(ws + P.o_exact);
+        p.exact_list = reinterpret_cast<int32_t*>(ws + P.o_exactlist);
+        p.hub_twin = reinterpret_cast<uint32_t*>(ws + P.o_twin);
+        p.hub_twin_mask = (uint32_t)(next_pow2(2 * P.n_hubs) - 1);
+    }
     if (P.reorder) p.gat = reinterpret_cast<int32_t*>(ws + P.o_gat);
     R.prefix = reinterpret_cast<uint2*>(ws + P.o_prefix);
     R.scan_tmp = reinterpret_cast<uint32_t*>(ws + P.o_scan);
@@ -1000,6 +1011,7 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
     }
     if (hub) {
         if (T) T->begin(KB_KERNEL_HUB_CHUNK);
+        if (R.P.sketch) kb::launch_hub_sketch(p, R.total_chunks, s);
         kb::launch_clear_hubs(p, (int64_t)(R.set_bytes / sizeof(uint64_t)), s);
         kb::launch_hub_chunk(p, R.total_chunks, s);
         if (T) T->end();
@@ -2093,6 +2105,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
                 for (int f = 0; f < 3; ++f) kb::launch_clear_bits(sv->frz[f], sv->planned_n, word_end, s);
             }
             SV_TRY(sv, prepare(ctx, &view, &o, sv->R, -1, true));
+            for (bool& on : sv->R.class_on) on = true;  // new vertices refine
             sv->planned_n = sv->n_used;
             std::vector<int64_t> voff((size_t)G + 1);
             for (int j = 0; j < G; ++j) voff[(size_t)j] = sv->slots[(size_t)j].vbase;
@@ -2161,6 +2174,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         if (ctx->h_ctr->err) {
             SV_TRY(sv, device_error(ctx));
         }
+        for (int c = 0; c < 3; ++c) sv->R.class_on[c] = ctx->h_ctr->class_on[c] > 0;
         // bookkeeping and retirement (one synchronisation for all copies)
         std::vector<std::pair<ServeRequest*, int>> finished;
         for (int j = 0; j < G; ++j) {

@@ -26,6 +26,11 @@ static_assert(kMaxHubChunk < 65536, "a chunk's edge count is packed in 16 bits")
 constexpr int kMaxMedSplit = 256;
 constexpr int kDefaultMedSplit = kMaxMedSplit;
 constexpr int kHubFinalThreads = 256;
+// Sketches (kb_hub.cu) go ahead of the exact sets from this many hub chunks on
+// (a million edges), where they cost less than the launches they add, and for
+// thresholds that leave room for one in every hub's set.
+constexpr int64_t kSketchMinChunks = 2048;
+constexpr int kSketchMinThreshold = 128;
 constexpr int kProbeLimit = 1 << 22;  // bound on block-table probes per vertex
 constexpr int kSmallDegree = 8;       // vertices with at most this many edges take a lane each (kb_small.cu),
 constexpr int kMidDegree = 32;        // with at most this many eight lanes each (kb_medium.cu)
@@ -50,6 +55,8 @@ struct Counters {
     int64_t keyed_e[3];
     int32_t dense_bad;  // a level-0 key outside [0, kDenseLabels) (launch_dense_labels)
     int64_t prev_count; // blocks at the level before
+    uint32_t most_pairs;    // most distinct pairs of a vertex of the medium CTA kernel this round
+    uint32_t exact_chunks;  // chunks of hubs that need their exact set (launch_hub_sketch)
     int64_t n_class[3]; // mid and medium vertices and hubs of the graph (launch_classes)
 };
 
@@ -139,6 +146,13 @@ struct RoundParams {
     uint64_t* hub_sets;
     uint64_t* hub_acc;  // [n_hubs] sum of pair mixes over unique pairs
     uint32_t* hub_cnt;  // [n_hubs] unique pairs
+    // Sketches first (kb_hub.cu): hub_exact[h] != 0 for the hubs that need their
+    // exact set, whose chunks are in exact_list (ctr->exact_chunks of them); the
+    // others that refine are alone in their new block.  nullptr: every hub does.
+    uint32_t* hub_exact;
+    int32_t* exact_list;
+    uint32_t* hub_twin;      // [hub_twin_mask + 1] table of hub indices + 1
+    uint32_t hub_twin_mask;
     // several graphs at once (batched refinement, serving); all null or 0 for one graph
     int32_t n_graphs;
     const int64_t* voff;       // [G+1] first vertex of every graph
@@ -284,6 +298,7 @@ void launch_medium_round(const RoundParams& p, cudaStream_t s);  //   after the 
 // Per-device kernel attributes (shared-memory carveouts); call once per device
 // before the first launch and outside any stream capture.
 void set_medium_kernel_attributes();
+void launch_hub_sketch(const RoundParams& p, int64_t total_chunks, cudaStream_t s);  // kb_hub.cu
 void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s);
 void launch_hub_final(const RoundParams& p, cudaStream_t s);
 // Several graphs, after the rank scan: gbase_cur, and the stop test of every

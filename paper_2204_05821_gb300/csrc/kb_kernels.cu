@@ -31,8 +31,13 @@ namespace {
 // new to the hub (the CAS that placed them found the slot empty) are counted
 // and summed into its hash.
 // ----------------------------------------------------------------------------
+// Whether hub h takes part in the exact path this round.
+__device__ __forceinline__ bool hub_is_exact(const RoundParams& p, int h) {
+    return p.hub_exact ? p.hub_exact[h] != 0u : vertex_refines(p, p.hub_v[h]);
+}
+
 template <int kChunk>
-__global__ void __launch_bounds__(kHubThreads) hub_chunk_kernel(const RoundParams p) {
+__device__ __forceinline__ void hub_chunk(const RoundParams& p, int64_t c) {
     constexpr int kHubSetCap = 2 * kChunk;  // the chunk's shared dedup set
     __shared__ uint64_t s_pair[kChunk];
     __shared__ uint64_t s_new[kChunk];
@@ -41,13 +46,12 @@ __global__ void __launch_bounds__(kHubThreads) hub_chunk_kernel(const RoundParam
     __shared__ uint64_t s_accsum;
 
     const int tid = threadIdx.x;
-    const int64_t c = blockIdx.x;
     // every thread reads the chunk's hub and packed extent (one broadcast word each)
     const int h = p.chunk_hub[c];
     const uint64_t ext = p.chunk_ext[c];
     const int64_t e0 = (int64_t)(ext >> 16);
     const int E = (int)(ext & 0xffffu);
-    if ((p.gmode || p.vmask || p.frozen) && !vertex_refines(p, p.hub_v[h])) return;  // uniform over the CTA
+    if (!hub_is_exact(p, h)) return;  // uniform over the CTA
     if (tid == 0) {
         s_nuniq = 0;
         s_nnew = 0;
@@ -172,6 +176,20 @@ __global__ void __launch_bounds__(kHubThreads) hub_chunk_kernel(const RoundParam
     }
 }
 
+// A chunk per CTA, or (after sketches) the listed chunks in strides of the grid.
+template <int kChunk>
+__global__ void __launch_bounds__(kHubThreads) hub_chunk_kernel(const RoundParams p) {
+    if (!p.exact_list) {
+        hub_chunk<kChunk>(p, blockIdx.x);
+        return;
+    }
+    const uint32_t total = p.ctr->exact_chunks;
+    for (uint32_t i = blockIdx.x; i < total; i += gridDim.x) {
+        hub_chunk<kChunk>(p, p.exact_list[i]);
+        __syncthreads();  // the shared sets start afresh
+    }
+}
+
 __device__ __forceinline__ bool hub_set_contains(const uint64_t* gset, uint64_t gcap, uint64_t pr) {
     uint64_t slot = hub_set_home(pr, gcap);
     for (uint64_t t = 0; t < gcap; ++t) {
@@ -199,6 +217,10 @@ __global__ void __launch_bounds__(kHubFinalThreads) hub_final_kernel(const Round
     const int h = blockIdx.x;
     const int32_t v = p.hub_v[h];
     if (!vertex_refines(p, v)) return;
+    if (!hub_is_exact(p, h)) {  // its sketch says that it is alone in its new block
+        if (tid == 0) toggle_min(p.bitmap, (uint32_t)v);
+        return;
+    }
     const int32_t own = own_of(p, v);
     const uint32_t cnt = p.hub_cnt[h];
     const uint64_t hv = vertex_hash(own, cnt, p.hub_acc[h], p.hash_mode);
@@ -403,6 +425,7 @@ __global__ void __launch_bounds__(kScanThreads) popc_scan_kernel(const uint32_t*
         for (int k = 0; k < 3; ++k) ctr->class_on[k] = 0;
         ctr->moved = 0;
         ctr->graphs_on = 0;
+        ctr->most_pairs = 0;
         if (rank_total) rank[nw] = make_uint2(all, 0u);
     }
 #pragma unroll
@@ -806,14 +829,16 @@ __global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p
         s_h0 = lo;
     }
     __syncthreads();
+    bool any = false;
     for (int i = threadIdx.x; i < kClearHubs; i += blockDim.x) {
         const int h = s_h0 + i;
         const bool in = h < p.n_hubs && p.hub_set_off[h] < t1;
         s_end[i] = in ? p.hub_set_off[h + 1] : t1;
-        s_ref[i] = in && vertex_refines(p, p.hub_v[h]);
+        s_ref[i] = in && hub_is_exact(p, h);
+        any |= s_ref[i] != 0;
         if (!in) break;  // later entries keep their stale values: the walk below stops at this one
     }
-    __syncthreads();
+    if (!__syncthreads_or(any)) return;
     ulonglong2* sets2 = reinterpret_cast<ulonglong2*>(p.hub_sets);
     const ulonglong2 e = make_ulonglong2(kEmptyPair, kEmptyPair);
     int j = 0;
@@ -1002,7 +1027,7 @@ void launch_clear_hubs(const RoundParams& p, int64_t total_slots, cudaStream_t s
     cudaMemsetAsync(p.hub_acc, 0, sizeof(uint64_t) * (size_t)p.n_hubs, s);
     cudaMemsetAsync(p.hub_cnt, 0, sizeof(uint32_t) * (size_t)p.n_hubs, s);
     if (total_slots <= 0) return;
-    if (!p.frozen) {
+    if (!p.frozen && !p.hub_exact) {
         cudaMemsetAsync(p.hub_sets, 0xff, sizeof(uint64_t) * (size_t)total_slots, s);
         return;
     }
@@ -1059,12 +1084,14 @@ void launch_clear_bits(uint32_t* words, int64_t a, int64_t b, cudaStream_t s) {
 
 void launch_hub_chunk(const RoundParams& p, int64_t total_chunks, cudaStream_t s) {
     if (p.n_hubs <= 0 || total_chunks <= 0) return;
+    // after sketches few chunks may be left: a grid that fills the chip walks them
+    const unsigned grid = (unsigned)(p.exact_list ? std::min<int64_t>(total_chunks, 152 * 12 * 4) : total_chunks);
     if (p.hub_chunk == 256)
-        hub_chunk_kernel<256><<<(unsigned)total_chunks, kHubThreads, 0, s>>>(p);
+        hub_chunk_kernel<256><<<grid, kHubThreads, 0, s>>>(p);
     else if (p.hub_chunk == 1024)
-        hub_chunk_kernel<1024><<<(unsigned)total_chunks, kHubThreads, 0, s>>>(p);
+        hub_chunk_kernel<1024><<<grid, kHubThreads, 0, s>>>(p);
     else
-        hub_chunk_kernel<kDefaultHubChunk><<<(unsigned)total_chunks, kHubThreads, 0, s>>>(p);
+        hub_chunk_kernel<kDefaultHubChunk><<<grid, kHubThreads, 0, s>>>(p);
 }
 
 void launch_hub_final(const RoundParams& p, cudaStream_t s) {

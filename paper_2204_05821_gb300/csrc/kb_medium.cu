@@ -490,7 +490,10 @@ __global__ void __launch_bounds__(kThreads) medium_cta_kernel(const RoundParams 
         // find or insert, with the full signature compare on every tag match
         const uint64_t h = vertex_hash(own, cnt, acc, p.hash_mode);
         const uint32_t hi = table_hi(h, p.epoch);
-        if (tid == 0) s_pos = h & p.mask;
+        if (tid == 0) {
+            s_pos = h & p.mask;
+            if (p.hub_exact && cnt > *(volatile uint32_t*)&p.ctr->most_pairs) atomicMax(&p.ctr->most_pairs, cnt);
+        }
         while (true) {
             if (tid == 0) {
                 uint64_t pos = s_pos;
