@@ -344,7 +344,7 @@ kb_status kb_summary(kb_context* ctx, const kb_graph* g, int direction, int use_
  * blocks then cost less than re-keying whole blocks; work reports n for every
  * computed level.  The result is the same either way.
  * KB_ERR_INVALID_ARG when an old level or a changed id lies outside [0, n).
- * Scratch: about 29 B x n of library-owned device memory.  Synchronises. */
+ * Scratch: about 9 B x n of library-owned device memory.  Synchronises. */
 kb_status kb_refine_update(kb_context* ctx, const kb_graph* g, const kb_options* opt, int k,
                            const int32_t* changed, int64_t n_changed, int32_t* levels,
                            int64_t* counts, int* levels_computed, int64_t* work);

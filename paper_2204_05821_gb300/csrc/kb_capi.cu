@@ -65,10 +65,9 @@ struct kb_context {
     // summary graph: triple table, first edges, edge bitmap and its ranks
     void* sum_buf = nullptr;
     size_t sum_buf_bytes = 0;
-    // incremental refinement: bitmaps, block flags, kept minima, id ranges
+    // incremental refinement: bitmaps, old blocks' smallest members
     void* upd_buf = nullptr;
     size_t upd_buf_bytes = 0;
-    unsigned long long* d_work = nullptr;  // |W| of the current round
     cudaStream_t copy_stream = nullptr;  // level rows back to the host (kb_refine_host)
     cudaEvent_t row_ev = nullptr;
     // timing: CUDA events per kernel family; with work, also the vertices and
@@ -1256,46 +1255,37 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     cudaStream_t s = ctx->stream;
     auto row = [&](int i) { return levels + (size_t)i * (size_t)n; };
 
-    // scratch: changed, dirty, moved and work-set bitmaps, block flags, kept
-    // minima, the old row of the current level, the new level 0, id ranges
-    const int64_t nw = (n >> 5) + 1;
-    const size_t szb = align_up(sizeof(uint32_t) * (size_t)nw), sz4 = align_up(sizeof(int32_t) * (size_t)n);
-    KB_TRY(ensure_buffer(ctx, &ctx->upd_buf, &ctx->upd_buf_bytes, 4 * szb + align_up((size_t)n) + 3 * sz4 + 4 * sz4));
-    if (!ctx->d_work && cudaMalloc(reinterpret_cast<void**>(&ctx->d_work), sizeof(unsigned long long)) != cudaSuccess) {
-        cudaGetLastError();
-        return fail(ctx, KB_ERR_OOM, "cannot allocate a counter");
-    }
+    // scratch: six bitmaps, the smallest vertex of every old block and, per
+    // vertex, of its old block
+    const size_t szb = align_up(sizeof(uint32_t) * (size_t)((n >> 5) + 1)), sz4 = align_up(sizeof(int32_t) * (size_t)n);
+    KB_TRY(ensure_buffer(ctx, &ctx->upd_buf, &ctx->upd_buf_bytes, 6 * szb + 2 * sz4));
     char* b = reinterpret_cast<char*>(ctx->upd_buf);
+    auto bits = [&](int j) { return reinterpret_cast<uint32_t*>(b + (size_t)j * szb); };
+    uint32_t *changed_bits = bits(0), *flag = bits(1), *taint = bits(2), *dirty = bits(3), *moved = bits(4), *wmask = bits(5);
+    uint32_t* old_min = reinterpret_cast<uint32_t*>(b + 6 * szb);
+    uint32_t* old_name = reinterpret_cast<uint32_t*>(b + 6 * szb + sz4);
 
-    // The first round re-keys at least every vertex of an old level-0 block
-    // that holds a changed vertex.  When that is over a quarter of the
-    // vertices (level-0 blocks are label classes, often huge), recomputing
-    // with the frozen blocks of a full refinement costs less than re-keying
-    // whole blocks round after round.
-    {
-        KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-        kb::launch_check_ids(n, row(0), ctx->d_ctr, s);
-        uint32_t* scratch = reinterpret_cast<uint32_t*>(b);
-        KB_CUDA(ctx, cudaMemsetAsync(scratch, 0, szb, s));
-        kb::launch_set_bits(n, n_changed, changed, scratch, ctx->d_ctr, s);
-        KB_TRY(read_counters(ctx));
-        if (ctx->h_ctr->err & kb::kErrInvalid)
-            return fail(ctx, KB_ERR_INVALID_ARG, "old levels or changed vertices hold ids outside [0, n)");
-        KB_CUDA(ctx, cudaMemsetAsync(scratch, 0, szb, s));
-        KB_CUDA(ctx, cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), s));
-        kb::launch_touched_size(n, n_changed, changed, row(0), scratch, ctx->d_work, s);
-        KB_CUDA(ctx, cudaGetLastError());
-        unsigned long long w1 = 0;
-        KB_CUDA(ctx, cudaMemcpyAsync(&w1, ctx->d_work, sizeof(w1), cudaMemcpyDeviceToHost, s));
-        KB_CUDA(ctx, cudaStreamSynchronize(s));
-        if ((int64_t)w1 * 4 > n) {
-            KB_TRY(refine_impl(ctx, g, opt, nullptr, 0, k, levels, counts, levels_computed));
-            if (work) {
-                const int lc = levels_computed ? *levels_computed : k;
-                for (int i = 0; i <= k; ++i) work[i] = i <= lc ? n : 0;
-            }
-            return KB_OK;
+    // The old levels must be partitions with ids in [0, n); the changed ids too.
+    // The first round re-keys at least every vertex of an old level-0 block that
+    // holds a changed vertex.  When that is over a quarter of the vertices
+    // (level-0 blocks are label classes, often huge), recomputing with the frozen
+    // blocks of a full refinement costs less than re-keying whole blocks round
+    // after round.
+    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
+    KB_CUDA(ctx, cudaMemsetAsync(changed_bits, 0, 3 * szb, s));
+    kb::launch_check_ids(n * (int64_t)(k + 1), n, levels, ctx->d_ctr, s);
+    kb::launch_changed(n, n_changed, changed, row(0), changed_bits, flag, ctx->d_ctr, s);
+    KB_CUDA(ctx, cudaGetLastError());
+    KB_TRY(read_counters(ctx));
+    if (ctx->h_ctr->err & kb::kErrInvalid)
+        return fail(ctx, KB_ERR_INVALID_ARG, "old levels or changed vertices hold ids outside [0, n)");
+    if (ctx->h_ctr->work_set * 4 > n) {
+        KB_TRY(refine_impl(ctx, g, opt, nullptr, 0, k, levels, counts, levels_computed));
+        if (work) {
+            const int lc = levels_computed ? *levels_computed : k;
+            for (int i = 0; i <= k; ++i) work[i] = i <= lc ? n : 0;
         }
+        return KB_OK;
     }
 
     Prepared R;
@@ -1303,80 +1293,53 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     const int32_t* init_key = opt->use_vertex_labels ? g->vertex_labels : nullptr;
     KB_TRY(prepare(ctx, g, opt, R, -1, false, nullptr, init_key));
     kb::RoundParams& p = R.p;
-    uint32_t* changed_bits = reinterpret_cast<uint32_t*>(b);
-    uint32_t* dirty = reinterpret_cast<uint32_t*>(b + szb);
-    uint32_t* moved = reinterpret_cast<uint32_t*>(b + 2 * szb);
-    uint32_t* wmask = reinterpret_cast<uint32_t*>(b + 3 * szb);
-    uint8_t* flag = reinterpret_cast<uint8_t*>(b + 4 * szb);
-    char* b2 = b + 4 * szb + align_up((size_t)n);
-    uint32_t* kmin = reinterpret_cast<uint32_t*>(b2);
-    int32_t* keep = reinterpret_cast<int32_t*>(b2 + sz4);
-    int32_t* level0 = reinterpret_cast<int32_t*>(b2 + 2 * sz4);
-    int32_t* ranges = reinterpret_cast<int32_t*>(b2 + 3 * sz4);
 
-    // the old levels must be partitions with ids in [0, n); the changed ids too
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-    for (int i = 0; i <= k; ++i) kb::launch_check_ids(n, row(i), ctx->d_ctr, s);
-    KB_CUDA(ctx, cudaMemsetAsync(changed_bits, 0, szb, s));
-    kb::launch_set_bits(n, n_changed, changed, changed_bits, ctx->d_ctr, s);
+    // level 0 from scratch, in place of the old one; its moved vertices start
+    // the dirty set
+    p.old_min = old_min;
+    p.old_name = old_name;
+    p.taint = taint;
+    p.keep_old = row(0);
+    kb::launch_old_min(n, row(0), old_min, s);
+    if (init_key)
+        KB_TRY(launch_level0(ctx, R, init_key, row(0), s));
+    else
+        kb::launch_one_block(p, row(0), s);
+    kb::launch_moved(n, nullptr, old_name, taint, moved, ctx->d_ctr, s);
     KB_CUDA(ctx, cudaGetLastError());
     KB_TRY(read_counters(ctx));
-    if (ctx->h_ctr->err & kb::kErrInvalid)
-        return fail(ctx, KB_ERR_INVALID_ARG, "old levels or changed vertices hold ids outside [0, n)");
-
-    // level 0 from scratch; its moved vertices start the dirty set
-    if (init_key) {
-        KB_TRY(launch_level0(ctx, R, init_key, level0, s));
-        KB_TRY(read_counters(ctx));
-        KB_TRY(device_error(ctx));
-        counts[0] = ctx->h_ctr->count;
-    } else {
-        kb::launch_fill_i32(level0, n, 0, s);
-        if (p.perm) kb::launch_fill_i32(p.gat, n, 0, s);
-        counts[0] = 1;
-    }
-    KB_CUDA(ctx, cudaMemsetAsync(wmask, 0xff, szb, s));
-    kb::launch_moved(n, wmask, row(0), level0, ranges, moved, s);
-    KB_CUDA(ctx, cudaMemcpyAsync(row(0), level0, sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-    kb::launch_count_bits(moved, nw, &ctx->d_ctr->moved, s);
-    KB_TRY(read_counters(ctx));
+    KB_TRY(device_error(ctx));
+    counts[0] = init_key ? ctx->h_ctr->count : 1;
     if (work) work[0] = n;
 
+    R.counters_clear = true;
+    R.compact = true;  // windows packed from the work set
     for (int i = 1; i <= k; ++i) {
         Timer T(ctx);
         // dirty = changed | moved | predecessors of moved; W = their previous-level blocks
         // (the pass over every edge only when some vertex moved)
         const bool any_moved = ctx->h_ctr->moved > 0;
-        kb::launch_or_words(nw, changed_bits, moved, dirty, s);
         if (any_moved) kb::launch_dirty_from_moved(n, R.P.m_proc, p.row, p.col, moved, dirty, s);
-        KB_CUDA(ctx, cudaMemsetAsync(ctx->d_work, 0, sizeof(unsigned long long), s));
-        kb::launch_work_set(n, row(i - 1), dirty, flag, wmask, ctx->d_work, s);
-        KB_CUDA(ctx, cudaMemcpyAsync(keep, row(i), sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, s));
-        kb::launch_keep_min(n, wmask, keep, kmin, s);
+        kb::launch_work_set(n, row(i - 1), changed_bits, moved, any_moved ? dirty : nullptr, flag, wmask, ctx->d_ctr, s);
+        kb::launch_old_min(n, row(i), old_min, s);
+        KB_CUDA(ctx, cudaMemsetAsync(taint, 0, szb, s));
         KB_TRY(next_epoch(ctx, R, s));
         KB_TRY(next_empty_round(ctx, R, s));
         p.prev = row(i - 1);
         p.vmask = wmask;
-        p.keep_old = keep;
-        p.kmin = kmin;
+        p.keep_old = row(i);
         KB_TRY(launch_round_body(ctx, R, s, &T));
-        kb::launch_keep_bits(n, wmask, keep, kmin, p.bitmap, s);
+        kb::launch_keep_bits(n, wmask, row(i), old_min, p.bitmap, s);
         T.begin(KB_KERNEL_RENUMBER);
         kb::launch_renumber(p, R.prefix, R.scan_tmp, row(i), nullptr, false, s);
         T.end();
-        kb::launch_moved(n, wmask, keep, row(i), ranges, moved, s);
-        kb::launch_count_bits(moved, nw, &ctx->d_ctr->moved, s);
+        kb::launch_moved(n, wmask, old_name, taint, moved, ctx->d_ctr, s);
         KB_CUDA(ctx, cudaGetLastError());
         KB_TRY(read_counters(ctx));
         ctx->round_ms.push_back(T.collect());
         KB_TRY(device_error(ctx));
         counts[i] = ctx->h_ctr->count;
-        if (work) {
-            unsigned long long w = 0;
-            KB_CUDA(ctx, cudaMemcpy(&w, ctx->d_work, sizeof(w), cudaMemcpyDeviceToHost));
-            work[i] = (int64_t)w;
-        }
+        if (work) work[i] = ctx->h_ctr->work_set;
         if (levels_computed) *levels_computed = i;
         if (opt->early_stop && counts[i] == counts[i - 1]) {
             if (i < k) kb::launch_copy_rows(levels, n, i, i + 1, k, s);
@@ -1388,9 +1351,6 @@ kb_status update_impl(kb_context* ctx, const kb_graph* g, const kb_options* opt,
             break;
         }
     }
-    p.vmask = nullptr;
-    p.keep_old = nullptr;
-    p.kmin = nullptr;
     KB_CUDA(ctx, cudaStreamSynchronize(s));
     return KB_OK;
 }
@@ -2292,7 +2252,6 @@ kb_status kb_destroy(kb_context* ctx) {
     cudaFree(ctx->fix_buf);
     cudaFree(ctx->sum_buf);
     cudaFree(ctx->upd_buf);
-    cudaFree(ctx->d_work);
     if (ctx->copy_stream) cudaStreamDestroy(ctx->copy_stream);
     if (ctx->row_ev) cudaEventDestroy(ctx->row_ev);
 

@@ -56,6 +56,16 @@ __device__ __forceinline__ void join_slot(const RoundParams& p, uint64_t pos, ui
     p.slot_of[v] = (int32_t)pos;
 }
 
+// Incremental refinement: vertex v's new block goes by `name`.  Where its old
+// one went by another, both names are tainted (RoundParams::taint).
+__device__ __forceinline__ void note_old_name(const RoundParams& p, int64_t v, uint32_t name) {
+    const uint32_t old = p.old_min[p.keep_old[v]];
+    p.old_name[v] = old;
+    if (old == name) return;
+    atomicOr(&p.taint[old >> 5], 1u << (old & 31));
+    atomicOr(&p.taint[name >> 5], 1u << (name & 31));
+}
+
 __device__ __forceinline__ bool vertex_active(const RoundParams& p, int64_t v) {
     return !p.vmask || ((p.vmask[v >> 5] >> (v & 31)) & 1u);
 }

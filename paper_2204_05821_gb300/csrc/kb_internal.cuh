@@ -48,6 +48,7 @@ struct Counters {
     int64_t frozen; // vertices frozen for the next round (launch_freeze_clean)
     int64_t class_on[3]; // mid and medium vertices and hubs that refine next round (launch_freeze_clean)
     int64_t moved;  // re-keyed vertices whose smallest block member changed (renumbering)
+    int64_t work_set;   // vertices re-keyed by a round of an incremental refinement
     int64_t graphs_on;  // graphs of a batch that refine next round (launch_graph_bases)
     // vertices re-keyed this round and their edges in the processed
     // direction, per kernel family: small, medium, hub
@@ -82,12 +83,16 @@ struct RoundParams {
     // bisimulation).
     const int32_t* own_key;
     // Incremental refinement (kb_refine_update): only vertices with their bit
-    // set in vmask are re-keyed; every other vertex keeps its old grouping at
-    // this level: keep_old is the level's old row and kmin[b] the smallest
-    // such vertex of old block b.  nullptr when every vertex is re-keyed.
+    // set in vmask are re-keyed (nullptr: all); every other vertex keeps its old
+    // grouping at this level: keep_old is the level's old row and old_min[b] the
+    // smallest vertex of old block b.  The renumbering writes old_name[v], the
+    // smallest vertex of v's old block, for every re-keyed vertex, and sets the
+    // bits of its old and new block's names in taint where they differ.
     const uint32_t* vmask;
     const int32_t* keep_old;
-    const uint32_t* kmin;
+    const uint32_t* old_min;
+    uint32_t* old_name;
+    uint32_t* taint;
     // Frozen blocks (stratified rounds, whose keys hold the own previous block):
     // a block that cannot change this round, because it has one member (a
     // vertex alone in its previous block stays alone) or because all its
@@ -410,22 +415,20 @@ void launch_levels_differ(const int32_t* a, const int32_t* b, int64_t n, Counter
 // Incremental refinement (kb_update.cu)
 void launch_dirty_from_moved(int64_t n, int64_t m, const int64_t* row, const int32_t* col, const uint32_t* moved,
                              uint32_t* dirty, cudaStream_t s);
-void launch_or_words(int64_t nw, const uint32_t* a, const uint32_t* b, uint32_t* out, cudaStream_t s);
-void launch_work_set(int64_t n, const int32_t* prev, const uint32_t* dirty, uint8_t* flag, uint32_t* wmask,
-                     unsigned long long* count, cudaStream_t s);
-void launch_keep_min(int64_t n, const uint32_t* wmask, const int32_t* old, uint32_t* kmin, cudaStream_t s);
-void launch_keep_bits(int64_t n, const uint32_t* wmask, const int32_t* old, const uint32_t* kmin, uint32_t* bitmap,
+void launch_work_set(int64_t n, const int32_t* prev, const uint32_t* changed, const uint32_t* moved,
+                     const uint32_t* dirty, uint32_t* flag, uint32_t* wmask, Counters* ctr, cudaStream_t s);
+void launch_old_min(int64_t n, const int32_t* level, uint32_t* old_min, cudaStream_t s);
+void launch_keep_bits(int64_t n, const uint32_t* wmask, const int32_t* old, const uint32_t* old_min, uint32_t* bitmap,
                       cudaStream_t s);
-void launch_moved(int64_t n, const uint32_t* wmask, const int32_t* old, const int32_t* cur, int32_t* ranges,
-                  uint32_t* moved, cudaStream_t s);
-void launch_check_ids(int64_t n, const int32_t* a, Counters* ctr, cudaStream_t s);
-// *out += vertices in the blocks of `level` that hold a vertex of ids
-// (touched: a zeroed bitmap of n bits; ids and level values in [0, n)).
-void launch_touched_size(int64_t n, int64_t count, const int32_t* ids, const int32_t* level, uint32_t* touched,
-                         unsigned long long* out, cudaStream_t s);
-// *out += set bits of words[0..nw) (kb_kernels.cu)
-void launch_count_bits(const uint32_t* words, int64_t nw, int64_t* out, cudaStream_t s);
-void launch_set_bits(int64_t n, int64_t count, const int32_t* ids, uint32_t* bits, Counters* ctr, cudaStream_t s);
+void launch_moved(int64_t n, const uint32_t* wmask, const uint32_t* old_name, const uint32_t* taint, uint32_t* moved,
+                  Counters* ctr, cudaStream_t s);
+// Level 0 without labels: {V} (out all 0), with RoundParams::old_name and taint.
+void launch_one_block(const RoundParams& p, int32_t* out, cudaStream_t s);
+void launch_check_ids(int64_t count, int64_t n, const int32_t* a, Counters* ctr, cudaStream_t s);
+// Bits of the changed vertices; ctr->work_set += vertices in the blocks of
+// `level` that hold one (touched: a zeroed bitmap of n bits).
+void launch_changed(int64_t n, int64_t count, const int32_t* ids, const int32_t* level, uint32_t* bits,
+                    uint32_t* touched, Counters* ctr, cudaStream_t s);
 // Copy row src of the level store to the rows [first, last] of levels (src not among them).
 void launch_copy_rows(int32_t* levels, int64_t n, int src, int first, int last, cudaStream_t s);
 

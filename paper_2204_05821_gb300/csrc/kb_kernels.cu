@@ -467,11 +467,14 @@ __global__ void __launch_bounds__(256) assign_kernel(const RoundParams p, const 
     for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < p.n; v += stride) {
         uint32_t mn = (uint32_t)v;
         if (!vertex_active(p, v)) {
-            mn = p.kmin[p.keep_old[v]];  // incremental: the smallest kept member of its old block
+            mn = p.old_min[p.keep_old[v]];  // incremental: its old block stays
             if ((int64_t)mn >= p.n) mn = (uint32_t)v;
-        } else if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
-            mn = block_min(p, v);
-            if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
+        } else {
+            if (!((p.bitmap[v >> 5] >> (v & 31)) & 1u)) {
+                mn = block_min(p, v);
+                if ((int64_t)mn >= p.n) mn = (uint32_t)v;  // only after a reported device error
+            }
+            if (p.taint) note_old_name(p, v, mn);
         }
         const uint2 rw = rank[mn >> 5];
         const int32_t b = (int32_t)(rw.x + __popc(rw.y & ((1u << (mn & 31)) - 1u)));
@@ -787,23 +790,6 @@ __global__ void clear_bits_kernel(uint32_t* words, int64_t a, int64_t b) {
     }
 }
 
-// *out += set bits of words[0..nw): a few hundred atomics in all
-__global__ void __launch_bounds__(256) count_bits_kernel(const uint32_t* words, int64_t nw, int64_t* out) {
-    __shared__ unsigned long long s_sum[8];
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    unsigned long long c = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nw; i += stride) c += __popc(words[i]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(kFull, c, o);
-    if ((threadIdx.x & 31) == 0) s_sum[threadIdx.x >> 5] = c;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned long long t = 0;
-        for (int w = 0; w < 8; ++w) t += s_sum[w];
-        if (t) atomicAdd(reinterpret_cast<unsigned long long*>(out), t);
-    }
-}
-
 // Refill the sets of the hubs that refine this round with the empty pair, in
 // tiles of kClearTile consecutive slots of all sets together (one hub's set
 // can hold 10^8 slots; large tiles keep the per-tile search for the first hub
@@ -944,6 +930,7 @@ __global__ void __launch_bounds__(256) dense_assign_kernel(const RoundParams p, 
         }
         const uint2 e = __ldg(lpair + l);
         const uint32_t mn = e.x;
+        if (p.taint) note_old_name(p, v, mn);
         out[v] = (int32_t)e.y;
         if (p.perm) p.gat[p.perm[v]] = (int32_t)mn;  // the block by its smallest member
         if (p.minof) p.minof[v] = mn;
@@ -1069,11 +1056,6 @@ void launch_round_work(const RoundParams& p, cudaStream_t s) {
     if (p.n <= 0) return;
     const int g = grid_for(p.n, 256) < 1216 ? grid_for(p.n, 256) : 1216;
     round_work_kernel<<<g, 256, 0, s>>>(p.n, p.row, p.frozen, p.mid_max, p.hub_threshold, p.ctr);
-}
-
-void launch_count_bits(const uint32_t* words, int64_t nw, int64_t* out, cudaStream_t s) {
-    if (nw <= 0) return;
-    count_bits_kernel<<<grid_for(nw, 256) < 1216 ? grid_for(nw, 256) : 1216, 256, 0, s>>>(words, nw, out);
 }
 
 void launch_clear_bits(uint32_t* words, int64_t a, int64_t b, cudaStream_t s) {
