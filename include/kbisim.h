@@ -204,7 +204,8 @@ kb_status kb_set_workspace(kb_context* ctx, void* device_ptr, size_t bytes);
  *   counts           HOST int64[k+1]; counts[i] = number of blocks at level i
  *   levels_computed  HOST, may be NULL; the last level actually refined (< k when
  *                    early_stop found a stable partition; rows after it are copies)
- * Synchronises the stream once per round to read the block count, and once
+ * Synchronises the stream once per round to read the block count (a graph of at
+ * most 2^21 vertices and processed edges: once per 64 rounds), and once
  * more at level 0 when it has keys (vertex labels or a starting partition): a
  * range check decides whether they all lie in [0, 8192), which takes a path
  * without the block table. */
@@ -357,7 +358,8 @@ kb_status kb_refine_host(kb_context* ctx, const kb_graph* g, const kb_options* o
 
 /* Per-round and per-kernel timing of the last refine call, in milliseconds,
  * measured with CUDA events on the context stream when enabled.
- *   kb_set_timing(ctx, 1) enables event recording (small overhead); 2 also
+ *   kb_set_timing(ctx, 1) enables event recording (small overhead; a small
+ *   graph's rounds then run as one kernel per pass instead of in one kernel); 2 also
  *   records the work of every round (kb_get_round_work; one extra pass over
  *   the row offsets per round); 0 disables both.
  *   round_ms[i] for i < n_rounds: device time of refinement round i+1.

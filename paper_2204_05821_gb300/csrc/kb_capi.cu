@@ -32,6 +32,7 @@ struct kb_context {
     kb::Counters* d_ctr = nullptr;
     kb::Counters* h_ctr = nullptr;  // pinned: the last counters read, and a slot per round in flight (queue_counters)
     cudaEvent_t slot_ev[4] = {};
+    int fused_ctas = 0;  // largest grid of the fused kernel (launch_fused_rounds)
     uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
     char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
     void* class_tmp = nullptr;    // degree-class bitmaps, tile counts and hub list during planning
@@ -344,6 +345,7 @@ kb_status device_error(kb_context* ctx) {
     if (e & kb::kErrInvalid)
         return fail(ctx, KB_ERR_INVALID_ARG, "row_offsets not monotone from 0 to m, or a neighbour id out of [0, n)");
     if (e & kb::kErrTableFull) return fail(ctx, KB_ERR_TABLE_FULL, "block table probe limit reached");
+    if (e & kb::kErrWait) return fail(ctx, KB_ERR_TIMEOUT, "a wait for the whole grid gave up");
     if (e & (kb::kErrStage | kb::kErrHubSet)) return fail(ctx, KB_ERR_DEVICE_CHECK, "device consistency check failed (%d)", e);
     return KB_OK;
 }
@@ -906,7 +908,7 @@ kb_status next_epoch(kb_context* ctx, Prepared& R, cudaStream_t s) {
 // The round word of the next round's empty-signature minima: smaller than any
 // before.
 kb_status next_empty_round(kb_context* ctx, Prepared& R, cudaStream_t s) {
-    if (*R.round >= 0xfffffff0u) {
+    if (*R.round >= 0xffffff00u) {
         KB_CUDA(ctx, cudaMemsetAsync(R.p.emin, 0xff, R.emin_bytes, s));
         *R.round = 0;
     }
@@ -1062,6 +1064,79 @@ struct RowCopyGuard {
     }
 };
 
+// Graphs up to this size (vertices and processed edges) take the fused kernel.
+// Its passes have fewer CTAs in flight (80 registers and the largest of all
+// passes' shared memory), so larger graphs lose by it what the launches cost.
+// Prepared power-law graphs, whole calls in us without it / with it:
+//   vertices + edges     2.3e5      9.3e5      1.9e6      3.7e6      7.5e6
+//   labelled, out      374/261    412/329    464/400    542/565    715/717
+//   kaushik, in        386/267    462/393    578/498    673/738    909/910
+//   schaetzle, out     350/232    459/382    627/555    674/741    946/950
+constexpr int64_t kFusedSize = (int64_t)1 << 21;
+
+// Rounds i_start + 1 .. k after the starting level is queued, kb::kFusedRounds at
+// a time.  all_on: no freeze pass ran yet.
+kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int i_start, int k, bool stop, bool all_on,
+                       int64_t* counts, int* levels_computed, int64_t* last_count, bool* stopped_stable) {
+    cudaStream_t s = ctx->stream;
+    kb::FusedRounds a;
+    a.p = R.p;
+    a.p.prev = reinterpret_cast<const int32_t*>(R.p.minof);  // blocks by name
+    a.p.frozen = R.frozen;
+    a.p.moved = R.moved;
+    a.f = freeze_pass(ctx, R);
+    a.rank = R.prefix;
+    a.sums = ctx->d_dense;  // the starting level is through with it
+    a.levels = rows.levels;
+    a.ping[0] = rows.ping[0];
+    a.ping[1] = rows.ping[1];
+    a.total_chunks = R.total_chunks;
+    a.k = k;
+    a.stop_stable = stop;
+    if (R.p.n_hubs) {
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_sets, 0xff, R.set_bytes, s));
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_acc, 0, sizeof(uint64_t) * (size_t)R.p.n_hubs, s));
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_cnt, 0, sizeof(uint32_t) * (size_t)R.p.n_hubs, s));
+    }
+    if (all_on) KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
+    bool stable = false;
+    for (int first = i_start + 1; first <= k && !stable;) {
+        // every round takes an epoch of the table and a round word of the minima
+        KB_TRY(next_epoch(ctx, R, s));
+        KB_TRY(next_empty_round(ctx, R, s));
+        a.first = first;
+        a.last = std::min({k, first + kb::kFusedRounds - 1, first + (int)(255u - *R.epoch)});
+        a.p.epoch = R.p.epoch;
+        a.p.ehigh = R.p.ehigh;
+        a.all_on = all_on && first == i_start + 1;
+        *R.epoch += (uint32_t)(a.last - first);
+        *R.round += (uint32_t)(a.last - first);
+        KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, s));
+        KB_TRY(read_counters(ctx));
+        KB_TRY(device_error(ctx));
+        const Counters& hc = *ctx->h_ctr;
+        if (hc.last_round < first || hc.last_round > a.last)
+            return fail(ctx, KB_ERR_DEVICE_CHECK, "the fused rounds ended at %d of %d..%d", hc.last_round, first, a.last);
+        if (counts && first == i_start + 1) counts[i_start] = hc.start_count;
+        for (int i = first; i <= hc.last_round; ++i) {
+            ctx->round_ms.push_back(0.f);
+            if (counts) counts[i] = hc.round_count[i - first];
+        }
+        if (last_count) *last_count = hc.count;
+        if (levels_computed) *levels_computed = hc.last_round;
+        stable = stop && hc.count == hc.prev_count;
+        if (stable && counts)
+            for (int i = hc.last_round + 1; i <= k; ++i) counts[i] = hc.count;
+        first = hc.last_round + 1;
+    }
+    if (stable && stopped_stable) *stopped_stable = true;
+    if (rows.host) {
+        KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
+        KB_TRY(emit_rows(ctx, rows, i_start + 1, k));
+    }
+    return KB_OK;
+}
+
 // The refinement driver shared by kb_refine, kb_refine_from and
 // kb_refine_fixpoint.  counts (k+1 entries) may be NULL in fixpoint mode;
 // *last_count receives the block count of the last level computed and
@@ -1103,6 +1178,10 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_CUDA(ctx, cudaGetLastError());
     }
 
+    // Small graphs run all their rounds in one kernel.
+    const bool fused = p.minof && ctx->fused_ctas > 0 && !ctx->timing && !ctx->work && !R.P.sketch && k > i_start &&
+                       R.P.m_proc + n <= kFusedSize;
+
     // ---- the starting level
     int32_t* row0 = rows.row(i_start);
     int64_t prev_count = 1;
@@ -1113,7 +1192,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         // At most kDenseLabels blocks after the small-label path: how many are
         // frozen decides nothing about the first round, and the count comes
         // back with that round's.
-        count_known = !(dense && R.P.freeze && !ctx->work && k > i_start);
+        count_known = !((dense || fused) && R.P.freeze && !ctx->work && k > i_start);
         if (count_known) {
             KB_TRY(read_counters(ctx));
             KB_TRY(device_error(ctx));
@@ -1138,6 +1217,10 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     if (last_count) *last_count = prev_count;
     if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
     KB_TRY(emit_rows(ctx, rows, i_start, i_start));
+
+    if (fused)
+        return fused_rounds(ctx, R, rows, i_start, k, opt->early_stop || fixpoint, !init_key, counts, levels_computed,
+                            last_count, stopped_stable);
 
     // ---- refinement rounds
     R.counters_clear = !R.P.subject;
@@ -2228,6 +2311,7 @@ kb_status kb_create(kb_context** out, int device, void* stream) {
     for (auto& e : ctx->ev) cudaEventCreate(&e);
     for (auto& e : ctx->slot_ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     kb::set_medium_kernel_attributes();
+    ctx->fused_ctas = kb::fused_max_ctas();
     cudaGetLastError();
     *out = ctx;
     return KB_OK;

@@ -78,7 +78,7 @@ __device__ __forceinline__ bool vertex_level0(const RoundParams& p, int64_t v) {
 
 // In a frozen block (RoundParams::frozen): it keeps its previous block.
 __device__ __forceinline__ bool vertex_frozen(const RoundParams& p, int64_t v) {
-    return p.frozen && ((__ldg(p.frozen + (v >> 5)) >> (v & 31)) & 1u);
+    return p.frozen && ((load_level(p.frozen + (v >> 5)) >> (v & 31)) & 1u);
 }
 
 // Active and refining by signature (not in level-0 mode, not frozen).

@@ -39,7 +39,10 @@ constexpr int kDefaultWarpVerts = 128;
 constexpr uint64_t kEmptyPair = ~0ull;  // block field 0x7fffffff never occurs (n <= 2^31-2)
 
 // bits of Counters::err
-enum : int32_t { kErrTableFull = 1, kErrInvalid = 2, kErrStage = 4, kErrHubSet = 8 };
+enum : int32_t { kErrTableFull = 1, kErrInvalid = 2, kErrStage = 4, kErrHubSet = 8, kErrWait = 16 };
+
+// Rounds that one launch of the fused kernel runs at most.
+constexpr int kFusedRounds = 64;
 
 struct Counters {
     int32_t err;
@@ -56,6 +59,13 @@ struct Counters {
     int64_t keyed_e[3];
     int32_t dense_bad;  // a level-0 key outside [0, kDenseLabels) (launch_dense_labels)
     int64_t prev_count; // blocks at the level before
+    // the fused rounds of small graphs (launch_fused_rounds): arrivals at the
+    // grid's barrier, the last round run, the count before its first round and
+    // after each one
+    uint32_t arrived;
+    int32_t last_round;
+    int64_t start_count;
+    int64_t round_count[kFusedRounds];
     uint32_t most_pairs;    // most distinct pairs of a vertex of the medium CTA kernel this round
     uint32_t exact_chunks;  // chunks of hubs that need their exact set (launch_hub_sketch)
     int64_t n_class[3]; // mid and medium vertices and hubs of the graph (launch_classes)
@@ -188,9 +198,22 @@ __host__ __device__ __forceinline__ const int32_t* gather_base(const RoundParams
     return p.perm ? p.gat : p.prev;
 }
 
+// Loads of what a kernel only reads: the previous level and the frozen bits.
+// The fused kernel of small graphs writes them between its phases, so its
+// translation unit (kb_fused.cu) asks for ordinary loads instead of the
+// read-only path; device code is compiled per translation unit.
+template <class T>
+__device__ __forceinline__ T load_level(const T* x) {
+#ifdef KB_LEVELS_WRITTEN
+    return *x;
+#else
+    return __ldg(x);
+#endif
+}
+
 // The previous block of neighbour word w (bit 31: direction).
 __device__ __forceinline__ int32_t gather_block(const RoundParams& p, int32_t w) {
-    return __ldg(gather_base(p) + (w & 0x7fffffff));
+    return load_level(gather_base(p) + (w & 0x7fffffff));
 }
 
 // ---------------------------------------------------------------- hashing
@@ -320,6 +343,24 @@ struct GraphStop {
     const uint8_t* mode = nullptr;    // [G]
     const int64_t* prev_count = nullptr;
 };
+// Rounds first..last (at most kFusedRounds) of one small graph in one cooperative
+// launch (kb_fused.cu): p, f and the buffers as for the single passes, with the
+// starting level's freeze pass done (or all_on: every vertex refines).
+struct FusedRounds {
+    RoundParams p;          // epoch and ehigh of round `first`
+    FreezePass f;
+    uint2* rank = nullptr;
+    uint32_t* sums = nullptr;    // [CTAs] scratch of the rank scan
+    int32_t* levels = nullptr;   // row i at levels + i * n, or
+    int32_t* ping[2] = {nullptr, nullptr};  // in turn
+    int64_t total_chunks = 0;
+    int first = 0, last = 0, k = 0;  // k: the call's last level
+    bool stop_stable = false;    // stop at a round that keeps the count; its row and all up to k are copied
+    bool all_on = false;
+};
+// CTAs that a cooperative launch may have (0: not available).
+int fused_max_ctas();
+cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, cudaStream_t s);
 // Canonical renumbering: prefix of block minima, then ids.
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
 // The frozen, class_on and moved counters restart at 0; with frozen
