@@ -497,17 +497,20 @@ const char* kb_server_last_error(const kb_server* server);
  * unchanged until the request has been admitted (kb_server_poll reports 1, 2
  * or 3): they are copied to the device at admission, not at submission.
  * levels_out is HOST int32[(k+1)*n] or NULL: when given, the levels are
- * written there when the request finishes (no host copy inside the library;
- * keep it alive until kb_server_fetch).  Checked here: sizes, the ends of
+ * written there by the time the request finishes (no host copy inside the
+ * library; rows of 512 KB and more of a pinned buffer as they become final; keep
+ * it alive until kb_server_fetch).  Pinned arrays of a KB_DIR_OUT request are read
+ * in place, once.  Checked here: sizes, the ends of
  * row_offsets and the arena's capacity; every offset and neighbour id is
  * checked on the device at admission, where a malformed graph fails alone
- * (state 3) without reaching the shared arena.  ticket receives the request's
+ * (state 3) without joining the shared arena.  ticket receives the request's
  * id.  Thread-safe with respect to kb_server_step. */
 kb_status kb_server_submit(kb_server* server, const kb_graph* g, const kb_options* opt, int k, int32_t* levels_out,
                            int64_t* ticket);
 /* Admit what fits, then run one round for every in-flight request and retire
- * finished ones (their levels are copied to host memory).  running / waiting
- * (may be NULL) receive the request counts after the step. */
+ * finished ones (their levels are copied to host memory; the copies may still run
+ * when it returns with others running, and kb_server_poll, kb_server_fetch and
+ * kb_server_get_stats wait for them).  running / waiting (may be NULL) receive the request counts after the step. */
 kb_status kb_server_step(kb_server* server, int32_t* running, int32_t* waiting);
 /* state: 0 waiting, 1 running, 2 done (fetchable), 3 rejected at admission
  * (kb_server_fetch returns KB_ERR_INVALID_ARG and forgets it); KB_ERR_NOT_FOUND

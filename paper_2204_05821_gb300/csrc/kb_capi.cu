@@ -1734,6 +1734,9 @@ struct ServeRequest {
     int32_t* d_levels = nullptr;
     size_t level_bytes = 0;
     int32_t* out = nullptr;               // caller's host levels, or null: kept in `levels`
+    bool early_rows = false;              // rows go to `out` as soon as they are final (kEarlyRowBytes)
+    int rows_queued = 0;                  // rows whose copies to `out` are queued
+    bool draining = false;                // finished but for the copies of its levels (state 1)
     std::unique_ptr<int32_t[]> levels;    // host copy after completion (when out is null)
     std::vector<int64_t> counts;
     int32_t levels_computed = 0;
@@ -1741,10 +1744,34 @@ struct ServeRequest {
     std::string error;
 };
 
+// Device copy of a waiting request's host arrays (and room for its processed
+// CSR).  Two of them, so that the next request's copies run while one is
+// checked and placed.
+struct Stage {
+    void* buf = nullptr;
+    size_t bytes = 0;
+    size_t o_row = 0, o_col = 0, o_lab = 0, o_vlab = 0, o_csr = 0;
+    int64_t ticket = 0;           // whose arrays it holds (0: nobody's)
+    cudaEvent_t full = nullptr;   // copied
+    cudaEvent_t free = nullptr;   // placed: may be overwritten
+};
+
+// A finished request's level store, returned once the copies out of it are done.
+struct Draining {
+    int64_t ticket;
+    int32_t* d_levels;
+    size_t level_bytes;
+};
+
 struct Slot {
     int64_t ticket = -1;  // -1: dead
     int64_t vbase = 0, n = 0, ebase = 0, m = 0;
 };
+
+// Rows of at least this size go to a pinned host buffer one by one, as soon as
+// they are final, while the next rounds run (a copy costs the host about what
+// the link takes for 400 KB); smaller ones together when the request finishes.
+constexpr size_t kEarlyRowBytes = 512 << 10;
 
 double now_s() {
     return std::chrono::duration<double>(std::chrono::steady_clock::now().time_since_epoch()).count();
@@ -1781,6 +1808,7 @@ struct kb_server {
     // vertices are told (false after a compaction, which renames blocks and
     // clears the frozen ones)
     bool history = false;
+    int64_t frozen = 0;  // frozen vertices after the last step
     // per-slot device arrays (capacity max_requests + dead slots: sized by max_slots)
     int32_t max_slots = 0;
     int32_t* vgraph = nullptr;
@@ -1792,9 +1820,19 @@ struct kb_server {
     char* slot_up = nullptr;
     std::vector<char> slot_up_h;
     std::vector<uint32_t> gbase_host;
-    // staging for admission (raw graph, processed CSR for IN / BOTH)
-    void* stage = nullptr;
-    size_t stage_bytes = 0;
+    // staging for admission (raw graph, processed CSR for IN / BOTH), and the
+    // streams of the copies in and out: they overlap the rounds
+    Stage stage[2];
+    cudaStream_t up = nullptr, down = nullptr;
+    // Requests placed straight from pinned host arrays in this step and not yet
+    // known to be well formed: tickets in the order of their slots, which are the
+    // last ones, and a device word each (kb::launch_place_checked)
+    std::vector<int64_t> unchecked;
+    int32_t* verdict = nullptr;           // [max_requests]
+    int32_t* verdict_h = nullptr;         // pinned
+    bool host_access = false;             // kernels can read all host memory
+    std::vector<Draining> draining;
+    cudaEvent_t drained = nullptr;  // after the last copy out of a store in `draining`
     // round state
     Prepared R;
     bool dirty = true;
@@ -1833,20 +1871,156 @@ kb_status sfail(kb_server* sv, kb_status st, const char* fmt, ...) {
         }                                                                    \
     } while (0)
 
-// Copy request r's graph into the arena at the tail as slot `slot`.
-kb_status place_request(kb_server* sv, ServeRequest& r, int slot, bool* rejected) {
+// Whether the device reads [x, x + bytes) in place: pinned at both ends, on a
+// device that can read what may lie between them in any case.
+bool device_reads(const void* x, size_t bytes) {
+    if (!x || !bytes) return true;
+    for (const void* q : {x, (const void*)((const char*)x + bytes - 1)}) {
+        cudaPointerAttributes a{};
+        if (cudaPointerGetAttributes(&a, q) != cudaSuccess || a.type != cudaMemoryTypeHost || a.devicePointer != q) {
+            cudaGetLastError();
+            return false;
+        }
+    }
+    return true;
+}
+
+// Out-edge requests in pinned memory are read in place (launch_place_checked):
+// their verdicts come back for all of them at once.
+bool read_in_place(const kb_server* sv, const ServeRequest& r) {
+    return sv->host_access && r.n > 0 && !needs_in_csr(r.opt.direction) &&
+           device_reads(r.row, sizeof(int64_t) * (size_t)(r.n + 1)) && device_reads(r.col, sizeof(int32_t) * (size_t)r.m) &&
+           device_reads(r.lab, sizeof(int32_t) * (size_t)r.m) && device_reads(r.vlab, sizeof(int32_t) * (size_t)r.n);
+}
+
+// Append a slot for r's graph, which is placed at the arena's tail.
+void push_slot(kb_server* sv, ServeRequest& r) {
+    Slot sl;
+    sl.ticket = r.ticket;
+    sl.vbase = sv->n_used;
+    sl.n = r.n;
+    sl.ebase = sv->m_used;
+    sl.m = r.m_proc;
+    r.slot = (int)sv->slots.size();
+    sv->slots.push_back(sl);
+    sv->n_used += r.n;
+    sv->m_used += r.m_proc;
+}
+
+// Request r is in the arena and runs from the next round on (sv->mu held).
+void start_request(ServeRequest& r) {
+    r.state = 1;
+    r.round = 0;
+    r.rows_queued = 0;
+    cudaPointerAttributes attr{};
+    r.early_rows = sizeof(int32_t) * (size_t)r.n >= kEarlyRowBytes && r.out &&
+                   cudaPointerGetAttributes(&attr, r.out) == cudaSuccess && attr.type == cudaMemoryTypeHost;
+    cudaGetLastError();
+    r.counts.assign((size_t)r.k + 1, 0);
+    r.row = nullptr;  // the caller's graph arrays are no longer read
+    r.col = r.lab = r.vlab = nullptr;
+}
+
+// Request r is malformed (sv->mu held).
+void reject_request(kb_server* sv, ServeRequest& r) {
+    sv->level_pool[r.level_bytes].push_back(r.d_levels);
+    sv->level_bytes_in_use -= r.level_bytes;
+    r.d_levels = nullptr;
+    r.state = 3;
+    r.error = "row_offsets not monotone from 0 to m, or a neighbour id out of [0, n)";
+    r.row = nullptr;
+    ++sv->failed;
+}
+
+// Settle the unchecked requests.  A malformed one leaves the arena, and with it
+// those behind it, which wait again.
+kb_status check_placed(kb_server* sv, bool* changed) {
+    const size_t count = sv->unchecked.size();
+    if (!count) return KB_OK;
+    cudaStream_t s = sv->ctx->stream;
+    SV_CUDA(sv, cudaMemcpyAsync(sv->verdict_h, sv->verdict, sizeof(int32_t) * count, cudaMemcpyDeviceToHost, s));
+    SV_CUDA(sv, cudaStreamSynchronize(s));
+    std::lock_guard<std::mutex> lk(sv->mu);
+    size_t good = 0;
+    while (good < count && !sv->verdict_h[good]) ++good;
+    for (size_t i = 0; i < good; ++i) start_request(sv->reqs[sv->unchecked[i]]);
+    if (good) *changed = true;
+    if (good < count) {
+        const size_t slot = sv->slots.size() - (count - good);
+        sv->n_used = sv->slots[slot].vbase;
+        sv->m_used = sv->slots[slot].ebase;
+        sv->slots.resize(slot);
+    }
+    for (size_t i = count; i-- > good;) {
+        ServeRequest& r = sv->reqs[sv->unchecked[i]];
+        r.slot = -1;
+        if (sv->verdict_h[i]) {
+            reject_request(sv, r);
+        } else {
+            sv->level_pool[r.level_bytes].push_back(r.d_levels);
+            sv->level_bytes_in_use -= r.level_bytes;
+            r.d_levels = nullptr;
+            sv->waiting.push_front(r.ticket);
+        }
+    }
+    sv->unchecked.clear();
+    return KB_OK;
+}
+
+// Queue the copies of a waiting request's arrays into S.
+kb_status stage_request(kb_server* sv, const ServeRequest& r, Stage& S) {
+    const int64_t n = r.n, m = r.m;
+    size_t off = 0;
+    auto take = [&](size_t b) { size_t o = off; off += align_up(b); return o; };
+    S.ticket = 0;
+    S.o_row = take(sizeof(int64_t) * (size_t)(n + 1));
+    S.o_col = take(sizeof(int32_t) * (size_t)m);
+    S.o_lab = take(sizeof(int32_t) * (size_t)m);
+    S.o_vlab = take(sizeof(int32_t) * (size_t)n);
+    Plan P;
+    P.n = n;
+    P.m = m;
+    P.dir = r.opt.direction;
+    P.m_proc = r.m_proc;
+    P.labels = r.lab != nullptr;
+    layout_csr(P);
+    S.o_csr = take(P.csr_bytes);
+    if (off > S.bytes) {
+        if (S.buf) cudaFree(S.buf);
+        S.buf = nullptr;
+        S.bytes = 0;
+        if (cudaMalloc(&S.buf, off) != cudaSuccess) {
+            cudaGetLastError();
+            return sfail(sv, KB_ERR_OOM, "cannot allocate %zu bytes of staging", off);
+        }
+        S.bytes = off;
+    }
+    char* b = reinterpret_cast<char*>(S.buf);
+    SV_CUDA(sv, cudaStreamWaitEvent(sv->up, S.free, 0));
+    SV_CUDA(sv, cudaMemcpyAsync(b + S.o_row, r.row, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice, sv->up));
+    if (m)
+        SV_CUDA(sv, cudaMemcpyAsync(b + S.o_col, r.col, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, sv->up));
+    if (m && P.labels)
+        SV_CUDA(sv, cudaMemcpyAsync(b + S.o_lab, r.lab, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, sv->up));
+    if (r.vlab)
+        SV_CUDA(sv, cudaMemcpyAsync(b + S.o_vlab, r.vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, sv->up));
+    SV_CUDA(sv, cudaEventRecord(S.full, sv->up));
+    S.ticket = r.ticket;
+    return KB_OK;
+}
+
+// Copy request r's graph into the arena at the tail, as a new slot.  next: the
+// request that is likely to follow (or null), whose arrays are copied meanwhile.
+kb_status place_request(kb_server* sv, ServeRequest& r, const ServeRequest* next, bool* rejected) {
     *rejected = false;
     kb_context* ctx = sv->ctx;
     cudaStream_t s = ctx->stream;
     Arena& A = sv->arena[sv->cur];
     const int64_t n = r.n, m = r.m, mp = r.m_proc;
-    // staging: raw CSR (+ processed CSR for IN / BOTH)
-    size_t off = 0;
-    auto take = [&](size_t b) { size_t o = off; off += align_up(b); return o; };
-    const size_t o_row = take(sizeof(int64_t) * (size_t)(n + 1));
-    const size_t o_col = take(sizeof(int32_t) * (size_t)m);
-    const size_t o_lab = take(sizeof(int32_t) * (size_t)m);
-    const size_t o_vlab = take(sizeof(int32_t) * (size_t)n);
+    const int at = sv->stage[1].ticket == r.ticket ? 1 : 0;
+    Stage& S = sv->stage[at];
+    if (S.ticket != r.ticket) SV_TRY(sv, stage_request(sv, r, S));
+    S.ticket = 0;
     Plan P;
     P.n = n;
     P.m = m;
@@ -1854,23 +2028,9 @@ kb_status place_request(kb_server* sv, ServeRequest& r, int slot, bool* rejected
     P.m_proc = mp;
     P.labels = r.lab != nullptr;
     layout_csr(P);
-    const size_t o_csr = take(P.csr_bytes);
-    if (off > sv->stage_bytes) {
-        if (sv->stage) cudaFree(sv->stage);
-        sv->stage = nullptr;
-        sv->stage_bytes = 0;
-        if (cudaMalloc(&sv->stage, off) != cudaSuccess) {
-            cudaGetLastError();
-            return sfail(sv, KB_ERR_OOM, "cannot allocate %zu bytes of staging", off);
-        }
-        sv->stage_bytes = off;
-    }
-    char* b = reinterpret_cast<char*>(sv->stage);
-    SV_CUDA(sv, cudaMemcpyAsync(b + o_row, r.row, sizeof(int64_t) * (size_t)(n + 1), cudaMemcpyHostToDevice, s));
-    if (m) SV_CUDA(sv, cudaMemcpyAsync(b + o_col, r.col, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, s));
-    if (m && P.labels)
-        SV_CUDA(sv, cudaMemcpyAsync(b + o_lab, r.lab, sizeof(int32_t) * (size_t)m, cudaMemcpyHostToDevice, s));
-    if (r.vlab) SV_CUDA(sv, cudaMemcpyAsync(b + o_vlab, r.vlab, sizeof(int32_t) * (size_t)n, cudaMemcpyHostToDevice, s));
+    const size_t o_row = S.o_row, o_col = S.o_col, o_lab = S.o_lab, o_vlab = S.o_vlab, o_csr = S.o_csr;
+    char* b = reinterpret_cast<char*>(S.buf);
+    SV_CUDA(sv, cudaStreamWaitEvent(s, S.full, 0));
     // the arena is shared: a malformed CSR is checked on the device before it
     // is placed, and the request fails alone
     SV_CUDA(sv, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
@@ -1878,10 +2038,13 @@ kb_status place_request(kb_server* sv, ServeRequest& r, int slot, bool* rejected
                         ctx->d_ctr, s);
     SV_CUDA(sv, cudaGetLastError());
     SV_CUDA(sv, cudaMemcpyAsync(ctx->h_ctr, ctx->d_ctr, sizeof(Counters), cudaMemcpyDeviceToHost, s));
+    if (next && stage_request(sv, *next, sv->stage[1 - at]) != KB_OK) {
+        sv->last_error.clear();  // staged when its turn comes
+        cudaGetLastError();
+    }
     SV_CUDA(sv, cudaStreamSynchronize(s));
     if (ctx->h_ctr->err & kb::kErrInvalid) {
         *rejected = true;
-        r.error = "row_offsets not monotone from 0 to m, or a neighbour id out of [0, n)";
         return KB_OK;
     }
     kb::PlaceArgs a{};
@@ -1909,17 +2072,8 @@ kb_status place_request(kb_server* sv, ServeRequest& r, int slot, bool* rejected
     a.dst_ebase = sv->m_used;
     kb::launch_place(a, s);
     SV_CUDA(sv, cudaGetLastError());
-    Slot sl;
-    sl.ticket = r.ticket;
-    sl.vbase = sv->n_used;
-    sl.n = n;
-    sl.ebase = sv->m_used;
-    sl.m = mp;
-    if ((int)sv->slots.size() != slot) return sfail(sv, KB_ERR_DEVICE_CHECK, "slot order broken");
-    sv->slots.push_back(sl);
-    sv->n_used += n;
-    sv->m_used += mp;
-    r.slot = slot;
+    SV_CUDA(sv, cudaEventRecord(S.free, s));
+    push_slot(sv, r);
     return KB_OK;
 }
 
@@ -1988,110 +2142,193 @@ size_t level_store_bytes(size_t bytes) {
     return b;
 }
 
+// A finished request whose levels have reached the host (sv->mu held).
+void publish(kb_server* sv, ServeRequest& r) {
+    r.draining = false;
+    r.t_done = now_s();
+    r.state = 2;
+    ++sv->completed;
+    sv->latencies_ms.push_back(1000.0 * (r.t_done - r.t_submit));
+    sv->edge_rounds += (double)r.m_proc * (double)r.levels_computed;
+}
+
+// Return the level stores whose copies are done; wait: all of them.
+kb_status release_drained(kb_server* sv, bool wait) {
+    if (sv->draining.empty()) return KB_OK;
+    if (wait) {
+        SV_CUDA(sv, cudaEventSynchronize(sv->drained));
+    } else {
+        const cudaError_t e = cudaEventQuery(sv->drained);
+        if (e == cudaErrorNotReady) return KB_OK;
+        SV_CUDA(sv, e);
+    }
+    std::lock_guard<std::mutex> lk(sv->mu);
+    for (const Draining& d : sv->draining) {
+        sv->level_pool[d.level_bytes].push_back(d.d_levels);
+        sv->level_bytes_in_use -= d.level_bytes;
+        auto it = sv->reqs.find(d.ticket);
+        if (it != sv->reqs.end() && it->second.draining) publish(sv, it->second);
+    }
+    sv->draining.clear();
+    return KB_OK;
+}
+
 // Admit waiting requests in arrival order while they fit.
 kb_status admit(kb_server* sv, bool* changed) {
-    std::vector<int64_t> admitted;
     while (true) {
-        int64_t t;
+        int64_t t = 0;
+        const ServeRequest* next = nullptr;
         {
             std::lock_guard<std::mutex> lk(sv->mu);
-            if (sv->waiting.empty()) break;
-            t = sv->waiting.front();
+            if (!sv->waiting.empty()) t = sv->waiting.front();
+            if (sv->waiting.size() > 1) next = &sv->reqs[sv->waiting[1]];
         }
+        if (!t) {
+            if (sv->unchecked.empty()) break;
+            SV_TRY(sv, check_placed(sv, changed));  // may leave requests waiting again
+            continue;
+        }
+        SV_TRY(sv, release_drained(sv, true));  // their stores may be needed
         ServeRequest& r = sv->reqs[t];
         int live = 0;
         for (const Slot& sl : sv->slots) live += sl.ticket >= 0;
-        if (live >= sv->cfg.max_requests) break;
         const size_t lb = level_store_bytes(sizeof(int32_t) * (size_t)r.n * (size_t)(r.k + 1));
         std::vector<int32_t*>& pooled = sv->level_pool[lb];
         const size_t budget = sv->cfg.memory_budget;
-        if (budget) {
-            if (sv->level_bytes_in_use + lb > budget) break;
-        } else if (pooled.empty()) {
-            const size_t fr = free_device_bytes();
-            if (fr < lb + ((size_t)1 << 30)) break;
+        bool fits = live < sv->cfg.max_requests;
+        if (fits && budget) {
+            fits = sv->level_bytes_in_use + lb <= budget;
+        } else if (fits && pooled.empty()) {
+            fits = free_device_bytes() >= lb + ((size_t)1 << 30);
         }
-        const bool fits_tail = sv->n_used + r.n <= sv->cfg.max_vertices && sv->m_used + r.m_proc <= sv->cfg.max_edges &&
-                               (int)sv->slots.size() < sv->max_slots;
-        if (!fits_tail) {
+        bool pack = false;
+        if (fits && !(sv->n_used + r.n <= sv->cfg.max_vertices && sv->m_used + r.m_proc <= sv->cfg.max_edges &&
+                      (int)sv->slots.size() < sv->max_slots)) {
             int64_t ln = 0, lm = 0;
             for (const Slot& sl : sv->slots)
                 if (sl.ticket >= 0) {
                     ln += sl.n;
                     lm += sl.m;
                 }
-            if (ln + r.n > sv->cfg.max_vertices || lm + r.m_proc > sv->cfg.max_edges) break;
-            SV_TRY(sv, compact(sv));
+            fits = ln + r.n <= sv->cfg.max_vertices && lm + r.m_proc <= sv->cfg.max_edges;
+            pack = fits;
         }
+        const bool direct = fits && !pack && read_in_place(sv, r);
+        if (!direct && !sv->unchecked.empty()) {
+            // (a malformed one among them may make room)
+            SV_TRY(sv, check_placed(sv, changed));
+            continue;
+        }
+        if (!fits) break;
+        if (pack) SV_TRY(sv, compact(sv));
         if (!pooled.empty()) {
             r.d_levels = pooled.back();
             pooled.pop_back();
         } else if (cudaMalloc(&r.d_levels, lb) != cudaSuccess) {
             cudaGetLastError();
             r.d_levels = nullptr;
-            break;
+            if (sv->unchecked.empty()) break;
+            SV_TRY(sv, check_placed(sv, changed));
+            continue;
         }
         r.level_bytes = lb;
         sv->level_bytes_in_use += lb;
+        if (direct) {
+            cudaStream_t s = sv->ctx->stream;
+            if (sv->unchecked.empty())
+                SV_CUDA(sv, cudaMemsetAsync(sv->verdict, 0, sizeof(int32_t) * (size_t)sv->cfg.max_requests, s));
+            Arena& A = sv->arena[sv->cur];
+            kb::PlaceArgs a{};
+            a.srow = r.row;
+            a.scol = r.col;
+            a.slab = r.lab;
+            a.svlab = r.vlab;
+            a.drow = A.row;
+            a.dcol = A.col;
+            a.dlab = A.lab;
+            a.dvlab = A.vlab;
+            a.n = r.n;
+            a.m = r.m;
+            a.dst_vbase = sv->n_used;
+            a.dst_ebase = sv->m_used;
+            kb::launch_place_checked(a, sv->verdict + sv->unchecked.size(), s);
+            SV_CUDA(sv, cudaGetLastError());
+            push_slot(sv, r);
+            sv->unchecked.push_back(t);
+            std::lock_guard<std::mutex> lk(sv->mu);
+            sv->waiting.pop_front();
+            continue;
+        }
+        // the next one's copies start already if it fits behind this one
+        if (next && (live + 2 > sv->cfg.max_requests || (int)sv->slots.size() + 2 > sv->max_slots ||
+                     sv->n_used + r.n + next->n > sv->cfg.max_vertices ||
+                     sv->m_used + r.m_proc + next->m_proc > sv->cfg.max_edges || read_in_place(sv, *next)))
+            next = nullptr;
         bool rejected = false;
-        SV_TRY(sv, place_request(sv, r, (int)sv->slots.size(), &rejected));
+        SV_TRY(sv, place_request(sv, r, next, &rejected));
         std::lock_guard<std::mutex> lk(sv->mu);
         sv->waiting.pop_front();
         if (rejected) {
-            sv->level_pool[lb].push_back(r.d_levels);
-            sv->level_bytes_in_use -= lb;
-            r.d_levels = nullptr;
-            r.state = 3;
-            r.row = nullptr;
-            ++sv->failed;
-            continue;
+            reject_request(sv, r);
+        } else {
+            start_request(r);
+            *changed = true;
         }
-        r.state = 1;
-        r.round = 0;
-        r.counts.assign((size_t)r.k + 1, 0);
-        r.row = nullptr;  // the caller's graph arrays are no longer read
-        r.col = r.lab = r.vlab = nullptr;
-        *changed = true;
     }
+    // one that did not follow after all is copied again when it is admitted
+    for (Stage& S : sv->stage)
+        if (S.ticket) {
+            SV_CUDA(sv, cudaEventSynchronize(S.full));
+            S.ticket = 0;
+        }
     return KB_OK;
 }
 
-// Finish request r after its last round, in two parts so that every request
-// retiring in a step shares one synchronisation: retire_copy queues the copy
-// of its levels to the host (the caller's buffer given at submission, else a
-// buffer of its own; rows after the last refined level repeat it), and
-// retire_finish, after the stream has drained, releases its level store.
-kb_status retire_copy(kb_server* sv, ServeRequest& r, int last) {
-    cudaStream_t s = sv->ctx->stream;
-    const size_t n = (size_t)r.n;
-    if (!r.out) {
+// Queue the copies of request r's rows up to `last`, which is final, to its host
+// levels (the caller's buffer given at submission, else a buffer of its own).
+kb_status copy_rows_out(kb_server* sv, ServeRequest& r, int last) {
+    const size_t n = (size_t)r.n, q = (size_t)r.rows_queued;
+    if (!r.out && !r.levels) {
         r.levels.reset(new (std::nothrow) int32_t[std::max<size_t>(n * (size_t)(r.k + 1), 1)]);
         if (!r.levels) return sfail(sv, KB_ERR_OOM, "cannot allocate host memory for the levels");
     }
     int32_t* dst = r.out ? r.out : r.levels.get();
-    if (n) {
-        SV_CUDA(sv, cudaMemcpyAsync(dst, r.d_levels, sizeof(int32_t) * n * (size_t)(last + 1), cudaMemcpyDeviceToHost, s));
-        for (int j = last + 1; j <= r.k; ++j)
-            SV_CUDA(sv, cudaMemcpyAsync(dst + (size_t)j * n, r.d_levels + (size_t)last * n, sizeof(int32_t) * n,
-                                        cudaMemcpyDeviceToHost, s));
-    }
+    if (n && r.rows_queued <= last)
+        SV_CUDA(sv, cudaMemcpyAsync(dst + q * n, r.d_levels + q * n, sizeof(int32_t) * n * ((size_t)last + 1 - q),
+                                    cudaMemcpyDeviceToHost, sv->down));
+    r.rows_queued = last + 1;
     return KB_OK;
 }
 
-void retire_finish(kb_server* sv, ServeRequest& r, int last) {
+// Finish request r after its last round: its slot is free, and its levels and
+// level store follow when the copies are done (publish, release_drained).  Rows
+// after the last refined level repeat it.
+kb_status retire(kb_server* sv, ServeRequest& r, int last) {
+    const size_t n = (size_t)r.n;
+    SV_TRY(sv, copy_rows_out(sv, r, last));
+    int32_t* dst = r.out ? r.out : r.levels.get();
+    for (int j = last + 1; n && j <= r.k; ++j)
+        SV_CUDA(sv, cudaMemcpyAsync(dst + (size_t)j * n, r.d_levels + (size_t)last * n, sizeof(int32_t) * n,
+                                    cudaMemcpyDeviceToHost, sv->down));
+    SV_CUDA(sv, cudaEventRecord(sv->drained, sv->down));
+    std::lock_guard<std::mutex> lk(sv->mu);
     for (int j = last + 1; j <= r.k; ++j) r.counts[(size_t)j] = r.counts[(size_t)last];
     r.levels_computed = last;
-    sv->level_pool[r.level_bytes].push_back(r.d_levels);
+    r.draining = true;
+    sv->draining.push_back({r.ticket, r.d_levels, r.level_bytes});
     r.d_levels = nullptr;
-    sv->level_bytes_in_use -= r.level_bytes;
     sv->slots[(size_t)r.slot].ticket = -1;
     r.slot = -1;
-    r.t_done = now_s();
-    std::lock_guard<std::mutex> lk(sv->mu);
-    r.state = 2;
-    ++sv->completed;
-    sv->latencies_ms.push_back(1000.0 * (r.t_done - r.t_submit));
-    sv->edge_rounds += (double)r.m_proc * (double)last;
+    return KB_OK;
+}
+
+// The caller asks for a request: one that has finished waits for the copies of
+// its levels (sv->mu held).
+kb_status settle(kb_server* sv, ServeRequest& r) {
+    if (!r.draining) return KB_OK;
+    SV_CUDA(sv, cudaEventSynchronize(sv->drained));
+    publish(sv, r);
+    return KB_OK;
 }
 
 kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
@@ -2194,7 +2431,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         p.frozen = sv->R.frozen;
         p.frozen_min = sv->R.frozen_min;
         p.moved = sv->history ? sv->R.moved : nullptr;
-        sv->R.compact = sv->history;  // retired graphs' vertices are frozen
+        sv->R.compact = sv->history && sv->frozen * 4 > sv->n_used;  // (retired graphs' vertices are frozen)
         SV_TRY(sv, launch_round_body(ctx, sv->R, s, nullptr));
         kb::GraphStop stop;
         stop.active = gactive;
@@ -2218,8 +2455,11 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
             SV_TRY(sv, device_error(ctx));
         }
         for (int c = 0; c < 3; ++c) sv->R.class_on[c] = ctx->h_ctr->class_on[c] > 0;
-        // bookkeeping and retirement (one synchronisation for all copies)
-        std::vector<std::pair<ServeRequest*, int>> finished;
+        sv->frozen = ctx->h_ctr->frozen;
+        // bookkeeping and retirement.  The copies out run on a stream of their
+        // own while the other requests refine: those of finished requests first,
+        // then the new rows of large ones.
+        SV_TRY(sv, release_drained(sv, false));
         for (int j = 0; j < G; ++j) {
             const Slot sl = sv->slots[(size_t)j];
             if (sl.ticket < 0) continue;
@@ -2230,20 +2470,19 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
             bool done = done_round >= r.k;
             if (done_round > 0 && r.opt.early_stop && cnt == r.counts[(size_t)done_round - 1]) done = true;
             ++r.round;
-            if (done) {
-                SV_TRY(sv, retire_copy(sv, r, done_round));
-                finished.push_back({&r, done_round});
-            }
+            if (done) SV_TRY(sv, retire(sv, r, done_round));
         }
-        if (!finished.empty()) {
-            SV_CUDA(sv, cudaStreamSynchronize(s));
-            for (auto& f : finished) retire_finish(sv, *f.first, f.second);
+        for (int j = 0; j < G; ++j) {
+            if (sv->slots[(size_t)j].ticket < 0) continue;
+            ServeRequest& r = sv->reqs[sv->slots[(size_t)j].ticket];
+            if (r.early_rows) SV_TRY(sv, copy_rows_out(sv, r, r.round - 1));
         }
         ++sv->steps;
     }
-    std::lock_guard<std::mutex> lk(sv->mu);
     int run = 0;
     for (const Slot& sl : sv->slots) run += sl.ticket >= 0;
+    if (run == 0) SV_TRY(sv, release_drained(sv, true));
+    std::lock_guard<std::mutex> lk(sv->mu);
     if (running) *running = run;
     if (waiting_out) *waiting_out = (int32_t)sv->waiting.size();
     return KB_OK;
@@ -2765,6 +3004,10 @@ kb_status kb_server_create(kb_server** out, int device, void* stream, const kb_s
     alloc((void**)&sv->emin, sizeof(uint64_t) * (size_t)N);
     const size_t bwN = sizeof(uint32_t) * (size_t)((N >> 5) + 1);
     for (int f = 0; f < 5; ++f) alloc((void**)&sv->frz[f], bwN);
+    alloc((void**)&sv->verdict, sizeof(int32_t) * (size_t)cfg->max_requests);
+    if (ok && cudaMallocHost(&sv->verdict_h, sizeof(int32_t) * (size_t)cfg->max_requests) != cudaSuccess) ok = false;
+    int access = 0;
+    if (cudaDeviceGetAttribute(&access, cudaDevAttrPageableMemoryAccess, device) == cudaSuccess) sv->host_access = access != 0;
     if (ok) {
         ok = cudaMemset(sv->arena[0].row, 0, sizeof(int64_t)) == cudaSuccess &&
              cudaMemset(sv->arena[1].row, 0, sizeof(int64_t)) == cudaSuccess &&
@@ -2773,7 +3016,14 @@ kb_status kb_server_create(kb_server** out, int device, void* stream, const kb_s
              cudaMemset(sv->frz[0], 0, bwN) == cudaSuccess && cudaMemset(sv->frz[1], 0, bwN) == cudaSuccess &&
              cudaMemset(sv->frz[2], 0, bwN) == cudaSuccess;
     }
+    ok = ok && cudaStreamCreateWithFlags(&sv->up, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaStreamCreateWithFlags(&sv->down, cudaStreamNonBlocking) == cudaSuccess &&
+         cudaEventCreateWithFlags(&sv->drained, cudaEventDisableTiming) == cudaSuccess;
+    for (Stage& S : sv->stage)
+        ok = ok && cudaEventCreateWithFlags(&S.full, cudaEventDisableTiming) == cudaSuccess &&
+             cudaEventCreateWithFlags(&S.free, cudaEventDisableTiming) == cudaSuccess;
     if (!ok) {
+        cudaGetLastError();
         kb_server_destroy(sv);
         return KB_ERR_OOM;
     }
@@ -2787,6 +3037,16 @@ kb_status kb_server_destroy(kb_server* sv) {
         cudaSetDevice(sv->ctx->device);
         if (sv->ctx->stream) cudaStreamSynchronize(sv->ctx->stream); else cudaDeviceSynchronize();
     }
+    // copies to and from the callers' arrays
+    for (cudaStream_t c : {sv->up, sv->down})
+        if (c) {
+            cudaStreamSynchronize(c);
+            cudaStreamDestroy(c);
+        }
+    if (sv->drained) cudaEventDestroy(sv->drained);
+    cudaFree(sv->verdict);
+    if (sv->verdict_h) cudaFreeHost(sv->verdict_h);
+    for (const Draining& d : sv->draining) cudaFree(d.d_levels);
     for (auto& kv : sv->reqs)
         if (kv.second.d_levels) cudaFree(kv.second.d_levels);
     for (auto& kv : sv->level_pool)
@@ -2806,7 +3066,11 @@ kb_status kb_server_destroy(kb_server* sv) {
     cudaFree(sv->voff);
     cudaFree(sv->bases);
     cudaFree(sv->slot_up);
-    cudaFree(sv->stage);
+    for (Stage& S : sv->stage) {
+        cudaFree(S.buf);
+        if (S.full) cudaEventDestroy(S.full);
+        if (S.free) cudaEventDestroy(S.free);
+    }
     kb_destroy(sv->ctx);
     delete sv;
     return KB_OK;
@@ -2867,6 +3131,7 @@ kb_status kb_server_poll(kb_server* sv, int64_t ticket, int32_t* state) {
     std::lock_guard<std::mutex> lk(sv->mu);
     auto it = sv->reqs.find(ticket);
     if (it == sv->reqs.end()) return KB_ERR_NOT_FOUND;
+    KB_TRY(settle(sv, it->second));
     *state = it->second.state;
     return KB_OK;
 }
@@ -2877,6 +3142,7 @@ kb_status kb_server_fetch(kb_server* sv, int64_t ticket, int32_t* levels, int64_
     auto it = sv->reqs.find(ticket);
     if (it == sv->reqs.end()) return KB_ERR_NOT_FOUND;
     ServeRequest& r = it->second;
+    KB_TRY(settle(sv, r));
     if (r.state == 3) {
         const std::string why = r.error;
         sv->reqs.erase(it);
@@ -2901,6 +3167,7 @@ kb_status kb_server_fetch(kb_server* sv, int64_t ticket, int32_t* levels, int64_
 kb_status kb_server_get_stats(kb_server* sv, kb_server_stats* st) {
     if (!sv || !st) return KB_ERR_INVALID_ARG;
     std::lock_guard<std::mutex> lk(sv->mu);
+    for (auto& kv : sv->reqs) KB_TRY(settle(sv, kv.second));
     std::memset(st, 0, sizeof(*st));
     st->submitted = sv->submitted;
     st->completed = sv->completed;

@@ -11,8 +11,8 @@
 //
 // What bounds it: the chain of dependent loads in each phase and some 2 us per
 // barrier, five to seven a round.  Whole calls, one launch per pass against this
-// kernel: 10^4 vertices and 3 x 10^4 edges, 6 rounds: 248 -> 183 us; a graph of
-// 5 x 10^4 edges with host buffers: 525 -> 450 us; 3 x 10^5 vertices to their
+// kernel: 10^4 vertices and 5 x 10^4 edges: 248 -> 183 us; a graph of
+// 7 x 10^5 edges with host buffers: 525 -> 450 us; 3 x 10^5 vertices to their
 // fixpoint in 11 rounds: 1066 -> 847 us.  Three CTAs per SM (a CTA per 256
 // vertices) as the occupancy allows: the last took 885 us with two and 1209 us
 // with one.

@@ -493,4 +493,7 @@ struct PlaceArgs {
     int64_t src_vbase, dst_vbase, src_ebase, dst_ebase;
 };
 void launch_place(const PlaceArgs& a, cudaStream_t s);
+// From arrays that the device may read in host memory (source bases 0), checked;
+// *verdict, cleared by the caller, becomes 1 when they are malformed.
+void launch_place_checked(const PlaceArgs& a, int32_t* verdict, cudaStream_t s);
 }  // namespace kb
