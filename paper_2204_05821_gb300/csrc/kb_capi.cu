@@ -34,8 +34,9 @@ struct kb_context {
     cudaEvent_t slot_ev[4] = {};
     int fused_ctas = 0;  // largest grid of the fused kernel (launch_fused_rounds)
     uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
+    bool dense_empty = false;     // the minima are all ones (launch_dense_level0 leaves them so)
     char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
-    void* class_tmp = nullptr;    // degree-class bitmaps, tile counts and hub list during planning
+    void* class_tmp = nullptr;    // degree-class bitmaps of the last plan; its tile counts and hub list
     size_t class_tmp_bytes = 0;
     void* plan_tmp = nullptr;    // in-degree scratch used by kb_workspace_size
     size_t plan_tmp_bytes = 0;
@@ -174,6 +175,7 @@ struct Plan {
     size_t o_emin = 0, o_mid = 0, o_med = 0, o_slot = 0, o_table = 0, o_bitmap = 0, o_prefix = 0, o_scan = 0, o_hubv = 0, o_chunk = 0, o_setoff = 0,
            o_chunkhub = 0, o_chunkext = 0, o_perm = 0, o_gat = 0, o_colr = 0, o_hist = 0, o_ownkey = 0, o_acc = 0, o_cnt = 0, o_sets = 0, o_exact = 0, o_exactlist = 0, o_twin = 0,
            o_frozen = 0, o_classes = 0, o_shared = 0, o_minof = 0, o_joined = 0, o_moved = 0, o_mark = 0;
+    size_t clear_bytes = 0;  // from o_bitmap on
     size_t total = 0;
     // bytes of one degree-class bitmap; four follow one another (kb::DegreeClass)
     size_t class_bytes() const { return align_up(sizeof(uint32_t) * (size_t)((n >> 5) + 1)); }
@@ -242,14 +244,21 @@ void layout_round(Plan& P) {
     // CSR is reordered in place
     P.o_colr = takeg(P.reorder && !needs_in_csr(P.dir) ? sizeof(int32_t) * (size_t)P.m_proc : 0);
     P.o_hist = takeg(P.reorder ? sizeof(unsigned long long) * 512 : 0);
-    P.o_classes = takeg((P.freeze || P.graph_ext) ? Plan::kClassBitmaps * P.class_bytes() : 0);
+    P.o_classes = takeg(P.graph_ext ? Plan::kClassBitmaps * P.class_bytes() : 0);  // (else ctx->class_tmp serves)
     P.graph_bytes = P.graph_ext ? goff : 0;
     size_t off = P.graph_ext ? 0 : goff;
     auto take = [&](size_t bytes) { size_t o = off; off += align_up(bytes); return o; };
     P.o_emin = take(P.ext_table ? 0 : sizeof(uint64_t) * (size_t)std::max<int64_t>(P.n, 1));
     P.o_slot = take(sizeof(int32_t) * (size_t)std::max<int64_t>(P.n, 1));
     P.o_table = take(P.ext_table ? 0 : sizeof(uint64_t) * (size_t)P.cap);
+    // what starts a call clear, together
+    const bool own_freeze = P.freeze && !P.ext_freeze;
     P.o_bitmap = take(sizeof(uint32_t) * (size_t)nw);
+    P.o_frozen = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
+    P.o_shared = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
+    P.o_moved = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
+    P.o_joined = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
+    P.clear_bytes = off - P.o_bitmap;
     P.o_prefix = take(sizeof(uint2) * (size_t)(nw + 1));
     P.o_scan = take(sizeof(uint32_t) * kb::scan_tmp_words(nw));
     P.o_acc = take(sizeof(uint64_t) * H);
@@ -261,12 +270,7 @@ void layout_round(Plan& P) {
     P.o_twin = take(P.sketch ? sizeof(uint32_t) * (size_t)next_pow2(2 * H) : 0);
     P.o_gat = take(P.reorder ? sizeof(int32_t) * (size_t)P.n : 0);
     P.o_ownkey = take(P.subject ? sizeof(int32_t) * (size_t)P.n : 0);
-    const bool own_freeze = P.freeze && !P.ext_freeze;
-    P.o_frozen = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
-    P.o_shared = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_minof = take(own_freeze ? sizeof(uint32_t) * (size_t)P.n : 0);
-    P.o_joined = take(P.freeze ? sizeof(uint32_t) * (size_t)nw : 0);
-    P.o_moved = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.o_mark = take(own_freeze ? sizeof(uint32_t) * (size_t)nw : 0);
     P.total = off;
 }
@@ -379,11 +383,18 @@ struct ClassScratch {
     }
 };
 
+// The tile counts lie in the counters, which are cleared in any case, or in the
+// scratch.
+uint32_t* tile_counts(kb_context* ctx, const Plan& P, const ClassScratch& C) {
+    if (kb::kClassLists * kb::class_tiles(P.n) <= sizeof(Counters::tiles) / sizeof(uint32_t)) return ctx->d_ctr->tiles;
+    return reinterpret_cast<uint32_t*>(reinterpret_cast<char*>(ctx->class_tmp) + C.counts);
+}
+
 // Degree classes of the processed CSR and the host side of the plan: hubs,
 // their chunks and sets, the number of medium vertices.  One round trip, which
 // also brings back ctx->h_ctr (errors of the validation, the level-0 key
 // check).
-kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::CheckRows check) {
+kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::CheckRows check, const kb::CheckIds& ids) {
     cudaStream_t s = ctx->stream;
     P.hub_v.clear();
     P.chunk_off.assign(1, 0);
@@ -394,18 +405,29 @@ kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::Check
     const ClassScratch C(P);
     KB_TRY(ensure_buffer(ctx, &ctx->class_tmp, &ctx->class_tmp_bytes, C.total));
     char* b = reinterpret_cast<char*>(ctx->class_tmp);
-    uint32_t* counts = reinterpret_cast<uint32_t*>(b + C.counts);
+    uint32_t* counts = tile_counts(ctx, P, C);
+    if (counts != ctx->d_ctr->tiles)
+        KB_CUDA(ctx, cudaMemsetAsync(counts, 0, kb::kClassLists * sizeof(uint32_t) * kb::class_tiles(P.n), s));
     uint32_t* bits = reinterpret_cast<uint32_t*>(b);
     const int64_t pitch = (int64_t)(P.class_bytes() / sizeof(uint32_t));
     const kb::ClassBounds bounds{std::min(P.small_max, kb::kSmallDegree), P.small_max, P.thr};
-    kb::launch_classes(P.n, P.m_proc, row_p, bounds, bits, pitch, counts, check, ctx->d_ctr, s);
-    kb::launch_class_list(P.n, row_p, bits, pitch, counts, kb::kHub, C.hub_cap, reinterpret_cast<int32_t*>(b + C.hub_v),
-                          reinterpret_cast<int64_t*>(b + C.hub_deg), s);
-    KB_CUDA(ctx, cudaGetLastError());
+    // A graph with few possible hubs has them written to pinned memory as they are
+    // found; otherwise they are listed, and the first ones copied.
     const int64_t eager = std::min(C.hub_cap, kEagerHubs);
-    char* h_deg = ctx->h_hubs + sizeof(int32_t) * kEagerHubs;
-    KB_CUDA(ctx, cudaMemcpyAsync(ctx->h_hubs, b + C.hub_v, sizeof(int32_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
-    KB_CUDA(ctx, cudaMemcpyAsync(h_deg, b + C.hub_deg, sizeof(int64_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
+    int32_t* h_v = reinterpret_cast<int32_t*>(ctx->h_hubs);
+    int64_t* h_deg = reinterpret_cast<int64_t*>(ctx->h_hubs + sizeof(int32_t) * kEagerHubs);
+    kb::HubSink sink;
+    if (C.hub_cap <= kEagerHubs) sink = {h_v, h_deg, (uint32_t)C.hub_cap};
+    kb::launch_classes(P.n, P.m_proc, row_p, bounds, bits, pitch, counts, check, ids, sink, ctx->d_ctr, s);
+    if (!sink.cap) {
+        kb::launch_class_lists(P.n, row_p, bits, pitch, counts,
+                               {kb::kHub, C.hub_cap, reinterpret_cast<int32_t*>(b + C.hub_v),
+                                reinterpret_cast<int64_t*>(b + C.hub_deg)},
+                               kb::ClassList{}, s);
+        KB_CUDA(ctx, cudaMemcpyAsync(h_v, b + C.hub_v, sizeof(int32_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
+        KB_CUDA(ctx, cudaMemcpyAsync(h_deg, b + C.hub_deg, sizeof(int64_t) * (size_t)eager, cudaMemcpyDeviceToHost, s));
+    }
+    KB_CUDA(ctx, cudaGetLastError());
     KB_TRY(read_counters(ctx));
     KB_TRY(device_error(ctx));
     P.n_mid = ctx->h_ctr->n_class[0];
@@ -415,8 +437,16 @@ kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::Check
     if (H <= 0) return KB_OK;
     P.hub_v.resize((size_t)H);
     std::vector<int64_t> deg((size_t)H);
-    if (H <= eager) {
-        std::memcpy(P.hub_v.data(), ctx->h_hubs, sizeof(int32_t) * (size_t)H);
+    if (sink.cap) {
+        std::vector<std::pair<int32_t, int64_t>> found((size_t)H);
+        for (size_t i = 0; i < (size_t)H; ++i) found[i] = {h_v[i], h_deg[i]};
+        std::sort(found.begin(), found.end());
+        for (size_t i = 0; i < (size_t)H; ++i) {
+            P.hub_v[i] = found[i].first;
+            deg[i] = found[i].second;
+        }
+    } else if (H <= eager) {
+        std::memcpy(P.hub_v.data(), h_v, sizeof(int32_t) * (size_t)H);
         std::memcpy(deg.data(), h_deg, sizeof(int64_t) * (size_t)H);
     } else {
         KB_CUDA(ctx, cudaMemcpyAsync(P.hub_v.data(), b + C.hub_v, sizeof(int32_t) * (size_t)H, cudaMemcpyDeviceToHost, s));
@@ -516,7 +546,13 @@ kb_status make_plan(kb_context* ctx, const kb_graph* g, const kb_options* opt, P
         KB_TRY(build_processed_csr(ctx, g, P, csr_base));
         row_p = reinterpret_cast<const int64_t*>(csr_base + P.o_rowp);
     }
-    KB_TRY(plan_classes(ctx, P, row_p, opt->validate && !for_query ? kb::CheckRows::kAll : kb::CheckRows::kNone));
+    const bool check = opt->validate && !for_query;
+    kb::CheckIds ids;
+    if (check && !needs_in_csr(P.dir)) {
+        ids.a[0] = g->col_indices;
+        ids.count[0] = g->m;
+    }
+    KB_TRY(plan_classes(ctx, P, row_p, check ? kb::CheckRows::kAll : kb::CheckRows::kNone, ids));
     layout_round(P);
     return KB_OK;
 }
@@ -592,6 +628,7 @@ struct Prepared {
     uint32_t* edgeless = nullptr;
     // clean blocks (frozen blocks on): moved vertices and marked (dirty)
     // blocks; RoundParams::minof
+    bool bitmap_fresh = false, counters_fresh = false;  // both clear since prepare
     bool bitmap_ready = false;  // the round's bitmap holds the minima of its frozen blocks already
     bool counters_clear = false;  // the round need not clear the counters (no errors so far; see launch_renumber)
     uint32_t* moved = nullptr;
@@ -681,12 +718,11 @@ kb_status bind_graph_part(kb_context* ctx, const kb_graph* g, const Plan& P, cha
         const ClassScratch C(P);
         const char* b = reinterpret_cast<const char*>(ctx->class_tmp);
         const uint32_t* bits = reinterpret_cast<const uint32_t*>(b);
-        const uint32_t* counts = reinterpret_cast<const uint32_t*>(b + C.counts);
         const int64_t pitch = (int64_t)(P.class_bytes() / sizeof(uint32_t));
-        kb::launch_class_list(n, p.row, bits, pitch, counts, kb::kMid, P.n_mid, const_cast<int32_t*>(p.mid_v), nullptr, s);
-        kb::launch_class_list(n, p.row, bits, pitch, counts, kb::kMedium, P.n_med, const_cast<int32_t*>(p.med_v), nullptr,
-                              s);
-        if (P.freeze || P.graph_ext)  // laid out only then
+        kb::launch_class_lists(n, p.row, bits, pitch, tile_counts(ctx, P, C),
+                               {kb::kMid, P.n_mid, const_cast<int32_t*>(p.mid_v), nullptr},
+                               {kb::kMedium, P.n_med, const_cast<int32_t*>(p.med_v), nullptr}, s);
+        if (P.graph_ext)  // laid out only then
             KB_CUDA(ctx, cudaMemcpyAsync(gws + P.o_classes, b, Plan::kClassBitmaps * P.class_bytes(),
                                          cudaMemcpyDeviceToDevice, s));
         KB_CUDA(ctx, cudaGetLastError());
@@ -738,22 +774,21 @@ kb_status bind_table(kb_context* ctx, const Plan& P, Prepared& R, cudaStream_t s
     return KB_OK;
 }
 
-// Queue the validation of the caller's CSR.  Its verdict comes back with the
-// degree classes (plan_classes), which only read the offsets of an out-edge CSR;
-// before in-edges are counted it has to be known.
+// Validate the caller's CSR before its in-edges are counted.  An out-edge CSR is
+// checked along with the degree classes (plan_classes), which only read its offsets.
 kb_status check_input(kb_context* ctx, const kb_graph* g, const kb_options* opt) {
-    if (!opt->validate) return KB_OK;
-    const bool in = needs_in_csr(opt->direction);
-    kb::launch_validate(g->n, g->m, in ? g->row_offsets : nullptr, g->col_indices, ctx->d_ctr, ctx->stream);
+    if (!opt->validate || !needs_in_csr(opt->direction)) return KB_OK;
+    kb::launch_validate(g->n, g->m, g->row_offsets, g->col_indices, ctx->d_ctr, ctx->stream);
     KB_CUDA(ctx, cudaGetLastError());
-    if (!in) return KB_OK;
     KB_TRY(read_counters(ctx));
     return device_error(ctx);
 }
 
 // Queue the small-label minima of a level 0 (launch_dense_labels).
 kb_status check_small_labels(kb_context* ctx, int64_t n, const int32_t* key) {
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_dense, 0xff, sizeof(uint32_t) * kb::kDenseLabels, ctx->stream));
+    if (!ctx->dense_empty)
+        KB_CUDA(ctx, cudaMemsetAsync(ctx->d_dense, 0xff, sizeof(uint32_t) * kb::kDenseLabels, ctx->stream));
+    ctx->dense_empty = false;
     kb::launch_dense_labels(n, key, ctx->d_dense, ctx->d_ctr, ctx->stream);
     KB_CUDA(ctx, cudaGetLastError());
     return KB_OK;
@@ -769,6 +804,7 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     cudaStream_t s = ctx->stream;
     const int64_t n = g->n;
     KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
+    R.counters_fresh = true;
     Plan& P = R.P;
     char* csr = nullptr;
     char* gws = nullptr;
@@ -861,15 +897,16 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
     R.total_chunks = P.n_chunks;
     R.set_bytes = sizeof(uint64_t) * (size_t)P.set_slots;
     if (P.freeze) {
-        R.edgeless = reinterpret_cast<uint32_t*>(gws + P.o_classes);
+        char* classes = P.graph_ext ? gws + P.o_classes : reinterpret_cast<char*>(ctx->class_tmp);
+        R.edgeless = reinterpret_cast<uint32_t*>(classes);
         const int64_t members[3] = {P.n_mid, P.n_med, (int64_t)P.n_hubs};
         for (int c = 0; c < 3; ++c)
-            R.class_bits[c] = members[c] ? reinterpret_cast<uint32_t*>(gws + P.o_classes + (size_t)(c + 1) * P.class_bytes())
+            R.class_bits[c] = members[c] ? reinterpret_cast<uint32_t*>(classes + (size_t)(c + 1) * P.class_bytes())
                                          : nullptr;
         p.joined = reinterpret_cast<uint32_t*>(ws + P.o_joined);  // all clear between rounds
-        KB_CUDA(ctx, cudaMemsetAsync(p.joined, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
         if (R.ext_frozen) {
             // the caller's state, kept as it is
+            KB_CUDA(ctx, cudaMemsetAsync(p.joined, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
             R.frozen = R.ext_frozen;
             R.frozen_min = R.ext_frozen_min;
             p.shared = R.ext_shared;
@@ -877,17 +914,15 @@ kb_status prepare(kb_context* ctx, const kb_graph* g, const kb_options* opt, Pre
             R.moved = R.ext_moved;
             R.mark = R.ext_mark;
         } else {
-            // nothing frozen before the starting level; shared starts empty
-            const size_t bw = sizeof(uint32_t) * (size_t)((n >> 5) + 1);
+            // nothing frozen before the starting level; shared starts empty, and
+            // the locality order's moved bits are set one by one
             R.frozen = reinterpret_cast<uint32_t*>(ws + P.o_frozen);
             p.shared = reinterpret_cast<uint32_t*>(ws + P.o_shared);
             p.minof = reinterpret_cast<uint32_t*>(ws + P.o_minof);
             R.moved = reinterpret_cast<uint32_t*>(ws + P.o_moved);
             R.mark = reinterpret_cast<uint32_t*>(ws + P.o_mark);
-            KB_CUDA(ctx, cudaMemsetAsync(R.frozen, 0, bw, s));
-            KB_CUDA(ctx, cudaMemsetAsync(p.shared, 0, bw, s));
-            // the locality order's moved bits are set one by one
-            if (P.reorder) KB_CUDA(ctx, cudaMemsetAsync(R.moved, 0, bw, s));
+            KB_CUDA(ctx, cudaMemsetAsync(p.bitmap, 0, P.clear_bytes, s));
+            R.bitmap_fresh = true;
         }
         KB_CUDA(ctx, cudaGetLastError());
     }
@@ -943,8 +978,10 @@ kb::FreezePass freeze_pass(kb_context* ctx, const Prepared& R) {
 kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_t* out, cudaStream_t s,
                         bool* dense_path = nullptr) {
     KB_TRY(next_epoch(ctx, R, s));
-    KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
-    KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
+    if (!R.counters_fresh) KB_CUDA(ctx, cudaMemsetAsync(ctx->d_ctr, 0, sizeof(Counters), s));
+    if (!R.bitmap_fresh)
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
+    R.counters_fresh = R.bitmap_fresh = false;
     R.p.prev = key;
     R.p.frozen = nullptr;
     R.p.frozen_min = nullptr;
@@ -966,6 +1003,7 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
     if (dense) {
         kb::launch_dense_level0(R.p, key, ctx->d_dense, reinterpret_cast<uint2*>(ctx->d_dense + kb::kDenseLabels),
                                 R.prefix, R.scan_tmp, out, s);
+        ctx->dense_empty = true;
     } else {
         kb::launch_small_round(R.p, true, kb::SmallWindows::kConsecutive, s);
         kb::launch_renumber(R.p, R.prefix, R.scan_tmp, out, nullptr, false, s);
@@ -1086,7 +1124,7 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
     a.p.moved = R.moved;
     a.f = freeze_pass(ctx, R);
     a.rank = R.prefix;
-    a.sums = ctx->d_dense;  // the starting level is through with it
+    a.sums = ctx->d_dense + kb::kDenseLabels;  // the pairs, with which the starting level is through
     a.levels = rows.levels;
     a.ping[0] = rows.ping[0];
     a.ping[1] = rows.ping[1];
@@ -1098,7 +1136,8 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_acc, 0, sizeof(uint64_t) * (size_t)R.p.n_hubs, s));
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_cnt, 0, sizeof(uint32_t) * (size_t)R.p.n_hubs, s));
     }
-    if (all_on) KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
+    if (all_on && !R.bitmap_fresh)
+        KB_CUDA(ctx, cudaMemsetAsync(R.p.bitmap, 0, sizeof(uint32_t) * (size_t)((R.p.n >> 5) + 1), s));
     bool stable = false;
     for (int first = i_start + 1; first <= k && !stable;) {
         // every round takes an epoch of the table and a round word of the minima
@@ -1111,7 +1150,7 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
         a.all_on = all_on && first == i_start + 1;
         *R.epoch += (uint32_t)(a.last - first);
         *R.round += (uint32_t)(a.last - first);
-        KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, s));
+        KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, first > i_start + 1, s));
         KB_TRY(read_counters(ctx));
         KB_TRY(device_error(ctx));
         const Counters& hc = *ctx->h_ctr;
@@ -1209,8 +1248,10 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         if (p.minof) {
             // P_0 = {V}: one block, whose smallest member is vertex 0
             kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.minof), n, 0, s);
-            KB_CUDA(ctx, cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
-            kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.bitmap), 1, 1, s);
+            if (!fused) {
+                KB_CUDA(ctx, cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
+                kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.bitmap), 1, 1, s);
+            }
         }
     }
     if (counts) counts[i_start] = prev_count;

@@ -287,7 +287,7 @@ int fused_max_ctas() {
     return sms * per_sm;
 }
 
-cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, cudaStream_t s) {
+cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, bool again, cudaStream_t s) {
     FusedRounds b = a;
     // a CTA per 256 vertices: more only lengthen the barriers
     const int64_t want = (a.p.n + 255) / 256;
@@ -296,8 +296,10 @@ cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, cudaStream_t
         const int64_t per = (a.p.n + (int64_t)grid * kFusedWarps - 1) / ((int64_t)grid * kFusedWarps);
         b.p.warp_verts = (int32_t)std::min<int64_t>(kDefaultWarpVerts, std::max<int64_t>(32, (per + 31) & ~(int64_t)31));
     }
-    cudaError_t e = cudaMemsetAsync(&a.p.ctr->arrived, 0, sizeof(uint32_t), s);
-    if (e != cudaSuccess) return e;
+    if (again) {
+        const cudaError_t e = cudaMemsetAsync(&a.p.ctr->arrived, 0, sizeof(uint32_t), s);
+        if (e != cudaSuccess) return e;
+    }
     void* args[] = {&b};
     return cudaLaunchCooperativeKernel(reinterpret_cast<const void*>(fused_rounds_kernel), dim3(grid), dim3(kFusedThreads),
                                        args, sizeof(FusedSmem), s);

@@ -69,6 +69,8 @@ struct Counters {
     uint32_t most_pairs;    // most distinct pairs of a vertex of the medium CTA kernel this round
     uint32_t exact_chunks;  // chunks of hubs that need their exact set (launch_hub_sketch)
     int64_t n_class[3]; // mid and medium vertices and hubs of the graph (launch_classes)
+    uint32_t hub_at;    // hubs handed out (HubSink)
+    uint32_t tiles[3 * 32];  // tile counts of launch_classes, up to 32 tiles
 };
 
 // Everything one refinement round reads and writes.
@@ -360,7 +362,8 @@ struct FusedRounds {
 };
 // CTAs that a cooperative launch may have (0: not available).
 int fused_max_ctas();
-cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, cudaStream_t s);
+// again: not the first launch since the counters were cleared.
+cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, bool again, cudaStream_t s);
 // Canonical renumbering: prefix of block minima, then ids.
 // rank: (n/32 + 2) words, rank[w] = (minima before word w, minima bits of word w).
 // The frozen, class_on and moved counters restart at 0; with frozen
@@ -380,9 +383,10 @@ size_t scan_tmp_words(int64_t n_items);
 // the general level-0 pass writes: the minima bitmap and the shared-block
 // marks of p, the rank words, ctr->count, the level (out), minof and the
 // locality order's copy gat.  lpair: kDenseLabels (minimum, id) words of scratch.
+// It leaves lmin all ones.
 constexpr int kDenseLabels = 8192;
 void launch_dense_labels(int64_t n, const int32_t* key, uint32_t* lmin, Counters* ctr, cudaStream_t s);
-void launch_dense_level0(const RoundParams& p, const int32_t* key, const uint32_t* lmin, uint2* lpair, uint2* rank,
+void launch_dense_level0(const RoundParams& p, const int32_t* key, uint32_t* lmin, uint2* lpair, uint2* rank,
                          uint32_t* scan_tmp, int32_t* out, cudaStream_t s);
 void launch_fill_i32(int32_t* out, int64_t n, int32_t value, cudaStream_t s);
 // vgraph[v] = graph owning v
@@ -415,13 +419,36 @@ struct ClassBounds {
     int32_t medium;  // of the medium class
 };
 enum class CheckRows { kNone, kOrder, kAll };
+// ids: two arrays whose entries have to lie in [0, n) (kErrInvalid).  hubs: room
+// for the hubs and their degrees in any order (cap 0: none wanted).  The caller
+// has cleared tile_counts and ctr.  One launch: on small graphs each costs more
+// than its work (ids, offsets, hub list and its copies in one launch, both lists
+// in one, and the bitmaps of a call cleared together: a whole call on 10^4
+// vertices and 5 x 10^4 edges 185 -> 160 us, on 7 x 10^5 edges with host buffers
+// 447 -> 403 us; on 10^8 edges 5070 -> 4990 us).
+struct CheckIds {
+    const int32_t* a[2] = {nullptr, nullptr};
+    int64_t count[2] = {0, 0};
+};
+struct HubSink {
+    int32_t* v = nullptr;
+    int64_t* deg = nullptr;
+    uint32_t cap = 0;
+};
 size_t class_tiles(int64_t n);
 void launch_classes(int64_t n, int64_t m, const int64_t* row, const ClassBounds& bounds, uint32_t* bits, int64_t pitch,
-                    uint32_t* tile_counts, CheckRows check, Counters* ctr, cudaStream_t s);
-// The vertices of a class, ascending, at most cap of them, with their degrees
-// unless deg is nullptr.
-void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
-                       DegreeClass c, int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s);
+                    uint32_t* tile_counts, CheckRows check, const CheckIds& ids, const HubSink& hubs, Counters* ctr,
+                    cudaStream_t s);
+// The vertices of one or two classes, ascending, at most cap of each, with their
+// degrees unless deg is nullptr.
+struct ClassList {
+    DegreeClass cls = kMid;
+    int64_t cap = 0;
+    int32_t* out = nullptr;
+    int64_t* deg = nullptr;
+};
+void launch_class_lists(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
+                        const ClassList& a, const ClassList& b, cudaStream_t s);
 // Hub and packed extent of every hub chunk (RoundParams::chunk_hub, chunk_ext).
 void launch_chunk_ext(int64_t chunks, int32_t n_hubs, const int32_t* hub_v, const int64_t* chunk_off,
                       const int64_t* row, int32_t chunk, int32_t* chunk_hub, uint64_t* out, cudaStream_t s);

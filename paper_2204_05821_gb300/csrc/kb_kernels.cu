@@ -388,13 +388,15 @@ __global__ void dense_mark_kernel(const RoundParams p, const uint32_t* lmin) {
     if (p.shared && !(e & kSingleBit)) atomicOr(&p.shared[m >> 5], 1u << (m & 31));
 }
 
-// (smallest vertex, canonical id) of every used label
-__global__ void dense_ids_kernel(const uint32_t* lmin, const uint2* rank, uint2* lpair) {
+// (smallest vertex, canonical id) of every used label; leaves the minima empty
+// for the next level 0
+__global__ void dense_ids_kernel(uint32_t* lmin, const uint2* rank, uint2* lpair) {
     const int l = blockIdx.x * blockDim.x + threadIdx.x;
     if (l >= kDenseLabels) return;
-    const uint32_t m = lmin[l] & kVertexMask;
+    const uint32_t e = lmin[l], m = e & kVertexMask;
     uint32_t id = 0u;
-    if (lmin[l] != kNoMember) {
+    if (e != kNoMember) {
+        lmin[l] = kNoMember;
         const uint2 rw = rank[m >> 5];
         id = rw.x + __popc(rw.y & ((1u << (m & 31)) - 1u));
     }
@@ -591,7 +593,7 @@ void launch_dense_labels(int64_t n, const int32_t* key, uint32_t* lmin, Counters
     dense_label_min_kernel<<<(unsigned)grid, kDenseThreads, 0, s>>>(n, key, lmin, ctr);
 }
 
-void launch_dense_level0(const RoundParams& p, const int32_t* key, const uint32_t* lmin, uint2* lpair, uint2* rank,
+void launch_dense_level0(const RoundParams& p, const int32_t* key, uint32_t* lmin, uint2* lpair, uint2* rank,
                          uint32_t* scan_tmp, int32_t* out, cudaStream_t s) {
     if (p.n <= 0) return;
     const int64_t nw = (p.n >> 5) + 1;

@@ -59,18 +59,6 @@ kb_status scratch_address(int device, unsigned char** out) {
     return KB_OK;
 }
 
-// Level i-1 must hold ids in [0, n) (they index the empty-signature minima);
-// with col given, the neighbour ids too.
-__global__ void check_ids_kernel(int64_t n, int64_t m, const int32_t* prev, const int32_t* col, kb::Counters* ctr) {
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    bool bad = false;
-    for (int64_t v = t; v < n; v += stride) bad |= prev[v] < 0 || (int64_t)prev[v] >= n;
-    if (col)
-        for (int64_t e = t; e < m; e += stride) bad |= col[e] < 0 || (int64_t)col[e] >= n;
-    if (bad) atomicOr(&ctr->err, kb::kErrInvalid);
-}
-
 uint64_t next_pow2(uint64_t x) {
     uint64_t p = 1;
     while (p < x) p <<= 1;
@@ -143,16 +131,22 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     NA_CUDA(cudaMemsetAsync(base, 0, kOffBitmap + sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
     NA_CUDA(cudaMemsetAsync(p.table, 0, sizeof(uint64_t) * cap, s));
     NA_CUDA(cudaMemsetAsync(p.emin, 0xff, sizeof(uint64_t) * (size_t)n, s));
-    const unsigned grid = (unsigned)std::min<int64_t>((std::max(n, g->m) + 255) / 256, 152 * 8);
-    check_ids_kernel<<<grid, 256, 0, s>>>(n, g->m, prev, opt->validate ? g->col_indices : nullptr, ctr);
     // the degree classes: no vertex may lie above the hub threshold (no hub path
-    // here) or have a negative degree
+    // here) or have a negative degree.  Level i-1 must hold ids in [0, n) (they
+    // index the empty-signature minima).
+    kb::CheckIds ids;
+    ids.a[0] = prev;
+    ids.count[0] = n;
+    if (opt->validate) {
+        ids.a[1] = g->col_indices;
+        ids.count[1] = g->m;
+    }
     uint32_t* bits = reinterpret_cast<uint32_t*>(base + kOffClasses);
     const int64_t pitch = (int64_t)(up(sizeof(uint32_t) * kWords) / sizeof(uint32_t));
     uint32_t* tiles = reinterpret_cast<uint32_t*>(base + kOffTiles);
     const kb::ClassBounds bounds{p.small_max, p.mid_max, thr};
     kb::launch_classes(n, g->m, p.row, bounds, bits, pitch, tiles,
-                       opt->validate ? kb::CheckRows::kAll : kb::CheckRows::kOrder, ctr, s);
+                       opt->validate ? kb::CheckRows::kAll : kb::CheckRows::kOrder, ids, kb::HubSink{}, ctr, s);
     NA_CUDA(cudaGetLastError());
     kb::Counters host_ctr{};
     NA_CUDA(cudaMemcpyAsync(&host_ctr, ctr, sizeof(host_ctr), cudaMemcpyDeviceToHost, s));
@@ -165,8 +159,8 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     int32_t* lists = reinterpret_cast<int32_t*>(base + kOffMed);
     p.mid_v = lists;
     p.med_v = lists + p.n_mid;
-    kb::launch_class_list(n, p.row, bits, pitch, tiles, kb::kMid, p.n_mid, lists, nullptr, s);
-    kb::launch_class_list(n, p.row, bits, pitch, tiles, kb::kMedium, p.n_med, lists + p.n_mid, nullptr, s);
+    kb::launch_class_lists(n, p.row, bits, pitch, tiles, {kb::kMid, p.n_mid, lists, nullptr},
+                           {kb::kMedium, p.n_med, lists + p.n_mid, nullptr}, s);
 
     kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
     kb::launch_mid_round(p, s);

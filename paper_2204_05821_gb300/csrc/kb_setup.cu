@@ -256,9 +256,32 @@ __global__ void remap_cols_kernel(int64_t m, const int32_t* col, const int32_t* 
 constexpr int kListTile = 131072;  // vertices whose words one CTA of the list kernel turns into ids
 constexpr int kClassPer = 4096;    // vertices per CTA of the class kernel, at most; a divisor of kListTile
 
+// The CTAs past the class_ctas first ones check ids (CheckIds) meanwhile.
 __global__ void __launch_bounds__(256) classes_kernel(int64_t n, int64_t m, const int64_t* row, ClassBounds bounds,
                                                       uint32_t* bits, int64_t pitch, uint32_t* tile_counts, int per,
-                                                      CheckRows check, Counters* ctr) {
+                                                      CheckRows check, unsigned class_ctas, CheckIds ids, HubSink hubs,
+                                                      Counters* ctr) {
+    if (blockIdx.x >= class_ctas) {
+        const int64_t stride = (int64_t)(gridDim.x - class_ctas) * 256;
+        const int64_t t0 = (int64_t)(blockIdx.x - class_ctas) * 256 + threadIdx.x;
+        bool wrong = false;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int32_t* a = ids.a[k];
+            const int64_t count = ids.count[k];
+            int64_t i = t0;
+            for (; i + 7 * stride < count; i += 8 * stride) {  // eight loads in flight
+                int32_t x[8];
+#pragma unroll
+                for (int u = 0; u < 8; ++u) x[u] = __ldcs(a + i + u * stride);
+#pragma unroll
+                for (int u = 0; u < 8; ++u) wrong |= x[u] < 0 || (int64_t)x[u] >= n;
+            }
+            for (; i < count; i += stride) wrong |= a[i] < 0 || (int64_t)a[i] >= n;
+        }
+        if (__any_sync(kFull, wrong) && (threadIdx.x & 31) == 0) atomicOr(&ctr->err, kErrInvalid);
+        return;
+    }
     __shared__ uint32_t s_n[kClassLists];
     if (threadIdx.x < kClassLists) s_n[threadIdx.x] = 0u;
     __syncthreads();
@@ -273,6 +296,13 @@ __global__ void __launch_bounds__(256) classes_kernel(int64_t n, int64_t m, cons
         const int64_t d = v < n ? row[v + 1] - row[v] : 1;
         bad |= d < 0;
         const bool mid = v < n && d > bounds.small && d <= bounds.mid, hub = v < n && d > bounds.medium;
+        if (hub && hubs.cap) {
+            const uint32_t at = atomicAdd(&ctr->hub_at, 1u);
+            if (at < hubs.cap) {
+                hubs.v[at] = (int32_t)v;
+                hubs.deg[at] = d;
+            }
+        }
         unsigned w[1 + kClassLists];
         w[kEdgeless] = __ballot_sync(kFull, d == 0);
         w[kMid] = __ballot_sync(kFull, mid);
@@ -334,10 +364,19 @@ __device__ __forceinline__ int64_t block_exscan_i64(int64_t x, int64_t* tmp, int
 // when deg is given): a CTA takes the words of one tile and finds its place from
 // the counts of the tiles before it.  Nothing is written at or past cap.
 static_assert(kListTile == kT * 4 * 32, "four words per thread");
-__global__ void __launch_bounds__(kT) class_list_kernel(int64_t n, const int64_t* row, const uint32_t* bits,
-                                                        const uint32_t* tile_counts, int64_t cap, int32_t* out,
-                                                        int64_t* deg) {
+struct TwoLists {
+    ClassList l[2];
+};
+__global__ void __launch_bounds__(kT) class_list_kernel(int64_t n, const int64_t* row, const uint32_t* all_bits,
+                                                        int64_t pitch, const uint32_t* all_counts,
+                                                        const TwoLists lists) {
     __shared__ int64_t tmp[32];
+    const ClassList& L = lists.l[blockIdx.y];
+    const uint32_t* bits = all_bits + L.cls * pitch;
+    const uint32_t* tile_counts = all_counts + L.cls - 1;
+    const int64_t cap = L.cap;
+    int32_t* out = L.out;
+    int64_t* deg = L.deg;
     if (tile_counts[kClassLists * (int64_t)blockIdx.x] == 0) return;  // uniform over the CTA
     int64_t before = 0, base;
     for (int64_t t = threadIdx.x; t < blockIdx.x; t += kT) before += tile_counts[kClassLists * t];
@@ -464,21 +503,27 @@ void launch_chunk_ext(int64_t chunks, int32_t n_hubs, const int32_t* hub_v, cons
 size_t class_tiles(int64_t n) { return (size_t)((n + kListTile - 1) / kListTile); }
 
 void launch_classes(int64_t n, int64_t m, const int64_t* row, const ClassBounds& bounds, uint32_t* bits, int64_t pitch,
-                    uint32_t* tile_counts, CheckRows check, Counters* ctr, cudaStream_t s) {
+                    uint32_t* tile_counts, CheckRows check, const CheckIds& ids, const HubSink& hubs, Counters* ctr,
+                    cudaStream_t s) {
     if (n <= 0) return;
-    cudaMemsetAsync(tile_counts, 0, kClassLists * sizeof(uint32_t) * class_tiles(n), s);
     int per = 256;  // short CTAs on small graphs (11 us for 10^5 vertices in CTAs of 4096, 4 us in CTAs of 256)
     while (per < kClassPer && n > (int64_t)per * 152 * 8) per *= 2;
     // (n >> 5) + 1 words: the last one may lie past the last vertex
-    classes_kernel<<<(unsigned)((n + per) / per), 256, 0, s>>>(n, m, row, bounds, bits, pitch, tile_counts, per, check,
-                                                               ctr);
+    const unsigned ctas = (unsigned)((n + per) / per);
+    const int64_t most = ids.count[0] > ids.count[1] ? ids.count[0] : ids.count[1];
+    const unsigned id_ctas = most > 0 ? (unsigned)grid_for(most, 256) : 0u;
+    classes_kernel<<<ctas + id_ctas, 256, 0, s>>>(n, m, row, bounds, bits, pitch, tile_counts, per, check, ctas, ids,
+                                                  hubs, ctr);
 }
 
-void launch_class_list(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
-                       DegreeClass c, int64_t cap, int32_t* out, int64_t* deg, cudaStream_t s) {
-    if (n <= 0 || cap <= 0) return;
-    class_list_kernel<<<(unsigned)class_tiles(n), kT, 0, s>>>(n, row, bits + c * pitch, tile_counts + c - 1, cap, out,
-                                                              deg);
+void launch_class_lists(int64_t n, const int64_t* row, const uint32_t* bits, int64_t pitch, const uint32_t* tile_counts,
+                        const ClassList& a, const ClassList& b, cudaStream_t s) {
+    TwoLists l;
+    int lists = 0;
+    for (const ClassList* x : {&a, &b})
+        if (x->cap > 0) l.l[lists++] = *x;
+    if (n <= 0 || !lists) return;
+    class_list_kernel<<<dim3((unsigned)class_tiles(n), (unsigned)lists), kT, 0, s>>>(n, row, bits, pitch, tile_counts, l);
 }
 
 void launch_locality_order(int64_t n, int64_t m, const int32_t* col, uint32_t* cnt, unsigned long long* hist,
