@@ -1114,8 +1114,10 @@ constexpr int64_t kFusedSize = (int64_t)1 << 21;
 
 // Rounds i_start + 1 .. k after the starting level is queued, kb::kFusedRounds at
 // a time.  all_on: no freeze pass ran yet.
+// key0: the starting level's keys, when it is not queued yet and they are small.
 kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int i_start, int k, bool stop, bool all_on,
-                       int64_t* counts, int* levels_computed, int64_t* last_count, bool* stopped_stable) {
+                       const int32_t* key0, int64_t* counts, int* levels_computed, int64_t* last_count,
+                       bool* stopped_stable) {
     cudaStream_t s = ctx->stream;
     kb::FusedRounds a;
     a.p = R.p;
@@ -1150,7 +1152,10 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
         a.all_on = all_on && first == i_start + 1;
         *R.epoch += (uint32_t)(a.last - first);
         *R.round += (uint32_t)(a.last - first);
+        a.key0 = first == i_start + 1 ? key0 : nullptr;
+        a.lmin = ctx->d_dense;
         KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, first > i_start + 1, s));
+        if (a.key0) ctx->dense_empty = true;
         KB_TRY(read_counters(ctx));
         KB_TRY(device_error(ctx));
         const Counters& hc = *ctx->h_ctr;
@@ -1171,7 +1176,7 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
     if (stable && stopped_stable) *stopped_stable = true;
     if (rows.host) {
         KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
-        KB_TRY(emit_rows(ctx, rows, i_start + 1, k));
+        KB_TRY(emit_rows(ctx, rows, key0 ? i_start : i_start + 1, k));
     }
     return KB_OK;
 }
@@ -1225,7 +1230,11 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     int32_t* row0 = rows.row(i_start);
     int64_t prev_count = 1;
     bool count_known = true;  // the starting level's block count is on the host
-    if (init_key) {
+    // with the rounds of a small graph when the keys are known to be small
+    const bool fused0 = fused && init_key && init_key == R.key_checked && R.key_dense && R.counters_fresh && R.bitmap_fresh;
+    if (fused0) {
+        R.key_checked = nullptr;
+    } else if (init_key) {
         bool dense = false;
         KB_TRY(launch_level0(ctx, R, init_key, row0, s, &dense));
         // At most kDenseLabels blocks after the small-label path: how many are
@@ -1256,12 +1265,14 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     }
     if (counts) counts[i_start] = prev_count;
     if (last_count) *last_count = prev_count;
-    if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
-    KB_TRY(emit_rows(ctx, rows, i_start, i_start));
+    if (!fused0) {
+        if (rows.host) KB_CUDA(ctx, cudaEventRecord(ctx->row_ev, s));
+        KB_TRY(emit_rows(ctx, rows, i_start, i_start));
+    }
 
     if (fused)
-        return fused_rounds(ctx, R, rows, i_start, k, opt->early_stop || fixpoint, !init_key, counts, levels_computed,
-                            last_count, stopped_stable);
+        return fused_rounds(ctx, R, rows, i_start, k, opt->early_stop || fixpoint, !init_key,
+                            fused0 ? init_key : nullptr, counts, levels_computed, last_count, stopped_stable);
 
     // ---- refinement rounds
     R.counters_clear = !R.P.subject;

@@ -1,4 +1,5 @@
-// All rounds of a small graph in one cooperative kernel.
+// All rounds of a small graph in one cooperative kernel, and the starting level
+// before them when its keys are small.
 //
 // A round is a chain of six or seven short passes, each of which takes a few
 // microseconds on a small graph, about as long as launching it and draining the
@@ -13,7 +14,8 @@
 // barrier, five to seven a round.  Whole calls, one launch per pass against this
 // kernel: 10^4 vertices and 5 x 10^4 edges: 248 -> 183 us; a graph of
 // 7 x 10^5 edges with host buffers: 525 -> 450 us; 3 x 10^5 vertices to their
-// fixpoint in 11 rounds: 1066 -> 847 us.  Three CTAs per SM (a CTA per 256
+// fixpoint in 11 rounds: 1066 -> 847 us.  The starting level's four passes in here
+// too: 159 -> 147 us for the first (with fewer setup operations since).  Three CTAs per SM (a CTA per 256
 // vertices) as the occupancy allows: the last took 885 us with two and 1209 us
 // with one.
 //
@@ -109,7 +111,8 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
     const int64_t thread = (int64_t)blockIdx.x * kFusedThreads + tid, threads = warps * 32;
     uint32_t target = 0;
 
-    for (int i = a.first; i <= a.last; ++i) {
+    for (int i = a.key0 ? a.first - 1 : a.first; i <= a.last; ++i) {
+        const bool level0 = i < a.first;
         RoundParams p = a.p;
         p.epoch = a.p.epoch + (uint32_t)(i - a.first);
         p.ehigh = a.p.ehigh - (uint32_t)(i - a.first);
@@ -119,21 +122,29 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
         const int64_t frozen = all ? 0 : *(volatile int64_t*)&ctr->frozen;
         bool on[3];
         for (int c = 0; c < 3; ++c) on[c] = all || *(volatile int64_t*)&ctr->class_on[c] > 0;
-        const bool hubs = p.n_hubs > 0 && on[2];
+        const bool hubs = p.n_hubs > 0 && on[2] && !level0;
 
         // ---- keys
-        if (frozen * 4 > n) {
+        if (level0) {  // every label's smallest vertex, shared when the label has others
+            for (int64_t l = thread; l < kDenseLabels; l += threads) {
+                const uint32_t e = a.lmin[l];
+                if (e == kNoMember) continue;
+                const uint32_t m = e & kVertexMask;
+                atomicOr(&p.bitmap[m >> 5], 1u << (m & 31));
+                if (!(e & kSingleBit)) atomicOr(&p.shared[m >> 5], 1u << (m & 31));
+            }
+        } else if (frozen * 4 > n) {
             if ((n - frozen) * 64 < n) p.warp_verts *= 4;  // few vertices refine: longer tasks
             small_body<false, true, true>(p, sm.compact, my_warp, warps);
         } else {
             small_body<false, false, true>(p, sm.small, my_warp, warps);
         }
-        if (p.n_mid > 0 && on[0]) {
+        if (p.n_mid > 0 && on[0] && !level0) {
             __syncthreads();
             const int32_t per = (int32_t)min((int64_t)kMedTask, (p.n_mid + warps - 1) / warps);
             for (int64_t t = my_warp * per; t < p.n_mid; t += warps * per) mid_task(p, sm.mid.set, sm.mid.mark, t, per);
         }
-        if (p.n_med > 0 && on[1]) {
+        if (p.n_med > 0 && on[1] && !level0) {
             const int32_t thr = min(p.hub_threshold, (int32_t)kMaxHubThreshold);
             const int32_t split = min(max(p.med_split, 1), (int32_t)kMedSplit);
             if (p.mid_max < min(thr, split)) {
@@ -208,7 +219,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             if (i == a.first) ctr->start_count = ctr->count;
             ctr->prev_count = ctr->count;
             ctr->count = (int64_t)base;
-            ctr->round_count[i - a.first] = (int64_t)base;
+            if (!level0) ctr->round_count[i - a.first] = (int64_t)base;
             ctr->last_round = i;
             ctr->frozen = 0;
             for (int c = 0; c < 3; ++c) ctr->class_on[c] = 0;
@@ -218,7 +229,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
         if (!grid_barrier(ctr, target)) return;
 
         // ---- ids; under early stop a round that kept the count is the last one
-        const bool stable = a.stop_stable &&
+        const bool stable = a.stop_stable && !level0 &&
                             *(volatile int64_t*)&ctr->count == *(volatile int64_t*)&ctr->prev_count;
         if (stable) {
             if (a.levels) {
@@ -233,7 +244,22 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             }
             return;
         }
-        assign_frozen(p, a.rank, out, p.moved, a.f.mark ? const_cast<uint32_t*>(a.f.mark) : nullptr, &sm.pass.word);
+        if (level0) {
+            for (int64_t v = thread; v < n; v += threads) {
+                const uint32_t l = (uint32_t)a.key0[v];
+                uint32_t m = l < (uint32_t)kDenseLabels ? a.lmin[l] & kVertexMask : (uint32_t)n;
+                if ((int64_t)m >= n) {  // the keys changed since they were checked
+                    set_error(ctr, kErrInvalid);
+                    m = (uint32_t)v;
+                }
+                const uint2 rw = a.rank[m >> 5];
+                out[v] = (int32_t)(rw.x + __popc(rw.y & ((1u << (m & 31)) - 1u)));
+                if (p.perm) p.gat[p.perm[v]] = (int32_t)m;
+                p.minof[v] = m;
+            }
+        } else {
+            assign_frozen(p, a.rank, out, p.moved, a.f.mark ? const_cast<uint32_t*>(a.f.mark) : nullptr, &sm.pass.word);
+        }
         if (hubs) {  // leave the used sets and sums empty for the next round
             for (int h = blockIdx.x; h < p.n_hubs; h += gridDim.x) {
                 if (!vertex_refines(p, p.hub_v[h])) continue;
@@ -250,7 +276,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
 
         // ---- frozen blocks of the next round
         const int per_warp = (int)min((int64_t)32, max((int64_t)1, nw / warps));
-        if (few_moved(p)) {  // (the count is read after the barrier and not written before the next)
+        if (!level0 && few_moved(p)) {  // (the count is read after the barrier and not written before the next)
             for (int64_t w0 = my_warp * per_warp; w0 < nw; w0 += warps * per_warp)
                 dirty_blocks(p, a.f.edgeless, p.moved, kMaxHubThreshold, const_cast<uint32_t*>(a.f.mark), per_warp, nullptr,
                              w0);
@@ -258,6 +284,12 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
         }
         FreezePass f = a.f;
         f.per_warp = per_warp;
+        if (level0) {  // only its singletons are frozen, as after launch_dense_level0
+            f.edgeless = nullptr;
+            f.mark = nullptr;
+            f.moved_clear = nullptr;
+            for (int64_t l = thread; l < kDenseLabels; l += threads) a.lmin[l] = kNoMember;
+        }
         __syncthreads();
         if (tid < 4) sm.pass.on[tid] = 0u;
         __syncthreads();

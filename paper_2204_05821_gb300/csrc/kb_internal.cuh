@@ -357,6 +357,10 @@ struct FusedRounds {
     int32_t* ping[2] = {nullptr, nullptr};  // in turn
     int64_t total_chunks = 0;
     int first = 0, last = 0, k = 0;  // k: the call's last level
+    // the starting level too, row first - 1, when its keys are small: they and the
+    // label minima (launch_dense_labels), which are left empty
+    const int32_t* key0 = nullptr;
+    uint32_t* lmin = nullptr;
     bool stop_stable = false;    // stop at a round that keeps the count; its row and all up to k are copied
     bool all_on = false;
 };
@@ -385,6 +389,7 @@ size_t scan_tmp_words(int64_t n_items);
 // locality order's copy gat.  lpair: kDenseLabels (minimum, id) words of scratch.
 // It leaves lmin all ones.
 constexpr int kDenseLabels = 8192;
+constexpr uint32_t kNoMember = 0xffffffffu;
 void launch_dense_labels(int64_t n, const int32_t* key, uint32_t* lmin, Counters* ctr, cudaStream_t s);
 void launch_dense_level0(const RoundParams& p, const int32_t* key, uint32_t* lmin, uint2* lpair, uint2* rank,
                          uint32_t* scan_tmp, int32_t* out, cudaStream_t s);

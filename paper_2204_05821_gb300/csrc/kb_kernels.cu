@@ -330,7 +330,6 @@ __global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p
 // ----------------------------------------------------------------------------
 constexpr int kDenseThreads = 512;
 
-constexpr uint32_t kNoMember = 0xffffffffu;
 
 // Lower an entry to `member`: a vertex, with kSingleBit when it is the only one
 // its side has seen.
