@@ -1022,6 +1022,19 @@ kb_status launch_level0(kb_context* ctx, Prepared& R, const int32_t* key, int32_
     return KB_OK;
 }
 
+// Up to this many vertices the small, mid and medium vertices of a round that
+// keys most of them go in one launch (kb::launch_keys).  It holds four CTAs of the
+// small body per SM instead of five, which costs large graphs more than the
+// draining between the classes.  Prepared power-law graphs, n = m/6, whole calls
+// in us apart / together:
+//   edges               3.2e6      6.4e6      1.3e7      2.6e7      5.1e7
+//   labelled, out     526/485    692/659    999/949  1618/1584  2742/2735
+//   kaushik, in       659/634    888/874  1321/1301  2082/2082  3767/3818
+//   schaetzle, out    633/605    938/914  1356/1330  2190/2175  3720/3739
+//   labelled, both    551/500    705/669  1054/1002  1664/1621  3023/2998
+// and 10^8 edges of 10^7 vertices 4970 / 5080.
+constexpr int64_t kKeysVertices = 6 << 20;
+
 // One refinement round up to (not including) the renumbering.
 kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer* T) {
     kb::RoundParams& p = R.p;
@@ -1036,17 +1049,24 @@ kb_status launch_round_body(kb_context* ctx, Prepared& R, cudaStream_t s, Timer*
     if (!R.bitmap_ready) kb::launch_clear_round(p, s);
     R.bitmap_ready = false;
     if (T) T->end();
-    if (T) T->begin(KB_KERNEL_SMALL);
-    kb::launch_small_round(p, false,
-                           R.sparse ? kb::SmallWindows::kSparse
-                                    : (R.compact ? kb::SmallWindows::kCompact : kb::SmallWindows::kConsecutive),
-                           s);
-    if (mid) kb::launch_mid_round(p, s);
-    if (T) T->end();
-    if (med) {
-        if (T) T->begin(KB_KERNEL_MEDIUM);
-        kb::launch_medium_round(p, s);
+    if ((mid || med) && !R.compact && !R.sparse && !ctx->timing && p.n <= kKeysVertices) {
+        kb::RoundParams q = p;
+        if (!mid) q.n_mid = 0;
+        if (!med) q.n_med = 0;
+        kb::launch_keys(q, s);
+    } else {
+        if (T) T->begin(KB_KERNEL_SMALL);
+        kb::launch_small_round(p, false,
+                               R.sparse ? kb::SmallWindows::kSparse
+                                        : (R.compact ? kb::SmallWindows::kCompact : kb::SmallWindows::kConsecutive),
+                               s);
+        if (mid) kb::launch_mid_round(p, s);
         if (T) T->end();
+        if (med) {
+            if (T) T->begin(KB_KERNEL_MEDIUM);
+            kb::launch_medium_round(p, s);
+            if (T) T->end();
+        }
     }
     if (hub) {
         if (T) T->begin(KB_KERNEL_HUB_CHUNK);

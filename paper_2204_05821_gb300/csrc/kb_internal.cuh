@@ -323,6 +323,9 @@ void launch_round_work(const RoundParams& p, cudaStream_t s);
 // (kCompact: worth it when many are frozen; kSparse: nearly all are).
 enum class SmallWindows { kConsecutive, kCompact, kSparse };
 void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s);
+int32_t default_task_vertices(int64_t n);  // per warp task, when the caller gives none
+// The small, mid and medium vertices in one launch (kb_keys.cu).
+void launch_keys(const RoundParams& p, cudaStream_t s);
 void launch_mid_round(const RoundParams& p, cudaStream_t s);     // kb_medium.cu: after the small vertices,
 void launch_medium_round(const RoundParams& p, cudaStream_t s);  //   after the mid ones
 // Per-device kernel attributes (shared-memory carveouts); call once per device

@@ -52,11 +52,21 @@ kb_status scratch_address(int device, unsigned char** out) {
             return KB_ERR_CUDA;
         }
         g_scratch_ptr[device] = ptr;
-        kb::set_medium_kernel_attributes();  // once per device, on the first call
-        cudaGetLastError();
     }
     *out = reinterpret_cast<unsigned char*>(g_scratch_ptr[device]);
     return KB_OK;
+}
+
+// What a call starts with: two runs of zeros and one of ones, in 16-byte words
+// (one launch in the place of three clears).
+__global__ void __launch_bounds__(256) reset_kernel(uint4* zero_a, int64_t a, uint4* zero_b, int64_t b, uint4* ones,
+                                                    int64_t c) {
+    const int64_t stride = (int64_t)gridDim.x * 256;
+    const int64_t t = (int64_t)blockIdx.x * 256 + threadIdx.x;
+    const uint4 z = make_uint4(0u, 0u, 0u, 0u), o = make_uint4(~0u, ~0u, ~0u, ~0u);
+    for (int64_t i = t; i < a; i += stride) zero_a[i] = z;
+    for (int64_t i = t; i < b; i += stride) zero_b[i] = z;
+    for (int64_t i = t; i < c; i += stride) ones[i] = o;
 }
 
 uint64_t next_pow2(uint64_t x) {
@@ -128,9 +138,13 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     p.n_hubs = 0;
 
     // The array keeps the previous call's contents: reset what must start clean.
-    NA_CUDA(cudaMemsetAsync(base, 0, kOffBitmap + sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
-    NA_CUDA(cudaMemsetAsync(p.table, 0, sizeof(uint64_t) * cap, s));
-    NA_CUDA(cudaMemsetAsync(p.emin, 0xff, sizeof(uint64_t) * (size_t)n, s));
+    // (every part of it is padded to 256 bytes)
+    auto words = [](size_t bytes) { return (int64_t)((bytes + sizeof(uint4) - 1) / sizeof(uint4)); };
+    const int64_t table_words = words(sizeof(uint64_t) * cap);
+    reset_kernel<<<(unsigned)std::min<int64_t>((table_words + 255) / 256, 152 * 8), 256, 0, s>>>(
+        reinterpret_cast<uint4*>(base), words(kOffBitmap + sizeof(uint32_t) * (size_t)((n >> 5) + 1)),
+        reinterpret_cast<uint4*>(p.table), table_words, reinterpret_cast<uint4*>(p.emin),
+        words(sizeof(uint64_t) * (size_t)n));
     // the degree classes: no vertex may lie above the hub threshold (no hub path
     // here) or have a negative degree.  Level i-1 must hold ids in [0, n) (they
     // index the empty-signature minima).
@@ -162,9 +176,7 @@ extern "C" kb_status kb_refine_round_noalloc(void* stream, const kb_graph* g, co
     kb::launch_class_lists(n, p.row, bits, pitch, tiles, {kb::kMid, p.n_mid, lists, nullptr},
                            {kb::kMedium, p.n_med, lists + p.n_mid, nullptr}, s);
 
-    kb::launch_small_round(p, false, kb::SmallWindows::kConsecutive, s);
-    kb::launch_mid_round(p, s);
-    kb::launch_medium_round(p, s);
+    kb::launch_keys(p, s);
     kb::launch_renumber(p, reinterpret_cast<uint2*>(base + kOffPrefix), reinterpret_cast<uint32_t*>(base + kOffScan),
                         out, nullptr, false, s);
     NA_CUDA(cudaGetLastError());

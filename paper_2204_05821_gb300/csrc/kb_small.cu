@@ -28,10 +28,12 @@ static int64_t task_vertices(int64_t n, int64_t lo, int64_t hi) {
     return std::min(hi, std::max(lo, (per + 7) & ~(int64_t)7));
 }
 
+int32_t default_task_vertices(int64_t n) { return (int32_t)task_vertices(n, 32, kDefaultWarpVerts); }
+
 void launch_small_round(const RoundParams& p, bool level0, SmallWindows windows, cudaStream_t s) {
     if (p.n <= 0) return;
     const bool compact = windows != SmallWindows::kConsecutive;
-    int64_t wv = p.warp_verts > 0 ? p.warp_verts : task_vertices(p.n, 32, kDefaultWarpVerts);
+    int64_t wv = p.warp_verts > 0 ? p.warp_verts : default_task_vertices(p.n);
     // few vertices refine: long warp tasks, so that far fewer CTAs set up and
     // flush a join map for a handful of vertices each
     if (windows == SmallWindows::kSparse) wv = task_vertices(p.n, kDefaultWarpVerts, 4096);
