@@ -44,12 +44,13 @@ METRIC = "k-bisim edges/s per round"
 # byte of a kernel, from one ncu capture of it on the large recipe at a tenth
 # of the size, where its traffic grows in proportion to its units.  Valid only for the kernel source it was measured
 # on: the SHA-1 of the kernel's file followed by the two shared device headers
-# must match.
+# must match (hub_chunk: the sketch kernel's, which reads nearly all of the hub
+# edges).
 KERNEL_HEADERS = ("paper_2204_05821_gb300/csrc/kb_device.cuh", "paper_2204_05821_gb300/csrc/kb_internal.cuh")
 TRAFFIC_PER_ALGO_BYTE = {
-    "hub_chunk": ("paper_2204_05821_gb300/csrc/kb_kernels.cu", "9734ccc8cb4fa02be0fff878a6f1f298d83277e3", 2.206),
-    "small": ("paper_2204_05821_gb300/csrc/kb_small.cu", "5fe82d2a0a4fa2dc30c2c8474321b9501eb6d7f1", 5.522),
-    "medium": ("paper_2204_05821_gb300/csrc/kb_medium.cu", "98941f79c3ef798d184d25adb0e052b61de81aa0", 1.965),
+    "hub_chunk": ("paper_2204_05821_gb300/csrc/kb_hub.cu", "9b30efa5eefeb6290ffc4a2729e74bb0886ea8b2", 1.071),
+    "small": ("paper_2204_05821_gb300/csrc/kb_small.cuh", "49d18be05b7a279b849882139d236cd3339060ab", 5.624),
+    "medium": ("paper_2204_05821_gb300/csrc/kb_medium.cuh", "e6f9879934724e8969fe577671fcddd926713405", 1.953),
 }
 
 
@@ -387,15 +388,15 @@ def run_ours(args, rank, world, local):
                 "kernel_share": {kname: fam_ms[kname] / sum(fam_ms.values()) for kname in fam_ms},
                 "per_launch_ms": {kname: fam_ms[kname] / max(1, fam_n[kname]) for kname in fam_ms}}
     # our kernels per family event: the medium family is a warp kernel and a
-    # CTA kernel, the hub-chunk family clears the refining hubs' sets first,
-    # renumbering is the 3-kernel rank scan, the stable-round copy, the
-    # assignment, the moved count, the dirty, freeze and frozen-count passes
-    # and the refining count; "other" is memsets only; per call add level 0
-    # over the small labels (label minima, minima marks, rank scan, label ids,
-    # assignment, freeze, frozen count, refining count); the setup kernels
-    # ran once, in kb_graph_prepare
-    per_event = {"small": 1, "medium": 2, "hub_chunk": 2, "hub_final": 1, "renumber": 10, "other": 0}
-    launches = int(sum(per_event.get(kname, 1) * cnt for kname, cnt in fam_n.items())) + 10 * args.steps
+    # CTA kernel, beside the mid kernel that mostly runs in the same rounds; the
+    # hub-chunk family makes and looks up the sketches (three kernels) and clears
+    # the refining hubs' sets first; renumbering is the two kernels of the rank
+    # scan, the assignment and the dirty and freeze passes; "other" is memsets
+    # only; per call add level 0 over the small labels (label minima, minima
+    # marks, rank scan, label ids, assignment, freeze) and the stable round's
+    # copy; the setup kernels ran once, in kb_graph_prepare
+    per_event = {"small": 1, "medium": 3, "hub_chunk": 5, "hub_final": 1, "renumber": 5, "other": 0}
+    launches = int(sum(per_event.get(kname, 1) * cnt for kname, cnt in fam_n.items())) + 8 * args.steps
     # Round 1 is the one round that keys every vertex and every edge (nothing
     # is frozen before it): the full-work figure, with the whole round's
     # algorithmic bytes taken as 12 B per edge (neighbour id, edge label,

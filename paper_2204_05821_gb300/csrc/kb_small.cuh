@@ -7,8 +7,8 @@
 // shared memory, sums their mixes, probes the table and, on a tag match, derives
 // the representative's pairs and looks each up among its own (the full
 // signature compare).  Representatives are small vertices too, as larger ones
-// enter the table after this kernel; in the fused kernel they may be of any
-// degree, so the compare has no limit.  Neighbouring lanes read neighbouring edges, so
+// enter the table after this kernel; where the classes share a launch
+// (kb_fused.cu, kb_keys.cu) they may be of any degree, so the compare has no limit.  Neighbouring lanes read neighbouring edges, so
 // the lines that one lane's load brings serve the others from L1.
 //
 // What bounds it: random 4-8 byte accesses (blocks, table, representatives) and
