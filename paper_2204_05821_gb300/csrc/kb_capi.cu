@@ -1250,6 +1250,12 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     int32_t* row0 = rows.row(i_start);
     int64_t prev_count = 1;
     bool count_known = true;  // the starting level's block count is on the host
+    if (fused && init_key && !R.key_checked && R.P.dense0) {  // (a prepared graph's plan checked no keys)
+        KB_TRY(check_small_labels(ctx, n, init_key));
+        KB_TRY(read_counters(ctx));
+        R.key_checked = init_key;
+        R.key_dense = ctx->h_ctr->dense_bad == 0;
+    }
     // with the rounds of a small graph when the keys are known to be small
     const bool fused0 = fused && init_key && init_key == R.key_checked && R.key_dense && R.counters_fresh && R.bitmap_fresh;
     if (fused0) {
