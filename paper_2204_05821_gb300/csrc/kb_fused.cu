@@ -134,7 +134,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
                 if (!(e & kSingleBit)) atomicOr(&p.shared[m >> 5], 1u << (m & 31));
             }
         } else if (frozen * 4 > n) {
-            if ((n - frozen) * 64 < n) p.warp_verts *= 4;  // few vertices refine: longer tasks
+            if ((n - frozen) * 64 < n) p.warp_verts = sparse_task(p.warp_verts);  // few vertices refine
             small_body<false, true, true>(p, sm.compact, my_warp, warps);
         } else {
             small_body<false, false, true>(p, sm.small, my_warp, warps);

@@ -49,7 +49,18 @@ constexpr int64_t kResidentWarps = 152 * kSmallMinBlocks * kSmallWarps;  // warp
 constexpr int kMapBits = 10;
 constexpr int kMapCap = 1 << kMapBits;
 constexpr uint64_t kMapEmpty = ~0ull;
+// Longest task: packed windows keep a vertex's place in its task in 16 bits.
+constexpr int32_t kMaxTaskVerts = 65536;
 constexpr uint64_t kEmptyKeyBit = 1ull << 63;  // map key of an empty-signature join: bit 63 | own
+
+// Task of a round in which few vertices refine: four times as long, so that fewer
+// warps walk windows that are nearly empty, up to the 4096 vertices that
+// launch_small_round takes there; a caller's longer task stays as it is.
+__host__ __device__ constexpr int32_t sparse_task(int32_t verts) {
+    return verts >= 4096 ? verts : (verts * 4 < 4096 ? verts * 4 : 4096);
+}
+static_assert(sparse_task(kMaxTaskVerts) == kMaxTaskVerts && sparse_task(4095) == 4096 && sparse_task(32) == 128,
+              "a task never grows past what its windows can address");
 
 struct JoinMap {
     uint64_t key[kMapCap];
@@ -138,7 +149,7 @@ __device__ __forceinline__ void small_body(const RoundParams& p, SmallSmem<kLeve
         // vertices take no lane.  The next window is picked, and its row offsets
         // and own blocks loaded, before the current one works.
         constexpr int kLook = kCompact ? 128 : 32;
-        const int span = (int)(ve - vb);  // task vertices (at most 65536)
+        const int span = (int)(ve - vb);  // task vertices (at most kMaxTaskVerts)
         int pf_off = -1;  // next window: this lane's vertex as an offset from vb (-1: none)
         int pf_next = 0;  // and where the window after it starts
         int64_t pf_a = 0;
