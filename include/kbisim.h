@@ -198,6 +198,16 @@ kb_status kb_workspace_size(kb_context* ctx, const kb_graph* g, const kb_options
  * library-allocated scratch.  Calls fail with KB_ERR_OOM if it is too small. */
 kb_status kb_set_workspace(kb_context* ctx, void* device_ptr, size_t bytes);
 
+/* Limits of the kernel that runs all rounds of a small graph (at most 2^21
+ * vertices and processed edges) in one launch, whose CTAs wait for one another
+ * between the passes of a round.
+ *   max_ctas   largest grid; -1: what the device holds at once (the default);
+ *              0: never use it (one kernel per pass)
+ *   max_polls  how often a CTA looks for the others before it gives up; 0: the
+ *              default, some seconds.  The call then returns KB_ERR_TIMEOUT.
+ * Results never depend on either. */
+kb_status kb_set_round_kernel(kb_context* ctx, int32_t max_ctas, int32_t max_polls);
+
 /* Refine levels 0..k.
  *   levels           DEVICE int32[(k+1)*n]; row i (levels + i*n) receives the
  *                    canonical block id of every vertex at level i

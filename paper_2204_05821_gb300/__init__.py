@@ -250,6 +250,11 @@ class Context:
         self._check(self._lib.kb_set_workspace(self._h, ctypes.c_void_p(self._ws.data_ptr()),
                                                self._ws.numel()))
 
+    def set_round_kernel(self, max_ctas: int = -1, max_polls: int = 0):
+        """``kb_set_round_kernel``: limits of the kernel that runs all rounds of
+        a small graph (0 CTAs: never use it)."""
+        self._check(self._lib.kb_set_round_kernel(self._h, int(max_ctas), int(max_polls)))
+
     # -- prepared graphs
     def prepare(self, graph: DeviceGraph, options: Options = None) -> "PreparedGraph":
         """``kb_graph_prepare``: the per-graph structures of every refinement

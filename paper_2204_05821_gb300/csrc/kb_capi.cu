@@ -32,7 +32,9 @@ struct kb_context {
     kb::Counters* d_ctr = nullptr;
     kb::Counters* h_ctr = nullptr;  // pinned: the last counters read, and a slot per round in flight (queue_counters)
     cudaEvent_t slot_ev[4] = {};
-    int fused_ctas = 0;  // largest grid of the fused kernel (launch_fused_rounds)
+    int fused_ctas = 0;  // largest grid of the fused kernel (launch_fused_rounds),
+    int fused_most = 0;  //   as the device has it,
+    uint32_t fused_polls = kb::kFusedPolls;  // and its limit of waiting (kb_set_round_kernel)
     uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
     bool dense_empty = false;     // the minima are all ones (launch_dense_level0 leaves them so)
     char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
@@ -1153,6 +1155,7 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
     a.total_chunks = R.total_chunks;
     a.k = k;
     a.stop_stable = stop;
+    a.max_polls = ctx->fused_polls;
     if (R.p.n_hubs) {
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_sets, 0xff, R.set_bytes, s));
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_acc, 0, sizeof(uint64_t) * (size_t)R.p.n_hubs, s));
@@ -1175,9 +1178,9 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
         a.key0 = first == i_start + 1 ? key0 : nullptr;
         a.lmin = ctx->d_dense;
         KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, first > i_start + 1, s));
-        if (a.key0) ctx->dense_empty = true;
         KB_TRY(read_counters(ctx));
         KB_TRY(device_error(ctx));
+        if (a.key0) ctx->dense_empty = true;  // (a kernel that gave up may have left minima)
         const Counters& hc = *ctx->h_ctr;
         if (hc.last_round < first || hc.last_round > a.last)
             return fail(ctx, KB_ERR_DEVICE_CHECK, "the fused rounds ended at %d of %d..%d", hc.last_round, first, a.last);
@@ -2628,7 +2631,7 @@ kb_status kb_create(kb_context** out, int device, void* stream) {
     for (auto& e : ctx->ev) cudaEventCreate(&e);
     for (auto& e : ctx->slot_ev) cudaEventCreateWithFlags(&e, cudaEventDisableTiming);
     kb::set_medium_kernel_attributes();
-    ctx->fused_ctas = kb::fused_max_ctas();
+    ctx->fused_ctas = ctx->fused_most = kb::fused_max_ctas();
     cudaGetLastError();
     *out = ctx;
     return KB_OK;
@@ -2686,6 +2689,14 @@ kb_status kb_set_workspace(kb_context* ctx, void* ptr, size_t bytes) {
     if (!ctx) return KB_ERR_INVALID_ARG;
     ctx->user_ws = ptr;
     ctx->user_ws_bytes = ptr ? bytes : 0;
+    return KB_OK;
+}
+
+kb_status kb_set_round_kernel(kb_context* ctx, int32_t max_ctas, int32_t max_polls) {
+    if (!ctx) return KB_ERR_INVALID_ARG;
+    if (max_ctas < -1 || max_polls < 0) return fail(ctx, KB_ERR_INVALID_ARG, "bad limits of the round kernel");
+    ctx->fused_ctas = max_ctas < 0 || ctx->fused_most == 0 ? ctx->fused_most : max_ctas;
+    ctx->fused_polls = max_polls > 0 ? (uint32_t)max_polls : (uint32_t)kb::kFusedPolls;
     return KB_OK;
 }
 

@@ -42,7 +42,6 @@ static_assert(kFusedThreads == kSmallThreads && kFusedWarps == kMidWarps && kFus
 // instead of exchanging sums across a barrier (hierarchy of 3 x 10^5 vertices:
 // 847 against 893 us with 9,376 words).
 constexpr int64_t kDirectWords = 16384;
-constexpr uint32_t kWaitLimit = 1u << 24;  // polls, each a round trip to the L2: some ten seconds
 
 union FusedSmem {
     SmallSmem<false, false> small;
@@ -61,7 +60,9 @@ union FusedSmem {
 };
 
 // Wait for the whole grid; false when the limit ran out (or did for another CTA).
-__device__ __forceinline__ bool grid_barrier(Counters* ctr, uint32_t& target) {
+// A CTA passes only when all of them arrived, so what it reads next is whole
+// even if others gave up meanwhile; it ends at the next barrier.
+__device__ __forceinline__ bool grid_barrier(Counters* ctr, uint32_t& target, uint32_t max_polls) {
     target += gridDim.x;
     __shared__ int s_go;
     __syncthreads();
@@ -70,10 +71,10 @@ __device__ __forceinline__ bool grid_barrier(Counters* ctr, uint32_t& target) {
         atomicAdd(&ctr->arrived, 1u);
         volatile uint32_t* arrived = &ctr->arrived;
         uint32_t polls = 0;
-        while ((int32_t)(*arrived - target) < 0 && ++polls < kWaitLimit) {
+        while ((int32_t)(*arrived - target) < 0 && ++polls < max_polls) {
         }
-        s_go = polls < kWaitLimit && !(*(volatile int32_t*)&ctr->err & kErrWait);
-        if (polls >= kWaitLimit) atomicOr(&ctr->err, kErrWait);
+        s_go = polls < max_polls && !(*(volatile int32_t*)&ctr->err & kErrWait);
+        if (polls >= max_polls) atomicOr(&ctr->err, kErrWait);
         __threadfence();
     }
     __syncthreads();
@@ -167,13 +168,13 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
                 all_chunks<1024>(p, sm.chunk1024, a.total_chunks);
             else
                 all_chunks<kDefaultHubChunk>(p, sm.chunk512, a.total_chunks);
-            if (!grid_barrier(ctr, target)) return;
+            if (!grid_barrier(ctr, target, a.max_polls)) return;
             for (int h = blockIdx.x; h < p.n_hubs; h += gridDim.x) {
                 __syncthreads();
                 hub_final(p, sm.hub, h);
             }
         }
-        if (!grid_barrier(ctr, target)) return;
+        if (!grid_barrier(ctr, target, a.max_polls)) return;
 
         // ---- ranks of the block minima: a CTA per run of words
         const int64_t run = ((nw + gridDim.x - 1) / gridDim.x + 3) & ~(int64_t)3;
@@ -191,7 +192,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             for (int64_t w = wa + tid; w < wb; w += kFusedThreads) own += __popc(p.bitmap[w]);
             own = cta_sum(own, sm.pass.warp);
             if (tid == 0) a.sums[blockIdx.x] = own;
-            if (!grid_barrier(ctr, target)) return;
+            if (!grid_barrier(ctr, target, a.max_polls)) return;
             for (int b = tid; b < (int)blockIdx.x; b += kFusedThreads) before += a.sums[b];
         }
         uint32_t base = cta_sum(before, sm.pass.warp);
@@ -226,7 +227,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             ctr->moved = 0;
             ctr->most_pairs = 0;
         }
-        if (!grid_barrier(ctr, target)) return;
+        if (!grid_barrier(ctr, target, a.max_polls)) return;
 
         // ---- ids; under early stop a round that kept the count is the last one
         const bool stable = a.stop_stable && !level0 &&
@@ -272,7 +273,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             }
         }
         if (i == a.k) return;
-        if (!grid_barrier(ctr, target)) return;
+        if (!grid_barrier(ctr, target, a.max_polls)) return;
 
         // ---- frozen blocks of the next round
         const int per_warp = (int)min((int64_t)32, max((int64_t)1, nw / warps));
@@ -280,7 +281,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
             for (int64_t w0 = my_warp * per_warp; w0 < nw; w0 += warps * per_warp)
                 dirty_blocks(p, a.f.edgeless, p.moved, kMaxHubThreshold, const_cast<uint32_t*>(a.f.mark), per_warp, nullptr,
                              w0);
-            if (!grid_barrier(ctr, target)) return;
+            if (!grid_barrier(ctr, target, a.max_polls)) return;
         }
         FreezePass f = a.f;
         f.per_warp = per_warp;
@@ -298,7 +299,7 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
         __syncthreads();
         add_frozen(ctr, sm.pass.on);
         if (i == a.last) return;
-        if (!grid_barrier(ctr, target)) return;
+        if (!grid_barrier(ctr, target, a.max_polls)) return;
     }
 }
 

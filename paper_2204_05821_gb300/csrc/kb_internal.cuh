@@ -43,6 +43,9 @@ enum : int32_t { kErrTableFull = 1, kErrInvalid = 2, kErrStage = 4, kErrHubSet =
 
 // Rounds that one launch of the fused kernel runs at most.
 constexpr int kFusedRounds = 64;
+// How often one of its CTAs looks for the others before it gives up (each look a
+// round trip to the L2, some seconds in all).
+constexpr int32_t kFusedPolls = 1 << 24;
 
 struct Counters {
     int32_t err;
@@ -366,6 +369,7 @@ struct FusedRounds {
     uint32_t* lmin = nullptr;
     bool stop_stable = false;    // stop at a round that keeps the count; its row and all up to k are copied
     bool all_on = false;
+    uint32_t max_polls = kFusedPolls;
 };
 // CTAs that a cooperative launch may have (0: not available).
 int fused_max_ctas();
