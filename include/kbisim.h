@@ -47,7 +47,8 @@ typedef enum {
                                  retried.  The table holds n / load_factor slots, so this needs a
                                  clustered hash, e.g. hash_mode 1 on a previous block with millions
                                  of distinct signatures */
-    KB_ERR_TIMEOUT = 4,       /* a bounded device wait gave up */
+    KB_ERR_TIMEOUT = 4,       /* a bounded device wait gave up (no call returns it: the one kernel that
+                                 waits is replaced by kernels that do not, kb_set_round_kernel) */
     KB_ERR_CUDA = 5,          /* a CUDA runtime call failed */
     KB_ERR_DEVICE_CHECK = 6,  /* a device-side consistency check failed */
     KB_ERR_NOT_FOUND = 7      /* unknown server ticket */
@@ -204,9 +205,13 @@ kb_status kb_set_workspace(kb_context* ctx, void* device_ptr, size_t bytes);
  *   max_ctas   largest grid; -1: what the device holds at once (the default);
  *              0: never use it (one kernel per pass)
  *   max_polls  how often a CTA looks for the others before it gives up; 0: the
- *              default, some seconds.  The call then returns KB_ERR_TIMEOUT.
- * Results never depend on either. */
+ *              default, some seconds
+ * When it gives up, or the device refuses the launch, the call starts again with
+ * one kernel per pass.  Results never depend on either limit. */
 kb_status kb_set_round_kernel(kb_context* ctx, int32_t max_ctas, int32_t max_polls);
+/* How often that kernel was launched on this context, was refused by the device,
+ * and gave up (HOST, each may be NULL). */
+kb_status kb_get_round_kernel(const kb_context* ctx, int64_t* launches, int64_t* refused, int64_t* gave_up);
 
 /* Refine levels 0..k.
  *   levels           DEVICE int32[(k+1)*n]; row i (levels + i*n) receives the

@@ -255,6 +255,12 @@ class Context:
         a small graph (0 CTAs: never use it)."""
         self._check(self._lib.kb_set_round_kernel(self._h, int(max_ctas), int(max_polls)))
 
+    def round_kernel(self):
+        """``kb_get_round_kernel``: (launches, refused, gave up)."""
+        c = np.zeros(3, dtype=np.int64)
+        self._check(self._lib.kb_get_round_kernel(self._h, *[ctypes.c_void_p(c.ctypes.data + 8 * i) for i in range(3)]))
+        return tuple(int(x) for x in c)
+
     # -- prepared graphs
     def prepare(self, graph: DeviceGraph, options: Options = None) -> "PreparedGraph":
         """``kb_graph_prepare``: the per-graph structures of every refinement

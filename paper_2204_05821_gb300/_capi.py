@@ -135,6 +135,7 @@ SIGNATURES = [
                                ctypes.POINTER(ctypes.c_size_t)]),
     ("kb_set_workspace", _I, [_P, _P, ctypes.c_size_t]),
     ("kb_set_round_kernel", _I, [_P, _I32, _I32]),
+    ("kb_get_round_kernel", _I, [_P, _P, _P, _P]),
     ("kb_refine", _I, [_P, ctypes.POINTER(KbGraph), ctypes.POINTER(KbOptions), _I, _P, _P, _P]),
     ("kb_refine_from", _I, [_P, ctypes.POINTER(KbGraph), ctypes.POINTER(KbOptions), _P, _I, _I, _P, _P, _P]),
     ("kb_refine_host", _I, [_P, ctypes.POINTER(KbGraph), ctypes.POINTER(KbOptions), _I, _P, _P, _P]),

@@ -35,6 +35,7 @@ struct kb_context {
     int fused_ctas = 0;  // largest grid of the fused kernel (launch_fused_rounds),
     int fused_most = 0;  //   as the device has it,
     uint32_t fused_polls = kb::kFusedPolls;  // and its limit of waiting (kb_set_round_kernel)
+    int64_t fused_launches = 0, fused_refused = 0, fused_gave_up = 0;  // kb_get_round_kernel
     uint32_t* d_dense = nullptr;  // label minima and (minimum, id) pairs of a small-label level 0
     bool dense_empty = false;     // the minima are all ones (launch_dense_level0 leaves them so)
     char* h_hubs = nullptr;       // pinned: the first kEagerHubs hubs of a plan and their degrees
@@ -1137,10 +1138,15 @@ constexpr int64_t kFusedSize = (int64_t)1 << 21;
 // Rounds i_start + 1 .. k after the starting level is queued, kb::kFusedRounds at
 // a time.  all_on: no freeze pass ran yet.
 // key0: the starting level's keys, when it is not queued yet and they are small.
+// broken_off: -1, or when the launch was refused or a wait of the kernel ran out
+// (then nothing else is reported) the last level that it got to; the level before
+// it is whole.
 kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int i_start, int k, bool stop, bool all_on,
                        const int32_t* key0, int64_t* counts, int* levels_computed, int64_t* last_count,
-                       bool* stopped_stable) {
+                       bool* stopped_stable, int* broken_off) {
     cudaStream_t s = ctx->stream;
+    *broken_off = -1;
+    int reached = i_start;
     kb::FusedRounds a;
     a.p = R.p;
     a.p.prev = reinterpret_cast<const int32_t*>(R.p.minof);  // blocks by name
@@ -1177,9 +1183,22 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
         *R.round += (uint32_t)(a.last - first);
         a.key0 = first == i_start + 1 ? key0 : nullptr;
         a.lmin = ctx->d_dense;
-        KB_CUDA(ctx, kb::launch_fused_rounds(a, ctx->fused_ctas, first > i_start + 1, s));
+        if (kb::launch_fused_rounds(a, ctx->fused_ctas, first > i_start + 1, s) != cudaSuccess) {
+            cudaGetLastError();  // (an error of the device itself comes back with the next call)
+            ++ctx->fused_refused;
+            *broken_off = reached;
+            return KB_OK;
+        }
+        ++ctx->fused_launches;
         KB_TRY(read_counters(ctx));
-        KB_TRY(device_error(ctx));
+        reached = std::max(reached, (int)ctx->h_ctr->last_round);
+        const kb_status st = device_error(ctx);
+        if (st == KB_ERR_TIMEOUT) {
+            ++ctx->fused_gave_up;
+            *broken_off = reached;
+            return KB_OK;
+        }
+        KB_TRY(st);
         if (a.key0) ctx->dense_empty = true;  // (a kernel that gave up may have left minima)
         const Counters& hc = *ctx->h_ctr;
         if (hc.last_round < first || hc.last_round > a.last)
@@ -1207,10 +1226,11 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
 // The refinement driver shared by kb_refine, kb_refine_from and
 // kb_refine_fixpoint.  counts (k+1 entries) may be NULL in fixpoint mode;
 // *last_count receives the block count of the last level computed and
-// *stopped_stable whether a round reproduced its input partition.
+// *stopped_stable whether a round reproduced its input partition.  may_fuse:
+// small graphs may run all rounds in one kernel.
 kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt, const int32_t* start, int i_start,
                       int k, const LevelRows& rows, int64_t* counts, int* levels_computed, int64_t* last_count,
-                      bool* stopped_stable = nullptr, const kb_prepared* pg = nullptr) {
+                      bool* stopped_stable = nullptr, const kb_prepared* pg = nullptr, bool may_fuse = true) {
     const int64_t n = g->n;
     const bool fixpoint = rows.levels == nullptr;
     if (levels_computed) *levels_computed = i_start;
@@ -1246,7 +1266,7 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
     }
 
     // Small graphs run all their rounds in one kernel.
-    const bool fused = p.minof && ctx->fused_ctas > 0 && !ctx->timing && !ctx->work && !R.P.sketch && k > i_start &&
+    const bool fused = may_fuse && p.minof && ctx->fused_ctas > 0 && !ctx->timing && !ctx->work && !R.P.sketch && k > i_start &&
                        R.P.m_proc + n <= kFusedSize;
 
     // ---- the starting level
@@ -1260,7 +1280,10 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         R.key_dense = ctx->h_ctr->dense_bad == 0;
     }
     // with the rounds of a small graph when the keys are known to be small
-    const bool fused0 = fused && init_key && init_key == R.key_checked && R.key_dense && R.counters_fresh && R.bitmap_fresh;
+    // (not in place: a kernel that is broken off while it writes the level would leave neither the keys nor the level)
+    const bool in_place = init_key < row0 + n && row0 < init_key + n;
+    const bool fused0 = fused && init_key && init_key == R.key_checked && R.key_dense && R.counters_fresh &&
+                        R.bitmap_fresh && !in_place;
     if (fused0) {
         R.key_checked = nullptr;
     } else if (init_key) {
@@ -1299,9 +1322,19 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_TRY(emit_rows(ctx, rows, i_start, i_start));
     }
 
-    if (fused)
-        return fused_rounds(ctx, R, rows, i_start, k, opt->early_stop || fixpoint, !init_key,
-                            fused0 ? init_key : nullptr, counts, levels_computed, last_count, stopped_stable);
+    if (fused) {
+        int broken_off = -1;
+        KB_TRY(fused_rounds(ctx, R, rows, i_start, k, opt->early_stop || fixpoint, !init_key, fused0 ? init_key : nullptr,
+                            counts, levels_computed, last_count, stopped_stable, &broken_off));
+        if (broken_off < 0) return KB_OK;
+        // Again, one kernel per pass.  Once the starting level is written, it is
+        // started from: the caller's start may be a later row of the levels, which the
+        // rounds have overwritten (the two levels of a fixpoint are the library's own).
+        const bool level_written = rows.levels && init_key && (!fused0 || broken_off > i_start);
+        ctx->round_ms.clear();
+        return refine_core(ctx, g, opt, level_written ? row0 : start, i_start, k, rows, counts, levels_computed, last_count,
+                           stopped_stable, pg, false);
+    }
 
     // ---- refinement rounds
     R.counters_clear = !R.P.subject;
@@ -2697,6 +2730,14 @@ kb_status kb_set_round_kernel(kb_context* ctx, int32_t max_ctas, int32_t max_pol
     if (max_ctas < -1 || max_polls < 0) return fail(ctx, KB_ERR_INVALID_ARG, "bad limits of the round kernel");
     ctx->fused_ctas = max_ctas < 0 || ctx->fused_most == 0 ? ctx->fused_most : max_ctas;
     ctx->fused_polls = max_polls > 0 ? (uint32_t)max_polls : (uint32_t)kb::kFusedPolls;
+    return KB_OK;
+}
+
+kb_status kb_get_round_kernel(const kb_context* ctx, int64_t* launches, int64_t* refused, int64_t* gave_up) {
+    if (!ctx) return KB_ERR_INVALID_ARG;
+    if (launches) *launches = ctx->fused_launches;
+    if (refused) *refused = ctx->fused_refused;
+    if (gave_up) *gave_up = ctx->fused_gave_up;
     return KB_OK;
 }
 
