@@ -1162,6 +1162,7 @@ kb_status fused_rounds(kb_context* ctx, Prepared& R, const LevelRows& rows, int 
     a.k = k;
     a.stop_stable = stop;
     a.max_polls = ctx->fused_polls;
+    a.edges = R.P.m_proc;
     if (R.p.n_hubs) {
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_sets, 0xff, R.set_bytes, s));
         KB_CUDA(ctx, cudaMemsetAsync(R.p.hub_acc, 0, sizeof(uint64_t) * (size_t)R.p.n_hubs, s));

@@ -322,8 +322,12 @@ int fused_max_ctas() {
 
 cudaError_t launch_fused_rounds(const FusedRounds& a, int max_ctas, bool again, cudaStream_t s) {
     FusedRounds b = a;
-    // a CTA per 256 vertices: more only lengthen the barriers
-    const int64_t want = (a.p.n + 255) / 256;
+    // a CTA per 256 vertices or 1024 edges, whichever are more: more only lengthen
+    // the barriers, fewer leave vertices of high degree to a few CTAs (whole calls by
+    // vertices alone / with edges: 1500 vertices of 1000 edges 1567 / 149 us, 10^4 of
+    // 100 469 / 212, 300 of 500 755 / 120; Erdos-Renyi and power-law graphs of 2 x 10^4
+    // to 1.7 x 10^6 edges with 3 to 12 a vertex: within 3% or up to 12% faster)
+    const int64_t want = std::max((a.p.n + 255) / 256, (a.edges + 1023) / 1024);
     const unsigned grid = (unsigned)std::max<int64_t>(1, std::min<int64_t>(max_ctas, want));
     if (b.p.warp_verts <= 0) {  // a task per warp, at least a window
         const int64_t per = (a.p.n + (int64_t)grid * kFusedWarps - 1) / ((int64_t)grid * kFusedWarps);

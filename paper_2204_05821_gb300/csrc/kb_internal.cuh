@@ -361,6 +361,7 @@ struct FusedRounds {
     uint32_t* sums = nullptr;    // [CTAs] scratch of the rank scan
     int32_t* levels = nullptr;   // row i at levels + i * n, or
     int32_t* ping[2] = {nullptr, nullptr};  // in turn
+    int64_t edges = 0;           // of the processed CSR
     int64_t total_chunks = 0;
     int first = 0, last = 0, k = 0;  // k: the call's last level
     // the starting level too, row first - 1, when its keys are small: they and the
