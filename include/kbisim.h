@@ -514,8 +514,8 @@ const char* kb_server_last_error(const kb_server* server);
  * levels_out is HOST int32[(k+1)*n] or NULL: when given, the levels are
  * written there by the time the request finishes (no host copy inside the
  * library; rows of 512 KB and more of a pinned buffer as they become final; keep
- * it alive until kb_server_fetch).  Pinned arrays of a KB_DIR_OUT request are read
- * in place, once.  Checked here: sizes, the ends of
+ * it alive until kb_server_fetch).  Pinned arrays of a KB_DIR_OUT request that are
+ * aligned to their elements are read in place, once.  Checked here: sizes, the ends of
  * row_offsets and the arena's capacity; every offset and neighbour id is
  * checked on the device at admission, where a malformed graph fails alone
  * (state 3) without joining the shared arena.  ticket receives the request's

@@ -1986,11 +1986,15 @@ kb_status sfail(kb_server* sv, kb_status st, const char* fmt, ...) {
         }                                                                    \
     } while (0)
 
-// Whether the device reads [x, x + bytes) in place: pinned at both ends, on a
-// device that can read what may lie between them in any case.
-bool device_reads(const void* x, size_t bytes) {
-    if (!x || !bytes) return true;
-    for (const void* q : {x, (const void*)((const char*)x + bytes - 1)}) {
+// Whether the device reads `count` elements at x in place: aligned (a kernel's
+// loads are, a copy takes any address), pinned at both ends, on a device that can
+// read what may lie between them in any case.
+template <class T>
+bool device_reads(const T* x, int64_t count) {
+    if (!x || !count) return true;
+    if (reinterpret_cast<uintptr_t>(x) % sizeof(T)) return false;
+    const size_t bytes = sizeof(T) * (size_t)count;
+    for (const void* q : {(const void*)x, (const void*)((const char*)x + bytes - 1)}) {
         cudaPointerAttributes a{};
         if (cudaPointerGetAttributes(&a, q) != cudaSuccess || a.type != cudaMemoryTypeHost || a.devicePointer != q) {
             cudaGetLastError();
@@ -2004,8 +2008,7 @@ bool device_reads(const void* x, size_t bytes) {
 // their verdicts come back for all of them at once.
 bool read_in_place(const kb_server* sv, const ServeRequest& r) {
     return sv->host_access && r.n > 0 && !needs_in_csr(r.opt.direction) &&
-           device_reads(r.row, sizeof(int64_t) * (size_t)(r.n + 1)) && device_reads(r.col, sizeof(int32_t) * (size_t)r.m) &&
-           device_reads(r.lab, sizeof(int32_t) * (size_t)r.m) && device_reads(r.vlab, sizeof(int32_t) * (size_t)r.n);
+           device_reads(r.row, r.n + 1) && device_reads(r.col, r.m) && device_reads(r.lab, r.m) && device_reads(r.vlab, r.n);
 }
 
 // Append a slot for r's graph, which is placed at the arena's tail.
