@@ -180,8 +180,9 @@ __global__ void __launch_bounds__(kFusedThreads, 3) fused_rounds_kernel(const Fu
         const int64_t run = ((nw + gridDim.x - 1) / gridDim.x + 3) & ~(int64_t)3;
         const int64_t wa = min(nw, (int64_t)blockIdx.x * run), wb = min(nw, wa + run);
         uint32_t before = 0;
-        if (nw <= kDirectWords) {  // every CTA counts the words before its own
-            const uint4* words = reinterpret_cast<const uint4*>(p.bitmap);
+        const uint4* words = reinterpret_cast<const uint4*>(p.bitmap);
+        // (a caller's workspace may start at any 8 bytes)
+        if (nw <= kDirectWords && (reinterpret_cast<uintptr_t>(words) & 15) == 0) {  // every CTA counts the words before its own
 #pragma unroll 4
             for (int64_t w = tid; w < wa >> 2; w += kFusedThreads) {  // (wa is nw or a multiple of 4)
                 const uint4 x = words[w];

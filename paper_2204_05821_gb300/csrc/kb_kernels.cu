@@ -311,10 +311,15 @@ __global__ void __launch_bounds__(256) clear_hub_sets_kernel(const RoundParams p
     if (!__syncthreads_or(any)) return;
     ulonglong2* sets2 = reinterpret_cast<ulonglong2*>(p.hub_sets);
     const ulonglong2 e = make_ulonglong2(kEmptyPair, kEmptyPair);
+    const bool pairs = (reinterpret_cast<uintptr_t>(sets2) & 15) == 0;  // (a caller's workspace may start at any 8 bytes)
     int j = 0;
     for (int64_t s = t0 + 2 * threadIdx.x; s < t1; s += 2 * blockDim.x) {
         while (j < kClearHubs - 1 && s_end[j] <= s) ++j;
-        if (s_ref[j]) sets2[s >> 1] = e;
+        if (!s_ref[j]) continue;
+        if (pairs)
+            sets2[s >> 1] = e;
+        else
+            p.hub_sets[s] = p.hub_sets[s + 1] = kEmptyPair;
     }
 }
 
