@@ -235,8 +235,13 @@ void layout_round(Plan& P) {
     auto takeg = [&](size_t bytes) { size_t o = goff; goff += align_up(bytes); return o; };
     const int64_t nw = (P.n >> 5) + 1;
     const size_t H = P.n_hubs;
-    P.o_mid = takeg(sizeof(int32_t) * (size_t)P.n_mid);
-    P.o_med = takeg(sizeof(int32_t) * (size_t)P.n_med);
+    // The mid and medium vertices, one list behind the other.  A prepared graph's are
+    // as long as they are; a call's have room for as many as n and the edges allow, so
+    // that a workspace of the queried size serves every graph of that size without
+    // hubs, also one that was changed in place since the query.
+    const int64_t most = P.m_proc / (std::min(P.small_max, kb::kSmallDegree) + 1);
+    P.o_mid = takeg(sizeof(int32_t) * (size_t)(P.graph_ext ? P.n_mid + P.n_med : std::min(P.n, most)));
+    P.o_med = P.o_mid + sizeof(int32_t) * (size_t)P.n_mid;
     P.o_hubv = takeg(sizeof(int32_t) * H);
     P.o_chunk = takeg(sizeof(int64_t) * (H + 1));
     P.o_setoff = takeg(sizeof(int64_t) * (H + 1));
@@ -436,7 +441,7 @@ kb_status plan_classes(kb_context* ctx, Plan& P, const int64_t* row_p, kb::Check
     P.n_mid = ctx->h_ctr->n_class[0];
     P.n_med = ctx->h_ctr->n_class[1];
     const int64_t H = ctx->h_ctr->n_class[2];
-    if (H > C.hub_cap || P.n_mid + P.n_med > P.n) return fail(ctx, KB_ERR_DEVICE_CHECK, "degree class larger than the graph allows");
+    if (H > C.hub_cap || P.n_mid + P.n_med > std::min(P.n, P.m_proc / (bounds.small + 1))) return fail(ctx, KB_ERR_DEVICE_CHECK, "degree class larger than the graph allows");
     if (H <= 0) return KB_OK;
     P.hub_v.resize((size_t)H);
     std::vector<int64_t> deg((size_t)H);

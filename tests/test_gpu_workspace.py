@@ -43,3 +43,26 @@ def test_any_eight_byte_address(offset, n, m, hub):
                 assert res.levels_computed == lc
             torch.cuda.synchronize()
             ctx._check(ctx._lib.kb_set_workspace(ctx._h, None, 0))
+
+
+@pytest.mark.parametrize("d", [kb.DIR_OUT, kb.DIR_IN, kb.DIR_BOTH])
+def test_graph_changed_in_place(d):
+    # the same tensors, vertices and edges; no vertex above eight edges, then some of 30 and of 200
+    n, m = 20_000, 60_000
+    few = graphgen.from_edges(n, np.arange(m) % n, (np.arange(m) * 7 + 1) % n, np.arange(m) % 3, np.arange(n) % 4)
+    deg = np.zeros(n, dtype=np.int64)
+    deg[:1_600] = 30
+    deg[1_600:1_660] = 200
+    src = np.repeat(np.arange(n), deg)
+    rng = np.random.Generator(np.random.PCG64(2))
+    ends = np.repeat(np.arange(n), deg[::-1])  # in-degrees of the same kind
+    many = graphgen.from_edges(n, src, rng.permutation(ends), rng.integers(0, 3, size=m), np.arange(n) % 4)
+    dg = kb.DeviceGraph.from_numpy(few, "cuda:0")
+    opts = kb.Options(direction=d)
+    with kb.Context(0, torch_workspace=True) as ctx:
+        for g in (few, many, few):
+            for t, a in ((dg.row_offsets, g.row_offsets), (dg.col, g.col), (dg.elabel, g.elabel), (dg.vlabel, g.vlabel)):
+                t.copy_(torch.from_numpy(a))
+            res = ctx.refine(dg, 4, opts)
+            L, C, _ = oracle.refine_graph(g, d, True, True, k=4)
+            assert np.array_equal(res.levels.cpu().numpy(), L[:5]) and np.array_equal(res.counts, C)
