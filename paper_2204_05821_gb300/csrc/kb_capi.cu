@@ -1691,6 +1691,7 @@ kb_status fixpoint_impl(kb_context* ctx, const kb_graph* g, const kb_options* op
 // key.  Stopping is decided per graph on the device, which freezes all blocks of
 // a stopped graph.  The host queues every round before it looks at the one
 // before, and stops once no graph refines.
+constexpr size_t kBatchStage = 512 << 10;  // some 30,000 graphs
 kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, int64_t G, const int32_t* k_h,
                      const kb_options* opt, int32_t* levels, int64_t* counts, int32_t* lc_out) {
     if (!g || !opt) return fail(ctx, KB_ERR_INVALID_ARG, "graph and options must not be NULL");
@@ -1732,7 +1733,7 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
     const size_t o_k = take(sizeof(int32_t) * (size_t)G);
     const size_t o_act = take((size_t)G);
     const size_t o_last = take(sizeof(int32_t) * (size_t)G);
-    const size_t up_bytes = off - o_voff;  // voff .. glast come from the host in one copy
+    const size_t up_bytes = off - o_voff;  // voff .. glast
     const size_t o_bases = take(sizeof(uint32_t) * (size_t)(G + 1) * (size_t)(kmax + 1));
     KB_TRY(ensure_buffer(ctx, &ctx->batch_ws, &ctx->batch_ws_bytes, off));
     char* b = reinterpret_cast<char*>(ctx->batch_ws);
@@ -1742,11 +1743,22 @@ kb_status batch_impl(kb_context* ctx, const kb_graph* g, const int64_t* voff_h, 
     uint8_t* gact = reinterpret_cast<uint8_t*>(b + o_act);
     int32_t* glast = reinterpret_cast<int32_t*>(b + o_last);
     uint32_t* bases = reinterpret_cast<uint32_t*>(b + o_bases);
-    std::vector<char> up(up_bytes, 0);
-    std::memcpy(up.data(), voff_h, sizeof(int64_t) * (size_t)(G + 1));
-    std::memcpy(up.data() + (o_k - o_voff), k_h, sizeof(int32_t) * (size_t)G);
-    for (int64_t j = 0; j < G; ++j) up[o_act - o_voff + (size_t)j] = k_h[j] > 0 ? 1 : 0;
-    KB_CUDA(ctx, cudaMemcpyAsync(voff, up.data(), up_bytes, cudaMemcpyHostToDevice, s));  // staged before it returns
+    // From the host in one copy (staged before it returns), but with many graphs what
+    // is here already from where it lies: filling a buffer with it took longer than the
+    // copies (5 x 10^6 graphs of two vertices: 38.4 -> 44.7 ms).
+    const bool together = up_bytes <= kBatchStage;
+    const size_t up_from = together ? o_voff : o_act, up_to = together ? o_voff + up_bytes : o_last;
+    std::vector<char> up(up_to - up_from, 0);
+    if (together) {
+        std::memcpy(up.data(), voff_h, sizeof(int64_t) * (size_t)(G + 1));
+        std::memcpy(up.data() + (o_k - o_voff), k_h, sizeof(int32_t) * (size_t)G);
+    } else {
+        KB_CUDA(ctx, cudaMemcpyAsync(voff, voff_h, sizeof(int64_t) * (size_t)(G + 1), cudaMemcpyHostToDevice, s));
+        KB_CUDA(ctx, cudaMemcpyAsync(kd, k_h, sizeof(int32_t) * (size_t)G, cudaMemcpyHostToDevice, s));
+        KB_CUDA(ctx, cudaMemsetAsync(glast, 0, sizeof(int32_t) * (size_t)G, s));
+    }
+    for (int64_t j = 0; j < G; ++j) up[o_act - up_from + (size_t)j] = k_h[j] > 0 ? 1 : 0;
+    KB_CUDA(ctx, cudaMemcpyAsync(b + up_from, up.data(), up.size(), cudaMemcpyHostToDevice, s));
     kb::launch_vertex_graph(voff, (int32_t)G, n, vgraph, s);
     p.voff = voff;
     p.n_graphs = (int32_t)G;
