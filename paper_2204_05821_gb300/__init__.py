@@ -570,10 +570,17 @@ class Server:
         return int(st.value)
 
     def fetch(self, ticket: int):
-        levels, _graph = self._meta.pop(ticket)
+        levels, _graph = self._meta[ticket]
         counts = np.zeros(levels.shape[0], dtype=np.int64)
         lc = ctypes.c_int32(0)
-        self._check(self._lib.kb_server_fetch(self._h, int(ticket), _np_ptr(levels), _np_ptr(counts), ctypes.byref(lc)))
+        st = self._lib.kb_server_fetch(self._h, int(ticket), _np_ptr(levels), _np_ptr(counts), ctypes.byref(lc))
+        if st != _capi.KB_OK:
+            error = KbError(st, self._lib.kb_server_last_error(self._h).decode())
+            # an unfinished request still reads and writes its arrays; a rejected one is forgotten
+            if self._lib.kb_server_poll(self._h, int(ticket), ctypes.byref(lc)) == _capi.KB_ERR_NOT_FOUND:
+                del self._meta[ticket]
+            raise error
+        del self._meta[ticket]
         return levels, counts, int(lc.value)
 
     def stats(self) -> dict:
