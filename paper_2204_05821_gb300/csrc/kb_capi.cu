@@ -2028,6 +2028,14 @@ bool read_in_place(const kb_server* sv, const ServeRequest& r) {
            device_reads(r.row, r.n + 1) && device_reads(r.col, r.m) && device_reads(r.lab, r.m) && device_reads(r.vlab, r.n);
 }
 
+// A request by its ticket, for the stepping thread, which does not hold sv->mu:
+// other threads submit and fetch meanwhile.  (A request stays where it is while
+// others come and go, and is only fetched once the step is through with it.)
+ServeRequest& request(kb_server* sv, int64_t ticket) {
+    std::lock_guard<std::mutex> lk(sv->mu);
+    return sv->reqs.find(ticket)->second;
+}
+
 // Append a slot for r's graph, which is placed at the arena's tail.
 void push_slot(kb_server* sv, ServeRequest& r) {
     Slot sl;
@@ -2245,7 +2253,7 @@ kb_status compact(kb_server* sv) {
         Slot ns = o;
         ns.vbase = nv;
         ns.ebase = ne;
-        sv->reqs[o.ticket].slot = (int)live.size();
+        request(sv, o.ticket).slot = (int)live.size();
         live.push_back(ns);
         nv += o.n;
         ne += o.m;
@@ -2324,7 +2332,7 @@ kb_status admit(kb_server* sv, bool* changed) {
             continue;
         }
         SV_TRY(sv, release_drained(sv, true));  // their stores may be needed
-        ServeRequest& r = sv->reqs[t];
+        ServeRequest& r = request(sv, t);
         int live = 0;
         for (const Slot& sl : sv->slots) live += sl.ticket >= 0;
         const size_t lb = level_store_bytes(sizeof(int32_t) * (size_t)r.n * (size_t)(r.k + 1));
@@ -2539,7 +2547,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         for (int j = 0; j < G; ++j) {
             const Slot& sl = sv->slots[(size_t)j];
             if (sl.ticket < 0) continue;
-            ServeRequest& r = sv->reqs[sl.ticket];
+            ServeRequest& r = request(sv, sl.ticket);
             lev[j] = r.d_levels + (size_t)r.round * (size_t)r.n;
             before[j] = r.round > 0 ? r.counts[(size_t)r.round - 1] : 0;
             up[o_act + (size_t)j] = 1;
@@ -2598,7 +2606,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         for (int j = 0; j < G; ++j) {
             const Slot sl = sv->slots[(size_t)j];
             if (sl.ticket < 0) continue;
-            ServeRequest& r = sv->reqs[sl.ticket];
+            ServeRequest& r = request(sv, sl.ticket);
             const int64_t cnt = (int64_t)(sv->gbase_host[(size_t)j + 1] - sv->gbase_host[(size_t)j]);
             r.counts[(size_t)r.round] = cnt;
             const int done_round = r.round;
@@ -2609,7 +2617,7 @@ kb_status server_step(kb_server* sv, int32_t* running, int32_t* waiting_out) {
         }
         for (int j = 0; j < G; ++j) {
             if (sv->slots[(size_t)j].ticket < 0) continue;
-            ServeRequest& r = sv->reqs[sv->slots[(size_t)j].ticket];
+            ServeRequest& r = request(sv, sv->slots[(size_t)j].ticket);
             if (r.early_rows) SV_TRY(sv, copy_rows_out(sv, r, r.round - 1));
         }
         ++sv->steps;
@@ -3323,9 +3331,7 @@ kb_status kb_server_get_stats(kb_server* sv, kb_server_stats* st) {
     st->submitted = sv->submitted;
     st->completed = sv->completed;
     st->failed = sv->failed;
-    int run = 0;
-    for (const Slot& sl : sv->slots) run += sl.ticket >= 0;
-    st->running = run;
+    for (const auto& kv : sv->reqs) st->running += kv.second.state == 1;  // (the slots are the stepping thread's)
     st->waiting = (int64_t)sv->waiting.size();
     st->steps = sv->steps;
     st->compactions = sv->compactions;
