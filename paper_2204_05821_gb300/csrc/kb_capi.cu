@@ -1312,14 +1312,8 @@ kb_status refine_core(kb_context* ctx, const kb_graph* g, const kb_options* opt,
         KB_CUDA(ctx, cudaMemsetAsync(&ctx->d_ctr->count, 1, 1, s));
         kb::launch_fill_i32(row0, n, 0, s);
         if (p.perm) kb::launch_fill_i32(p.gat, n, 0, s);
-        if (p.minof) {
-            // P_0 = {V}: one block, whose smallest member is vertex 0
-            kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.minof), n, 0, s);
-            if (!fused) {
-                KB_CUDA(ctx, cudaMemsetAsync(p.bitmap, 0, sizeof(uint32_t) * (size_t)((n >> 5) + 1), s));
-                kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.bitmap), 1, 1, s);
-            }
-        }
+        // P_0 = {V}: one block, named by vertex 0 (no freeze pass reads its bitmap)
+        if (p.minof) kb::launch_fill_i32(reinterpret_cast<int32_t*>(p.minof), n, 0, s);
     }
     if (counts) counts[i_start] = prev_count;
     if (last_count) *last_count = prev_count;
