@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(256) hub_alone_kernel(const RoundParams p) {
         while (true) {  // at most half full
             const uint32_t old = atomicCAS(&p.hub_twin[slot], 0u, (uint32_t)h + 1u);
             if (old == 0u) break;
+            __threadfence();  // the index before the hash that it leads to: a stale one would hide a twin
             if (volatile_load(&p.hub_acc[old - 1u]) == hash) {
                 other = (int)old - 1;
                 break;
