@@ -48,9 +48,9 @@ METRIC = "k-bisim edges/s per round"
 # edges).
 KERNEL_HEADERS = ("paper_2204_05821_gb300/csrc/kb_device.cuh", "paper_2204_05821_gb300/csrc/kb_internal.cuh")
 TRAFFIC_PER_ALGO_BYTE = {
-    "hub_chunk": ("paper_2204_05821_gb300/csrc/kb_hub.cu", "9b30efa5eefeb6290ffc4a2729e74bb0886ea8b2", 1.071),
-    "small": ("paper_2204_05821_gb300/csrc/kb_small.cuh", "49d18be05b7a279b849882139d236cd3339060ab", 5.624),
-    "medium": ("paper_2204_05821_gb300/csrc/kb_medium.cuh", "e6f9879934724e8969fe577671fcddd926713405", 1.953),
+    "hub_chunk": ("paper_2204_05821_gb300/csrc/kb_hub.cu", "e541b794a75b6f10f0d6cd0a28bfb160e687b71d", 1.071),
+    "small": ("paper_2204_05821_gb300/csrc/kb_small.cuh", "82a78967db22c1329134ee4e9fef6a2bec5782c9", 5.624),
+    "medium": ("paper_2204_05821_gb300/csrc/kb_medium.cuh", "20884106dc387bbdccb4a94e99da503bbee02843", 1.953),
 }
 
 

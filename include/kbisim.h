@@ -195,7 +195,8 @@ kb_status kb_workspace_size(kb_context* ctx, const kb_graph* g, const kb_options
                             size_t* bytes);
 
 /* Use caller-owned device memory as scratch (e.g. a torch tensor).  The
- * buffer must stay alive while calls that use it run.  ptr = NULL reverts to
+ * buffer starts at a multiple of eight bytes and must stay alive while calls that
+ * use it run.  ptr = NULL reverts to
  * library-allocated scratch.  Calls fail with KB_ERR_OOM if it is too small. */
 kb_status kb_set_workspace(kb_context* ctx, void* device_ptr, size_t bytes);
 

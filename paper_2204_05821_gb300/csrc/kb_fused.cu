@@ -16,12 +16,13 @@
 // 7 x 10^5 edges with host buffers: 525 -> 450 us; 3 x 10^5 vertices to their
 // fixpoint in 11 rounds: 1066 -> 847 us.  The starting level's four passes in here
 // too: 159 -> 147 us for the first (with fewer setup operations since).  Three CTAs per SM (a CTA per 256
-// vertices) as the occupancy allows: the last took 885 us with two and 1209 us
-// with one.
+// vertices or 1024 edges) as the occupancy allows: the last took 885 us with two and
+// 1209 us with one.
 //
 // The grid is launched cooperatively, so all its CTAs run at once and the
 // barrier's wait ends; it has a limit all the same, after which the kernel
-// reports an error and returns.
+// reports an error and returns, and the call runs again with one kernel per pass
+// (as it does when the device refuses the launch).
 #define KB_LEVELS_WRITTEN
 #include <cuda_runtime.h>
 
